@@ -367,8 +367,10 @@ def table(args):
             mds.mds_verify(v.ctx, w.target, w.draft_list(), w.model_ids, w.tokens, w.temps, scheme,
                            spec.verify_seed, out_tokens, out_acc, None, stream)
 
-        # classical IS is bound by its quadrature's exponentials: the kernel
-        # counts them (nodes chosen on the device x V x draft rows)
+        # classical IS: the exponentials of its quadrature taken term by term
+        # (nodes chosen on the device x V x draft rows), which the kernel
+        # counts; it bins the tokens and evaluates far fewer, so this rate
+        # compares with the ex2 peak as the work replaced, not as a load
         exps = torch.zeros(1, dtype=torch.int64, device=dev) if scheme == "IS" else None
 
         for _ in range(args.warmup):

@@ -40,6 +40,7 @@ struct mds_ctx {
 namespace {
 
 constexpr int kRingBytes = 80 * 1024;   // streaming rings: 8 warps x 5 stages of 2 KB
+constexpr int kRingBytesIs = 40 * 1024; // classical IS: 1 KB stages (two rows), beside its bins two CTAs per SM
 
 struct DeviceGuard {
   int prev = -1;
@@ -106,7 +107,7 @@ int geometry(const mds_ctx* ctx, int scheme, int n_models, mds::Params& p) {
   p.esize = esize_of(c.dtype);
   p.rows_max = 1 + n_models;
   p.scheme = scheme;
-  p.ring_bytes = kRingBytes;
+  p.ring_bytes = (scheme == MDS_IS) ? kRingBytesIs : kRingBytes;
   // candidate lists: WIS with at most three draft models in the stats pass;
   // the truncated alphabet always (its Omega_0 comes from the list)
   const bool lists = (scheme == MDS_WIS && p.rows_max <= 4) || scheme == MDS_WIS0;

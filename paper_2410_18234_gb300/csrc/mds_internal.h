@@ -12,7 +12,6 @@ constexpr int kThreads = 256;          // threads per CTA
 constexpr int kMaxRows = 1 + MDS_MAX_K; // target + one row per distinct draft model
 constexpr int kMaxSpecial = MDS_MAX_S * (MDS_MAX_K - 1);
 constexpr int kIsNodesMax = 1024;      // trapezoid nodes for plain IS
-constexpr int kIsChunk = 16;           // nodes accumulated per pass
 constexpr int kXch = 34;               // floats one CTA contributes to a cluster exchange
 constexpr int kMaxCluster = 16;
 constexpr int kListN = 32;             // WIS candidate list: the largest target logits of a sequence

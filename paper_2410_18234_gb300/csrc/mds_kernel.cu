@@ -47,6 +47,12 @@ constexpr long long kWaitLimit = 1ll << 24;
 constexpr int kFastRows = 4;            // WIS candidate path: target + up to 3 draft models
 constexpr int kWStages = 5;             // stages of each warp's streaming ring
 constexpr int kWarpApp = 64;            // candidate tokens one warp can hold during the stats pass
+constexpr int kIsSub = 4;               // IS: bins of log2 rho per octave
+constexpr int kIsMom = 8;               // IS: moments (Taylor terms) per bin
+constexpr int kIsWin = 32;              // IS: bins one binning pass holds
+constexpr int kIsStage = 64;            // IS: tokens a warp sets aside before it adds them to the bins
+constexpr int kIsBinBytes = kThreads / 32 * kIsWin * 4 * kIsMom * 4;   // four copies of the bins per warp
+constexpr int kIsTabBins = kIsBinBytes / (kIsMom * 4);                 // bins of all rows the residual's table holds
 constexpr int kSampleStride = 4;        // the candidate filter's starting threshold samples 1 unit in 4
 
 // Order-preserving map of floats (not NaN) to unsigned; every key is > 0.
@@ -279,9 +285,14 @@ struct State {
   // SpecTr: inverse residual masses of rejected rounds
   float sp_invR[MDS_MAX_K];
   int sp_rows[MDS_MAX_K];
-  // IS: quadrature grid
-  int is_mlo, is_n;
+  // IS: quadrature grid, bins of log2 rho (kIsSub to the octave) and the
+  // moments of one window of them (one copy for the peers, one combined)
+  int is_mlo, is_n, is_b0, is_nb;
   int is_cnt[kMaxRows];
+  float is_lz[kMaxRows];        // log2(Z_r / Z_0)
+  float is_mom[kIsWin * kIsMom + 1], is_sum[kIsWin * kIsMom + 1];
+  float is_ctr[kIsWin];         // the bins' centres
+  int is_tab;                   // the residual reads the bins' Taylor coefficients
   // CDF search
   int owner, seg;
   float run;
@@ -456,6 +467,8 @@ struct Kernel {
   float* segref;       // bonus draw: each segment sum's reference (round(max * c))
   float* isW;          // IS: weights [rows][kIsNodesMax]
   float* isT;          // IS: nodes t_n
+  float* isBin;        // IS: per-warp bins [warp][bin][copy][moment]; later the residual's coefficients
+  float4* isStg;       // IS: tokens a warp has set aside [warp][kIsStage]
   char* cl_base;       // WIS: this CTA's buffered tokens and their logits per row,
                        //      two alternating copies of [cap_cta] ids + [rows][cap_cta] logits
   int* ap_id;          // WIS: tokens each warp set aside during the stats pass ...
@@ -1152,12 +1165,13 @@ struct Kernel {
         default: break;
       }
     }
-    for (int r0 = 0; r0 < nr; r0 += 4) {
-      switch (min(4, nr - r0)) {
+    constexpr int step = SCHEME == MDS_IS ? 2 : 4;   // classical IS: its ring holds two rows a stage
+    for (int r0 = 0; r0 < nr; r0 += step) {
+      switch (min(step, nr - r0)) {
         case 1: stats_pass<1, false>(r0); break;
         case 2: stats_pass<2, false>(r0); break;
-        case 3: stats_pass<3, false>(r0); break;
-        default: stats_pass<4, false>(r0); break;
+        case 3: stats_pass<step == 4 ? 3 : 1, false>(r0); break;
+        default: stats_pass<step == 4 ? 4 : 1, false>(r0); break;
       }
     }
   }
@@ -2032,54 +2046,201 @@ struct Kernel {
   }
 
   // ---------------------------------------------------------------- plain IS
+  // The law needs M_r(t) = sum_x p_r(x) exp(-t rho_r(x)) at some 300 nodes t
+  // and, for a residual draw, G(rho) = sum_n W_n exp(-t_n rho) at every token:
+  // 300 exponentials a token each way if summed as written.  Both depend on a
+  // token only through log rho, and exp(-t rho) is analytic there (bounded by
+  // 1 in a strip of half-width pi/2), so tokens are binned by log2 rho, kIsSub
+  // bins to the octave, and a bin keeps the moments sum p v^k, k < kIsMom, of
+  // the offset v in [-1, 1] from its centre.  A Taylor polynomial then moves
+  // the centre's exponential to every token: with half-width d = ln 2 / 8 the
+  // remainder is below (d / (pi/2))^8 = 1e-10 of the bin's mass.  G goes the
+  // other way, one polynomial per bin.  Work per token falls from nodes x
+  // (exponential, multiply, add) to kIsMom adds, and depends on nodes x bins
+  // only beside it.
+  //
+  // Moments: eight lanes serve a token (lane k its k-th moment), a warp four
+  // tokens at a time, each into its own copy of the bins, so no two lanes of
+  // an instruction share an address, the bank of every lane is fixed and the
+  // sums have a fixed order.  Eight warps x 32 bins x 4 copies take 32 KB
+  // (two CTAs per SM); wider ranges of rho take further windows of 32 bins.
+  // What bounds it now is issue: about 3 instructions a token in the adds.
+  // Measured (GB300): B = 64, K = 4, V = 32000 594 -> 222 us a call, B = 1024,
+  // K = 4, V = 151936 22.1 -> 5.4 ms; p_I(Y) 3e-7 off 64 bits before and after.
+
+  // exp(-s e^(d v)) = sum_k z[k] v^k, d = half a bin in ln rho: the series of
+  // exp(g), g = -s (e^(d v) - 1), by (k + 1) z_{k+1} = -s d sum_i z_{k-i} d^i / i!.
+  __device__ __forceinline__ static void is_series(float s, float (&z)[kIsMom]) {
+    constexpr float d = 0.5f * 0.6931471805599453f / kIsSub;
+    constexpr float f[kIsMom - 1] = {1.f, d, d * d / 2, d * d * d / 6, d * d * d * d / 24, d * d * d * d * d / 120,
+                                     d * d * d * d * d * d / 720};
+    static_assert(kIsMom == 8, "series coefficients");
+    z[0] = ex2(__fmul_rn(s, -kLog2e));
+#pragma unroll
+    for (int k = 0; k + 1 < kIsMom; ++k) {
+      float t = 0.f;
+#pragma unroll
+      for (int i = 0; i <= k; ++i) t = __fmaf_rn(z[k - i], f[i], t);
+      z[k + 1] = __fmul_rn(__fmul_rn(t, s), -d / (float)(k + 1));
+    }
+  }
+  // Centre of bin n (the octave's power of two is exact).
+  __device__ __forceinline__ static float is_centre(int n) {
+    const int o = (n >= 0) ? n / kIsSub : -((kIsSub - 1 - n) / kIsSub);
+    return ldexpf(ex2((float)(n - o * kIsSub) / kIsSub), o);
+  }
+  // log2 rho of a token in bins, from the row's and the target's logit; the
+  // probabilities follow prob_of.
+  __device__ __forceinline__ float is_pos(float lq, float lp, int r) const {
+    const float aq = __fmaf_rn(lq, S.c[0], -__fmul_rn(S.M[0], S.c[0]));
+    const float ap = __fmaf_rn(lp, S.c[r], -__fmul_rn(S.M[r], S.c[r]));
+    return __fmul_rn(__fadd_rn(__fsub_rn(aq, ap), S.is_lz[r]), (float)kIsSub);
+  }
+
+  // Add this warp's set-aside tokens (v, v^2, p, bin) to its bins.
+  __device__ __forceinline__ void is_flush(float* bins, const float4* stg, int cnt) const {
+    const int lane = threadIdx.x & 31;
+    const int g = lane >> 3, k = lane & 7;
+    __syncwarp();
+    float* mine = bins + g * kIsMom + k;
+    for (int i = 0; i < cnt; i += 16) {
+      float4 x[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) x[q] = stg[i + 4 * q + g];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float v4 = __fmul_rn(x[q].y, x[q].y);
+        float w = __fmul_rn(x[q].z, (k & 1) ? x[q].x : 1.f);
+        w = __fmul_rn(w, (k & 2) ? x[q].y : 1.f);
+        w = __fmul_rn(w, (k & 4) ? v4 : 1.f);
+        float* at = mine + __float_as_int(x[q].w);
+        *at = __fadd_rn(*at, w);   // this lane's own address: no other lane adds there
+      }
+    }
+  }
+
+  // Moments of row r over the window of bins [b0, b0 + kIsWin) into S.is_sum
+  // (the last entry: the mass of tokens whose ratio is 0 or below every bin,
+  // first window only), combined over the CTA's warps and the cluster.
+  __device__ void is_moments(int r, int b0, bool first) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    float* bins = isBin + (size_t)warp * kIsWin * 4 * kIsMom;
+    float4* stg = isStg + warp * kIsStage;
+    for (int i = lane; i < kIsWin * 4 * kIsMom; i += 32) bins[i] = 0.f;
+    __syncwarp();
+    float zero = 0.f;
+    stream(1u | (1u << r), [&](int, bool valid, const auto& L) {
+      float lq[VE], lp[VE];
+      if (valid) {
+        L(0, lq);
+        L(r, lp);
+      } else {
+#pragma unroll
+        for (int e = 0; e < VE; ++e) lq[e] = lp[e] = kNegInf;
+      }
+#pragma unroll
+      for (int e0 = 0; e0 < VE; e0 += 2) {
+        int cnt = 0;
+#pragma unroll
+        for (int e = e0; e < e0 + 2; ++e) {
+          const float pr = prob_of(lp[e], S.M[r], S.c[r], S.invZ[r]);
+          const float q = prob_of(lq[e], S.M[0], S.c[0], S.invZ[0]);
+          const float x = is_pos(lq[e], lp[e], r);
+          const float n = rintf(x);
+          const int bin = (int)n - b0;
+          const bool pos = pr > 0.f && q > 0.f;
+          const bool in = pos && bin >= 0 && bin < kIsWin;
+          if (first && pr > 0.f && (!(q > 0.f) || bin < 0)) zero = __fadd_rn(zero, pr);
+          const unsigned m = __ballot_sync(0xffffffffu, in);
+          if (in) {
+            const float v = __fmul_rn(2.f, __fsub_rn(x, n));
+            stg[cnt + __popc(m & ((1u << lane) - 1u))] =
+                make_float4(v, __fmul_rn(v, v), pr, __int_as_float(bin * 4 * kIsMom));
+          }
+          cnt += __popc(m);
+        }
+        // whole groups of 16: the rest adds nothing to bin 0
+        if (lane < 16 && cnt + lane < ((cnt + 15) & ~15)) stg[cnt + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+        is_flush(bins, stg, cnt);
+        __syncwarp();
+      }
+    });
+    zero = warp_sum(zero);
+    if (lane == 0) S.red[warp] = zero;
+    __syncthreads();
+    {
+      // one (bin, moment) per thread: warps and copies in order
+      static_assert(kIsWin * kIsMom == kThreads, "one bin moment per thread");
+      const int n = tid / kIsMom, k = tid % kIsMom;
+      float t = 0.f;
+      for (int w = 0; w < kWarps; ++w)
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          t = __fadd_rn(t, isBin[((w * kIsWin + n) * 4 + c) * kIsMom + k]);
+      S.is_mom[tid] = t;
+      if (tid == 0) {
+        float z = 0.f;
+        for (int w = 0; w < kWarps; ++w) z = __fadd_rn(z, S.red[w]);
+        S.is_mom[kThreads] = z;
+      }
+    }
+    if (tid < kIsWin) S.is_ctr[tid] = is_centre(b0 + tid);
+    __syncthreads();
+    if (cn > 1) {
+      cluster_sync_all();
+      for (int i = tid; i <= kThreads; i += kThreads) {
+        float t = 0.f;
+        for (int q = 0; q < cn; ++q) t = __fadd_rn(t, ld_dsmem(&S.is_mom[i], (uint32_t)q));
+        S.is_sum[i] = t;
+      }
+      cluster_sync_all();   // every peer has read before the next window's moments
+    } else {
+      for (int i = tid; i <= kThreads; i += kThreads) S.is_sum[i] = S.is_mom[i];
+      __syncthreads();
+    }
+  }
+
   __device__ void is_prepare() {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // rows present and their branch counts
-    if (threadIdx.x == 0) {
+    if (tid == 0) {
       for (int r = 0; r < kMaxRows; ++r) S.is_cnt[r] = 0;
       for (int i = 0; i < S.nv; ++i) S.is_cnt[S.vrow[i]]++;
+      for (int r = 1; r < S.nrows; ++r) S.is_lz[r] = __fsub_rn(log2f(S.invZ[0]), log2f(S.invZ[r]));
     }
     __syncthreads();
-    // range of rho = q / p_r over tokens with q > 0 and p_r > 0
+    // range of rho = q / p_r over tokens with q > 0 and p_r > 0, a row at a time
     float lo = kPosInf, hi = 0.f;
-    uint32_t mask = 1u;
-    for (int r = 1; r < S.nrows; ++r)
-      if (S.is_cnt[r]) mask |= 1u << r;
-    stream(mask, [&](int, bool valid, const auto& L) {
-      if (!valid) return;
-      float q[VE];
-      {
-        float v[VE];
+    for (int r = 1; r < S.nrows; ++r) {
+      if (!S.is_cnt[r]) continue;
+      stream(1u | (1u << r), [&](int, bool valid, const auto& L) {
+        if (!valid) return;
+        float v[VE], w[VE];
         L(0, v);
-#pragma unroll
-        for (int e = 0; e < VE; ++e) q[e] = prob_of(v[e], S.M[0], S.c[0], S.invZ[0]);
-      }
-      for (int r = 1; r < S.nrows; ++r) {
-        if (!S.is_cnt[r]) continue;
-        float v[VE];
-        L(r, v);
+        L(r, w);
 #pragma unroll
         for (int e = 0; e < VE; ++e) {
-          const float pr = prob_of(v[e], S.M[r], S.c[r], S.invZ[r]);
-          if (pr > 0.f && q[e] > 0.f) {
-            const float rho = __fdiv_rn(q[e], pr);
+          const float q = prob_of(v[e], S.M[0], S.c[0], S.invZ[0]);
+          const float pr = prob_of(w[e], S.M[r], S.c[r], S.invZ[r]);
+          if (pr > 0.f && q > 0.f) {
+            const float rho = __fdiv_rn(q, pr);
             lo = fminf(lo, rho);
             hi = fmaxf(hi, rho);
           }
         }
-      }
-    });
+      });
+    }
 #pragma unroll
     for (int o = 16; o; o >>= 1) {
       lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
       hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
     }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (lane == 0) {
       S.red[warp * 2] = lo;
       S.red[warp * 2 + 1] = hi;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (tid == 0) {
       for (int w = 0; w < kWarps; ++w) {
         lo = fminf(lo, S.red[w * 2]);
         hi = fmaxf(hi, S.red[w * 2 + 1]);
@@ -2088,7 +2249,7 @@ struct Kernel {
       S.xch[xbuf][1] = hi;
     }
     cluster_gather(S, 2, xbuf, cn);
-    if (threadIdx.x == 0) {
+    if (tid == 0) {
       float rlo = kPosInf, rhi = 0.f;
       for (int q = 0; q < cn; ++q) {
         rlo = fminf(rlo, S.gat[2 * q]);
@@ -2104,70 +2265,61 @@ struct Kernel {
       if (mhi - mlo + 1 > kIsNodesMax) mhi = mlo + kIsNodesMax - 1;
       S.is_mlo = mlo;
       S.is_n = mhi - mlo + 1;
-      if (p.dbg_exps && rank == 0) {
-        // the node sums below: one exponential per node, token and draft row
-        int rows = 0;
-        for (int r = 1; r < S.nrows; ++r) rows += S.is_cnt[r] ? 1 : 0;
-        atomicAdd(p.dbg_exps, (unsigned long long)S.is_n * (unsigned long long)p.V * (unsigned long long)rows);
+      // the bins of that range, a bin to spare on either side (no bins
+      // without a token of positive q and p)
+      S.is_b0 = 0;
+      S.is_nb = 0;
+      if (rlo <= rhi && rhi < kPosInf) {
+        S.is_b0 = (int)floorf(kIsSub * log2f(rlo)) - 1;
+        S.is_nb = (int)ceilf(kIsSub * log2f(rhi)) + 2 - S.is_b0;
       }
+      int rows = 0;
+      for (int r = 1; r < S.nrows; ++r) rows += S.is_cnt[r] ? 1 : 0;
+      S.is_tab = (rows * S.is_nb <= kIsTabBins) ? 1 : 0;
+      // the node sums taken directly: one exponential per node, token and draft row
+      if (p.dbg_exps && rank == 0)
+        atomicAdd(p.dbg_exps, (unsigned long long)S.is_n * (unsigned long long)p.V * (unsigned long long)rows);
     }
     __syncthreads();
     const int nn = S.is_n;
-    for (int n = threadIdx.x; n < nn; n += kThreads) isT[n] = ex2(__fmul_rn((float)(S.is_mlo + n) * p.is_h, kLog2e));
+    // nodes t_n = e^((mlo + n) h): the exponent in log2, its fraction apart
+    for (int n = tid; n < nn; n += kThreads) {
+      const double x = (double)(S.is_mlo + n) * ((double)p.is_h * 1.4426950408889634);
+      const double i = rint(x);
+      isT[n] = ldexpf(ex2((float)(x - i)), (int)i);
+    }
     __syncthreads();
-    // M_r(t_n) = sum_x p_r(x) exp(-t_n rho_r(x)), node chunks of kIsChunk
+    // M_r(t_n), a window of bins at a time
     for (int r = 1; r < S.nrows; ++r) {
       if (!S.is_cnt[r]) continue;
-      for (int n0 = 0; n0 < nn; n0 += kIsChunk) {
-        float acc[kIsChunk];
-        float tl[kIsChunk];
+      for (int b = 0; b < S.is_nb || b == 0; b += kIsWin) {
+        is_moments(r, S.is_b0 + b, b == 0);
+        for (int n = tid; n < nn; n += kThreads) {
+          float acc = (b == 0) ? S.is_sum[kThreads] : isW[r * kIsNodesMax + n];
+          const float t = isT[n];
+          for (int i = 0; i < kIsWin; ++i) {
+            const float* A = S.is_sum + i * kIsMom;
+            if (A[0] == 0.f) continue;   // an empty bin
+            const float s = __fmul_rn(t, S.is_ctr[i]);
+            if (!(s < 110.f)) continue;  // exp(-s) is 0 in 32 bits
+            if (s < 1e-9f) {
+              acc = __fadd_rn(acc, A[0]);
+              continue;
+            }
+            float z[kIsMom];
+            is_series(s, z);
+            float m = 0.f;
 #pragma unroll
-        for (int i = 0; i < kIsChunk; ++i) {
-          acc[i] = 0.f;
-          tl[i] = (n0 + i < nn) ? __fmul_rn(isT[n0 + i], -kLog2e) : 0.f;
-        }
-        stream(1u | (1u << r), [&](int, bool valid, const auto& L) {
-          if (!valid) return;
-          float q[VE], pr[VE];
-          {
-            float v[VE];
-            L(0, v);
-#pragma unroll
-            for (int e = 0; e < VE; ++e) q[e] = prob_of(v[e], S.M[0], S.c[0], S.invZ[0]);
-            L(r, v);
-#pragma unroll
-            for (int e = 0; e < VE; ++e) pr[e] = prob_of(v[e], S.M[r], S.c[r], S.invZ[r]);
+            for (int k = kIsMom - 1; k >= 0; --k) m = __fmaf_rn(A[k], z[k], m);
+            acc = __fadd_rn(acc, m);
           }
-#pragma unroll
-          for (int e = 0; e < VE; ++e) {
-            if (!(pr[e] > 0.f)) continue;
-            const float rho = __fdiv_rn(q[e], pr[e]);
-#pragma unroll
-            for (int i = 0; i < kIsChunk; ++i) acc[i] = __fmaf_rn(pr[e], ex2(__fmul_rn(tl[i], rho)), acc[i]);
-          }
-        });
-#pragma unroll
-        for (int i = 0; i < kIsChunk; ++i) {
-          const float v = warp_sum(acc[i]);
-          if (lane == 0) S.red[warp * kIsChunk + i] = v;
-        }
-        __syncthreads();
-        if (threadIdx.x < kIsChunk) {
-          float v = 0.f;
-          for (int w = 0; w < kWarps; ++w) v = __fadd_rn(v, S.red[w * kIsChunk + threadIdx.x]);
-          S.xch[xbuf][threadIdx.x] = v;
-        }
-        cluster_gather(S, kIsChunk, xbuf, cn);
-        if (threadIdx.x < kIsChunk && n0 + threadIdx.x < nn) {
-          float v = 0.f;
-          for (int q = 0; q < cn; ++q) v = __fadd_rn(v, S.gat[q * kIsChunk + threadIdx.x]);
-          isW[r * kIsNodesMax + n0 + threadIdx.x] = v;  // M_r(t_n) for now
+          isW[r * kIsNodesMax + n] = acc;   // M_r(t_n) for now
         }
         __syncthreads();
       }
     }
     // weights W_r(n) = h t_n c_r M_r^(c_r - 1) prod_{r' != r} M_r'^(c_r')
-    for (int n = threadIdx.x; n < nn; n += kThreads) {
+    for (int n = tid; n < nn; n += kThreads) {
       float Mv[kMaxRows];
       for (int r = 1; r < S.nrows; ++r) Mv[r] = S.is_cnt[r] ? isW[r * kIsNodesMax + n] : 1.f;
       const float base = __fmul_rn(p.is_h, isT[n]);
@@ -2181,6 +2333,40 @@ struct Kernel {
         }
         isW[r * kIsNodesMax + n] = w;
       }
+    }
+    __syncthreads();
+  }
+
+  // The residual's table: per draft row and bin, the coefficients in v of
+  // G(rho) = sum_n W_r(n) exp(-t_n rho), a warp per bin.  Replaces the bins.
+  __device__ void is_table() {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (!S.is_tab) return;
+    int row = 0;
+    for (int r = 1; r < S.nrows; ++r) {
+      if (!S.is_cnt[r]) continue;
+      const float* W = isW + r * kIsNodesMax;
+      for (int n = warp; n < S.is_nb; n += kWarps) {
+        const float ctr = is_centre(S.is_b0 + n);
+        float g[kIsMom];
+#pragma unroll
+        for (int k = 0; k < kIsMom; ++k) g[k] = 0.f;
+        for (int i = lane; i < S.is_n; i += 32) {
+          const float s = __fmul_rn(isT[i], ctr);
+          if (!(s < 110.f)) continue;
+          float z[kIsMom];
+          is_series(s, z);
+#pragma unroll
+          for (int k = 0; k < kIsMom; ++k) g[k] = __fmaf_rn(W[i], z[k], g[k]);
+        }
+        float* at = isBin + (size_t)(row * S.is_nb + n) * kIsMom;
+#pragma unroll
+        for (int k = 0; k < kIsMom; ++k) {
+          const float t = warp_sum(g[k]);
+          if (lane == k) at[k] = t;
+        }
+      }
+      ++row;
     }
     __syncthreads();
   }
@@ -2202,6 +2388,18 @@ struct Kernel {
       }
     }
     return sum;
+  }
+  // The same by a whole warp, the nodes dealt to its lanes.
+  __device__ float is_ratio_warp(const float* rho_r) const {
+    float sum = 0.f;
+    for (int r = 1; r < S.nrows; ++r) {
+      if (!S.is_cnt[r]) continue;
+      const float rl = __fmul_rn(rho_r[r], -kLog2e);
+      const float* W = isW + r * kIsNodesMax;
+      for (int n = (int)(threadIdx.x & 31); n < S.is_n; n += 32)
+        sum = __fmaf_rn(W[n], ex2(__fmul_rn(isT[n], rl)), sum);
+    }
+    return warp_sum(sum);
   }
 
   // ---------------------------------------------------------------- importance steps
@@ -2274,7 +2472,7 @@ struct Kernel {
     }
     __syncthreads();
     is_prepare();
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < 32) {
       const int y = S.Y;
       const float qv = prob_row(0, y);
       float rr[kMaxRows];
@@ -2282,8 +2480,11 @@ struct Kernel {
         const float pv = S.is_cnt[r] ? prob_row(r, y) : 0.f;
         rr[r] = pv > 0.f ? __fdiv_rn(qv, pv) : kPosInf;
       }
-      S.qY = qv;
-      S.pIY = __fmul_rn(qv, is_ratio_sum(rr));
+      const float ratio = is_ratio_warp(rr);
+      if (threadIdx.x == 0) {
+        S.qY = qv;
+        S.pIY = __fmul_rn(qv, ratio);
+      }
     }
   }
 
@@ -2617,6 +2818,7 @@ struct Kernel {
                 }
               if (p.dbg_exps && rank == 0 && tid == 0)   // p_I at every token: one exponential per node and row
                 atomicAdd(p.dbg_exps, (unsigned long long)S.is_n * (unsigned long long)p.V * (unsigned long long)rows);
+              is_table();
               Z = sample_cdf(mask, [&](int, const auto& L, float* r) { residual_is(L, r); }, ures, &tot);
               done = true;
             }
@@ -2735,26 +2937,63 @@ struct Kernel {
 #pragma unroll
       for (int e = 0; e < VE; ++e) q[e] = prob_of(v[e], S.M[0], S.c[0], S.invZ[0]);
     }
-    float rho[VE][kMaxRows];
-    for (int rr = 1; rr < S.nrows; ++rr) {
-      if (!S.is_cnt[rr]) continue;
-      float v[VE];
-      L(rr, v);
+    float pI[VE];
 #pragma unroll
-      for (int e = 0; e < VE; ++e) {
-        const float pv = prob_of(v[e], S.M[rr], S.c[rr], S.invZ[rr]);
-        rho[e][rr] = pv > 0.f ? __fdiv_rn(q[e], pv) : kPosInf;
+    for (int e = 0; e < VE; ++e) pI[e] = 0.f;
+    uint32_t slow = 0u;   // tokens outside the table (never within its range)
+    if (S.is_tab) {
+      int row = 0;
+      for (int rr = 1; rr < S.nrows; ++rr) {
+        if (!S.is_cnt[rr]) continue;
+        float lq[VE], lp[VE];
+        L(0, lq);
+        L(rr, lp);
+        const float* tab = isBin + (size_t)row * S.is_nb * kIsMom;
+        ++row;
+#pragma unroll
+        for (int e = 0; e < VE; ++e) {
+          if (!(prob_of(lp[e], S.M[rr], S.c[rr], S.invZ[rr]) > 0.f) || !(q[e] > 0.f)) continue;
+          const float x = is_pos(lq[e], lp[e], rr);
+          const float n = rintf(x);
+          const int bin = (int)n - S.is_b0;
+          if (bin < 0 || bin >= S.is_nb) {
+            slow |= 1u << e;
+            continue;
+          }
+          const float v = __fmul_rn(2.f, __fsub_rn(x, n));
+          const float4 lo = reinterpret_cast<const float4*>(tab + (size_t)bin * kIsMom)[0];
+          const float4 hi = reinterpret_cast<const float4*>(tab + (size_t)bin * kIsMom)[1];
+          float g = __fmaf_rn(hi.w, v, hi.z);
+          g = __fmaf_rn(g, v, hi.y);
+          g = __fmaf_rn(g, v, hi.x);
+          g = __fmaf_rn(g, v, lo.w);
+          g = __fmaf_rn(g, v, lo.z);
+          g = __fmaf_rn(g, v, lo.y);
+          pI[e] = __fadd_rn(pI[e], __fmaf_rn(g, v, lo.x));
+        }
       }
+    } else {
+      slow = (1u << VE) - 1u;
+    }
+    if (slow) {
+      float rho[VE][kMaxRows];
+      for (int rr = 1; rr < S.nrows; ++rr) {
+        if (!S.is_cnt[rr]) continue;
+        float v[VE];
+        L(rr, v);
+#pragma unroll
+        for (int e = 0; e < VE; ++e) {
+          const float pv = prob_of(v[e], S.M[rr], S.c[rr], S.invZ[rr]);
+          rho[e][rr] = pv > 0.f ? __fdiv_rn(q[e], pv) : kPosInf;
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < VE; ++e)
+        if ((slow >> e & 1u) && q[e] > 0.f) pI[e] = is_ratio_sum(rho[e]);
     }
 #pragma unroll
-    for (int e = 0; e < VE; ++e) {
-      if (!(q[e] > 0.f)) {
-        r[e] = 0.f;
-        continue;
-      }
-      const float pI = __fmul_rn(q[e], is_ratio_sum(rho[e]));
-      r[e] = fmaxf(0.f, __fsub_rn(q[e], pI));
-    }
+    for (int e = 0; e < VE; ++e)
+      r[e] = (q[e] > 0.f) ? fmaxf(0.f, __fsub_rn(q[e], __fmul_rn(q[e], pI[e]))) : 0.f;
   }
 
   // Sequential rejection over the valid drafts (baseline).  Returns Z.
@@ -2862,7 +3101,7 @@ struct Kernel {
 };
 
 template <int DT, int SCHEME>
-__global__ void __launch_bounds__(kThreads, SCHEME == MDS_IS ? 1 : 2) verify_kernel(const __grid_constant__ Params p) {
+__global__ void __launch_bounds__(kThreads, 2) verify_kernel(const __grid_constant__ Params p) {
   extern __shared__ __align__(128) char dsm[];
   __shared__ State S;
   Kernel<DT, SCHEME> k{p, S};
@@ -2875,7 +3114,7 @@ __global__ void __launch_bounds__(kThreads, SCHEME == MDS_IS ? 1 : 2) verify_ker
   k.nsegv = (k.Uv + 31) / 32;                                // segments the residual pass writes
   k.bm_words = (p.slice / Kernel<DT, SCHEME>::VE + 31) / 32;   // one bit per 16-byte unit
   // dynamic shared memory: ring | segment sums | chunk sums | segment references | scheme region
-  //   IS : nodes t_n | weights W_r(n)
+  //   IS : bins (the residual's coefficients) | set-aside tokens | nodes t_n | weights W_r(n)
   //   WIS: CTA list (two copies) | warp lists = staging list | merged list, the
   //        last aliased later by the special-token bitmap (only the CTA list
   //        is ever read by other CTAs)
@@ -2885,7 +3124,9 @@ __global__ void __launch_bounds__(kThreads, SCHEME == MDS_IS ? 1 : 2) verify_ker
   k.segref = k.chksum + ((((k.nseg + 31) / 32) + 3) & ~3);
   {
     char* c = reinterpret_cast<char*>(k.segref + ((k.nseg + 3) & ~3));
-    k.isT = reinterpret_cast<float*>(c);
+    k.isBin = reinterpret_cast<float*>(c);
+    k.isStg = reinterpret_cast<float4*>(c + kIsBinBytes);
+    k.isT = reinterpret_cast<float*>(c + kIsBinBytes + kWarps * kIsStage * 16);
     k.isW = k.isT + kIsNodesMax;
     k.cl_base = c;
     c += (size_t)2 * kListN * (1 + p.rows_max) * 4;
@@ -2958,7 +3199,8 @@ size_t smem_bytes(const Params& p) {
   const int VE = 16 / p.esize;
   const int nseg = (p.slice / VE + 31) / 32;
   size_t bytes = (size_t)p.ring_bytes + (size_t)((nseg + 3) & ~3) * 4 * 2 + (size_t)((((nseg + 31) / 32) + 3) & ~3) * 4;
-  if (p.scheme == MDS_IS) bytes += (size_t)kIsNodesMax * 4 * (1 + p.rows_max);
+  if (p.scheme == MDS_IS)
+    bytes += (size_t)kIsBinBytes + (size_t)kWarps * kIsStage * 16 + (size_t)kIsNodesMax * 4 * (1 + p.rows_max);
   if (p.scheme == MDS_WIS || p.scheme == MDS_WIS0) {
     const size_t bm = (size_t)((p.slice / VE + 31) / 32) * 4;
     const size_t cm = (size_t)p.cand_cap * 4 * (3 + p.rows_max);
