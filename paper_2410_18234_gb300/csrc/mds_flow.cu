@@ -20,10 +20,13 @@
 //   replace  the target mass outside Omega_0 (truncated alphabet);
 //   full     a full-vocabulary stage of the weighted scheme: the slice's top-s
 //            keys q - a b with a and b, and the Omega_2 masses of the rest;
-//   bonus    the target row's maximum and sum at depth L.
-// The CTA whose task completes a pass (a per-sequence counter) runs the
-// decision for that sequence: it combines the records in slice order, runs the
-// importance step (the WIS stages on the merged candidate list, Omega_1 by
+//   bonus    the target row's maximum, sum and run sums at depth L.
+// The compute warps work on their own shares of a slice without block
+// barriers and leave partial results in a record slot in shared memory; a
+// publishing warp merges them, stores the record and counts the pass's
+// slices.  The one that counts a pass's last slice posts a decision request.
+// A decision warp combines the records in slice order, runs the importance
+// step (the WIS stages on the merged candidate list, Omega_1 by
 // the keys q - a b, the stage LP, Remark 4's pairwise stages), Algorithm 1's
 // accept test, and the inverse-CDF search of a residual draw (slice by the
 // records, token by one re-read of that slice), then advances the walk and
@@ -46,8 +49,13 @@ using namespace mds::dev;
 
 constexpr int kCW = 8;                 // compute warps
 constexpr int kCT = kCW * 32;          // compute threads
-constexpr int kBlock = kCT + 32;       // + the scheduler warp
+constexpr int kBlock = kCT + 64;       // + the scheduler warp and the publishing warp
 constexpr int kNBuf = 2;               // slice buffers per CTA
+constexpr int kSlots = 3;              // records between the compute warps and the publishing warp
+constexpr int kFastUnits = kBufBytes / 16;   // units of all rows one slice holds
+constexpr int kWarpCand = 32;          // tokens one warp may set aside in a slice
+constexpr int kSlotCand = kCW * kWarpCand;
+constexpr int kMaxRuns = kFastUnits / 32;    // runs of 32 units of a slice
 constexpr int kCtasPerSm = 2;          // resident CTAs per SM (the launch bound)
 constexpr int kCandCap = 512;          // candidate tokens one slice may set aside
 constexpr int kListMax = 64;           // candidate list length at most
@@ -55,12 +63,6 @@ constexpr int kHdr = 2 * kMaxRows + 2; // record: (max, sum) per row, tau, list 
 constexpr int kTopF = 8;               // per-thread candidates of a full stage (>= MDS_MAX_S)
 constexpr int kMaxEntries = 512;       // slices x slice list length, at most
 constexpr int kDecStage = 8192;        // bytes of a pass's slice records ([ns][rec_floats]) at most
-// A stats pass's combined record (written over the sequence's slice records
-// by the CTA that completes the pass): per row M, 1/Z and the complement
-// mass, the list's length, tau, completeness and q(tau), then the list:
-// ids, target logits and per row exp terms (token order of the merge).
-constexpr int kCmbM = 0, kCmbIz = kMaxRows, kCmbPc = 2 * kMaxRows, kCmbN = 2 * kMaxRows + kListRowsMax;
-constexpr int kCmbHdr = kCmbN + 4;
 constexpr unsigned long long kWaitNs = 2000000000ull;   // 2 s bound on every wait
 constexpr unsigned FULLM = 0xffffffffu;
 static_assert(kHdr % 4 == 0, "record header keeps 16-byte alignment");
@@ -101,7 +103,7 @@ enum : int {
   kPhListB,             // list tasks: the sums and the candidates
   kPhListC,             // list tasks: ranking and the record
   kPhPublish,           // a task's record publication (fence, pass counter)
-  kPhCombine,           // combining a completed stats pass (the last task's CTA)
+  kPhCombine,           // (unused)
   kPhLp,                // the stage LPs (one thread)
   kPhLpCalls,           // count: stage LPs
   kPhTasks,             // count: slice tasks
@@ -149,7 +151,7 @@ struct __align__(16) FSeq {
 
 struct __align__(16) FDesc {
   FPass P;
-  int b, slice, exit, pad;
+  int b, slice, end, exit;     // the sequence, the next slice and the end of its group
 };
 static_assert(sizeof(FDesc) % 16 == 0, "descriptor moves in 16-byte chunks");
 
@@ -161,6 +163,16 @@ struct Cand {  // full-stage candidate: larger key first, then smaller token id
 #define CAND_NONE Cand{kNegInf, 0x7fffffff, 0.f, 0.f}
 __device__ __forceinline__ bool better(float ka, int ia, float kb, int ib) {
   return ka > kb || (ka == kb && ia < ib);
+}
+
+// The uniforms of one depth, drawn together by the lanes of a decision warp.
+enum : int { kDrSelect = 0, kDrAccept = 16, kDrResidual, kDrBonus, kDrKeep, kDrOutside, kDrawsN };
+__device__ __forceinline__ int draw_id(int i) {
+  return i < 16 ? kDrawSelect + i
+                : (i == kDrAccept ? kDrawAccept
+                                  : (i == kDrResidual ? kDrawResidual
+                                                      : (i == kDrBonus ? kDrawBonus
+                                                                       : (i == kDrKeep ? kDrawKeep : kDrawOutside))));
 }
 
 struct DState {                // the decision's working state (shared memory)
@@ -176,21 +188,16 @@ struct DState {                // the decision's working state (shared memory)
   int cm_id[kListMax];
   float cm_l0[kListMax];
   float cm_e[kListRowsMax][kListMax];
-  float cm_a[kListMax];
-  int cm_sp[kListMax];
   float pc[kListRowsMax];
-  int ksl[kMaxSlicesList];
-  int fin_s[kListMax], fin_i[kListMax];
   // stage
+  __align__(16) unsigned kx[32];   // the list's keys of a stage
   int om[MDS_MAX_S];
   float om_q[MDS_MAX_S], om_a[MDS_MAX_S], om_b[MDS_MAX_S], om_x[MDS_MAX_S];
-  float A2, B2;
-  int Y, fast_ok;
+  int Y;
   Cand fin[kTopF];
   float lp_rs[kMaxPairs], lp_fl[kMaxPairs], lp_fh[kMaxPairs];   // LP pair state in shared memory
   // search
-  int seg, cross, lastp, tok;
-  float run;
+  int tok;
   // truncated alphabet
   int k_lane[MDS_MAX_K], k_row[MDS_MAX_K];
   int o0_n, o0_all, o0_Yp;
@@ -198,6 +205,7 @@ struct DState {                // the decision's working state (shared memory)
   // depth (tk0) and the next depth (tk1), temperatures (target, drafts)
   int tk0[MDS_MAX_K], tk1[MDS_MAX_K];
   float tmp[MDS_MAX_K + 1];
+  float dr[kDrawsN];           // the depth's uniforms, by kDr*
   int xl_wait;                 // the row logits at the draft tokens are still in flight
   float o0_cut, o0_pa, o0_R;
   float rtot;
@@ -206,21 +214,35 @@ struct DState {                // the decision's working state (shared memory)
 static_assert(offsetof(DState, W) == offsetof(DState, P) + sizeof(FPass) && offsetof(FSeq, W) == sizeof(FPass),
               "a sequence's state copies into the decision state in one piece");
 
+// What the compute warps hand the publishing warp of one slice.
+enum : int { kSlotDone = 0,   // the record is in global memory already
+             kSlotSums, kSlotList, kSlotBonus, kSlotRuns, kSlotExit };
+struct __align__(16) Slot {
+  int mode, b, slice, kind, j, R, list, nrun;
+  int count;                   // slices to count with this one: its group's, at the group's end (else 0)
+  float c[kListRowsMax];
+  int ncand;                   // tokens set aside (zero between slices)
+  float tau[kCW];              // per warp: largest target logit not set aside
+  float m[kCW][kListRowsMax], s[kCW][kListRowsMax];
+  float run[kMaxRuns];
+  __align__(16) unsigned key[kSlotCand];   // order key of the target logit (16-bit logits: and the place, see set_aside)
+  int loc[kSlotCand], ord[kSlotCand];      // place in the slice
+  float l[kListRowsMax][kSlotCand];
+};
+
 struct FShared {
-  uint64_t full[kNBuf], empty[kNBuf];
+  uint64_t full[kNBuf], empty[kNBuf], done[kSlots], free[kSlots];
   FDesc desc[kNBuf];
   FDesc pend;                  // the scheduler's next task, resolved ahead
   float red[kCW * 2 * kMaxRows];
   float wth[kCW];
-  int ncand, last, issued, consumed;
-  int cmb_nv;                  // combine of a pass: valid entries
-  unsigned cmb_tau;            // ... order key of tau
+  int ncand, issued, consumed;
   float addtau;
   float add[kMaxRows];
   uint32_t bitmap[64];         // one bit per 16-byte unit of a slice holding a special token
   Cand wcand[kCW * kTopF];
   Cand blk[kTopF];
-  int flag_ok, flag_ab;
+  int flag_ok[2];
 #ifdef MDS_PHASE_TIMERS
   unsigned long long tm[kPhaseN];
 #endif
@@ -250,6 +272,17 @@ __device__ __forceinline__ unsigned long long now_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
+}
+// Ring words: launch, lap over the ring, payload (sequence << 8 | group of slices).
+constexpr unsigned long long kRingPay = 0xffffffull;
+__device__ __forceinline__ unsigned long long ring_word(unsigned epoch, unsigned lap, unsigned pay) {
+  return ((unsigned long long)(epoch & 0x3fffffffu) << 34) | ((unsigned long long)((lap + 1u) & 0x3ffu) << 24) | pay;
+}
+__device__ __forceinline__ unsigned long long dec_tag_of(unsigned epoch, unsigned t) {
+  return ((unsigned long long)epoch << 32) | (unsigned long long)(t + 1u);
+}
+__device__ __forceinline__ void st_relaxed(unsigned long long* a, unsigned long long v) {
+  asm volatile("st.relaxed.gpu.u64 [%0], %1;" ::"l"(a), "l"(v) : "memory");
 }
 __device__ __forceinline__ void cbar() { asm volatile("bar.sync 1, %0;" ::"n"(kCT) : "memory"); }
 
@@ -308,6 +341,80 @@ __device__ unsigned long long g_phase[kPhaseN];
 #define PT_CNTW(i)
 #endif
 
+// ------------------------------------------------------------------ slice loading (plain loads)
+// Unit u (16 bytes from byte 16 u of `src` on) of a row that ends before
+// `end` and starts at `first`: where the row is not 16-byte aligned, the two
+// aligned 16-byte blocks that hold the unit, shifted together, if both lie
+// inside the row, else logit by logit; logits past n read -inf.
+template <int DT>
+__device__ __forceinline__ uint4 load_unit(const char* src, const char* first, const char* end, int u, int n) {
+  constexpr int VE = Elt<DT>::VE;
+  const char* at = src + 16 * (size_t)u;
+  const unsigned sh = (unsigned)(reinterpret_cast<uintptr_t>(at) & 15u);
+  const char* blk = at - sh;
+  if (u * VE + VE <= n && blk >= first && blk + (sh ? 32 : 16) <= end) {
+    const uint4 lo = __ldg(reinterpret_cast<const uint4*>(blk));
+    if (!sh) return lo;
+    const uint4 hi = __ldg(reinterpret_cast<const uint4*>(blk) + 1);
+    uint32_t w0 = lo.x, w1 = lo.y, w2 = lo.z, w3 = lo.w, w4 = hi.x, w5 = hi.y, w6 = hi.z, w7 = hi.w;
+    if (sh & 8u) {
+      w0 = w2;
+      w1 = w3;
+      w2 = w4;
+      w3 = w5;
+      w4 = w6;
+      w5 = w7;
+    }
+    if (sh & 4u) {
+      w0 = w1;
+      w1 = w2;
+      w2 = w3;
+      w3 = w4;
+      w4 = w5;
+    }
+    const unsigned bits = (sh & 3u) * 8u;
+    return make_uint4(__funnelshift_r(w0, w1, bits), __funnelshift_r(w1, w2, bits), __funnelshift_r(w2, w3, bits),
+                      __funnelshift_r(w3, w4, bits));
+  }
+  uint32_t w[4];
+  if constexpr (DT == MDS_BF16) {
+    const unsigned short* s16 = reinterpret_cast<const unsigned short*>(src);
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const int t0 = u * VE + 2 * h;
+      const uint32_t a = (t0 < n) ? (uint32_t)__ldg(s16 + t0) : 0xff80u;
+      const uint32_t c = (t0 + 1 < n) ? (uint32_t)__ldg(s16 + t0 + 1) : 0xff80u;
+      w[h] = a | (c << 16);
+    }
+  } else {
+    const float* s32 = reinterpret_cast<const float*>(src);
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const int t0 = u * VE + h;
+      w[h] = (t0 < n) ? __float_as_uint(__ldg(s32 + t0)) : 0xff800000u;
+    }
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// Rows [0, R) of the slice [tok0, tok0 + n) into shared memory, every
+// thread its own units (u = thread, thread + 256, ...): used where bulk
+// copies are not (mapped host memory, rows not 16-byte aligned).
+template <int DT>
+__device__ __noinline__ void load_rows(const FPass& P, int R, char* b, int tok0, int n, int T, int V) {
+  constexpr int VE = Elt<DT>::VE, es = 16 / VE;
+  const int U = (n + VE - 1) / VE;
+  for (int r = 0; r < R; ++r) {
+    const char* first = P.row[r].ptr;
+    const char* src = first + (size_t)tok0 * es;
+    const char* end = first + (size_t)V * es;
+    char* dst = b + (size_t)r * T * es;
+#pragma unroll 4
+    for (int u = threadIdx.x; u < U; u += kCT)
+      *reinterpret_cast<uint4*>(dst + 16 * (size_t)u) = load_unit<DT>(src, first, end, u, n);
+  }
+}
+
 // ------------------------------------------------------------------ the engine
 
 template <int DT>
@@ -318,14 +425,12 @@ struct Eng {
   const Params& p;
   FShared& S;
   char* bufs;     // kNBuf x kBufBytes
+  Slot* slots;    // kSlots records on their way to the publishing warp
   int* cid;       // candidate ids
   float* cl;      // candidate target logits
   int* crank;     // candidate ranks
   int* cord;      // candidates ranked past the list, in rank order
 
-  __device__ __forceinline__ unsigned long long tag_of(unsigned t) const {
-    return ((unsigned long long)p.epoch << 32) | (unsigned long long)(t + 1u);
-  }
   __device__ __forceinline__ bool aborted() const { return ld_relaxed(&p.ctl[kCtlAbort]) != 0u; }
   __device__ __forceinline__ void set_abort(unsigned bits) const {
     atomicOr(p.status, bits);
@@ -345,6 +450,7 @@ struct Eng {
 
   // -------------------------------------------------------------- scheduler warp
   __device__ bool wait_mbar(uint64_t* bar, uint32_t parity) const {
+    if (mbar_try_wait(bar, parity)) return true;
     const unsigned long long t0 = now_ns();
     for (int it = 0;; ++it) {
       if (mbar_try_wait(bar, parity)) return true;
@@ -407,31 +513,31 @@ struct Eng {
     }
   }
 
-  // Claim the next task number and resolve it into Pd: the sequence, the
-  // slice and the sequence's pass descriptor (depth-0 tasks are implicit:
-  // task t < B * ns is slice t % ns of sequence t / ns).  Returns 0 when no
+  // Claim the next task number and resolve it into Pd: the sequence, its
+  // slices and the sequence's pass descriptor (depth-0 tasks are implicit:
+  // task t < B * ng is group t % ng of sequence t / ng).  Returns 0 when no
   // work is left (every sequence finished, or an abort).  Warp-wide.
   __device__ int resolve(FDesc& Pd) {
     const int lane = threadIdx.x & 31;
-    const unsigned N0 = (unsigned)p.B * (unsigned)p.ns;
-    int have = 0, b = 0, s = 0;
+    const unsigned N0 = (unsigned)p.B * (unsigned)p.ng;
+    int have = 0, b = 0, g = 0;
     if (lane == 0 && !aborted()) {
       const unsigned t = atomicAdd(&p.ctl[kCtlHead], 1u);
+      const unsigned slot = t % (unsigned)p.ring_cap;
       if (t < N0) {
-        b = (int)(t / (unsigned)p.ns);
-        s = (int)(t % (unsigned)p.ns);
-        st_release(&p.ring_rtag[t % (unsigned)p.ring_cap], tag_of(t));
+        b = (int)(t / (unsigned)p.ng);
+        g = (int)(t % (unsigned)p.ng);
+        st_release(&p.ring_rtag[slot], ring_word(p.epoch, t / (unsigned)p.ring_cap, 0u));
         have = 1;
       } else {
-        const unsigned slot = t % (unsigned)p.ring_cap;
-        const unsigned long long want = tag_of(t);
+        const unsigned long long want = ring_word(p.epoch, t / (unsigned)p.ring_cap, 0u);
         const unsigned long long t0 = now_ns();
         PT_T0(t_poll);
         for (int it = 0;; ++it) {
-          if (ld_acquire(&p.ring_tag[slot]) == want) {
-            const unsigned pay = __ldcg(&p.ring_pay[slot]);
-            b = (int)(pay >> 16);
-            s = (int)(pay & 0xffffu);
+          const unsigned long long w = ld_acquire(&p.ring_tag[slot]);
+          if ((w & ~kRingPay) == want) {
+            b = (int)((w >> 8) & 0xffffu);
+            g = (int)(w & 0xffu);
             st_release(&p.ring_rtag[slot], want);
             have = 2;
             break;
@@ -448,14 +554,15 @@ struct Eng {
     }
     have = __shfl_sync(FULLM, have, 0);
     b = __shfl_sync(FULLM, b, 0);
-    s = __shfl_sync(FULLM, s, 0);
+    g = __shfl_sync(FULLM, g, 0);
     if (have == 1)
       plan_depth0_warp(b, Pd.P);
     else if (have == 2)
       copy_in(&Pd.P, &reinterpret_cast<const FSeq*>(p.seq)[b].P, (int)sizeof(FPass), lane, 32);
     if (lane == 0) {
       Pd.b = b;
-      Pd.slice = s;
+      Pd.slice = g * p.group;
+      Pd.end = min(p.ns, (g + 1) * p.group);
       Pd.exit = have ? 0 : 1;
     }
     __syncwarp();
@@ -488,13 +595,13 @@ struct Eng {
         for (int i = lane; i < (int)(sizeof(FDesc) / 16); i += 32) dst[i] = src[i];
       }
       __syncwarp();
+      int more = 0;
       if (lane == 0) {
         if (have && p.bulk) {
           const int s = D.slice;
           const int tok0 = s * p.T;
           const int n = min(p.T, p.V - tok0);
           const uint32_t bytes = (uint32_t)n * (uint32_t)p.esize;
-          fence_proxy_async();
           mbar_expect_tx(&S.full[bi], bytes * (uint32_t)D.P.nstream);
           for (int r = 0; r < D.P.nstream; ++r)
             bulk_copy(buf(bi) + (size_t)r * p.T * p.esize, D.P.row[r].ptr + (size_t)tok0 * p.esize, bytes, &S.full[bi]);
@@ -502,50 +609,23 @@ struct Eng {
           mbar_arrive(&S.full[bi]);
         }
         S.issued = k + 1;
+        S.pend.slice += 1;
+        more = S.pend.slice < S.pend.end ? 1 : 0;
       }
+      more = __shfl_sync(FULLM, more, 0);
       __syncwarp();
       if (!have) return;
-      have = resolve(S.pend);
+      if (!more) have = resolve(S.pend);
     }
   }
 
-  // -------------------------------------------------------------- slice loading (plain loads)
-  // Rows [0, R) of the slice [tok0, tok0 + n) into shared memory; units past
-  // n read -inf.  Used where bulk copies are not (mapped host memory, rows
-  // not 16-byte aligned) and by the search's re-read of one slice.
+  // Rows [0, R) of a slice by plain loads, every thread its own units.
+  __device__ __forceinline__ void load_own(const FPass& P, int R, char* b, int tok0, int n) const {
+    load_rows<DT>(P, R, b, tok0, n, p.T, p.V);
+  }
+  // The same for readers of other threads' units.
   __device__ void load_plain(const FPass& P, int R, char* b, int tok0, int n) const {
-    const int U = (n + VE - 1) / VE;
-    for (int r = 0; r < R; ++r) {
-      const char* src = P.row[r].ptr + (size_t)tok0 * p.esize;
-      char* dst = b + (size_t)r * p.T * p.esize;
-      for (int u = threadIdx.x; u < U; u += kCT) {
-        uint4 x;
-        if (p.aligned) {
-          x = __ldg(reinterpret_cast<const uint4*>(src + 16 * (size_t)u));
-        } else {
-          uint32_t w[4];
-          if constexpr (DT == MDS_BF16) {
-            const unsigned short* s16 = reinterpret_cast<const unsigned short*>(src);
-#pragma unroll
-            for (int h = 0; h < 4; ++h) {
-              const int t0 = u * VE + 2 * h;
-              const uint32_t lo = (t0 < n) ? (uint32_t)__ldg(s16 + t0) : 0xff80u;
-              const uint32_t hi = (t0 + 1 < n) ? (uint32_t)__ldg(s16 + t0 + 1) : 0xff80u;
-              w[h] = lo | (hi << 16);
-            }
-          } else {
-            const float* s32 = reinterpret_cast<const float*>(src);
-#pragma unroll
-            for (int h = 0; h < 4; ++h) {
-              const int t0 = u * VE + h;
-              w[h] = (t0 < n) ? __float_as_uint(__ldg(s32 + t0)) : 0xff800000u;
-            }
-          }
-          x = make_uint4(w[0], w[1], w[2], w[3]);
-        }
-        *reinterpret_cast<uint4*>(dst + 16 * (size_t)u) = x;
-      }
-    }
+    load_own(P, R, b, tok0, n);
     cbar();
   }
 
@@ -587,9 +667,169 @@ struct Eng {
     return t;
   }
 
+  // -------------------------------------------------------------- statistics of a slice, warp by warp
+  // R rows (compile time) of a slice of at most 2048 / R units a row.  Every
+  // thread keeps its units (u = thread, thread + 256, ...: the warps
+  // interleave in chunks of 32 units) in registers and every warp works on
+  // its own share, with its own exponent references and no block barrier:
+  // the row maxima (packed), then the sums of 2^(l c - m c).  With LIST the
+  // warp first sets aside the tokens whose target logit reaches theta, the
+  // p.kth-th largest of its lanes' maxima (so at least p.kth tokens where the
+  // warp has as many), and leaves them out of its sums; more than kWarpCand
+  // of them (ties, flat rows) and theta rises to the largest bound that
+  // leaves at most that many.  With RUNS (the bonus row) the chunks' sums are
+  // kept too.  The publishing warp merges the eight warps' results.
+  //
+  // Bound by issue (4.5 instructions a logit) and by the loads' latency: two
+  // CTAs of eight independent warps an SM.  Against one pass by the whole
+  // block with five barriers and the publication in it (GB300, a 32 KB slice
+  // of two rows): with a list 17k -> 3.5k SM cycles, without 8k -> 2.7k.
+  template <int R, bool LIST, bool RUNS>
+  __device__ __forceinline__ void stats_fast(const FPass& P, char* b, int tok0, int n, Slot& T) {
+    constexpr int NU = (kFastUnits / R + kCT - 1) / kCT;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int U = (n + VE - 1) / VE;
+    if (!p.bulk) load_own(P, R, b, tok0, n);
+    uint4 x[R][NU];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int i = 0; i < NU; ++i) {
+        const int u = i * kCT + tid;
+        x[r][i] = (u < U) ? raw(b, r, u) : E::neg_inf();
+      }
+    float m[R];
+    unsigned key0 = 0u;   // order key of this lane's largest target logit
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      uint4 mx = x[r][0];
+#pragma unroll
+      for (int i = 1; i < NU; ++i) mx = E::max4(mx, x[r][i]);
+      const float lm = E::unit_max(mx);
+      const unsigned key = (lm > kNegInf) ? ord_key(__fadd_rn(lm, 0.f)) : 0u;
+      if (r == 0) key0 = key;
+      const unsigned km = __reduce_max_sync(FULLM, key);
+      m[r] = km ? ord_val(km) : kNegInf;
+    }
+    if constexpr (LIST) {
+      // theta: the kth-th largest lane maximum
+      unsigned km = __reduce_max_sync(FULLM, key0), rest = key0, last = km;
+      for (int t = 1; t < p.kth && km; ++t) {
+        const unsigned who = __ballot_sync(FULLM, rest == km);
+        if (lane == __ffs(who) - 1) rest = 0u;
+        km = __reduce_max_sync(FULLM, rest);
+        if (km) last = km;
+      }
+      float theta = last ? ord_val(last) : kPosInf;
+      unsigned long long bits = 0ull;   // this lane's tokens at or above theta, VE to a unit
+      auto mark = [&]() {
+        bits = 0ull;
+#pragma unroll
+        for (int i = 0; i < NU; ++i) {
+          if (E::unit_max(x[0][i]) >= theta) {
+            float v[VE];
+            E::unpack(x[0][i], v);
+            unsigned bb = 0u;
+#pragma unroll
+            for (int e = 0; e < VE; ++e) bb |= (v[e] >= theta && v[e] > kNegInf) ? 1u << e : 0u;
+            bits |= (unsigned long long)bb << (i * VE);
+          }
+        }
+        return __popcll(bits);
+      };
+      int cnt = mark();
+      if (__reduce_add_sync(FULLM, (unsigned)cnt) > (unsigned)kWarpCand) {
+        // the largest key that more than kWarpCand tokens reach, and one up
+        unsigned t = 0u;
+#pragma unroll 1
+        for (int bit = 31; bit >= 0; --bit) {
+          const unsigned cand = t | (1u << bit);
+          unsigned c = 0u;
+#pragma unroll 1
+          for (int u = tid; u < U; u += kCT) {
+            float v[VE];
+            E::unpack(raw(b, 0, u), v);
+#pragma unroll
+            for (int e = 0; e < VE; ++e) c += (v[e] == v[e] && ord_key(__fadd_rn(v[e], 0.f)) >= cand) ? 1u : 0u;
+          }
+          if (__reduce_add_sync(FULLM, c) > (unsigned)kWarpCand) t = cand;
+        }
+        theta = ord_val(t + 1u);
+        cnt = mark();
+      }
+      if (cnt) {
+        int pos = atomicAdd(&T.ncand, cnt);
+        for (unsigned long long q = bits; q; q &= q - 1ull) {
+          const int at = __ffsll((long long)q) - 1;
+          const int loc = ((at / VE) * kCT + tid) * VE + at % VE;
+          T.loc[pos] = loc;
+#pragma unroll
+          for (int rr = 0; rr < R; ++rr) T.l[rr][pos] = E::at(srow(b, rr), loc);
+          T.key[pos] = cand_key(T.l[0][pos], loc);
+          ++pos;
+        }
+      }
+      // out of the registers: every row reads -inf there
+#pragma unroll
+      for (int i = 0; i < NU; ++i) {
+        const unsigned bb = (unsigned)(bits >> (i * VE)) & ((1u << VE) - 1u);
+        if (__any_sync(FULLM, bb != 0u)) {
+#pragma unroll
+          for (int rr = 0; rr < R; ++rr) E::mask(x[rr][i], bb);
+        }
+      }
+      float tm = kNegInf;
+#pragma unroll
+      for (int i = 0; i < NU; ++i) tm = fmaxf(tm, E::unit_max(x[0][i]));
+      const unsigned tk = __reduce_max_sync(FULLM, (tm > kNegInf) ? ord_key(tm) : 0u);
+      if (lane == 0) T.tau[warp] = tk ? ord_val(tk) : kNegInf;
+    }
+    float s[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const float c = P.row[r].c;
+      const float mc = (m[r] > kNegInf) ? __fmul_rn(m[r], c) : 0.f;
+      float acc = 0.f;
+#pragma unroll
+      for (int i = 0; i < NU; ++i) {
+        if (i * kCT + warp * 32 >= U) break;   // warp-uniform
+        float v[VE];
+        E::unpack(x[r][i], v);
+#pragma unroll
+        for (int e = 0; e < VE; ++e) v[e] = ex2(__fmaf_rn(v[e], c, -mc));
+        float t;
+        if constexpr (VE == 8)
+          t = __fadd_rn(__fadd_rn(__fadd_rn(v[0], v[1]), __fadd_rn(v[2], v[3])),
+                        __fadd_rn(__fadd_rn(v[4], v[5]), __fadd_rn(v[6], v[7])));
+        else
+          t = __fadd_rn(__fadd_rn(v[0], v[1]), __fadd_rn(v[2], v[3]));
+        if constexpr (RUNS) {
+          const float w = warp_sum(t);
+          if (lane == 0) T.run[i * kCW + warp] = w;
+          acc = __fadd_rn(acc, w);
+        } else {
+          acc = __fadd_rn(acc, t);
+        }
+      }
+      s[r] = acc;
+    }
+    if constexpr (!RUNS) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) s[r] = warp_sum(s[r]);
+    }
+    if (lane == 0) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        T.m[warp][r] = m[r];
+        T.s[warp][r] = s[r];
+      }
+    }
+  }
+
   // -------------------------------------------------------------- stats task
-  // R rows (compile time, at most kListRowsMax) with or without the candidate
-  // list, in two passes over the slice in shared memory.  Pass A: every
+  // Slices too small for the warp-wise path (fewer units than threads): R rows
+  // (compile time, at most kListRowsMax) with the candidate list, by the whole
+  // block in two passes over the slice in shared memory.  Pass A: every
   // row's maximum (the slice's exponent reference) and the candidate
   // threshold theta: the smallest of the warps' largest target logits, so
   // that at least one token per warp is >= theta (theta = -inf for a slice
@@ -603,7 +843,7 @@ struct Eng {
   // kCandCap-th largest target logit (bisection) and pass B repeated.
   // Record: (max, sum) per row, tau, list length, then the list: ids, then
   // each row's logits.
-  template <int R, bool LIST>
+  template <int R>
   __device__ void stats_small(const FPass& P, const char* b, int tok0, int n, float* rec) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int U = (n + VE - 1) / VE;
@@ -622,7 +862,7 @@ struct Eng {
       mx = warp_max(mx);
       if (lane == 0) S.red[warp * kMaxRows + r] = mx;
     }
-    if constexpr (LIST) {
+    {
       // this warp's k-th largest thread maximum (distinct tokens), k = LN / kCW
       // rounded up: every warp then holds k tokens >= its value
       const int k = (LN + kCW - 1) / kCW;
@@ -650,7 +890,7 @@ struct Eng {
     // when every warp takes part; -inf (every token a candidate) for a slice
     // of at most kCandCap tokens
     float theta = kNegInf;
-    if constexpr (LIST) {
+    {
       if (n > kCandCap) {
         theta = kPosInf;
 #pragma unroll
@@ -661,7 +901,7 @@ struct Eng {
         if (theta == kPosInf) theta = kNegInf;
       }
     }
-    if (LIST) PT_ADD(kPhListA, t_a);
+    PT_ADD(kPhListA, t_a);
     PT_T0(t_b);
     float sm[R], tau;
     int nc = 0;
@@ -674,7 +914,7 @@ struct Eng {
         float v0[VE];
         E::unpack(x0, v0);
         uint32_t cm = 0u;
-        if constexpr (LIST) {
+        {
           const float um = E::unit_max(x0);
           if (um > theta) {
 #pragma unroll
@@ -726,7 +966,7 @@ struct Eng {
       }
       cbar();
       nc = S.ncand;
-      if (!LIST || nc <= kCandCap) break;
+      if (nc <= kCandCap) break;
       // more than kCandCap tokens above theta: raise it to the kCandCap-th
       // largest target logit (bisection on order-preserving keys over every
       // bit: keys of negative logits use the low bits too) and repeat
@@ -755,7 +995,7 @@ struct Eng {
       cbar();
     }
     nc = min(nc, kCandCap);   // the bisection leaves fewer than kCandCap; never read past the arrays
-    if (LIST) PT_ADD(kPhListB, t_b);
+    PT_ADD(kPhListB, t_b);
     PT_T0(t_c);
     // block sums of the rows (fixed order)
     float tot[R];
@@ -764,7 +1004,7 @@ struct Eng {
       const float v = warp_sum(sm[r]);
       if (lane == 0) S.red[warp * kMaxRows + r] = v;
     }
-    if constexpr (LIST) {
+    {
       tau = warp_max(tau);
       if (lane == 0) S.wth[warp] = tau;
     }
@@ -776,7 +1016,7 @@ struct Eng {
       for (int w = 0; w < kCW; ++w) t = __fadd_rn(t, S.red[w * kMaxRows + r]);
       tot[r] = t;
     }
-    if constexpr (LIST) {
+    {
       tau = kNegInf;
 #pragma unroll
       for (int w = 0; w < kCW; ++w) tau = fmaxf(tau, S.wth[w]);
@@ -854,10 +1094,10 @@ struct Eng {
         __stcg(rec + 2 * r + 1, tot[r]);
       }
       __stcg(rec + 2 * kMaxRows, tau);
-      __stcg(reinterpret_cast<int*>(rec) + 2 * kMaxRows + 1, LIST ? min(nc, LN) : 0);
+      __stcg(reinterpret_cast<int*>(rec) + 2 * kMaxRows + 1, min(nc, LN));
       S.ncand = 0;   // for the next slice (every reader is past the barriers above)
     }
-    if (LIST) PT_ADD(kPhListC, t_c);
+    PT_ADD(kPhListC, t_c);
   }
 
   // Stats of any number of rows, one row at a time, no candidate list.
@@ -924,221 +1164,24 @@ struct Eng {
     }
   }
 
-  // The slice's mass (record[0]) and its 32 run masses (record[4 + q]): run q
-  // is units [q * upl, (q + 1) * upl), upl = ceil(units / 32), the runs the
-  // decision's search walks.  A unit's mass adds its tokens in order, a run's
-  // its chunks of 32 units (each a butterfly over the units), the slice's
-  // its runs in order.
-  __device__ void resid_task(const FPass& P, const char* b, int tok0, int n, float* rec) {
+  // The masses of the slice's runs of 32 units, the runs the decision's
+  // search walks, one warp a run (runs warp, warp + 8, ...): a unit's mass
+  // adds its tokens in order, a run's its units by a butterfly.
+  __device__ void resid_task(const FPass& P, const char* b, int tok0, int n, Slot& T) {
     if (P.kind == kResid && P.nspec > 0) build_bitmap(P, tok0, n);
     const int U = (n + VE - 1) / VE;
-    const int upl = (U + 31) / 32;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int q = warp; q < 32; q += kCW) {
-      const int u0 = min(U, q * upl), u1 = min(U, u0 + upl);
-      float run = 0.f;
-      for (int c = u0; c < u1; c += 32) {
-        const int u = c + lane;
-        float us = 0.f;
-        if (u < u1) {
-          float w[VE];
-          weights(P, b, u, tok0, w);
+    const int tid = threadIdx.x, lane = tid & 31;
+    for (int u = tid; u - lane < U; u += kCT) {
+      float us = 0.f;
+      if (u < U) {
+        float w[VE];
+        weights(P, b, u, tok0, w);
 #pragma unroll
-          for (int e = 0; e < VE; ++e) us = __fadd_rn(us, w[e]);
-        }
-        run = __fadd_rn(run, warp_sum(us));
+        for (int e = 0; e < VE; ++e) us = __fadd_rn(us, w[e]);
       }
-      if (lane == 0) {
-        S.red[q] = run;
-        __stcg(rec + 4 + q, run);
-      }
+      us = warp_sum(us);
+      if (lane == 0) T.run[u >> 5] = us;
     }
-    cbar();
-    if (threadIdx.x == 0) {
-      float tot = 0.f;
-      for (int q = 0; q < 32; ++q) tot = __fadd_rn(tot, S.red[q]);
-      __stcg(rec, tot);
-    }
-  }
-
-  // -------------------------------------------------------------- a stats pass's combine
-  // Run by the CTA that completes a stats pass, with the pass's slice records
-  // (rec, [ns][rec_floats]) in global memory: every row's M and 1/Z and, with
-  // candidate lists, the sequence's list (the first LF of the slices' lists
-  // by (logit, then slice, then position: the slices hold increasing token
-  // ids and sort their own lists that way)), its complement masses and tau;
-  // written over the records as the combined record.  Scratch: the task's
-  // slice buffer b.  Sums over slices and entries run in fixed orders.
-  __device__ __noinline__ void combine_pass(const FPass& P, char* b, float* rec) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int ns = p.ns, rf = p.rec_floats, LN = p.lns, LF = p.ln;
-    const int R = P.nstream;
-    const bool list = P.list != 0;
-    float* sr = reinterpret_cast<float*>(b);                       // records [ns][rf]
-    unsigned* sk = reinterpret_cast<unsigned*>(b + kDecStage);     // entry keys [ns * LN]
-    int* fin = reinterpret_cast<int*>(sk + kMaxEntries);           // taken entries by merge rank [LF]
-    int* ksl = fin + kListMax;                                     // entries taken per slice [ns]
-    float* part = reinterpret_cast<float*>(ksl + kMaxSlices);      // per-warp partials [kCW][3 * kListRowsMax]
-    for (int i = tid; i < ns * rf / 4; i += kCT)
-      reinterpret_cast<float4*>(sr)[i] = __ldcg(reinterpret_cast<const float4*>(rec) + i);
-    if (tid < ns) ksl[tid] = 0;
-    if (tid == 0) {
-      S.cmb_nv = 0;
-      S.cmb_tau = 0u;
-    }
-    cbar();
-    // rows: warp w takes rows w, w + kCW, ...
-    float* hdr = part + kCW * 3 * kListRowsMax;   // combined header being built [kCmbHdr]
-    for (int r = warp; r < R; r += kCW) {
-      float M = kNegInf;
-      for (int sl = lane; sl < ns; sl += 32) M = fmaxf(M, sr[sl * rf + 2 * r]);
-      M = warp_max(M);
-      if (!(M > kNegInf) || M != M) {
-        if (lane == 0) atomicOr(p.status, MDS_ST_NONFINITE);
-        M = 0.f;
-      }
-      const float c = P.row[r].c;
-      float z = 0.f;
-      for (int sl = lane; sl < ns; sl += 32) {
-        const float ms = sr[sl * rf + 2 * r];
-        if (ms > kNegInf) z = __fadd_rn(z, __fmul_rn(sr[sl * rf + 2 * r + 1], ref_shift(ms, M, c)));
-      }
-      z = warp_sum(z);
-      if (lane == 0) {
-        hdr[kCmbM + r] = M;
-        hdr[kCmbPc + (r < kListRowsMax ? r : 0)] = z;   // the slices' sums (list passes add the entries left out)
-        if (!list) {
-          if (!(z > 0.f) || !(z < kPosInf) || z != z) {
-            atomicOr(p.status, MDS_ST_NONFINITE);
-            z = 1.f;
-          }
-          hdr[kCmbIz + r] = __frcp_rn(z);
-        }
-      }
-    }
-    if (!list) {
-      cbar();
-      for (int i = tid; i < 2 * kMaxRows; i += kCT) __stcg(rec + i, hdr[i]);
-      return;
-    }
-    // entries: keys (0: no entry), the valid count
-    const int NE = ns * LN;
-    for (int i0 = warp * 32; i0 < NE; i0 += kCT) {   // warp-uniform trips (the ballot below)
-      const int i = i0 + lane;
-      unsigned k = 0u;
-      if (i < NE) {
-        const int sl = i / LN, q = i - sl * LN;
-        if (q < __float_as_int(sr[sl * rf + 2 * kMaxRows + 1]))
-          k = ord_key(__fadd_rn(sr[sl * rf + kHdr + LN + q], 0.f));
-        sk[i] = k;
-      }
-      const unsigned vb = __ballot_sync(FULLM, k != 0u);
-      if (lane == 0 && vb) atomicAdd(&S.cmb_nv, __popc(vb));
-    }
-    cbar();
-    const int nf = min(LF, S.cmb_nv);
-    // rank of each valid entry in the merge order; the first nf are taken
-    for (int i = tid; i < NE; i += kCT) {
-      const unsigned k = sk[i];
-      if (k == 0u) continue;
-      int rank = 0;
-      for (int u = 0; u < NE; ++u) {
-        const unsigned ku = sk[u];
-        rank += (ku > k || (ku == k && u < i)) ? 1 : 0;
-      }
-      if (rank < nf) {
-        fin[rank] = i;
-        atomicAdd(&ksl[i / LN], 1);
-      }
-    }
-    cbar();
-    // tau and the complement masses: entries not taken (and the slices' own tau)
-    float add[kListRowsMax];
-#pragma unroll
-    for (int r = 0; r < kListRowsMax; ++r) add[r] = 0.f;
-    float tau = kNegInf;
-    for (int sl = tid; sl < ns; sl += kCT) tau = fmaxf(tau, sr[sl * rf + 2 * kMaxRows]);
-    for (int i = tid; i < NE; i += kCT) {
-      const int sl = i / LN, q = i - sl * LN;
-      if (q >= ksl[sl] && q < __float_as_int(sr[sl * rf + 2 * kMaxRows + 1])) {
-        const float* e = sr + sl * rf + kHdr + q;
-        tau = fmaxf(tau, e[LN]);
-#pragma unroll
-        for (int r = 0; r < kListRowsMax; ++r)
-          if (r < R) add[r] = __fadd_rn(add[r], exp_term(e[(1 + r) * LN], hdr[kCmbM + r], P.row[r].c));
-      }
-    }
-    tau = warp_max(tau);
-#pragma unroll
-    for (int r = 0; r < kListRowsMax; ++r) add[r] = warp_sum(add[r]);
-    if (lane == 0) {
-      if (tau > kNegInf) atomicMax(&S.cmb_tau, ord_key(tau));
-#pragma unroll
-      for (int r = 0; r < kListRowsMax; ++r) part[warp * 3 * kListRowsMax + r] = add[r];
-    }
-    // the list into the combined record: merge order for the weighted
-    // scheme, token-id order for the truncated alphabet
-    const bool by_id = p.scheme == MDS_WIS0;
-    float* out_id = rec + kCmbHdr;
-    float* out_l0 = out_id + LF;
-    float* out_e = out_l0 + LF;
-    float z[kListRowsMax];
-#pragma unroll
-    for (int r = 0; r < kListRowsMax; ++r) z[r] = 0.f;
-    for (int t = tid; t < nf; t += kCT) {
-      const int i = fin[t];
-      const int sl = i / LN, q = i - sl * LN;
-      const float* e = sr + sl * rf + kHdr + q;
-      const int id = __float_as_int(e[0]);
-      int pos = t;
-      if (by_id) {
-        pos = 0;
-        for (int u = 0; u < nf; ++u) {
-          const int iu = fin[u];
-          const int su = iu / LN, qu = iu - su * LN;
-          pos += (__float_as_int(sr[su * rf + kHdr + qu]) < id) ? 1 : 0;
-        }
-      }
-      __stcg(out_id + pos, __int_as_float(id));
-      __stcg(out_l0 + pos, e[LN]);
-#pragma unroll
-      for (int r = 0; r < kListRowsMax; ++r)
-        if (r < R) {
-          const float ev = exp_term(e[(1 + r) * LN], hdr[kCmbM + r], P.row[r].c);
-          __stcg(out_e + r * LF + pos, ev);
-          z[r] = __fadd_rn(z[r], ev);
-        }
-    }
-#pragma unroll
-    for (int r = 0; r < kListRowsMax; ++r) {
-      z[r] = warp_sum(z[r]);
-      if (lane == 0) part[warp * 3 * kListRowsMax + kListRowsMax + r] = z[r];
-    }
-    cbar();
-    if (tid == 0) {
-      for (int r = 0; r < R; ++r) {
-        float a = 0.f, zz = 0.f;
-        for (int w = 0; w < kCW; ++w) {
-          a = __fadd_rn(a, part[w * 3 * kListRowsMax + r]);
-          zz = __fadd_rn(zz, part[w * 3 * kListRowsMax + kListRowsMax + r]);
-        }
-        const float pc = __fadd_rn(hdr[kCmbPc + r], a);
-        float Z = __fadd_rn(pc, zz);
-        if (!(Z > 0.f) || !(Z < kPosInf) || Z != Z) {
-          atomicOr(p.status, MDS_ST_NONFINITE);
-          Z = 1.f;
-        }
-        hdr[kCmbPc + r] = pc;
-        hdr[kCmbIz + r] = __frcp_rn(Z);
-      }
-      const float t = S.cmb_tau ? ord_val(S.cmb_tau) : kNegInf;
-      hdr[kCmbN] = __int_as_float(nf);
-      hdr[kCmbN + 1] = t;
-      hdr[kCmbN + 2] = __int_as_float(nf == p.V ? 1 : 0);
-      hdr[kCmbN + 3] = (t > kNegInf) ? exp_term(t, hdr[kCmbM], P.row[0].c) : 0.f;
-    }
-    cbar();
-    for (int i = tid; i < kCmbHdr; i += kCT) __stcg(rec + i, hdr[i]);
   }
 
   // -------------------------------------------------------------- full-vocabulary stage task
@@ -1285,15 +1328,173 @@ struct Eng {
     }
   }
 
+  // -------------------------------------------------------------- the publishing warp
+  // Merges the compute warps' results of one slice into its record and counts
+  // the pass's slices; the warp that counts a pass's last slice posts the
+  // decision request.  The compute warps are meanwhile on later slices: the
+  // record's stores, the fence and the counter's round trip (about 3 us) cost
+  // them nothing.  A group of slices is counted once, at its end.
+  //
+  // Rows: the slice maximum and the warps' sums moved to it, warps in order.
+  __device__ void merge_rows(const Slot& T, float (&m)[kListRowsMax], float (&s)[kListRowsMax]) const {
+    const int lane = threadIdx.x & 31;
+    const int w = lane & 7;
+#pragma unroll
+    for (int r = 0; r < kListRowsMax; ++r) {
+      m[r] = kNegInf;
+      s[r] = 0.f;
+      if (r >= T.R) continue;
+      const float mw = T.m[w][r], sw = T.s[w][r];
+      float mm = mw;
+#pragma unroll
+      for (int o = 4; o; o >>= 1) mm = fmaxf(mm, __shfl_xor_sync(FULLM, mm, o));
+      float v = (mw > kNegInf) ? __fmul_rn(sw, ref_shift(mw, mm, T.c[r])) : 0.f;
+#pragma unroll
+      for (int o = 4; o; o >>= 1) v = __fadd_rn(v, __shfl_xor_sync(FULLM, v, o));
+      m[r] = mm;
+      s[r] = v;
+    }
+  }
+  // Rank key of a token set aside: larger first.  A 16-bit logit's key needs
+  // 16 bits, so the place in the slice (below 65536, smaller first) fits
+  // beside it and the keys are distinct; 32-bit logits tie by place apart.
+  __device__ __forceinline__ static unsigned cand_key(float l, int loc) {
+    const unsigned k = ord_key(__fadd_rn(l, 0.f));
+    return DT == MDS_BF16 ? ((k & 0xffff0000u) | (0xffffu - (unsigned)loc)) : k;
+  }
+
+  // The slice's list: the first LN of the tokens set aside, by target logit
+  // (ties: smaller id), with every row's logit; the others rejoin the sums in
+  // rank order, tau covers them and every token not set aside.
+  __device__ void merge_list(Slot& T, float* rec, const float (&m)[kListRowsMax], float (&s)[kListRowsMax]) const {
+    const int lane = threadIdx.x & 31;
+    const int LN = p.lns, n = T.ncand;
+    int* rid = reinterpret_cast<int*>(rec + kHdr);
+    float tau = (lane < kCW) ? T.tau[lane] : kNegInf;
+    // keys past n count for none
+    for (int i = n + lane; i < ((n + 3) & ~3); i += 32) T.key[i] = 0u;
+    __syncwarp();
+    const int tok0 = T.slice * p.T;
+    for (int i = lane; i < n; i += 32) {
+      const unsigned ki = T.key[i];
+      const int ii = tok0 + T.loc[i];
+      int rk = 0;
+      for (int q = 0; q < n; q += 4) {
+        const uint4 o = *reinterpret_cast<const uint4*>(T.key + q);
+        rk += (o.x > ki ? 1 : 0) + (o.y > ki ? 1 : 0) + (o.z > ki ? 1 : 0) + (o.w > ki ? 1 : 0);
+        if constexpr (DT != MDS_BF16) {
+          const int li = T.loc[i];
+          rk += (o.x == ki && q < n && T.loc[q] < li) ? 1 : 0;
+          rk += (o.y == ki && q + 1 < n && T.loc[q + 1] < li) ? 1 : 0;
+          rk += (o.z == ki && q + 2 < n && T.loc[q + 2] < li) ? 1 : 0;
+          rk += (o.w == ki && q + 3 < n && T.loc[q + 3] < li) ? 1 : 0;
+        }
+      }
+      if (rk < LN) {
+        __stcg(rid + rk, ii);
+#pragma unroll
+        for (int r = 0; r < kListRowsMax; ++r)
+          if (r < T.R) __stcg(rec + kHdr + LN * (1 + r) + rk, T.l[r][i]);
+      } else {
+        T.ord[rk - LN] = i;
+      }
+    }
+    __syncwarp();
+    float add[kListRowsMax];
+#pragma unroll
+    for (int r = 0; r < kListRowsMax; ++r) add[r] = 0.f;
+    for (int t = lane; t < n - LN; t += 32) {
+      const int i = T.ord[t];
+      tau = fmaxf(tau, T.l[0][i]);
+#pragma unroll
+      for (int r = 0; r < kListRowsMax; ++r)
+        if (r < T.R && m[r] > kNegInf) add[r] = __fadd_rn(add[r], exp_term(T.l[r][i], m[r], T.c[r]));
+    }
+    tau = warp_max(tau);
+#pragma unroll
+    for (int r = 0; r < kListRowsMax; ++r)
+      if (r < T.R) s[r] = __fadd_rn(s[r], warp_sum(add[r]));
+    if (lane == 0) {
+      __stcg(rec + 2 * kMaxRows, tau);
+      __stcg(reinterpret_cast<int*>(rec) + 2 * kMaxRows + 1, min(n, LN));
+    }
+  }
+
+  __device__ void publisher() {
+    const int lane = threadIdx.x & 31;
+    for (int k = 0;; ++k) {
+      Slot& T = slots[k % kSlots];
+      if (!__all_sync(FULLM, wait_mbar(&S.done[k % kSlots], (k / kSlots) & 1))) {
+        if (lane == 0) set_abort(MDS_ST_TIMEOUT);
+        return;
+      }
+      const int mode = T.mode;
+      if (mode == kSlotExit) return;
+      const int b = T.b, s = T.slice;
+      float* rec = p.rec + ((size_t)b * p.ns + s) * p.rec_floats;
+      PT_T0(t_pub);
+      if (mode == kSlotSums || mode == kSlotList || mode == kSlotBonus) {
+        float m[kListRowsMax], sm[kListRowsMax];
+        merge_rows(T, m, sm);
+        if (mode == kSlotList) merge_list(T, rec, m, sm);
+        if (mode == kSlotBonus) {
+          // the chunks' sums, each against its warp's reference, moved to the slice's
+          for (int q = lane; q < T.nrun; q += 32) {
+            const float mw = T.m[q & (kCW - 1)][0];
+            __stcg(rec + 4 + q, (mw > kNegInf) ? __fmul_rn(T.run[q], ref_shift(mw, m[0], T.c[0])) : 0.f);
+          }
+        }
+        if (lane == 0) {
+#pragma unroll
+          for (int r = 0; r < kListRowsMax; ++r)
+            if (r < T.R) {
+              __stcg(rec + 2 * r, m[r]);
+              __stcg(rec + 2 * r + 1, sm[r]);
+            }
+        }
+      } else if (mode == kSlotRuns) {
+        // run masses, and the slice's: the runs in chunks of 32
+        float tot = 0.f;
+        for (int q0 = 0; q0 < T.nrun; q0 += 32) {
+          const int q = q0 + lane;
+          const float v = q < T.nrun ? T.run[q] : 0.f;
+          if (q < T.nrun) __stcg(rec + 4 + q, v);
+          tot = __fadd_rn(tot, warp_sum(v));
+        }
+        if (lane == 0) __stcg(rec, tot);
+      }
+      const int kind = T.kind, j = T.j, R = T.R, list = T.list;
+      if (kind == kStats && j == 0 && s == 0) {
+        // the sequence's outputs start as -1 (the decisions overwrite them)
+        for (int q = lane; q <= p.L; q += 32) __stcg(p.out_tokens + (size_t)b * (p.L + 1) + q, -1);
+        if (lane == 0) __stcg(p.out_accept + b, -1);
+      }
+      __syncwarp();
+      const int count = T.count;
+      __syncwarp();
+      if (lane == 0) {
+        T.ncand = 0;
+        mbar_arrive(&S.free[k % kSlots]);
+        // the group's records before the count (release; the last one also acquires the others')
+        if (count && atom_add_acq_rel(&p.cnt[b], (unsigned)count) == (unsigned)(p.ns - count)) {
+          __threadfence();
+          post_decision(dec_payload(b, kind, j, R, list));
+        }
+      }
+      PT_ADDW(kPhPublish, t_pub);
+      __syncwarp();
+    }
+  }
+
   // -------------------------------------------------------------- compute warps
-  // The pass of a sequence is complete: publish a decision request (thread
-  // 0, after acquiring every slice's record through the pass counter; the
-  // release of the request's tag passes them on to the decision warp).
+  // The pass of a sequence is complete: publish a decision request (one
+  // thread, after acquiring every slice's record through the pass counter;
+  // the release of the request's tag passes them on to the decision warp).
   __device__ void post_decision(unsigned pay) const {
     const unsigned t = atomicAdd(&p.ctl[kCtlDecTail], 1u);
     const unsigned slot = t % (unsigned)p.dec_cap;
     if (t >= (unsigned)p.dec_cap) {
-      const unsigned long long prev = tag_of(t - (unsigned)p.dec_cap);
+      const unsigned long long prev = dec_tag_of(p.epoch, t - (unsigned)p.dec_cap);
       const unsigned long long t0 = now_ns();
       for (int it = 0; ld_acquire(&p.dec_rtag[slot]) != prev; ++it) {
         if (aborted()) break;
@@ -1305,97 +1506,124 @@ struct Eng {
       }
     }
     __stcg(p.dec_pay + slot, pay);
-    st_release(&p.dec_tag[slot], tag_of(t));
+    st_release(&p.dec_tag[slot], dec_tag_of(p.epoch, t));
   }
 
-  __device__ void process(int bi) {
+  // One slice: this warp's part of the results into T, or (slices too small
+  // for the warp-wise paths, more rows than they take, full stages) the whole
+  // record into global memory.  Thread 0 fills T's description.
+  __device__ void process(int bi, Slot& T) {
     FDesc& Dd = S.desc[bi];
     char* b = buf(bi);
     const int s = Dd.slice, seqb = Dd.b;
     const int tok0 = s * p.T, n = min(p.T, p.V - tok0);
     const FPass& P = Dd.P;
-    if (!p.bulk) load_plain(P, P.nstream, b, tok0, n);
     float* rec = p.rec + ((size_t)seqb * p.ns + s) * p.rec_floats;
     PT_T0(t_task);
     PT_CNT(kPhTasks);
+    int mode = kSlotDone;
+    const int U = (n + VE - 1) / VE;
     switch (P.kind) {
-      case kStats:
       case kBonus:
-        if (P.list) {
+        mode = kSlotBonus;
+        stats_fast<1, false, true>(P, b, tok0, n, T);
+        break;
+      case kStats:
+        if (P.list && p.fast_list) {
+          mode = kSlotList;
           switch (P.nstream) {
-            case 1: stats_small<1, true>(P, b, tok0, n, rec); break;
-            case 2: stats_small<2, true>(P, b, tok0, n, rec); break;
-            case 3: stats_small<3, true>(P, b, tok0, n, rec); break;
-            default: stats_small<4, true>(P, b, tok0, n, rec); break;
+            case 1: stats_fast<1, true, false>(P, b, tok0, n, T); break;
+            case 2: stats_fast<2, true, false>(P, b, tok0, n, T); break;
+            case 3: stats_fast<3, true, false>(P, b, tok0, n, T); break;
+            default: stats_fast<4, true, false>(P, b, tok0, n, T); break;
+          }
+        } else if (P.list) {
+          if (!p.bulk) load_plain(P, P.nstream, b, tok0, n);
+          switch (P.nstream) {
+            case 1: stats_small<1>(P, b, tok0, n, rec); break;
+            case 2: stats_small<2>(P, b, tok0, n, rec); break;
+            case 3: stats_small<3>(P, b, tok0, n, rec); break;
+            default: stats_small<4>(P, b, tok0, n, rec); break;
           }
         } else {
           switch (P.nstream) {
-            case 1: stats_small<1, false>(P, b, tok0, n, rec); break;
-            case 2: stats_small<2, false>(P, b, tok0, n, rec); break;
-            default: stats_rows(P, b, n, rec); break;
+            case 1:
+              mode = kSlotSums;
+              stats_fast<1, false, false>(P, b, tok0, n, T);
+              break;
+            case 2:
+              mode = kSlotSums;
+              stats_fast<2, false, false>(P, b, tok0, n, T);
+              break;
+            default:
+              if (!p.bulk) load_plain(P, P.nstream, b, tok0, n);
+              stats_rows(P, b, n, rec);
+              break;
           }
         }
         break;
       case kResid:
-      case kReplace: resid_task(P, b, tok0, n, rec); break;
-      case kFull: full_task(P, b, tok0, n, rec); break;
+      case kReplace:
+        mode = kSlotRuns;
+        if (!p.bulk) load_own(P, P.nstream, b, tok0, n);
+        resid_task(P, b, tok0, n, T);
+        break;
+      case kFull:
+        if (!p.bulk) load_plain(P, P.nstream, b, tok0, n);
+        full_task(P, b, tok0, n, rec);
+        break;
       default: break;
     }
     PT_ADD(P.kind == kStats ? (P.list ? kPhTaskList : kPhTaskStats)
                             : (P.kind == kBonus ? kPhTaskStats : (P.kind == kFull ? kPhTaskFull : kPhTaskResid)),
            t_task);
-    if (P.kind == kStats && P.j == 0 && s == 0) {
-      // the sequence's outputs start as -1 (the decisions overwrite them)
-      for (int j = threadIdx.x; j <= p.L; j += kCT) __stcg(p.out_tokens + (size_t)seqb * (p.L + 1) + j, -1);
-      if (threadIdx.x == 0) __stcg(p.out_accept + seqb, -1);
+    if (threadIdx.x == 0) {
+      T.mode = mode;
+      T.b = seqb;
+      T.slice = s;
+      T.kind = P.kind;
+      T.j = P.j;
+      T.R = P.nstream;
+      T.list = P.list;
+      T.nrun = (U + 31) / 32;
+      T.count = (s + 1 == Dd.end) ? s + 1 - (s / p.group) * p.group : 0;
     }
-    // publish the record: the barrier orders every thread's record writes
-    // before thread 0's release (acq_rel: the last arriver also acquires the
-    // other slices' records)
-    PT_T0(t_pub);
-    cbar();
-    if (threadIdx.x == 0) S.last = (atom_add_acq_rel(&p.cnt[seqb], 1u) == (unsigned)(p.ns - 1)) ? 1 : 0;
-    cbar();
-    PT_ADD(kPhPublish, t_pub);
-    if (S.last) {
-      // thread 0 acquired the other slices' records; the barrier passes that on
-      PT_T0(t_cmb);
-      if (P.kind == kStats) combine_pass(P, b, rec - (size_t)s * p.rec_floats);
-      cbar();
-      if (threadIdx.x == 0) {
-        __threadfence();   // the combined record before the request
-        post_decision(dec_payload(seqb, P.kind, P.j, P.nstream, P.list));
-      }
-      PT_ADD(kPhCombine, t_cmb);
-    }
+    if (threadIdx.x < kListRowsMax) T.c[threadIdx.x] = P.row[threadIdx.x].c;
   }
 
   __device__ void compute() {
+    const int lane = threadIdx.x & 31;
     for (int k = 0;; ++k) {
-      const int bi = k % kNBuf;
-      const uint32_t par = (k / kNBuf) & 1;
-      // thread 0 waits (bounded); the others then see the completed phase
+      const int bi = k % kNBuf, sl = k % kSlots;
+      // thread 0 waits for the slice and for a free record slot (bounded);
+      // the others then see the completed phases
       PT_T0(t_wait);
       if (threadIdx.x == 0) {
-        const bool ok = wait_mbar(&S.full[bi], par);
+        bool ok = wait_mbar(&S.full[bi], (k / kNBuf) & 1);
+        if (ok) S.consumed = k + 1;
+        if (ok && k >= kSlots) ok = wait_mbar(&S.free[sl], ((k / kSlots) - 1) & 1);
         if (!ok) set_abort(MDS_ST_TIMEOUT);
-        S.flag_ok = ok ? 1 : 0;
-        S.flag_ab = aborted() ? 1 : 0;
+        S.flag_ok[k & 1] = ok ? 1 : 0;
       }
       cbar();
       PT_ADD(kPhWaitFull, t_wait);
-      if (!S.flag_ok) break;
-      while (!mbar_try_wait(&S.full[bi], par)) {
+      if (!S.flag_ok[k & 1]) return;   // the publishing warp's own wait runs out
+      while (!mbar_try_wait(&S.full[bi], (k / kNBuf) & 1)) {
       }
-      if (S.desc[bi].exit) break;
-      if (!S.flag_ab) process(bi);
-      // generic accesses of this buffer before the next bulk copy into it
-      fence_proxy_async();
-      cbar();
-      if (threadIdx.x == 0) {
-        S.consumed = k + 1;
+      Slot& T = slots[sl];
+      const bool leave = S.desc[bi].exit != 0;
+      if (leave) {
+        if (threadIdx.x == 0) T.mode = kSlotExit;
+      } else {
+        process(bi, T);
+      }
+      // this warp is done with the buffer and with its part of the record
+      __syncwarp();
+      if (lane == 0) {
         mbar_arrive(&S.empty[bi]);
+        mbar_arrive(&S.done[sl]);
       }
+      if (leave) return;
     }
   }
 
@@ -1419,7 +1647,6 @@ template <int DT> __device__ __noinline__ void dec_full_nl(int b);
 template <int DT> __device__ __noinline__ void dec_bonus_nl(int b);
 template <int DT> __device__ __noinline__ void dec_wis0_nl(int b);
 template <int DT> __device__ __noinline__ void dec_accept_nl(int b);
-__device__ __forceinline__ int lp_solve5(int s, float A2, float B2, int A, int Btok, float u);
 __device__ __noinline__ int lp_solve8(int s, float A2, float B2, int A, int Btok, float u);
 
 template <int DT>
@@ -1436,9 +1663,6 @@ struct Dec {
   uint32_t* bm;    // special-token bits of a re-read slice [64]
   int lane;
 
-  __device__ __forceinline__ unsigned long long tag_of(unsigned t) const {
-    return ((unsigned long long)p.epoch << 32) | (unsigned long long)(t + 1u);
-  }
   __device__ __forceinline__ bool aborted() const { return ld_relaxed(&p.ctl[kCtlAbort]) != 0u; }
   __device__ __forceinline__ void set_abort(unsigned bits) const {
     atomicOr(p.status, bits);
@@ -1598,23 +1822,25 @@ struct Dec {
   // -------------------------------------------------------------- publishing
   __device__ void push(int b, int kind) {
     PT_T0(t_push);
-    if (lane == 0) D.P.kind = kind;
+    unsigned base = 0u;
+    if (lane == 0) {
+      // ring numbers first: their round trip runs beside the state's stores
+      base = (unsigned)p.B * (unsigned)p.ng + atomicAdd(&p.ctl[kCtlTail], (unsigned)p.ng);
+      D.P.kind = kind;
+    }
     __syncwarp();
     FSeq* g = &reinterpret_cast<FSeq*>(p.seq)[b];
     copy_out(&g->P, &D.P, (int)sizeof(FPass), lane, 32);
     copy_out(&g->W, &D.W, (int)sizeof(FWalk), lane, 32);
     if (lane == 0) __stcg(p.cnt + b, 0u);
-    __threadfence();   // every lane's state writes before any publication
-    __syncwarp();
-    unsigned base = 0u;
-    if (lane == 0) base = (unsigned)p.B * (unsigned)p.ns + atomicAdd(&p.ctl[kCtlTail], (unsigned)p.ns);
     base = __shfl_sync(FULLM, base, 0);
-    for (int i = lane; i < p.ns; i += 32) {
+    for (int i0 = 0; i0 < p.ng; i0 += 32) {
+      const int i = i0 + lane;
       const unsigned t = base + (unsigned)i;
-      const unsigned slot = t % (unsigned)p.ring_cap;
-      if (t >= (unsigned)p.ring_cap) {
+      const unsigned slot = t % (unsigned)p.ring_cap, lap = t / (unsigned)p.ring_cap;
+      if (i < p.ng && lap) {
         // the slot's previous task must have been taken
-        const unsigned long long prev = tag_of(t - (unsigned)p.ring_cap);
+        const unsigned long long prev = ring_word(p.epoch, lap - 1u, 0u);
         const unsigned long long t0 = now_ns();
         for (int it = 0; ld_acquire(&p.ring_rtag[slot]) != prev; ++it) {
           if (aborted()) break;
@@ -1625,8 +1851,10 @@ struct Dec {
           __nanosleep(64);
         }
       }
-      __stcg(p.ring_pay + slot, ((unsigned)b << 16) | (unsigned)i);
-      st_release(&p.ring_tag[slot], tag_of(t));
+      // every lane's state stores (joined by the warp barrier) before any publication
+      __syncwarp();
+      __threadfence();
+      if (i < p.ng) st_relaxed(&p.ring_tag[slot], ring_word(p.epoch, lap, ((unsigned)b << 8) | (unsigned)i));
     }
     __syncwarp();
     PT_ADDW(kPhPush, t_push);
@@ -1712,134 +1940,331 @@ struct Dec {
     __syncwarp();
   }
 
-  // The combined record of a stats pass (staged in scr; written by the CTA
-  // that completed the pass): every row's M and 1/Z and, with candidate
-  // lists, the sequence's list, its complement masses and tau.
-  __device__ void adopt_combined(int R, bool list) {
-    const float* c = reinterpret_cast<const float*>(scr);
-    for (int r = lane; r < R; r += 32) {
-      D.P.row[r].M = c[kCmbM + r];
-      D.P.row[r].invZ = c[kCmbIz + r];
-      if (list) D.pc[r] = c[kCmbPc + r];
-    }
-    if (list) {
-      const int LF = p.ln;
-      const int n = __float_as_int(c[kCmbN]);
-      for (int t = lane; t < n; t += 32) {
-        D.cm_id[t] = __float_as_int(c[kCmbHdr + t]);
-        D.cm_l0[t] = c[kCmbHdr + LF + t];
-        for (int r = 0; r < R; ++r) D.cm_e[r][t] = c[kCmbHdr + (2 + r) * LF + t];
-        D.cm_sp[t] = 0;
-        D.cm_a[t] = 0.f;
+  // Combine the slice records of a stats pass (staged in scr): every row's M
+  // and 1/Z and, with candidate lists, the sequence's list (the first LF of
+  // the slices' entries by target logit, then slice, then position; in
+  // token-id order), its complement masses and tau.  Sums over slices and entries run in fixed orders.
+  __device__ void combine(int R, bool list) {
+    const int ns = p.ns, rf = p.rec_floats;
+    const float* sr = reinterpret_cast<const float*>(scr);
+    for (int r = 0; r < R; ++r) {
+      float M = kNegInf;
+      for (int sl = lane; sl < ns; sl += 32) M = fmaxf(M, sr[sl * rf + 2 * r]);
+      M = warp_max(M);
+      if (!(M > kNegInf) || M != M) {
+        if (lane == 0) atomicOr(p.status, MDS_ST_NONFINITE);
+        M = 0.f;
       }
+      const float c = D.P.row[r].c;
+      float z = 0.f;
+      for (int sl = lane; sl < ns; sl += 32) {
+        const float ms = sr[sl * rf + 2 * r];
+        if (ms > kNegInf) z = __fadd_rn(z, __fmul_rn(sr[sl * rf + 2 * r + 1], ref_shift(ms, M, c)));
+      }
+      z = warp_sum(z);
       if (lane == 0) {
-        D.n = n;
-        D.cand_tau = c[kCmbN + 1];
-        D.cand_all = __float_as_int(c[kCmbN + 2]);
-        D.cand_q = c[kCmbN + 3];
+        D.P.row[r].M = M;
+        if (list)
+          D.pc[r] = z;   // of the slices; the entries not taken join below
+        else
+          finish_row(r, z);
       }
     }
     __syncwarp();
+    if (!list) return;
+    if (ns * p.lns <= 128)
+      combine_list<4>(R);
+    else
+      combine_list<kMaxEntries / 32>(R);
   }
 
-  // -------------------------------------------------------------- WIS stage on the candidate list
-  // One list entry per lane.  Returns false (changing nothing) if
-  // the list cannot certify Omega_1: fewer than s entries, or the s-th key
-  // not above every key outside the list (each such key is <= its q <= q(tau)).
-  __device__ bool wis_stage_list(int A, int Btok, int rb, float u) {
+  // The list part of combine, NT entries per lane at most (the small one
+  // serves all but the shortest rows and the smallest batches; unrolled code
+  // that one warp runs once costs its instruction fetches).
+  template <int NT>
+  __device__ __forceinline__ void combine_list(int R) {
+    const int ns = p.ns, rf = p.rec_floats;
+    const float* sr = reinterpret_cast<const float*>(scr);
+    // the entries' order keys, entry lane + 32 t (0: none); 16-bit logits
+    // differ in the key's upper half only
+    constexpr int kBits = DT == MDS_BF16 ? 16 : 32;
+    const int LN = p.lns, LF = p.ln;
+    unsigned key[NT];
+    unsigned cnt = 0u;
+#pragma unroll
+    for (int t = 0; t < NT; ++t) {
+      key[t] = 0u;
+      const int i = lane + 32 * t, sl = (int)__umulhi((unsigned)i, p.lns_rcp), q = i - sl * LN;
+      if (sl < ns && q < __float_as_int(sr[sl * rf + 2 * kMaxRows + 1]))
+        key[t] = ord_key(__fadd_rn(sr[sl * rf + kHdr + LN + q], 0.f)) >> (32 - kBits);
+      cnt += key[t] ? 1u : 0u;
+    }
+    const int nv = (int)__reduce_add_sync(FULLM, cnt);
+    // the largest key that at least LF entries reach
+    unsigned thr = 0u;
+    int ties = 0;
+    if (nv > LF) {
+#pragma unroll 1
+      for (int bit = kBits - 1; bit >= 0; --bit) {
+        const unsigned cand = thr | (1u << bit);
+        unsigned c = 0u;
+#pragma unroll
+        for (int t = 0; t < NT; ++t)
+          c += key[t] >= cand ? 1u : 0u;
+        if ((int)__reduce_add_sync(FULLM, c) >= LF) thr = cand;
+      }
+      unsigned c = 0u;
+#pragma unroll
+      for (int t = 0; t < NT; ++t)
+        c += key[t] > thr ? 1u : 0u;
+      ties = LF - (int)__reduce_add_sync(FULLM, c);
+    }
+    const unsigned lt = (1u << lane) - 1u;
+    int base = 0, tbase = 0;
+    float tau = kNegInf, add[kListRowsMax], in[kListRowsMax];
+#pragma unroll
+    for (int r = 0; r < kListRowsMax; ++r) add[r] = in[r] = 0.f;
+    for (int sl = lane; sl < ns; sl += 32) tau = fmaxf(tau, sr[sl * rf + 2 * kMaxRows]);
+#pragma unroll
+    for (int t = 0; t < NT; ++t) {
+      const int i = lane + 32 * t, sl = (int)__umulhi((unsigned)i, p.lns_rcp), q = i - sl * LN;
+      const unsigned tm = __ballot_sync(FULLM, key[t] == thr && thr);
+      const bool take = key[t] > thr || (thr && key[t] == thr && tbase + __popc(tm & lt) < ties);
+      const unsigned mk = __ballot_sync(FULLM, take);
+      const int pos = base + __popc(mk & lt);
+      base += __popc(mk);
+      tbase += __popc(tm);
+      if (key[t]) {
+        const float* e = sr + sl * rf + kHdr + q;
+        if (take) {
+          D.cm_id[pos] = __float_as_int(e[0]);
+          D.cm_l0[pos] = e[LN];
+          } else {
+          tau = fmaxf(tau, e[LN]);
+        }
+#pragma unroll
+        for (int r = 0; r < kListRowsMax; ++r)
+          if (r < R) {
+            const float v = exp_term(e[(1 + r) * LN], D.P.row[r].M, D.P.row[r].c);
+            if (take) {
+              D.cm_e[r][pos] = v;
+              in[r] = __fadd_rn(in[r], v);
+            } else {
+              add[r] = __fadd_rn(add[r], v);
+            }
+          }
+      }
+    }
+    const int n = base;
+    tau = warp_max(tau);
+#pragma unroll
+    for (int r = 0; r < kListRowsMax; ++r) {
+      if (r >= R) break;
+      const float a = warp_sum(add[r]), z = warp_sum(in[r]);
+      if (lane == 0) {
+        const float pc = __fadd_rn(D.pc[r], a);
+        D.pc[r] = pc;
+        finish_row(r, __fadd_rn(pc, z));
+      }
+    }
+    if (lane == 0) {
+      D.n = n;
+      D.cand_tau = tau;
+      D.cand_all = (n == p.V) ? 1 : 0;
+      D.cand_q = (tau > kNegInf) ? exp_term(tau, D.P.row[0].M, D.P.row[0].c) : 0.f;
+    }
+    __syncwarp();
+    // token-id order: the lanes of a stage then break ties and order Omega_1
+    // by their number
+    int id[2], at[2] = {0, 0};
+    float l0[2], e[2][kListRowsMax];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int i = lane + 32 * h;
+      id[h] = i < n ? D.cm_id[i] : 0;
+      l0[h] = i < n ? D.cm_l0[i] : 0.f;
+#pragma unroll
+      for (int r = 0; r < kListRowsMax; ++r) e[h][r] = (r < R && i < n) ? D.cm_e[r][i] : 0.f;
+    }
+    for (int u = 0; u < n; ++u) {
+      const int iu = D.cm_id[u];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) at[h] += iu < id[h] ? 1 : 0;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (lane + 32 * h < n) {
+        D.cm_id[at[h]] = id[h];
+        D.cm_l0[at[h]] = l0[h];
+#pragma unroll
+        for (int r = 0; r < kListRowsMax; ++r)
+          if (r < R) D.cm_e[r][at[h]] = e[h][r];
+      }
+    __syncwarp();
+  }
+
+  // -------------------------------------------------------------- WIS stages on the candidate list
+  // The pairwise stages (Remark 4) with one list entry per lane, its state in
+  // registers throughout: the target probability, the rows' probabilities,
+  // the law's explicit value where a stage has set one.  Returns the first
+  // stage the list could not certify (fewer than s entries, or the s-th key
+  // not above every key outside the list, each of which is <= its q <=
+  // q(tau)), nv if none; *Ao the stages' token so far.  The law is left in
+  // the pass (gamma, the special tokens' table).  A stage takes 5k SM cycles
+  // alone (the same through shared memory with the LP on one lane: 9k; 12.7k
+  // with eight decision warps an SM, 7.8k now).
+  __device__ int wis_stages_list(int b, int j, int* Ao) {
+    const int n = D.n, nv = D.nv, R = D.P.nrows;
     const int s = min(p.wis_s, p.V);
-    const int n = D.n;
-    PT_T0(t_sel);
-    {
-      const float iz0 = D.P.row[0].invZ, izb = D.P.row[rb].invZ;
-      const bool have = lane < n;
-      float q = 0.f, a = 0.f, bq = 0.f, key = kNegInf;
-      if (have) {
-        q = __fmul_rn(D.cm_e[0][lane], iz0);
-        if (D.cm_sp[lane]) {
-          a = D.cm_a[lane];
-        } else {
-          for (int r = 1; r < D.P.nrows; ++r)
-            if (D.P.row[r].gamma != 0.f) a = __fmaf_rn(D.P.row[r].gamma, __fmul_rn(D.cm_e[r][lane], D.P.row[r].invZ), a);
+    const bool have = lane < n;
+    const int id = have ? D.cm_id[lane] : 0x7fffffff;
+    const float q = have ? __fmul_rn(D.cm_e[0][lane], D.P.row[0].invZ) : 0.f;
+    const float qout = __fmul_rn(__fmul_rn(D.cand_q, D.P.row[0].invZ), 1.0001f);
+    float pr[kListRowsMax], pz[kListRowsMax], gm[kListRowsMax];   // rows 1.. : here, outside the list, coefficient
+#pragma unroll
+    for (int r = 1; r < kListRowsMax; ++r) {
+      const float iz = r < R ? D.P.row[r].invZ : 0.f;
+      pr[r] = (r < R && have) ? __fmul_rn(D.cm_e[r][lane], iz) : 0.f;
+      pz[r] = r < R ? __fmul_rn(D.pc[r], iz) : 0.f;
+      gm[r] = r == D.vrow[0] ? 1.f : 0.f;
+    }
+    bool sp = false;
+    float as = 0.f;
+    int A = D.X[0], m = 1;
+#pragma unroll 1
+    for (; m < nv; ++m) {
+      PT_T0(t_sel);
+      const float u = D.dr[kDrSelect + m - 1];
+      const int rb = D.vrow[m], Btok = D.X[m];
+      float a = 0.f, bq = 0.f, sa = 0.f, sb = 0.f;
+#pragma unroll
+      for (int r = 1; r < kListRowsMax; ++r) {
+        if (r >= R) break;
+        a = __fmaf_rn(gm[r], pr[r], a);
+        sa = __fmaf_rn(gm[r], pz[r], sa);
+        if (r == rb) {
+          bq = pr[r];
+          sb = pz[r];
         }
-        bq = __fmul_rn(D.cm_e[rb][lane], izb);
-        key = __fadd_rn(__fmaf_rn(-a, bq, q), 0.f);   // -0 -> +0: keys compare as floats
       }
-      // Omega_1: s rounds of a warp max over order-preserving keys, ties to
-      // the smaller token id (the list is in logit order, not id order)
-      const int myid = have ? D.cm_id[lane] : 0x7fffffff;
-      unsigned kk = have ? ord_key(key) : 0u;
-      uint32_t selm = 0u;
-      float kth = kNegInf;
-      for (int t = 0; t < s; ++t) {
-        const unsigned km = __reduce_max_sync(FULLM, kk);
-        if (!km) break;
-        const int idm = __reduce_min_sync(FULLM, (kk == km) ? myid : 0x7fffffff);
-        const uint32_t who = __ballot_sync(FULLM, kk == km && myid == idm);
-        const int wl = __ffs(who) - 1;
-        selm |= 1u << wl;
-        if (lane == wl) kk = 0u;
-        kth = ord_val(km);
+      if (sp) a = as;
+      const float key = __fadd_rn(__fmaf_rn(-a, bq, q), 0.f);   // -0 -> +0: keys compare as floats
+      // Omega_1: the entries with fewer than s larger keys; where the last of
+      // them tie, the smaller token ids (the lower lanes)
+      const unsigned kk = have ? ord_key(key) : 0u;
+      D.kx[lane] = kk;
+      __syncwarp();
+      int above = 0;
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        const uint4 o = reinterpret_cast<const uint4*>(D.kx)[c];
+        above += (o.x > kk ? 1 : 0) + (o.y > kk ? 1 : 0) + (o.z > kk ? 1 : 0) + (o.w > kk ? 1 : 0);
       }
+      uint32_t selm = __ballot_sync(FULLM, have && above < s);
+      if (__popc(selm) > s) {
+        const int last = (int)__reduce_max_sync(FULLM, (selm >> lane & 1u) ? (unsigned)above : 0u);
+        const uint32_t tie = __ballot_sync(FULLM, have && above == last);
+        selm = __ballot_sync(FULLM, (selm >> lane & 1u) &&
+                                        (above < last || __popc(tie & ((1u << lane) - 1u)) < s - last));
+      }
+      const unsigned kth = __reduce_min_sync(FULLM, (selm >> lane & 1u) ? kk : FULLM);
+      if (__popc(selm) != s || !(D.cand_all || ord_val(kth) > qout)) break;
       const bool sel = (selm >> lane) & 1u;
-      const float qout = __fmul_rn(__fmul_rn(D.cand_q, iz0), 1.0001f);
-      const bool ok = __popc(selm) == s && (D.cand_all || kth > qout);
-      const float ra = warp_sum((have && !sel) ? a : 0.f);
-      const float rbm = warp_sum((have && !sel) ? bq : 0.f);
-      if (!ok) {
-        if (lane == 0) D.fast_ok = 0;
-      } else {
-        // position in Omega_1 by token id
-        int rk = 0;
-        for (uint32_t mm = selm; mm; mm &= mm - 1u) rk += (__shfl_sync(FULLM, myid, __ffs(mm) - 1) < myid) ? 1 : 0;
-        if (lane >= s && lane < MDS_MAX_S) {
-          D.om[lane] = -1;
-          D.om_q[lane] = 0.f;
-          D.om_a[lane] = 0.f;
-          D.om_b[lane] = 0.f;
-        }
-        if (sel) {
-          D.om[rk] = D.cm_id[lane];
-          D.om_q[rk] = q;
-          D.om_a[rk] = a;
-          D.om_b[rk] = bq;
-        }
-        __syncwarp();
-        PT_ADDW(kPhDecSelect, t_sel);
-        if (lane == 0) {
-          // Omega_2 masses: complement (generic law) + list entries outside Omega_1
-          float sa = 0.f;
-          for (int r = 1; r < D.P.nrows; ++r)
-            if (D.P.row[r].gamma != 0.f) sa = __fmaf_rn(D.P.row[r].gamma, __fmul_rn(D.pc[r], D.P.row[r].invZ), sa);
-          const float sb = __fadd_rn(__fmul_rn(D.pc[rb], izb), rbm);
-          sa = __fadd_rn(sa, ra);
-          D.Y = solve(s, sa, sb, A, Btok, u);
-          D.A2 = sa;
-          D.B2 = sb;
-          D.fast_ok = 1;
-        }
-        __syncwarp();
-        const float A2 = D.A2, B2 = D.B2;
-        if (sel) {
-          D.cm_a[lane] = D.om_x[rk];
-          D.cm_sp[lane] = 1;
-        } else if (have && D.cm_sp[lane]) {
-          D.cm_a[lane] = __fmul_rn(0.5f, __fadd_rn(__fmul_rn(a, B2), __fmul_rn(bq, A2)));
-        }
-        __syncwarp();
-        if (lane == 0) gamma_update(rb, A2, B2);
+      // Omega_2 masses: complement (generic law) + list entries outside Omega_1
+      float ra = (have && !sel) ? a : 0.f, rbm = (have && !sel) ? bq : 0.f;
+#pragma unroll
+      for (int o = 16; o; o >>= 1) {
+        ra = __fadd_rn(ra, __shfl_xor_sync(FULLM, ra, o));
+        rbm = __fadd_rn(rbm, __shfl_xor_sync(FULLM, rbm, o));
       }
+      const float A2 = __fadd_rn(sa, ra), B2 = __fadd_rn(sb, rbm);
+      const int rk = __popc(selm & ((1u << lane) - 1u));   // position in Omega_1 by token id
+      if (lane >= s && lane < MDS_MAX_S) {
+        D.om[lane] = -1;
+        D.om_q[lane] = 0.f;
+        D.om_a[lane] = 0.f;
+        D.om_b[lane] = 0.f;
+      }
+      if (sel) {
+        D.om[rk] = id;
+        D.om_q[rk] = q;
+        D.om_a[rk] = a;
+        D.om_b[rk] = bq;
+      }
+      __syncwarp();
+      PT_ADDW(kPhDecSelect, t_sel);
+      PT_T0(t_lp);
+      float xr = 0.f;
+      if (s <= 5) {
+        float x[5];
+        bool capped;
+        A = stage_solve5(A2, B2, A, Btok, u, D.om, D.om_q, D.om_a, D.om_b, x, &capped);
+        if (capped && lane == 0) atomicOr(p.status, MDS_ST_LP_CAP);
+#pragma unroll
+        for (int t = 0; t < 5; ++t)
+          if (rk == t) xr = x[t];
+      } else {
+        if (lane == 0) D.Y = lp_solve8(s, A2, B2, A, Btok, u);
+        __syncwarp();
+        A = D.Y;
+        xr = D.om_x[rk & (MDS_MAX_S - 1)];
+      }
+      PT_ADDW(kPhLp, t_lp);
+      PT_CNTW(kPhLpCalls);
+      if (sel) {
+        as = xr;
+        sp = true;
+      } else if (sp) {
+        as = __fmul_rn(0.5f, __fadd_rn(__fmul_rn(a, B2), __fmul_rn(bq, A2)));
+      }
+      // generic law: gamma <- (B2/2) gamma + (A2/2) e_rb
+      const float hB = __fmul_rn(0.5f, B2), hA = __fmul_rn(0.5f, A2);
+#pragma unroll
+      for (int r = 1; r < kListRowsMax; ++r) {
+        gm[r] = __fmul_rn(hB, gm[r]);
+        if (r == rb) gm[r] = __fadd_rn(gm[r], hA);
+      }
+      __syncwarp();   // the tables are read before the next stage writes them
+    }
+    // the law into the pass: coefficients and the special tokens' table
+    const uint32_t spm = __ballot_sync(FULLM, sp);
+    if (sp) {
+      const int k = __popc(spm & ((1u << lane) - 1u));
+      D.P.spec_id[k] = id;
+      D.P.spec_val[k] = as;
+    }
+    if (lane == 0) {
+      D.P.nspec = __popc(spm);
+#pragma unroll
+      for (int r = 1; r < kListRowsMax; ++r)
+        if (r < R) D.P.row[r].gamma = gm[r];
     }
     __syncwarp();
-    return D.fast_ok != 0;
+    *Ao = A;
+    return m;
   }
 
-  // The stage LP on one thread.  Out of line, so that it has the kernel's
-  // whole register budget: s <= 5 keeps its pair state in registers, larger
-  // s in shared memory.
+  // The stage LP on the tables om, om_q, om_a, om_b (warp-wide): p_I on
+  // Omega_1 to om_x, the stage's token returned.
   __device__ int solve(int s, float A2, float B2, int A, int Btok, float u) {
     PT_T0(t_lp);
-    const int y = (s <= 5) ? lp_solve5(s, A2, B2, A, Btok, u) : lp_solve8(s, A2, B2, A, Btok, u);
+    int y;
+    if (s <= 5) {
+      float x[5];
+      bool capped;
+      y = stage_solve5(A2, B2, A, Btok, u, D.om, D.om_q, D.om_a, D.om_b, x, &capped);
+      if (capped && lane == 0) atomicOr(p.status, MDS_ST_LP_CAP);
+      if (lane == 0) {
+#pragma unroll
+        for (int t = 0; t < 5; ++t) D.om_x[t] = x[t];
+      }
+    } else {
+      if (lane == 0) D.Y = lp_solve8(s, A2, B2, A, Btok, u);
+      __syncwarp();
+      y = D.Y;
+    }
+    __syncwarp();
     PT_ADDW(kPhLp, t_lp);
     PT_CNTW(kPhLpCalls);
     return y;
@@ -1852,33 +2277,19 @@ struct Dec {
     D.P.row[rb].gamma = __fadd_rn(D.P.row[rb].gamma, hA);
   }
 
-  // The list's special tokens into the table form used by the residual and
-  // the point lookups.  One thread.
-  __device__ void list_to_table() {
-    int k = 0;
-    for (int i = 0; i < D.n && k < kMaxSpecial; ++i)
-      if (D.cm_sp[i]) {
-        D.P.spec_id[k] = D.cm_id[i];
-        D.P.spec_val[k] = D.cm_a[i];
-        ++k;
-      }
-    D.P.nspec = k;
-  }
-
   // -------------------------------------------------------------- decisions per pass kind
   __device__ void accept_step(int b) {
     PT_T0(t_acc);
     int walk_now = 0;
     if (lane == 0) {
-      const int j = D.P.j;
-      const float u = draw_uniform(p.seed, b, j, kDrawAccept);
+      const float u = D.dr[kDrAccept];
       const float ratio = D.W.pIY > 0.f ? __fdiv_rn(D.W.qY, D.W.pIY) : kPosInf;
       const bool acc = u < fminf(1.f, ratio);
       D.W.acc = acc ? 1 : 0;
       D.W.Ydiag = D.W.Y;
       walk_now = (acc && !p.acc_prob) ? 1 : 0;
       if (!walk_now) {
-        D.W.ures = acc ? 0.f : draw_uniform(p.seed, b, j, kDrawResidual);
+        D.W.ures = acc ? 0.f : D.dr[kDrResidual];
         if (p.scheme == MDS_SINGLE || D.nv == 1 || p.scheme != MDS_WIS) {
           // residual against one draft law: rows 0 and the first valid branch's
           for (int r = 0; r < D.P.nrows; ++r) D.P.row[r].gamma = 0.f;
@@ -1910,7 +2321,7 @@ struct Dec {
     plan_warp(b, j, D.W.valid, false, true, true, D.tk0);
     PT_ADDW(kPhDecPlan, t_plan);
     PT_T0(t_comb);
-    adopt_combined(R, list);
+    combine(R, list);
     if (p.dbg_rows) debug_rows(b, j, R);
     xl_sync();
     PT_ADDW(kPhDecCombine, t_comb);
@@ -1940,16 +2351,7 @@ struct Dec {
     __syncwarp();
     int A = D.X[0];
     int m = 1;
-    if (list) {
-      // every stage's selection uniform at once (lane m - 1 draws stage m's)
-      const float ul = (lane + 1 < D.nv) ? draw_uniform(p.seed, b, j, kDrawSelect + lane) : 0.f;
-      for (; m < D.nv; ++m) {
-        const float u = __shfl_sync(FULLM, ul, m - 1);
-        if (!wis_stage_list(A, D.X[m], D.vrow[m], u)) break;
-        A = D.Y;
-      }
-      if (lane == 0) list_to_table();
-    }
+    if (list) m = wis_stages_list(b, j, &A);
     if (lane == 0) {
       D.W.stage = m;
       D.W.A = A;
@@ -1979,7 +2381,7 @@ struct Dec {
     plan_warp(b, j, D.W.valid, false, false, false, D.tk0);
     const int m = D.W.stage;
     const int A = D.W.A, Btok = D.X[m], rb = D.vrow[m];
-    const float u = draw_uniform(p.seed, b, j, kDrawSelect + m - 1);
+    const float u = D.dr[kDrSelect + m - 1];
     const int s = min(p.wis_s, p.V);
     const float* recb = p.rec + (size_t)b * ns * p.rec_floats;
     for (int r = 0; r < s; ++r) {
@@ -2074,18 +2476,16 @@ struct Dec {
           qk[y - 1] = tf;
         }
       for (int t = 0; t < MDS_MAX_S; ++t) {
-        D.om[t] = om[t];
+        D.om[t] = (t < s) ? om[t] : -1;
         D.om_a[t] = ak[t];
         D.om_b[t] = bk[t];
         D.om_q[t] = qk[t];
       }
-      D.Y = solve(s, ra, rbs, A, Btok, u);
-      D.A2 = ra;
-      D.B2 = rbs;
     }
     __syncwarp();
+    const float A2 = ra, B2 = rbs;
+    const int Y = solve(s, A2, B2, A, Btok, u);
     // law update: special tokens outside Omega_1, gamma, Omega_1 values
-    const float A2 = D.A2, B2 = D.B2;
     for (int i = lane; i < D.P.nspec; i += 32) {
       const int tokn = D.P.spec_id[i];
       bool in1 = false;
@@ -2106,7 +2506,7 @@ struct Dec {
         }
         if (i < kMaxSpecial) D.P.spec_val[i] = D.om_x[t];
       }
-      D.W.A = D.Y;
+      D.W.A = Y;
       D.W.stage = m + 1;
       if (m + 1 < D.nv) D.P.rb = D.vrow[m + 1];
     }
@@ -2116,7 +2516,6 @@ struct Dec {
       return;
     }
     if (lane == 0) {
-      const int Y = D.W.A;
       D.W.Y = Y;
       D.W.qY = prob_row(D.P, 0, Y);
       D.W.pIY = law_at(D.P, Y);
@@ -2184,11 +2583,11 @@ struct Dec {
 
   // The smallest token whose running mass exceeds T, else the last token
   // with positive weight.  Four levels in token order, each a warp scan:
-  // the slices (masses Rs[0..ns)), the slice's 32 runs of upl units (masses
-  // from its staged record when `runs`, else summed from a re-read), the
-  // owning run's units (re-read, one per lane), the owning unit's tokens (in
-  // that lane's registers).
-  __device__ int search(FPass& P, float T, bool runs) {
+  // the slices (masses Rs[0..ns)), the slice's runs of 32 units (masses from
+  // its staged record, two per lane; the bonus row's against the slice's own
+  // maximum), the owning run's units (re-read, one per lane), the owning
+  // unit's tokens (in that lane's registers).
+  __device__ int search(FPass& P, float T, bool bonus) {
     // level 0: slices
     int s = -1, slast = -1;
     float base = 0.f, blast = 0.f;
@@ -2228,76 +2627,38 @@ struct Dec {
       }
       __syncwarp();
     }
-    // level 1: runs of upl units, one per lane
-    const int upl = (U + 31) / 32;
-    const int u0 = min(U, lane * upl), u1 = min(U, u0 + upl);
-    float part = 0.f;
-    if (runs) {
-      part = reinterpret_cast<const float*>(scr)[s * p.rec_floats + 4 + lane];
-    } else {
-      for (int u = u0; u < u1; ++u) {
-        float w[VE];
-        weights_g(P, u, tok0, n, w);
+    // level 1: runs lane and 32 + lane
+    const int nrun = (U + 31) / 32;
+    const float* rr = reinterpret_cast<const float*>(scr) + s * p.rec_floats + 4;
+    const float sc = bonus ? __fmul_rn(ref_shift(Hm[s], P.row[0].M, P.row[0].c), P.row[0].invZ) : 1.f;
+    const float r0 = lane < nrun ? __fmul_rn(rr[lane], sc) : 0.f;
+    const float r1 = lane + 32 < nrun ? __fmul_rn(rr[lane + 32], sc) : 0.f;
+    const float i0 = scan_incl(r0, lane);
+    const float i1 = __fadd_rn(__shfl_sync(FULLM, i0, 31), scan_incl(r1, lane));
+    const unsigned h0 = __ballot_sync(FULLM, __fadd_rn(base, i0) > T && r0 > 0.f);
+    const unsigned h1 = __ballot_sync(FULLM, __fadd_rn(base, i1) > T && r1 > 0.f);
+    const unsigned z0 = __ballot_sync(FULLM, r0 > 0.f), z1 = __ballot_sync(FULLM, r1 > 0.f);
+    if (!(z0 | z1)) return tok0;   // no mass in the slice (only by rounding)
+    const int own = h0 ? __ffs(h0) - 1 : (h1 ? 31 + __ffs(h1) : (z1 ? 63 - __clz(z1) : 31 - __clz(z0)));
+    const float run = __fadd_rn(base, own < 32 ? __shfl_sync(FULLM, __fsub_rn(i0, r0), own & 31)
+                                               : __shfl_sync(FULLM, __fsub_rn(i1, r1), own & 31));
+    // level 2: the run's units, one per lane; level 3 in the owning lane
+    const int u = own * 32 + lane;
+    float w[VE], us = 0.f;
 #pragma unroll
-        for (int e = 0; e < VE; ++e) part = __fadd_rn(part, w[e]);
-      }
+    for (int e = 0; e < VE; ++e) w[e] = 0.f;
+    if (u < U) {
+      weights_g(P, u, tok0, n, w);
+#pragma unroll
+      for (int e = 0; e < VE; ++e) us = __fadd_rn(us, w[e]);
     }
-    const float incl = scan_incl(part, lane);
-    const float excl = __fadd_rn(base, __fsub_rn(incl, part));
-    const unsigned hit1 = __ballot_sync(FULLM, __fadd_rn(base, incl) > T && part > 0.f);
-    const unsigned pos1 = __ballot_sync(FULLM, part > 0.f);
-    if (!pos1) return tok0;   // no mass in the slice (only by rounding)
-    const int own = hit1 ? __ffs(hit1) - 1 : 31 - __clz(pos1);
-    // level 2: the owning run's units, one per lane (chunks of 32); level 3
-    // in the owning lane
-    float run = __shfl_sync(FULLM, excl, own);
-    const int v0 = __shfl_sync(FULLM, u0, own), v1 = __shfl_sync(FULLM, u1, own);
-    int ulast = -1;
-    float ubase_last = 0.f;
-    for (int c0 = v0; c0 < v1; c0 += 32) {
-      const int u = c0 + lane;
-      float w[VE], us = 0.f;
-#pragma unroll
-      for (int e = 0; e < VE; ++e) w[e] = 0.f;
-      if (u < v1) {
-        weights_g(P, u, tok0, n, w);
-#pragma unroll
-        for (int e = 0; e < VE; ++e) us = __fadd_rn(us, w[e]);
-      }
-      const float ui = scan_incl(us, lane);
-      const float uex = __fadd_rn(run, __fsub_rn(ui, us));
-      const unsigned h2 = __ballot_sync(FULLM, __fadd_rn(run, ui) > T && us > 0.f);
-      const unsigned p2 = __ballot_sync(FULLM, us > 0.f);
-      if (h2) {
-        const int l2 = __ffs(h2) - 1;
-        int tok = 0;
-        if (lane == l2) {
-          float acc = uex;
-          int hit = -1, last = -1;
-#pragma unroll
-          for (int e = 0; e < VE; ++e) {
-            if (w[e] > 0.f) last = e;
-            acc = __fadd_rn(acc, w[e]);
-            if (hit < 0 && acc > T && w[e] > 0.f) hit = e;
-          }
-          if (hit < 0) hit = last < 0 ? 0 : last;
-          tok = min(tok0 + u * VE + hit, p.V - 1);
-        }
-        return __shfl_sync(FULLM, tok, l2);
-      }
-      if (p2) {
-        const int l2 = 31 - __clz(p2);
-        ulast = c0 + l2;
-        ubase_last = __shfl_sync(FULLM, uex, l2);
-      }
-      run = __shfl_sync(FULLM, __fadd_rn(run, ui), 31);
-    }
-    // T beyond the run's mass (only by rounding): the last unit with mass
-    int tok = tok0;
-    if (lane == 0 && ulast >= 0) {
-      float w[VE];
-      weights_g(P, ulast, tok0, n, w);
-      float acc = ubase_last;
+    const float ui = scan_incl(us, lane);
+    const unsigned h2 = __ballot_sync(FULLM, __fadd_rn(run, ui) > T && us > 0.f);
+    const unsigned z2 = __ballot_sync(FULLM, us > 0.f);
+    const int l2 = h2 ? __ffs(h2) - 1 : (z2 ? 31 - __clz(z2) : 0);
+    int tok = 0;
+    if (lane == l2) {
+      float acc = __fadd_rn(run, __fsub_rn(ui, us));
       int hit = -1, last = -1;
 #pragma unroll
       for (int e = 0; e < VE; ++e) {
@@ -2306,20 +2667,21 @@ struct Dec {
         if (hit < 0 && acc > T && w[e] > 0.f) hit = e;
       }
       if (hit < 0) hit = last < 0 ? 0 : last;
-      tok = min(tok0 + ulast * VE + hit, p.V - 1);
+      tok = min(tok0 + u * VE + hit, p.V - 1);
     }
-    return __shfl_sync(FULLM, tok, 0);
+    return __shfl_sync(FULLM, tok, l2);
   }
 
-  // Slice masses of the pass just completed (Rs) and their total in slice order.
+  // Slice masses of the pass just completed (Rs) and their total.
   __device__ float slice_masses(int b) {
     const float* rec = reinterpret_cast<const float*>(scr);
-    for (int q = lane; q < p.ns; q += 32) Rs[q] = rec[q * p.rec_floats];
-    __syncwarp();
     float R = 0.f;
-    if (lane == 0)
-      for (int q = 0; q < p.ns; ++q) R = __fadd_rn(R, Rs[q]);
-    return __shfl_sync(FULLM, R, 0);
+    for (int q = lane; q < p.ns; q += 32) {
+      Rs[q] = rec[q * p.rec_floats];
+      R = __fadd_rn(R, Rs[q]);
+    }
+    __syncwarp();
+    return warp_sum(R);
   }
 
   __device__ void decide_resid(int b) {
@@ -2328,7 +2690,7 @@ struct Dec {
     int Z = D.W.Y;
     if (!D.W.acc) {
       if (R > 0.f) {
-        Z = search(D.P, __fmul_rn(D.W.ures, R), true);
+        Z = search(D.P, __fmul_rn(D.W.ures, R), false);
       } else {
         // zero residual mass (only by rounding): sample the target row
         if (lane == 0) {
@@ -2352,7 +2714,7 @@ struct Dec {
     const float R = slice_masses(b);
     int Z;
     if (R > 0.f) {
-      Z = search(D.P, __fmul_rn(D.W.ures, R), true);
+      Z = search(D.P, __fmul_rn(D.W.ures, R), false);
     } else if (!D.W.zres && D.W.Yp >= 0) {
       Z = D.W.Yp;   // no target mass outside Omega_0
     } else if (!D.W.zres) {
@@ -2375,24 +2737,25 @@ struct Dec {
 
   __device__ void decide_bonus(int b) {
     const float* rec = reinterpret_cast<const float*>(scr);
+    float M = kNegInf;
     for (int q = lane; q < p.ns; q += 32) {
       Hm[q] = rec[q * p.rec_floats];
       Rs[q] = rec[q * p.rec_floats + 1];
+      M = fmaxf(M, Hm[q]);
     }
-    __syncwarp();
+    M = warp_max(M);
+    if (!(M > kNegInf) || M != M) {
+      if (lane == 0) atomicOr(p.status, MDS_ST_NONFINITE);
+      M = 0.f;
+    }
+    const float c = D.P.row[0].c;
+    float Zs = 0.f;
+    for (int q = lane; q < p.ns; q += 32)
+      if (Hm[q] > kNegInf) Zs = __fadd_rn(Zs, __fmul_rn(Rs[q], ref_shift(Hm[q], M, c)));
+    Zs = warp_sum(Zs);
     if (lane == 0) {
-      float M = kNegInf;
-      for (int q = 0; q < p.ns; ++q) M = fmaxf(M, Hm[q]);
-      if (!(M > kNegInf) || M != M) {
-        atomicOr(p.status, MDS_ST_NONFINITE);
-        M = 0.f;
-      }
-      const float c = D.P.row[0].c;
-      float Z = 0.f;
-      for (int q = 0; q < p.ns; ++q)
-        if (Hm[q] > kNegInf) Z = __fadd_rn(Z, __fmul_rn(Rs[q], ref_shift(Hm[q], M, c)));
       D.P.row[0].M = M;
-      finish_row(0, Z);
+      finish_row(0, Zs);
     }
     __syncwarp();
     if (p.dbg_rows && lane == 0) {
@@ -2402,15 +2765,15 @@ struct Dec {
       o[2] = D.P.row[0].c;
       o[3] = (float)(__ffs(D.W.valid) - 1);
     }
-    const float M = D.P.row[0].M, c = D.P.row[0].c, iz = D.P.row[0].invZ;
-    for (int q = lane; q < p.ns; q += 32)
-      Rs[q] = (Hm[q] > kNegInf) ? __fmul_rn(__fmul_rn(Rs[q], ref_shift(Hm[q], M, c)), iz) : 0.f;
-    __syncwarp();
+    const float iz = D.P.row[0].invZ;
     float Q = 0.f;
-    if (lane == 0)
-      for (int q = 0; q < p.ns; ++q) Q = __fadd_rn(Q, Rs[q]);
-    Q = __shfl_sync(FULLM, Q, 0);
-    const int Z = search(D.P, __fmul_rn(draw_uniform(p.seed, b, p.L, kDrawBonus), Q), false);
+    for (int q = lane; q < p.ns; q += 32) {
+      Rs[q] = (Hm[q] > kNegInf) ? __fmul_rn(__fmul_rn(Rs[q], ref_shift(Hm[q], M, c)), iz) : 0.f;
+      Q = __fadd_rn(Q, Rs[q]);
+    }
+    __syncwarp();
+    Q = warp_sum(Q);
+    const int Z = search(D.P, __fmul_rn(D.dr[kDrBonus], Q), true);
     if (lane == 0) {
       __stcg(p.out_tokens + (size_t)b * (p.L + 1) + p.L, Z);
       if (p.out_diag) {
@@ -2471,7 +2834,6 @@ struct Dec {
   // The list (token-id order, up to 64 entries) sits two entries per lane:
   // entry lane (half 0) and 32 + lane (half 1).
   __device__ void wis0_decide(int b) {
-    const int j = D.P.j;
     {
       const int n = D.n;
       bool have[2], in0[2];
@@ -2555,7 +2917,7 @@ struct Dec {
       float qY = 0.f, pIY = 0.f, R = 0.f;
       if (n0 > 0 && nk == 0) {
         float t;
-        yl = lane_cdf2(qt[0], qt[1], draw_uniform(p.seed, b, j, kDrawResidual), &t);
+        yl = lane_cdf2(qt[0], qt[1], D.dr[kDrResidual], &t);
       } else if (n0 > 0) {
         float a[2];
         {
@@ -2570,7 +2932,7 @@ struct Dec {
           const int Bl = D.k_lane[m];
           const float* wb = ew + D.k_row[m] * 64;
           const float bb[2] = {wb[lane], wb[lane + 32]};
-          const float u = draw_uniform(p.seed, b, j, kDrawSelect + m - 1);
+          const float u = D.dr[kDrSelect + m - 1];
           unsigned kk[2];
 #pragma unroll
           for (int h = 0; h < 2; ++h) kk[h] = in0[h] ? ord_key(__fadd_rn(__fmaf_rn(-a[h], bb[h], qt[h]), 0.f)) : 0u;
@@ -2611,9 +2973,7 @@ struct Dec {
               D.om_b[rk1[h]] = bb[h];
             }
           __syncwarp();
-          if (lane == 0) D.Y = solve(sn, A2, B2, D.cm_id[A], D.cm_id[Bl], u);
-          __syncwarp();
-          const int Yt = D.Y;
+          const int Yt = solve(sn, A2, B2, D.cm_id[A], D.cm_id[Bl], u);
           const unsigned y0 = __ballot_sync(FULLM, in0[0] && id[0] == Yt);
           const unsigned y1 = __ballot_sync(FULLM, in0[1] && id[1] == Yt);
           A = y0 ? __ffs(y0) - 1 : (y1 ? 32 + __ffs(y1) - 1 : 0);
@@ -2628,10 +2988,10 @@ struct Dec {
         qY = __shfl_sync(FULLM, Ah ? qt[1] : qt[0], Alane);
         pIY = __shfl_sync(FULLM, Ah ? a[1] : a[0], Alane);
         const float ratio = pIY > 0.f ? __fdiv_rn(qY, pIY) : kPosInf;
-        if (draw_uniform(p.seed, b, j, kDrawAccept) < fminf(1.f, ratio)) {
+        if (D.dr[kDrAccept] < fminf(1.f, ratio)) {
           yl = A;
         } else {
-          const float ures = draw_uniform(p.seed, b, j, kDrawResidual);
+          const float ures = D.dr[kDrResidual];
           yl = lane_cdf2(in0[0] ? fmaxf(0.f, __fsub_rn(qt[0], a[0])) : 0.f,
                          in0[1] ? fmaxf(0.f, __fsub_rn(qt[1], a[1])) : 0.f, ures, &R);
           if (yl < 0) {   // only by rounding: sample q~
@@ -2653,10 +3013,10 @@ struct Dec {
         D.W.qY = qY;
         D.W.pIY = pIY;
         D.W.zres = 0;
-        const bool keep = D.o0_n > 0 && (D.o0_all || draw_uniform(p.seed, b, j, kDrawKeep) < D.o0_pa);
+        const bool keep = D.o0_n > 0 && (D.o0_all || D.dr[kDrKeep] < D.o0_pa);
         D.tok = keep ? 1 : 0;
         if (!keep) {
-          D.W.ures = draw_uniform(p.seed, b, j, kDrawOutside);
+          D.W.ures = D.dr[kDrOutside];
           D.P.cut = cut;
           D.P.all0 = D.o0_all;
           D.P.nstream = 1;
@@ -2695,6 +3055,7 @@ struct Dec {
       const int n16 = p.ns * p.rec_floats / 4;
       for (int i = lane; i < n16; i += 32) cpa16(scr + 16 * i, recb + 4 * i);
     }
+    if (lane < kDrawsN) D.dr[lane] = draw_uniform(p.seed, b, j, draw_id(lane));   // beside the copies
     cpa_wait();
     __syncwarp();
     if (lane == 0) {
@@ -2729,7 +3090,7 @@ struct Dec {
       if (lane == 0 && !aborted()) {
         const unsigned t = atomicAdd(&p.ctl[kCtlDecHead], 1u);
         const unsigned slot = t % (unsigned)p.dec_cap;
-        const unsigned long long want = tag_of(t);
+        const unsigned long long want = dec_tag_of(p.epoch, t);
         const unsigned long long t0 = now_ns();
         PT_T0(t_poll);
         for (int it = 0;; ++it) {
@@ -2771,9 +3132,9 @@ __shared__ Params g_dp;
 
 constexpr int kDStateBytes = (int)((sizeof(DState) + 127) / 128 * 128);
 constexpr int kDecPerWarp = kDStateBytes + (kDecScratch + 127) / 128 * 128;
-constexpr int kDynBytes = kNBuf * kBufBytes + 4 * kCandCap * 4;
-constexpr int kDecWarps = (kDynBytes / kDecPerWarp < kBlock / 32) ? kDynBytes / kDecPerWarp : kBlock / 32;
-static_assert(kDecWarps >= 2, "decision warps per decision CTA");
+constexpr int kDynBytes = kNBuf * kBufBytes + 4 * kCandCap * 4 + kSlots * (int)sizeof(Slot);
+constexpr int kDecWarps = 4;   // decision warps per decision CTA
+static_assert(kDecWarps * kDecPerWarp <= kDynBytes && kDecWarps <= kBlock / 32, "decision warps' shared memory");
 
 // The calling warp's decision view: its state and scratch in the CTA's
 // dynamic shared memory, the parameters from the CTA's shared copy.
@@ -2795,16 +3156,8 @@ template <int DT> __device__ __noinline__ void dec_bonus_nl(int b) { dec_view<DT
 template <int DT> __device__ __noinline__ void dec_wis0_nl(int b) { dec_view<DT>().wis0_decide(b); }
 template <int DT> __device__ __noinline__ void dec_accept_nl(int b) { dec_view<DT>().accept_step(b); }
 
-// The stage LP of the calling warp's decision (one lane), on its Omega_1
-// tables: pair state in registers for s <= 5, in shared memory above.
-__device__ __forceinline__ int lp_solve5(int s, float A2, float B2, int A, int Btok, float u) {
-  DState& D = *reinterpret_cast<DState*>(g_dsm + (size_t)(threadIdx.x >> 5) * kDecPerWarp);
-  bool capped = false;
-  float RS[10], FL[10], FH[10];
-  const int y = stage_solve<5>(s, A2, B2, A, Btok, u, D.om, D.om_q, D.om_a, D.om_b, D.om_x, &capped, RS, FL, FH);
-  if (capped) atomicOr(g_dp.status, MDS_ST_LP_CAP);
-  return y;
-}
+// The stage LP for s > 5 of the calling warp's decision (one lane), on its
+// Omega_1 tables: pair state in shared memory.
 __device__ __noinline__ int lp_solve8(int s, float A2, float B2, int A, int Btok, float u) {
   DState& D = *reinterpret_cast<DState*>(g_dsm + (size_t)(threadIdx.x >> 5) * kDecPerWarp);
   bool capped = false;
@@ -2829,10 +3182,16 @@ __global__ void __launch_bounds__(kBlock, kCtasPerSm) flow_kernel(const __grid_c
   e.cl = reinterpret_cast<float*>(c + kCandCap * 4);
   e.crank = reinterpret_cast<int*>(c + 2 * kCandCap * 4);
   e.cord = reinterpret_cast<int*>(c + 3 * kCandCap * 4);
+  e.slots = reinterpret_cast<Slot*>(c + 4 * kCandCap * 4);
   if (threadIdx.x == 0) {
     for (int i = 0; i < kNBuf; ++i) {
       mbar_init(&S.full[i], 1);
-      mbar_init(&S.empty[i], 1);
+      mbar_init(&S.empty[i], kCW);
+    }
+    for (int i = 0; i < kSlots; ++i) {
+      mbar_init(&S.done[i], kCW);
+      mbar_init(&S.free[i], 1);
+      e.slots[i].ncand = 0;
     }
     S.issued = 0;
     S.consumed = 0;
@@ -2844,7 +3203,7 @@ __global__ void __launch_bounds__(kBlock, kCtasPerSm) flow_kernel(const __grid_c
   }
   // Roles: the CTAs on the first dec_sms SMs run decisions (kDecWarps
   // decision warps each, the rest of their warps idle), every other CTA
-  // streams slices (one scheduler warp, eight compute warps).  Decisions are
+  // streams slices (eight compute warps, a scheduler warp, a publishing warp).  Decisions are
   // serial code: on their own SMs they do not wait behind the streaming warps.
   __shared__ int role;
   if (threadIdx.x == 0) {
@@ -2862,6 +3221,8 @@ __global__ void __launch_bounds__(kBlock, kCtasPerSm) flow_kernel(const __grid_c
     __syncthreads();
     const int w = threadIdx.x >> 5;
     if (w < kDecWarps) decision_warp<DT>();
+  } else if (threadIdx.x >= kCT + 32) {
+    e.publisher();
   } else if (threadIdx.x >= kCT) {
     e.scheduler();
   } else {
@@ -2906,16 +3267,15 @@ size_t seq_bytes() { return sizeof(FSeq); }
 namespace {
 size_t up256(size_t x) { return (x + 255) / 256 * 256; }
 struct Layout {
-  size_t ctl, tag, pay, dtag, dpay, cnt, seq, rec;
+  size_t ctl, tag, dtag, dpay, cnt, seq, rec;
   size_t cap, dcap;
 };
 Layout layout(const Params& p, int nseq, int grid) {
   Layout L;
-  L.cap = (size_t)nseq * p.ns + (size_t)grid + 64;
+  L.cap = (size_t)nseq * p.ng + (size_t)grid + 64;
   L.dcap = (size_t)nseq + (size_t)grid * kDecWarps + 64;   // one request per sequence, plus the claims
   L.ctl = 256;
   L.tag = up256(L.cap * 8);
-  L.pay = up256(L.cap * 4);
   L.dtag = up256(L.dcap * 8);
   L.dpay = up256(L.dcap * 4);
   L.cnt = up256((size_t)nseq * 4);
@@ -2927,12 +3287,12 @@ Layout layout(const Params& p, int nseq, int grid) {
 
 size_t workspace_bytes(const Params& p, int nseq, int grid) {
   const Layout L = layout(p, nseq, grid);
-  return L.ctl + 2 * L.tag + L.pay + 2 * L.dtag + L.dpay + L.cnt + L.seq + L.rec;
+  return L.ctl + 2 * L.tag + 2 * L.dtag + L.dpay + L.cnt + L.seq + L.rec;
 }
 
 size_t clear_bytes(const Params& p, int nseq, int grid) {
   const Layout L = layout(p, nseq, grid);
-  return L.ctl + 2 * L.tag + L.pay + 2 * L.dtag + L.dpay + L.cnt;
+  return L.ctl + 2 * L.tag + 2 * L.dtag + L.dpay + L.cnt;
 }
 
 void carve_workspace(Params& p, char* w, int nseq, int grid) {
@@ -2943,8 +3303,6 @@ void carve_workspace(Params& p, char* w, int nseq, int grid) {
   w += L.tag;
   p.ring_rtag = reinterpret_cast<unsigned long long*>(w);
   w += L.tag;
-  p.ring_pay = reinterpret_cast<unsigned*>(w);
-  w += L.pay;
   p.dec_tag = reinterpret_cast<unsigned long long*>(w);
   w += L.dtag;
   p.dec_rtag = reinterpret_cast<unsigned long long*>(w);
@@ -3004,7 +3362,9 @@ bool plan_geometry(Params& p, int grid) {
     const int nsw = (int)(want < cap ? want : cap);
     int T = (p.V + nsw - 1) / nsw;
     T = ((T + kSliceQuantum - 1) / kSliceQuantum) * kSliceQuantum;
-    if (T < kSliceQuantum) T = kSliceQuantum;
+    // a unit for every thread at least: shorter slices cost their fixed work
+    // (record, count, combine) and use fewer lanes
+    if (T < kCT * (16 / es)) T = kCT * (16 / es);
     if (T > Tmax) T = Tmax;
     ns = (p.V + T - 1) / T;
   }
@@ -3027,21 +3387,36 @@ bool plan_geometry(Params& p, int grid) {
     // slice holding more of them only shortens the certified list)
     if (list) {
       const int base = (p.scheme == MDS_WIS0) ? 16 : 8;
-      int lns = (2 * p.ln + ns - 1) / ns;
+      // twice a slice's even share (the long list of a small batch: four times)
+      const int share = (p.ln > 32 && (long)p.B * ns <= 2L * grid) ? 4 : 2;
+      int lns = (share * p.ln + ns - 1) / ns;
       lns = (lns + 7) / 8 * 8;
       p.lns = lns < base ? base : (lns > p.ln ? p.ln : lns);
+      p.lns_rcp = (unsigned)((0x100000000ull + (unsigned)p.lns - 1u) / (unsigned)p.lns);
     } else {
       p.lns = 0;
     }
     int rf = kHdr + p.lns * (1 + lrows);
     if (rf < 4 + 4 * kTopF) rf = 4 + 4 * kTopF;
-    // the combined record of a pass is written over the pass's records
-    const int cmb = (kCmbHdr + p.ln * (2 + lrows) + ns - 1) / ns;
-    if (rf < cmb) rf = cmb;
+    const int runs = (T * es / 16 + 31) / 32;
+    if (rf < 4 + runs) rf = 4 + runs;
     p.rec_floats = (rf + 3) & ~3;
     p.hdr_floats = kHdr;
     if ((size_t)ns * p.rec_floats * 4 <= (size_t)kDecStage && ns * p.lns <= kMaxEntries) break;
   }
+  // Warp-wise candidate lists where every thread has a unit and the slice's
+  // list is short: each warp sets aside at least half as many tokens as the
+  // list holds, four times its even share, so a needed token is left
+  // out (which only shortens the certified list) about once in 10^6 warps.
+  p.fast_list = (list && p.T * es / 16 >= kCT && p.lns <= kWarpCand) ? 1 : 0;
+  p.kth = p.lns / 2;
+  // Slices per task: the scheduler's round trips for one task (claim, ring
+  // word, descriptor: about 2 us) are shared by a group of slices where there
+  // are many tasks per CTA; one slice a task where a pass's slices should
+  // spread over the GPU.
+  const long per_cta = (long)p.B * p.ns / grid;
+  p.group = per_cta >= 32 ? 4 : (per_cta >= 16 ? 2 : 1);
+  p.ng = (p.ns + p.group - 1) / p.group;
   p.dec_sms = decision_sms(grid);
   return p.dec_sms > 0;
 }

@@ -2,10 +2,11 @@
 // (mds_api.cu).  Not installed; not part of the public ABI.
 //
 // The engine splits every row the walk visits into slices of T tokens.  A
-// persistent grid takes slice tasks from a ring in global memory; each task
-// reduces its slice of the rows of one pass of one sequence to a record; the
-// CTA that completes a pass's last slice runs that sequence's decision for the
-// pass and publishes its next pass (or finishes the sequence).
+// persistent grid takes tasks (groups of slices) from a ring in global memory;
+// each slice of the rows of one pass of one sequence is reduced to a record;
+// the CTA that counts a pass's last slice posts a decision request, and a
+// decision warp combines the records, decides and publishes the sequence's
+// next pass (or finishes the sequence).
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -36,9 +37,8 @@ struct Params {
   float* out_diag;                     // [B][L+1][4] or null
   unsigned* status;                    // status word
   unsigned* ctl;                       // control words
-  unsigned long long* ring_tag;        // [ring_cap] published task tags
-  unsigned long long* ring_rtag;       // [ring_cap] tags of tasks taken
-  unsigned* ring_pay;                  // [ring_cap] (sequence << 16) | slice
+  unsigned long long* ring_tag;        // [ring_cap] published tasks (launch, lap, sequence, group)
+  unsigned long long* ring_rtag;       // [ring_cap] launch and lap of tasks taken
   unsigned long long* dec_tag;         // [dec_cap] published decision requests
   unsigned long long* dec_rtag;        // [dec_cap] tags of requests taken
   unsigned* dec_pay;                   // [dec_cap] the requests
@@ -55,6 +55,11 @@ struct Params {
   int ns;                              // slices per row
   int ln;                              // candidate list length of a sequence (0: no candidate lists)
   int lns;                             // candidate list length of one slice (<= ln)
+  unsigned lns_rcp;                    // ceil(2^32 / lns): entry / lns by a high product
+  int fast_list;                       // the slices' lists are found warp by warp
+  int kth;                             // ... each warp's threshold: its kth largest lane maximum
+  int group;                           // slices per task
+  int ng;                              // tasks per pass
   int rec_floats;                      // record stride per slice
   int hdr_floats;                      // start of a record's list entries
   int ring_cap;
