@@ -140,13 +140,8 @@ struct Elt<MDS_F32> {
   }
   // Logit i of a row in shared memory.
   __device__ static __forceinline__ float at(const char* row, int i) { return reinterpret_cast<const float*>(row)[i]; }
-  // -inf at the logits of `bits`.
-  __device__ static __forceinline__ void mask(uint4& x, unsigned bits) {
-    if (bits & 1u) x.x = kNegInfBits;
-    if (bits & 2u) x.y = kNegInfBits;
-    if (bits & 4u) x.z = kNegInfBits;
-    if (bits & 8u) x.w = kNegInfBits;
-  }
+  // -inf in its place.
+  __device__ static __forceinline__ void clear(char* row, int i) { reinterpret_cast<unsigned*>(row)[i] = kNegInfBits; }
 };
 template <>
 struct Elt<MDS_BF16> {
@@ -197,15 +192,8 @@ struct Elt<MDS_BF16> {
   __device__ static __forceinline__ float at(const char* row, int i) {
     return __uint_as_float((uint32_t) reinterpret_cast<const unsigned short*>(row)[i] << 16);
   }
-  __device__ static __forceinline__ void mask(uint4& x, unsigned bits) {
-    auto cut = [&](uint32_t& w, unsigned b) {
-      const uint32_t m = ((b & 1u) ? 0xffffu : 0u) | ((b & 2u) ? 0xffff0000u : 0u);
-      w = (w & ~m) | (kNegInfBits & m);
-    };
-    cut(x.x, bits);
-    cut(x.y, bits >> 2);
-    cut(x.z, bits >> 4);
-    cut(x.w, bits >> 6);
+  __device__ static __forceinline__ void clear(char* row, int i) {
+    reinterpret_cast<unsigned short*>(row)[i] = (unsigned short)kNegInfBits;
   }
 };
 
@@ -515,168 +503,127 @@ __device__ __forceinline__ int stage_solve(int s, float A2, float B2, int A, int
 }
 
 // The same stage for s <= 5 by a whole warp, same arithmetic in the same
-// order.  Every lane holds the whole network for the direct pass (uniform
-// code, no branches: a blocked step moves 0).  Only where supply and demand
-// are both left do augmenting paths follow: a lane then keeps one direction
-// of a pair, so that the residual graph is one ballot (its rows the tokens
-// that lead to a token), the search runs on its bits and a path's edges are
-// shuffles.
-// Entries past s are zero.  x: p_I on Omega_1, in every lane.
+// order.  Lane t < 5 keeps token t (law, demand), lane 5 a + b, a != b, one
+// direction of pair {a, b} (its flow to a and to b, its supply), so that the
+// code is a few small loops: one warp runs it serially, and what it costs is
+// latency and instruction fetches (unrolled over the ten pairs in uniform
+// registers it took twice as long, on one lane four times).  The residual
+// graph is one ballot (its rows the tokens that lead to a token), the search
+// runs on its bits and a path's edges are shuffles.  Entries past s are zero.
+// x: lane t's p_I on Omega_1.
 __device__ __forceinline__ int stage_solve5(float A2, float B2, int A, int Btok, float u, const int* om,
-                                            const float* om_q, const float* om_a, const float* om_b, float (&x)[5],
+                                            const float* om_q, const float* om_a, const float* om_b, float& x,
                                             bool* capped) {
-  constexpr int SM = 5, P = 10;
+  constexpr int SM = 5;
   constexpr unsigned full = 0xffffffffu;
   const int lane = (int)(threadIdx.x & 31);
-  float ak[SM], bk[SM], rd[SM], RS[P], FL[P], FH[P];
+  const bool tok = lane < SM;
+  const float av = tok ? om_a[lane] : 0.f, bv = tok ? om_b[lane] : 0.f, qv = tok ? om_q[lane] : 0.f;
+  const int id = tok ? om[lane] : -1;
+  x = __fadd_rn(__fadd_rn(__fmul_rn(av, bv), __fmul_rn(av, B2)), __fmul_rn(bv, A2));
+  float dem = fmaxf(0.f, __fsub_rn(qv, x));   // lanes past the tokens: 0
   float eps = 0.f;
+  {
+    const float qx = __fadd_rn(qv, x);
 #pragma unroll
-  for (int t = 0; t < SM; ++t) {
-    ak[t] = om_a[t];
-    bk[t] = om_b[t];
-    const float qk = om_q[t];
-    x[t] = __fadd_rn(__fadd_rn(__fmul_rn(ak[t], bk[t]), __fmul_rn(ak[t], B2)), __fmul_rn(bk[t], A2));
-    rd[t] = fmaxf(0.f, __fsub_rn(qk, x[t]));
-    eps = __fadd_rn(eps, __fadd_rn(qk, x[t]));
+    for (int t = 0; t < SM; ++t) eps = __fadd_rn(eps, __shfl_sync(full, qx, t));
+    eps = __fmul_rn(eps, kLpEpsRel);
   }
-  eps = __fmul_rn(eps, kLpEpsRel);
-  bool more_s = false, more_d = false;
-#pragma unroll
-  for (int i = 0; i < SM; ++i) {
-#pragma unroll
+  const int la = min(lane / SM, SM - 1), lb = lane % SM;
+  const float m = __fadd_rn(__fmul_rn(__shfl_sync(full, av, la), __shfl_sync(full, bv, lb)),
+                            __fmul_rn(__shfl_sync(full, av, lb), __shfl_sync(full, bv, la)));
+  float f = 0.f, g = 0.f, rs = (lane < SM * SM && la != lb) ? m : 0.f;
+  // (a) direct pass over the pairs (i, j), i < j
+#pragma unroll 1
+  for (int i = 0; i < SM - 1; ++i) {
+#pragma unroll 1
     for (int j = i + 1; j < SM; ++j) {
-      const int e = pidx(i, j, SM);
-      float rs = __fadd_rn(__fmul_rn(ak[i], bk[j]), __fmul_rn(ak[j], bk[i]));
-      const float dl = (rs > eps && rd[i] > eps) ? fminf(rs, rd[i]) : 0.f;
-      rs = __fsub_rn(rs, dl);
-      rd[i] = __fsub_rn(rd[i], dl);
-      const float dh = (rs > eps && rd[j] > eps) ? fminf(rs, rd[j]) : 0.f;
-      rs = __fsub_rn(rs, dh);
-      rd[j] = __fsub_rn(rd[j], dh);
-      FL[e] = dl;
-      FH[e] = dh;
-      RS[e] = rs;
-      more_s |= rs > eps;
+      const float r0 = __shfl_sync(full, rs, SM * i + j);
+      const float di = __shfl_sync(full, dem, i), dj = __shfl_sync(full, dem, j);
+      const float dl = (r0 > eps && di > eps) ? fminf(r0, di) : 0.f;
+      const float r1 = __fsub_rn(r0, dl);
+      const float dh = (r1 > eps && dj > eps) ? fminf(r1, dj) : 0.f;
+      const float r2 = __fsub_rn(r1, dh);
+      const bool lo = lane == SM * i + j, hi = lane == SM * j + i;
+      if (lo || hi) {
+        rs = r2;
+        f = lo ? dl : dh;
+        g = lo ? dh : dl;
+      }
+      if (lane == i) dem = __fsub_rn(di, dl);
+      if (lane == j) dem = __fsub_rn(dj, dh);
     }
   }
+  // (b) augmenting paths
+  int it = 0;
+#pragma unroll 1
+  for (; it < kLpMaxAugment; ++it) {
+    const unsigned dm = __ballot_sync(full, dem > eps);
+    const unsigned mS = __ballot_sync(full, rs > eps);
+    if (!dm || !mS) break;
+    const unsigned mG = __ballot_sync(full, g > eps);   // row v: the tokens that lead to v
+    unsigned visited = 0u;
 #pragma unroll
-  for (int t = 0; t < SM; ++t) more_d |= rd[t] > eps;
-  *capped = false;
-  if (more_s && more_d) {
-    // lane 5 a + b, a != b: pair {a, b} seen from a: its flow to a (f) and to
-    // b (g) and its supply; lanes 0..4 also the tokens' demands
-    float f = 0.f, g = 0.f, rs = 0.f, dem = 0.f;
+    for (int t = 0; t < SM; ++t) visited |= (mS >> (SM * t) & 31u) ? 1u << t : 0u;
+    unsigned frontier = visited, layers = visited, hit = visited & dm;
+    int lev = 0;
+#pragma unroll 1
+    while (!hit && frontier && lev < SM) {
+      unsigned nxt = 0u;
 #pragma unroll
-    for (int i = 0; i < SM; ++i)
-#pragma unroll
-      for (int j = i + 1; j < SM; ++j) {
-        const int e = pidx(i, j, SM);
-        if (lane == 5 * i + j) {
-          f = FL[e];
-          g = FH[e];
-        }
-        if (lane == 5 * j + i) {
-          f = FH[e];
-          g = FL[e];
-        }
-        if (lane == 5 * i + j || lane == 5 * j + i) rs = RS[e];
-      }
-#pragma unroll
-    for (int t = 0; t < SM; ++t)
-      if (lane == t) dem = rd[t];
-    int it = 0;
-    for (; it < kLpMaxAugment; ++it) {
-      const unsigned dm = __ballot_sync(full, dem > eps);
-      const unsigned mS = __ballot_sync(full, rs > eps);
-      if (!dm || !mS) break;
-      const unsigned mG = __ballot_sync(full, g > eps);   // row v: the tokens that lead to v
-      unsigned visited = 0u;
-#pragma unroll
-      for (int t = 0; t < SM; ++t) visited |= (mS >> (5 * t) & 31u) ? 1u << t : 0u;
-      unsigned frontier = visited, layers = visited, hit = visited & dm;
-      int lev = 0;
-      while (!hit && frontier && lev < SM) {
-        unsigned nxt = 0u;
-#pragma unroll
-        for (int t = 0; t < SM; ++t) nxt |= ((mG >> (5 * t)) & 31u & frontier) ? 1u << t : 0u;
-        nxt &= ~visited;
-        visited |= nxt;
-        frontier = nxt;
-        ++lev;
-        layers |= nxt << (5 * lev);
-        hit = nxt & dm;
-      }
-      if (!hit) break;
-      const int sink = __ffs(hit) - 1;
-      float delta = __shfl_sync(full, dem, sink);
-      int v = sink;
-      for (int l = lev; l > 0; --l) {
-        const int uu = __ffs((mG >> (5 * v)) & (layers >> (5 * (l - 1))) & 31u) - 1;
-        delta = fminf(delta, __shfl_sync(full, f, 5 * uu + v));
-        v = uu;
-      }
-      const int w = __ffs((mS >> (5 * v)) & 31u) - 1;   // the first pair of v with supply
-      delta = fminf(delta, __shfl_sync(full, rs, 5 * v + w));
-      if (lane == 5 * v + w) {
-        rs = __fsub_rn(rs, delta);
-        f = __fadd_rn(f, delta);
-      }
-      if (lane == 5 * w + v) {
-        rs = __fsub_rn(rs, delta);
-        g = __fadd_rn(g, delta);
-      }
-      v = sink;
-      for (int l = lev; l > 0; --l) {
-        const int uu = __ffs((mG >> (5 * v)) & (layers >> (5 * (l - 1))) & 31u) - 1;
-        const float d = lane == 5 * uu + v ? delta : (lane == 5 * v + uu ? -delta : 0.f);
-        f = __fsub_rn(f, d);
-        g = __fadd_rn(g, d);
-        v = uu;
-      }
-      if (lane == sink) dem = __fsub_rn(dem, delta);
+      for (int t = 0; t < SM; ++t) nxt |= ((mG >> (SM * t)) & 31u & frontier) ? 1u << t : 0u;
+      nxt &= ~visited;
+      visited |= nxt;
+      frontier = nxt;
+      ++lev;
+      layers |= nxt << (SM * lev);
+      hit = nxt & dm;
     }
-    *capped = it >= kLpMaxAugment;
-#pragma unroll
-    for (int i = 0; i < SM; ++i)
-#pragma unroll
-      for (int j = i + 1; j < SM; ++j) {
-        const int e = pidx(i, j, SM);
-        FL[e] = __shfl_sync(full, f, 5 * i + j);
-        FH[e] = __shfl_sync(full, g, 5 * i + j);
-        RS[e] = __shfl_sync(full, rs, 5 * i + j);
-      }
+    if (!hit) break;
+    const int sink = __ffs(hit) - 1;
+    float delta = __shfl_sync(full, dem, sink);
+    int v = sink;
+#pragma unroll 1
+    for (int l = lev; l > 0; --l) {
+      const int uu = __ffs((mG >> (SM * v)) & (layers >> (SM * (l - 1))) & 31u) - 1;
+      delta = fminf(delta, __shfl_sync(full, f, SM * uu + v));
+      v = uu;
+    }
+    const int w = __ffs((mS >> (SM * v)) & 31u) - 1;   // the first pair of v with supply
+    delta = fminf(delta, __shfl_sync(full, rs, SM * v + w));
+    if (lane == SM * v + w) {
+      rs = __fsub_rn(rs, delta);
+      f = __fadd_rn(f, delta);
+    }
+    if (lane == SM * w + v) {
+      rs = __fsub_rn(rs, delta);
+      g = __fadd_rn(g, delta);
+    }
+    v = sink;
+#pragma unroll 1
+    for (int l = lev; l > 0; --l) {
+      const int uu = __ffs((mG >> (SM * v)) & (layers >> (SM * (l - 1))) & 31u) - 1;
+      const float d = lane == SM * uu + v ? delta : (lane == SM * v + uu ? -delta : 0.f);
+      f = __fsub_rn(f, d);
+      g = __fadd_rn(g, d);
+      v = uu;
+    }
+    if (lane == sink) dem = __fsub_rn(dem, delta);
   }
+  *capped = it >= kLpMaxAugment;
+  // p_I on Omega_1: base + flow + half of the pair mass left over, pairs in order
+  const float add = __fadd_rn(f, __fmul_rn(0.5f, rs));
 #pragma unroll
-  for (int i = 0; i < SM; ++i) {
-#pragma unroll
-    for (int j = i + 1; j < SM; ++j) {
-      const int e = pidx(i, j, SM);
-      const float half = __fmul_rn(0.5f, RS[e]);
-      x[i] = __fadd_rn(x[i], __fadd_rn(FL[e], half));
-      x[j] = __fadd_rn(x[j], __fadd_rn(FH[e], half));
-    }
+  for (int w = 0; w < SM; ++w) {
+    const float t = __shfl_sync(full, add, tok ? SM * lane + w : 0);
+    if (tok && w != lane) x = __fadd_rn(x, t);
   }
   if (A == Btok) return A;
-  int pa = -1, pb = -1;
-#pragma unroll
-  for (int t = 0; t < SM; ++t) {
-    const int o = om[t];
-    if (o == A) pa = t;
-    if (o == Btok) pb = t;
-  }
+  const int pa = __ffs(__ballot_sync(full, id == A)) - 1, pb = __ffs(__ballot_sync(full, id == Btok)) - 1;
   if (pa >= 0 && pb >= 0) {
-    const int e = pidx(min(pa, pb), max(pa, pb), SM);
-    float fl = 0.f, rs = 0.f, m = 0.f;
-#pragma unroll
-    for (int i = 0; i < SM; ++i)
-#pragma unroll
-      for (int j = i + 1; j < SM; ++j)
-        if (pidx(i, j, SM) == e) {
-          fl = FL[pidx(i, j, SM)];
-          rs = RS[pidx(i, j, SM)];
-          m = __fadd_rn(__fmul_rn(ak[i], bk[j]), __fmul_rn(ak[j], bk[i]));
-        }
-    const float wlo = m > 0.f ? __fdiv_rn(__fadd_rn(fl, __fmul_rn(0.5f, rs)), m) : 0.5f;
+    const int e = SM * min(pa, pb) + max(pa, pb);   // seen from the lower token
+    const float to = __shfl_sync(full, add, e), mm = __shfl_sync(full, m, e);
+    const float wlo = mm > 0.f ? __fdiv_rn(to, mm) : 0.5f;
     const float wa = (pa < pb) ? wlo : __fsub_rn(1.f, wlo);
     return (u < wa) ? A : Btok;
   }

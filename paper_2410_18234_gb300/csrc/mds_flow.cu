@@ -51,7 +51,11 @@ constexpr int kCW = 8;                 // compute warps
 constexpr int kCT = kCW * 32;          // compute threads
 constexpr int kBlock = kCT + 64;       // + the scheduler warp and the publishing warp
 constexpr int kNBuf = 2;               // slice buffers per CTA
-constexpr int kSlots = 3;              // records between the compute warps and the publishing warp
+// Task descriptors: a buffer is released before its task is done, so task k's
+// descriptor lives on until task k + 3 is issued, which waits for every warp
+// to release task k + 1's buffer, so to have done task k.
+constexpr int kNDesc = kNBuf + 1;
+constexpr int kSlots = 3;              // records between the compute warps and the publishing warpss
 constexpr int kFastUnits = kBufBytes / 16;   // units of all rows one slice holds
 constexpr int kWarpCand = 32;          // tokens one warp may set aside in a slice
 constexpr int kSlotCand = kCW * kWarpCand;
@@ -70,11 +74,12 @@ static_assert(kTopF >= MDS_MAX_S, "full-stage candidates");
 
 enum : int { kNone = 0, kStats = 1, kResid = 2, kBonus = 3, kFull = 4, kReplace = 5 };
 
-// A decision request: sequence (16 bits), kind (3), depth (7), rows (5), list (1).
-__host__ __device__ constexpr unsigned dec_payload(int b, int kind, int j, int R, int list) {
-  return ((unsigned)b << 16) | ((unsigned)kind << 13) | ((unsigned)j << 6) | ((unsigned)R << 1) | (unsigned)(list != 0);
+// A decision request: sequence (16 bits), depth (7), whether the pass is the
+// sequence's first (its descriptor is not in memory yet).
+__host__ __device__ constexpr unsigned dec_payload(int b, int j, bool first) {
+  return ((unsigned)b << 8) | ((unsigned)j << 1) | (first ? 1u : 0u);
 }
-static_assert(MDS_MAX_L < 127 && kMaxRows < 32, "decision request fields");
+static_assert(MDS_MAX_L < 127, "decision request fields");
 
 // Phase-timer slots (SM cycles summed over CTAs, or counts).
 enum : int {
@@ -152,6 +157,7 @@ struct __align__(16) FSeq {
 struct __align__(16) FDesc {
   FPass P;
   int b, slice, end, exit;     // the sequence, the next slice and the end of its group
+  int first, pad[3];           // the group's first slice
 };
 static_assert(sizeof(FDesc) % 16 == 0, "descriptor moves in 16-byte chunks");
 
@@ -218,7 +224,7 @@ static_assert(offsetof(DState, W) == offsetof(DState, P) + sizeof(FPass) && offs
 enum : int { kSlotDone = 0,   // the record is in global memory already
              kSlotSums, kSlotList, kSlotBonus, kSlotRuns, kSlotExit };
 struct __align__(16) Slot {
-  int mode, b, slice, kind, j, R, list, nrun;
+  int mode, b, slice, kind, j, R, nrun;
   int count;                   // slices to count with this one: its group's, at the group's end (else 0)
   float c[kListRowsMax];
   int ncand;                   // tokens set aside (zero between slices)
@@ -226,13 +232,14 @@ struct __align__(16) Slot {
   float m[kCW][kListRowsMax], s[kCW][kListRowsMax];
   float run[kMaxRuns];
   __align__(16) unsigned key[kSlotCand];   // order key of the target logit (16-bit logits: and the place, see set_aside)
-  int loc[kSlotCand], ord[kSlotCand];      // place in the slice
+  unsigned short loc[kSlotCand], ord[kSlotCand];   // place in the slice; the tokens ranked past the list
   float l[kListRowsMax][kSlotCand];
 };
+static_assert(kListRowsMax * kSlotCand >= 2 * kCandCap, "the block-wise list's arrays lie over two slots' logits");
 
 struct FShared {
   uint64_t full[kNBuf], empty[kNBuf], done[kSlots], free[kSlots];
-  FDesc desc[kNBuf];
+  FDesc desc[kNDesc];
   FDesc pend;                  // the scheduler's next task, resolved ahead
   float red[kCW * 2 * kMaxRows];
   float wth[kCW];
@@ -273,13 +280,11 @@ __device__ __forceinline__ unsigned long long now_ns() {
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
 }
-// Ring words: launch, lap over the ring, payload (sequence << 8 | group of slices).
+// Ring words: launch, lap over the ring, payload of 24 bits (tasks: sequence
+// << 8 | group of slices; decisions: dec_payload).
 constexpr unsigned long long kRingPay = 0xffffffull;
 __device__ __forceinline__ unsigned long long ring_word(unsigned epoch, unsigned lap, unsigned pay) {
   return ((unsigned long long)(epoch & 0x3fffffffu) << 34) | ((unsigned long long)((lap + 1u) & 0x3ffu) << 24) | pay;
-}
-__device__ __forceinline__ unsigned long long dec_tag_of(unsigned epoch, unsigned t) {
-  return ((unsigned long long)epoch << 32) | (unsigned long long)(t + 1u);
 }
 __device__ __forceinline__ void st_relaxed(unsigned long long* a, unsigned long long v) {
   asm volatile("st.relaxed.gpu.u64 [%0], %1;" ::"l"(a), "l"(v) : "memory");
@@ -441,6 +446,12 @@ struct Eng {
   __device__ __forceinline__ uint4 raw(const char* b, int r, int u) const {
     return *reinterpret_cast<const uint4*>(srow(b, r) + 16 * u);
   }
+  // This warp has read its part of a buffer (the wait for the loads' values is
+  // the reads' own).
+  __device__ __forceinline__ void release(int bi) const {
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) mbar_arrive(&S.empty[bi]);
+  }
   // Explicit value of a special token of the current law, else fallback.
   __device__ __forceinline__ float spec_lookup(const FPass& P, int tok, float fallback) const {
     for (int i = 0; i < P.nspec; ++i)
@@ -515,22 +526,28 @@ struct Eng {
 
   // Claim the next task number and resolve it into Pd: the sequence, its
   // slices and the sequence's pass descriptor (depth-0 tasks are implicit:
-  // task t < B * ng is group t % ng of sequence t / ng).  Returns 0 when no
-  // work is left (every sequence finished, or an abort).  Warp-wide.
-  __device__ int resolve(FDesc& Pd) {
+  // task t < B * ng0 is group t % ng0 of sequence t / ng0).  Returns 0 when no
+  // work is left (every sequence finished, or an abort).  The number was
+  // claimed one task ahead (tn, lane 0), so that its round trip is over; the
+  // next one is claimed here.  Warp-wide.
+  __device__ int resolve(FDesc& Pd, unsigned& tn) {
     const int lane = threadIdx.x & 31;
-    const unsigned N0 = (unsigned)p.B * (unsigned)p.ng;
+    const unsigned N0 = (unsigned)p.B * (unsigned)p.ng0;
     int have = 0, b = 0, g = 0;
-    if (lane == 0 && !aborted()) {
-      const unsigned t = atomicAdd(&p.ctl[kCtlHead], 1u);
+    if (lane == 0) {
+      // the slot's word holds all of a task, and an acquire load orders the
+      // store that gives the slot back
+      const unsigned t = tn;
+      tn = atomicAdd(&p.ctl[kCtlHead], 1u);
+      const bool ab = aborted();
       const unsigned slot = t % (unsigned)p.ring_cap;
+      const unsigned long long want = ring_word(p.epoch, t / (unsigned)p.ring_cap, 0u);
       if (t < N0) {
-        b = (int)(t / (unsigned)p.ng);
-        g = (int)(t % (unsigned)p.ng);
-        st_release(&p.ring_rtag[slot], ring_word(p.epoch, t / (unsigned)p.ring_cap, 0u));
-        have = 1;
-      } else {
-        const unsigned long long want = ring_word(p.epoch, t / (unsigned)p.ring_cap, 0u);
+        b = (int)(t / (unsigned)p.ng0);
+        g = (int)(t % (unsigned)p.ng0);
+        st_relaxed(&p.ring_rtag[slot], want);
+        have = ab ? 0 : 1;
+      } else if (!ab) {
         const unsigned long long t0 = now_ns();
         PT_T0(t_poll);
         for (int it = 0;; ++it) {
@@ -538,16 +555,16 @@ struct Eng {
           if ((w & ~kRingPay) == want) {
             b = (int)((w >> 8) & 0xffffu);
             g = (int)(w & 0xffu);
-            st_release(&p.ring_rtag[slot], want);
+            st_relaxed(&p.ring_rtag[slot], want);
             have = 2;
             break;
           }
-          if (ld_relaxed(&p.ctl[kCtlDone]) >= (unsigned)p.B || aborted()) break;
+          if ((it & 3) == 3 && (ld_relaxed(&p.ctl[kCtlDone]) >= (unsigned)p.B || aborted())) break;
           if ((it & 15) == 15 && now_ns() - t0 > kWaitNs) {
             set_abort(MDS_ST_TIMEOUT);
             break;
           }
-          __nanosleep(it < 16 ? 32 : 256);
+          __nanosleep(it < 16 ? 32 : 128);
         }
         PT_ADD(kPhSchedPoll, t_poll);
       }
@@ -561,8 +578,9 @@ struct Eng {
       copy_in(&Pd.P, &reinterpret_cast<const FSeq*>(p.seq)[b].P, (int)sizeof(FPass), lane, 32);
     if (lane == 0) {
       Pd.b = b;
-      Pd.slice = g * p.group;
-      Pd.end = min(p.ns, (g + 1) * p.group);
+      const int group = have == 1 ? p.group0 : p.group;
+      Pd.slice = Pd.first = g * group;
+      Pd.end = min(p.ns, (g + 1) * group);
       Pd.exit = have ? 0 : 1;
     }
     __syncwarp();
@@ -574,10 +592,11 @@ struct Eng {
   // the descriptor move and the bulk copies.
   __device__ void scheduler() {
     const int lane = threadIdx.x & 31;
-    int have = resolve(S.pend);
+    unsigned tn = lane == 0 ? atomicAdd(&p.ctl[kCtlHead], 1u) : 0u;
+    int have = resolve(S.pend, tn);
     for (int k = 0;; ++k) {
       const int bi = k % kNBuf;
-      FDesc& D = S.desc[bi];
+      FDesc& D = S.desc[k % kNDesc];
       // the compute warps released this buffer (lane 0 waits; bounded)
       int ok = 1;
       PT_T0(t_empty);
@@ -615,7 +634,7 @@ struct Eng {
       more = __shfl_sync(FULLM, more, 0);
       __syncwarp();
       if (!have) return;
-      if (!more) have = resolve(S.pend);
+      if (!more) have = resolve(S.pend, tn);
     }
   }
 
@@ -685,7 +704,8 @@ struct Eng {
   // block with five barriers and the publication in it (GB300, a 32 KB slice
   // of two rows): with a list 17k -> 3.5k SM cycles, without 8k -> 2.7k.
   template <int R, bool LIST, bool RUNS>
-  __device__ __forceinline__ void stats_fast(const FPass& P, char* b, int tok0, int n, Slot& T) {
+  __device__ __forceinline__ void stats_fast(const FPass& P, int bi, int tok0, int n, Slot& T) {
+    char* b = buf(bi);
     constexpr int NU = (kFastUnits / R + kCT - 1) / kCT;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int U = (n + VE - 1) / VE;
@@ -723,17 +743,18 @@ struct Eng {
       float theta = last ? ord_val(last) : kPosInf;
       unsigned long long bits = 0ull;   // this lane's tokens at or above theta, VE to a unit
       auto mark = [&]() {
+        unsigned um = 0u;   // units that hold one
+#pragma unroll
+        for (int i = 0; i < NU; ++i) um |= E::unit_max(x[0][i]) >= theta ? 1u << i : 0u;
         bits = 0ull;
+        for (; um; um &= um - 1u) {
+          const int i = __ffs(um) - 1;
+          float v[VE];
+          E::unpack(i * kCT + tid < U ? raw(b, 0, i * kCT + tid) : E::neg_inf(), v);
+          unsigned bb = 0u;
 #pragma unroll
-        for (int i = 0; i < NU; ++i) {
-          if (E::unit_max(x[0][i]) >= theta) {
-            float v[VE];
-            E::unpack(x[0][i], v);
-            unsigned bb = 0u;
-#pragma unroll
-            for (int e = 0; e < VE; ++e) bb |= (v[e] >= theta && v[e] > kNegInf) ? 1u << e : 0u;
-            bits |= (unsigned long long)bb << (i * VE);
-          }
+          for (int e = 0; e < VE; ++e) bb |= (v[e] >= theta && v[e] > kNegInf) ? 1u << e : 0u;
+          bits |= (unsigned long long)bb << (i * VE);
         }
         return __popcll(bits);
       };
@@ -757,27 +778,36 @@ struct Eng {
         theta = ord_val(t + 1u);
         cnt = mark();
       }
+      // set aside: into the slot, and out of the slice (-inf in every row;
+      // this thread's own units, read back into its registers)
       if (cnt) {
         int pos = atomicAdd(&T.ncand, cnt);
         for (unsigned long long q = bits; q; q &= q - 1ull) {
           const int at = __ffsll((long long)q) - 1;
           const int loc = ((at / VE) * kCT + tid) * VE + at % VE;
-          T.loc[pos] = loc;
+          T.loc[pos] = (unsigned short)loc;
 #pragma unroll
-          for (int rr = 0; rr < R; ++rr) T.l[rr][pos] = E::at(srow(b, rr), loc);
+          for (int rr = 0; rr < R; ++rr) {
+            char* row = b + (size_t)rr * p.T * p.esize;
+            T.l[rr][pos] = E::at(row, loc);
+            E::clear(row, loc);
+          }
           T.key[pos] = cand_key(T.l[0][pos], loc);
           ++pos;
         }
-      }
-      // out of the registers: every row reads -inf there
+        asm volatile("" ::: "memory");
 #pragma unroll
-      for (int i = 0; i < NU; ++i) {
-        const unsigned bb = (unsigned)(bits >> (i * VE)) & ((1u << VE) - 1u);
-        if (__any_sync(FULLM, bb != 0u)) {
+        for (int r = 0; r < R; ++r)
 #pragma unroll
-          for (int rr = 0; rr < R; ++rr) E::mask(x[rr][i], bb);
-        }
+          for (int i = 0; i < NU; ++i)
+            if ((unsigned)(bits >> (i * VE)) & ((1u << VE) - 1u)) x[r][i] = raw(b, r, i * kCT + tid);
       }
+      fence_proxy_async();   // these stores before the next bulk copy into the buffer
+    }
+    // the slice is in registers: the buffer can be filled again (released at
+    // the task's end, a 32 KB slice's loads waited 1.5 to 3 us for it)
+    release(bi);
+    if constexpr (LIST) {
       float tm = kNegInf;
 #pragma unroll
       for (int i = 0; i < NU; ++i) tm = fmaxf(tm, E::unit_max(x[0][i]));
@@ -1128,45 +1158,102 @@ struct Eng {
   }
 
   // -------------------------------------------------------------- weights of the inverse-CDF draws
-  // Residual max(0, q - p_I) (kResid; p_I = sum_r gamma_r p_r with the
-  // special tokens' explicit values), or the target mass outside Omega_0
-  // (kReplace: tokens with a logit above `cut` weigh 0 unless all0 says
-  // Omega_0 is empty of them), or the target mass (kBonus).
+  // Residual max(0, q - p_I), p_I = sum_r gamma_r p_r with the special
+  // tokens' explicit values, of one unit.
   __device__ __forceinline__ void weights(const FPass& P, const char* b, int u, int tok0, float* w) const {
-    float v0[VE];
+    float v0[VE], a[VE];
     E::unpack(raw(b, 0, u), v0);
-    const float M0 = P.row[0].M, c0 = P.row[0].c, iz0 = P.row[0].invZ;
-    if (P.kind == kResid) {
-      float a[VE];
 #pragma unroll
-      for (int e = 0; e < VE; ++e) a[e] = 0.f;
-      for (int r = 1; r < P.nstream; ++r) {
-        const float g = P.row[r].gamma;
-        if (g == 0.f) continue;
-        float v[VE];
-        E::unpack(raw(b, r, u), v);
-        const float M = P.row[r].M, c = P.row[r].c, iz = P.row[r].invZ;
+    for (int e = 0; e < VE; ++e) a[e] = 0.f;
+    for (int r = 1; r < P.nstream; ++r) {
+      const float g = P.row[r].gamma;
+      if (g == 0.f) continue;
+      float v[VE];
+      E::unpack(raw(b, r, u), v);
+      const float M = P.row[r].M, c = P.row[r].c, iz = P.row[r].invZ;
 #pragma unroll
-        for (int e = 0; e < VE; ++e) a[e] = __fmaf_rn(g, prob_of(v[e], M, c, iz), a[e]);
-      }
-      if (P.nspec > 0 && ((S.bitmap[u >> 5] >> (u & 31)) & 1u)) {
-#pragma unroll
-        for (int e = 0; e < VE; ++e) a[e] = spec_lookup(P, tok0 + u * VE + e, a[e]);
-      }
-#pragma unroll
-      for (int e = 0; e < VE; ++e) w[e] = fmaxf(0.f, __fsub_rn(prob_of(v0[e], M0, c0, iz0), a[e]));
-    } else if (P.kind == kReplace) {
-#pragma unroll
-      for (int e = 0; e < VE; ++e) w[e] = (P.all0 || v0[e] > P.cut) ? 0.f : prob_of(v0[e], M0, c0, iz0);
-    } else {
-#pragma unroll
-      for (int e = 0; e < VE; ++e) w[e] = prob_of(v0[e], M0, c0, iz0);
+      for (int e = 0; e < VE; ++e) a[e] = __fmaf_rn(g, prob_of(v[e], M, c, iz), a[e]);
     }
+    if (P.nspec > 0 && ((S.bitmap[u >> 5] >> (u & 31)) & 1u)) {
+#pragma unroll
+      for (int e = 0; e < VE; ++e) a[e] = spec_lookup(P, tok0 + u * VE + e, a[e]);
+    }
+    const float M0 = P.row[0].M, c0 = P.row[0].c, iz0 = P.row[0].invZ;
+#pragma unroll
+    for (int e = 0; e < VE; ++e) w[e] = fmaxf(0.f, __fsub_rn(prob_of(v0[e], M0, c0, iz0), a[e]));
   }
 
   // The masses of the slice's runs of 32 units, the runs the decision's
   // search walks, one warp a run (runs warp, warp + 8, ...): a unit's mass
-  // adds its tokens in order, a run's its units by a butterfly.
+  // adds its tokens in order, a run's its units by a butterfly.  Up to four
+  // rows a thread's units are kept in registers (the buffer is released at
+  // once) with the rows' constants.
+  template <int R>
+  __device__ __forceinline__ void resid_fast(const FPass& P, int bi, int tok0, int n, Slot& T) {
+    constexpr int NU = (kFastUnits / R + kCT - 1) / kCT;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int U = (n + VE - 1) / VE;
+    char* b = buf(bi);
+    uint4 x[R][NU];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int i = 0; i < NU; ++i) {
+        const int u = i * kCT + tid;
+        x[r][i] = (u < U) ? raw(b, r, u) : E::neg_inf();
+      }
+    release(bi);
+    if (P.kind == kResid && P.nspec > 0) build_bitmap(P, tok0, n);
+    float mc[R], c[R], iz[R], gm[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      c[r] = P.row[r].c;
+      mc[r] = __fmul_rn(P.row[r].M, c[r]);
+      iz[r] = P.row[r].invZ;
+      gm[r] = r ? P.row[r].gamma : 1.f;
+    }
+    const bool resid = P.kind == kResid, special = resid && P.nspec > 0;
+    const bool none = P.kind == kReplace && P.all0;
+    const float cut = P.kind == kReplace ? P.cut : kPosInf;
+#pragma unroll
+    for (int i = 0; i < NU; ++i) {
+      if (i * kCT + warp * 32 >= U) break;   // warp-uniform
+      const int u = i * kCT + tid;
+      float q[VE], us = 0.f;
+      E::unpack(x[0][i], q);
+      if constexpr (R == 1) {
+        // the target mass outside Omega_0 (kReplace)
+#pragma unroll
+        for (int e = 0; e < VE; ++e) {
+          const float pq = __fmul_rn(ex2(__fmaf_rn(q[e], c[0], -mc[0])), iz[0]);
+          us = __fadd_rn(us, (none || q[e] > cut) ? 0.f : pq);
+        }
+      } else {
+        float a[VE];
+#pragma unroll
+        for (int e = 0; e < VE; ++e) a[e] = 0.f;
+#pragma unroll
+        for (int r = 1; r < R; ++r) {
+          if (gm[r] == 0.f) continue;
+          float v[VE];
+          E::unpack(x[r][i], v);
+#pragma unroll
+          for (int e = 0; e < VE; ++e)
+            a[e] = __fmaf_rn(gm[r], __fmul_rn(ex2(__fmaf_rn(v[e], c[r], -mc[r])), iz[r]), a[e]);
+        }
+        if (special && ((S.bitmap[u >> 5] >> (u & 31)) & 1u)) {
+#pragma unroll
+          for (int e = 0; e < VE; ++e) a[e] = spec_lookup(P, tok0 + u * VE + e, a[e]);
+        }
+#pragma unroll
+        for (int e = 0; e < VE; ++e)
+          us = __fadd_rn(us, fmaxf(0.f, __fsub_rn(__fmul_rn(ex2(__fmaf_rn(q[e], c[0], -mc[0])), iz[0]), a[e])));
+      }
+      us = warp_sum(us);
+      if (lane == 0) T.run[i * kCW + warp] = us;
+    }
+  }
+  // More rows than that.
   __device__ void resid_task(const FPass& P, const char* b, int tok0, int n, Slot& T) {
     if (P.kind == kResid && P.nspec > 0) build_bitmap(P, tok0, n);
     const int U = (n + VE - 1) / VE;
@@ -1396,7 +1483,7 @@ struct Eng {
         for (int r = 0; r < kListRowsMax; ++r)
           if (r < T.R) __stcg(rec + kHdr + LN * (1 + r) + rk, T.l[r][i]);
       } else {
-        T.ord[rk - LN] = i;
+        T.ord[rk - LN] = (unsigned short)i;
       }
     }
     __syncwarp();
@@ -1463,7 +1550,7 @@ struct Eng {
         }
         if (lane == 0) __stcg(rec, tot);
       }
-      const int kind = T.kind, j = T.j, R = T.R, list = T.list;
+      const int kind = T.kind, j = T.j;
       if (kind == kStats && j == 0 && s == 0) {
         // the sequence's outputs start as -1 (the decisions overwrite them)
         for (int q = lane; q <= p.L; q += 32) __stcg(p.out_tokens + (size_t)b * (p.L + 1) + q, -1);
@@ -1476,10 +1563,8 @@ struct Eng {
         T.ncand = 0;
         mbar_arrive(&S.free[k % kSlots]);
         // the group's records before the count (release; the last one also acquires the others')
-        if (count && atom_add_acq_rel(&p.cnt[b], (unsigned)count) == (unsigned)(p.ns - count)) {
-          __threadfence();
-          post_decision(dec_payload(b, kind, j, R, list));
-        }
+        if (count && atom_add_acq_rel(&p.cnt[b], (unsigned)count) == (unsigned)(p.ns - count))
+          post_decision(dec_payload(b, j, kind == kStats && j == 0));
       }
       PT_ADDW(kPhPublish, t_pub);
       __syncwarp();
@@ -1492,9 +1577,9 @@ struct Eng {
   // the release of the request's tag passes them on to the decision warp).
   __device__ void post_decision(unsigned pay) const {
     const unsigned t = atomicAdd(&p.ctl[kCtlDecTail], 1u);
-    const unsigned slot = t % (unsigned)p.dec_cap;
-    if (t >= (unsigned)p.dec_cap) {
-      const unsigned long long prev = dec_tag_of(p.epoch, t - (unsigned)p.dec_cap);
+    const unsigned slot = t % (unsigned)p.dec_cap, lap = t / (unsigned)p.dec_cap;
+    if (lap) {
+      const unsigned long long prev = ring_word(p.epoch, lap - 1u, 0u);
       const unsigned long long t0 = now_ns();
       for (int it = 0; ld_acquire(&p.dec_rtag[slot]) != prev; ++it) {
         if (aborted()) break;
@@ -1505,15 +1590,13 @@ struct Eng {
         __nanosleep(64);
       }
     }
-    __stcg(p.dec_pay + slot, pay);
-    st_release(&p.dec_tag[slot], dec_tag_of(p.epoch, t));
+    st_release(&p.dec_tag[slot], ring_word(p.epoch, lap, pay));
   }
 
   // One slice: this warp's part of the results into T, or (slices too small
   // for the warp-wise paths, more rows than they take, full stages) the whole
   // record into global memory.  Thread 0 fills T's description.
-  __device__ void process(int bi, Slot& T) {
-    FDesc& Dd = S.desc[bi];
+  __device__ void process(int bi, const FDesc& Dd, Slot& T) {
     char* b = buf(bi);
     const int s = Dd.slice, seqb = Dd.b;
     const int tok0 = s * p.T, n = min(p.T, p.V - tok0);
@@ -1526,16 +1609,16 @@ struct Eng {
     switch (P.kind) {
       case kBonus:
         mode = kSlotBonus;
-        stats_fast<1, false, true>(P, b, tok0, n, T);
+        stats_fast<1, false, true>(P, bi, tok0, n, T);
         break;
       case kStats:
         if (P.list && p.fast_list) {
           mode = kSlotList;
           switch (P.nstream) {
-            case 1: stats_fast<1, true, false>(P, b, tok0, n, T); break;
-            case 2: stats_fast<2, true, false>(P, b, tok0, n, T); break;
-            case 3: stats_fast<3, true, false>(P, b, tok0, n, T); break;
-            default: stats_fast<4, true, false>(P, b, tok0, n, T); break;
+            case 1: stats_fast<1, true, false>(P, bi, tok0, n, T); break;
+            case 2: stats_fast<2, true, false>(P, bi, tok0, n, T); break;
+            case 3: stats_fast<3, true, false>(P, bi, tok0, n, T); break;
+            default: stats_fast<4, true, false>(P, bi, tok0, n, T); break;
           }
         } else if (P.list) {
           if (!p.bulk) load_plain(P, P.nstream, b, tok0, n);
@@ -1545,19 +1628,21 @@ struct Eng {
             case 3: stats_small<3>(P, b, tok0, n, rec); break;
             default: stats_small<4>(P, b, tok0, n, rec); break;
           }
+          release(bi);
         } else {
           switch (P.nstream) {
             case 1:
               mode = kSlotSums;
-              stats_fast<1, false, false>(P, b, tok0, n, T);
+              stats_fast<1, false, false>(P, bi, tok0, n, T);
               break;
             case 2:
               mode = kSlotSums;
-              stats_fast<2, false, false>(P, b, tok0, n, T);
+              stats_fast<2, false, false>(P, bi, tok0, n, T);
               break;
             default:
               if (!p.bulk) load_plain(P, P.nstream, b, tok0, n);
               stats_rows(P, b, n, rec);
+              release(bi);
               break;
           }
         }
@@ -1566,13 +1651,23 @@ struct Eng {
       case kReplace:
         mode = kSlotRuns;
         if (!p.bulk) load_own(P, P.nstream, b, tok0, n);
-        resid_task(P, b, tok0, n, T);
+        switch (P.nstream) {
+          case 1: resid_fast<1>(P, bi, tok0, n, T); break;
+          case 2: resid_fast<2>(P, bi, tok0, n, T); break;
+          case 3: resid_fast<3>(P, bi, tok0, n, T); break;
+          case 4: resid_fast<4>(P, bi, tok0, n, T); break;
+          default:
+            resid_task(P, b, tok0, n, T);
+            release(bi);
+            break;
+        }
         break;
       case kFull:
         if (!p.bulk) load_plain(P, P.nstream, b, tok0, n);
         full_task(P, b, tok0, n, rec);
+        release(bi);
         break;
-      default: break;
+      default: release(bi); break;
     }
     PT_ADD(P.kind == kStats ? (P.list ? kPhTaskList : kPhTaskStats)
                             : (P.kind == kBonus ? kPhTaskStats : (P.kind == kFull ? kPhTaskFull : kPhTaskResid)),
@@ -1584,9 +1679,8 @@ struct Eng {
       T.kind = P.kind;
       T.j = P.j;
       T.R = P.nstream;
-      T.list = P.list;
       T.nrun = (U + 31) / 32;
-      T.count = (s + 1 == Dd.end) ? s + 1 - (s / p.group) * p.group : 0;
+      T.count = (s + 1 == Dd.end) ? s + 1 - Dd.first : 0;
     }
     if (threadIdx.x < kListRowsMax) T.c[threadIdx.x] = P.row[threadIdx.x].c;
   }
@@ -1610,20 +1704,17 @@ struct Eng {
       if (!S.flag_ok[k & 1]) return;   // the publishing warp's own wait runs out
       while (!mbar_try_wait(&S.full[bi], (k / kNBuf) & 1)) {
       }
-      Slot& T = slots[sl];
-      const bool leave = S.desc[bi].exit != 0;
-      if (leave) {
-        if (threadIdx.x == 0) T.mode = kSlotExit;
-      } else {
-        process(bi, T);
+      const FDesc& Dd = S.desc[k % kNDesc];
+      if (Dd.exit) {
+        if (threadIdx.x == 0) slots[sl].mode = kSlotExit;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&S.done[sl]);
+        return;
       }
-      // this warp is done with the buffer and with its part of the record
+      process(bi, Dd, slots[sl]);
+      // this warp is done with its part of the record
       __syncwarp();
-      if (lane == 0) {
-        mbar_arrive(&S.empty[bi]);
-        mbar_arrive(&S.done[sl]);
-      }
-      if (leave) return;
+      if (lane == 0) mbar_arrive(&S.done[sl]);
     }
   }
 
@@ -1640,7 +1731,7 @@ constexpr int kDecScratch = kDecStage + 2 * kMaxSlices * 4 + 64 * 4;   // + slic
 
 // Each kind of decision out of line (its own register allocation); each
 // rebuilds the warp's view of its shared state.
-template <int DT> __device__ __noinline__ void dec_stats_nl(int b, int j, int R, bool list);
+template <int DT> __device__ __noinline__ void dec_stats_nl(int b, int j);
 template <int DT> __device__ __noinline__ void dec_resid_nl(int b);
 template <int DT> __device__ __noinline__ void dec_replace_nl(int b);
 template <int DT> __device__ __noinline__ void dec_full_nl(int b);
@@ -1825,7 +1916,7 @@ struct Dec {
     unsigned base = 0u;
     if (lane == 0) {
       // ring numbers first: their round trip runs beside the state's stores
-      base = (unsigned)p.B * (unsigned)p.ng + atomicAdd(&p.ctl[kCtlTail], (unsigned)p.ng);
+      base = (unsigned)p.B * (unsigned)p.ng0 + atomicAdd(&p.ctl[kCtlTail], (unsigned)p.ng);
       D.P.kind = kind;
     }
     __syncwarp();
@@ -2197,13 +2288,11 @@ struct Dec {
       PT_T0(t_lp);
       float xr = 0.f;
       if (s <= 5) {
-        float x[5];
+        float x;
         bool capped;
         A = stage_solve5(A2, B2, A, Btok, u, D.om, D.om_q, D.om_a, D.om_b, x, &capped);
         if (capped && lane == 0) atomicOr(p.status, MDS_ST_LP_CAP);
-#pragma unroll
-        for (int t = 0; t < 5; ++t)
-          if (rk == t) xr = x[t];
+        xr = __shfl_sync(FULLM, x, rk & 31);
       } else {
         if (lane == 0) D.Y = lp_solve8(s, A2, B2, A, Btok, u);
         __syncwarp();
@@ -2251,14 +2340,11 @@ struct Dec {
     PT_T0(t_lp);
     int y;
     if (s <= 5) {
-      float x[5];
+      float x;
       bool capped;
       y = stage_solve5(A2, B2, A, Btok, u, D.om, D.om_q, D.om_a, D.om_b, x, &capped);
       if (capped && lane == 0) atomicOr(p.status, MDS_ST_LP_CAP);
-      if (lane == 0) {
-#pragma unroll
-        for (int t = 0; t < 5; ++t) D.om_x[t] = x[t];
-      }
+      if (lane < 5) D.om_x[lane] = x;
     } else {
       if (lane == 0) D.Y = lp_solve8(s, A2, B2, A, Btok, u);
       __syncwarp();
@@ -2310,7 +2396,7 @@ struct Dec {
     PT_ADDW(kPhDecAccept, t_acc);
   }
 
-  __device__ void decide_stats(int b, int j, int R, bool list) {
+  __device__ void decide_stats(int b, int j) {
     if (j == 0 && lane == 0) {
       D.W = FWalk{};
       D.W.valid = (p.K >= 32) ? FULLM : ((1u << p.K) - 1u);
@@ -2321,6 +2407,8 @@ struct Dec {
     plan_warp(b, j, D.W.valid, false, true, true, D.tk0);
     PT_ADDW(kPhDecPlan, t_plan);
     PT_T0(t_comb);
+    const int R = D.P.nstream;   // the planned pass is the completed one
+    const bool list = D.P.list != 0;
     combine(R, list);
     if (p.dbg_rows) debug_rows(b, j, R);
     xl_sync();
@@ -3031,15 +3119,15 @@ struct Dec {
   }
 
   // -------------------------------------------------------------- one decision
-  // Request fields: the sequence, the kind, depth, row count and list flag of
-  // the pass that just completed.
-  __device__ void decide(int b, int kind, int j, int R, bool list) {
+  // Request fields: the sequence, the depth of the pass that just completed
+  // and whether it is the sequence's first.
+  __device__ void decide(int b, int j, bool first) {
     // One round of asynchronous copies: the sequence's state (a depth-0
     // stats pass has none yet), its draft tokens at depths j and j + 1, its
     // temperatures and the slice records of the pass.
     const int K = p.K, L = p.L;
     PT_T0(t_load);
-    if (!(kind == kStats && j == 0)) {
+    if (!first) {
       const int4* src = reinterpret_cast<const int4*>(reinterpret_cast<const FSeq*>(p.seq) + b);
       int4* dst = reinterpret_cast<int4*>(&D.P);
       for (int i = lane; i < (int)(sizeof(FSeq) / 16); i += 32) cpa16(dst + i, src + i);
@@ -3066,8 +3154,9 @@ struct Dec {
     PT_ADDW(kPhDecLoad, t_load);
     PT_T0(t_dec);
     PT_CNTW(kPhDecisions);
+    const int kind = first ? kStats : D.P.kind;
     switch (kind) {
-      case kStats: dec_stats_nl<DT>(b, j, R, list); break;
+      case kStats: dec_stats_nl<DT>(b, j); break;
       case kResid: dec_resid_nl<DT>(b); break;
       case kReplace: dec_replace_nl<DT>(b); break;
       case kFull: dec_full_nl<DT>(b); break;
@@ -3090,34 +3179,30 @@ struct Dec {
       if (lane == 0 && !aborted()) {
         const unsigned t = atomicAdd(&p.ctl[kCtlDecHead], 1u);
         const unsigned slot = t % (unsigned)p.dec_cap;
-        const unsigned long long want = dec_tag_of(p.epoch, t);
+        const unsigned long long want = ring_word(p.epoch, t / (unsigned)p.dec_cap, 0u);
         const unsigned long long t0 = now_ns();
         PT_T0(t_poll);
         for (int it = 0;; ++it) {
-          if (ld_acquire(&p.dec_tag[slot]) == want) {
-            pay = __ldcg(&p.dec_pay[slot]);
-            st_release(&p.dec_rtag[slot], want);
+          const unsigned long long w = ld_acquire(&p.dec_tag[slot]);
+          if ((w & ~kRingPay) == want) {
+            pay = (unsigned)(w & kRingPay);
+            st_relaxed(&p.dec_rtag[slot], want);
             have = 1;
             break;
           }
-          if (ld_relaxed(&p.ctl[kCtlDone]) >= (unsigned)p.B || aborted()) break;
+          if ((it & 3) == 3 && (ld_relaxed(&p.ctl[kCtlDone]) >= (unsigned)p.B || aborted())) break;
           if ((it & 15) == 15 && now_ns() - t0 > kWaitNs) {
             set_abort(MDS_ST_TIMEOUT);
             break;
           }
-          __nanosleep(it < 16 ? 32 : 256);
+          __nanosleep(it < 16 ? 32 : 128);
         }
         PT_ADDW(kPhDecPoll, t_poll);
       }
       have = __shfl_sync(FULLM, have, 0);
       pay = __shfl_sync(FULLM, pay, 0);
       if (!have) return;
-      const int b = (int)(pay >> 16);
-      const int kind = (int)((pay >> 13) & 7u);
-      const int j = (int)((pay >> 6) & 127u);
-      const int R = (int)((pay >> 1) & 31u);
-      const bool list = (pay & 1u) != 0u;
-      decide(b, kind, j, R, list);
+      decide((int)(pay >> 8), (int)((pay >> 1) & 127u), (pay & 1u) != 0u);
     }
   }
 };
@@ -3132,7 +3217,8 @@ __shared__ Params g_dp;
 
 constexpr int kDStateBytes = (int)((sizeof(DState) + 127) / 128 * 128);
 constexpr int kDecPerWarp = kDStateBytes + (kDecScratch + 127) / 128 * 128;
-constexpr int kDynBytes = kNBuf * kBufBytes + 4 * kCandCap * 4 + kSlots * (int)sizeof(Slot);
+constexpr int kSlotOff = kNBuf * kBufBytes;
+constexpr int kDynBytes = kSlotOff + kSlots * (int)sizeof(Slot);
 constexpr int kDecWarps = 4;   // decision warps per decision CTA
 static_assert(kDecWarps * kDecPerWarp <= kDynBytes && kDecWarps <= kBlock / 32, "decision warps' shared memory");
 
@@ -3146,9 +3232,7 @@ __device__ __forceinline__ Dec<DT> dec_view() {
   return Dec<DT>{g_dp, g_S, *reinterpret_cast<DState*>(base), scr, rs, rs + kMaxSlices,
                  reinterpret_cast<uint32_t*>(rs + 2 * kMaxSlices), (int)(threadIdx.x & 31)};
 }
-template <int DT> __device__ __noinline__ void dec_stats_nl(int b, int j, int R, bool list) {
-  dec_view<DT>().decide_stats(b, j, R, list);
-}
+template <int DT> __device__ __noinline__ void dec_stats_nl(int b, int j) { dec_view<DT>().decide_stats(b, j); }
 template <int DT> __device__ __noinline__ void dec_resid_nl(int b) { dec_view<DT>().decide_resid(b); }
 template <int DT> __device__ __noinline__ void dec_replace_nl(int b) { dec_view<DT>().decide_replace(b); }
 template <int DT> __device__ __noinline__ void dec_full_nl(int b) { dec_view<DT>().decide_full(b); }
@@ -3177,12 +3261,12 @@ __global__ void __launch_bounds__(kBlock, kCtasPerSm) flow_kernel(const __grid_c
   FShared& S = g_S;
   Eng<DT> e{p, S};
   e.bufs = dsm;
-  char* c = dsm + (size_t)kNBuf * kBufBytes;
-  e.cid = reinterpret_cast<int*>(c);
-  e.cl = reinterpret_cast<float*>(c + kCandCap * 4);
-  e.crank = reinterpret_cast<int*>(c + 2 * kCandCap * 4);
-  e.cord = reinterpret_cast<int*>(c + 3 * kCandCap * 4);
-  e.slots = reinterpret_cast<Slot*>(c + 4 * kCandCap * 4);
+  e.slots = reinterpret_cast<Slot*>(dsm + kSlotOff);
+  // the block-wise list's arrays: a launch that uses them hands no lists over
+  e.cid = reinterpret_cast<int*>(&e.slots[0].l[0][0]);
+  e.cl = reinterpret_cast<float*>(e.cid + kCandCap);
+  e.crank = reinterpret_cast<int*>(&e.slots[1].l[0][0]);
+  e.cord = e.crank + kCandCap;
   if (threadIdx.x == 0) {
     for (int i = 0; i < kNBuf; ++i) {
       mbar_init(&S.full[i], 1);
@@ -3203,8 +3287,11 @@ __global__ void __launch_bounds__(kBlock, kCtasPerSm) flow_kernel(const __grid_c
   }
   // Roles: the CTAs on the first dec_sms SMs run decisions (kDecWarps
   // decision warps each, the rest of their warps idle), every other CTA
-  // streams slices (eight compute warps, a scheduler warp, a publishing warp).  Decisions are
-  // serial code: on their own SMs they do not wait behind the streaming warps.
+  // streams slices (eight compute warps, a scheduler warp, a publishing warp).
+  // Decisions are serial code of single warps, bound by latencies and
+  // instruction fetches: on their own SMs they share neither issue slots nor
+  // the instruction caches with the stream (B = 256, K = 8, V = 128256 WIS: a
+  // decision warp in every CTA instead took 1.2 times as long).
   __shared__ int role;
   if (threadIdx.x == 0) {
     unsigned smid;
@@ -3267,17 +3354,16 @@ size_t seq_bytes() { return sizeof(FSeq); }
 namespace {
 size_t up256(size_t x) { return (x + 255) / 256 * 256; }
 struct Layout {
-  size_t ctl, tag, dtag, dpay, cnt, seq, rec;
+  size_t ctl, tag, dtag, cnt, seq, rec;
   size_t cap, dcap;
 };
 Layout layout(const Params& p, int nseq, int grid) {
   Layout L;
   L.cap = (size_t)nseq * p.ng + (size_t)grid + 64;
   L.dcap = (size_t)nseq + (size_t)grid * kDecWarps + 64;   // one request per sequence, plus the claims
-  L.ctl = 256;
+  L.ctl = kCtlWords * 4;
   L.tag = up256(L.cap * 8);
   L.dtag = up256(L.dcap * 8);
-  L.dpay = up256(L.dcap * 4);
   L.cnt = up256((size_t)nseq * 4);
   L.seq = up256((size_t)nseq * sizeof(FSeq));
   L.rec = up256((size_t)nseq * p.ns * p.rec_floats * 4);
@@ -3287,12 +3373,12 @@ Layout layout(const Params& p, int nseq, int grid) {
 
 size_t workspace_bytes(const Params& p, int nseq, int grid) {
   const Layout L = layout(p, nseq, grid);
-  return L.ctl + 2 * L.tag + 2 * L.dtag + L.dpay + L.cnt + L.seq + L.rec;
+  return L.ctl + 2 * L.tag + 2 * L.dtag + L.cnt + L.seq + L.rec;
 }
 
 size_t clear_bytes(const Params& p, int nseq, int grid) {
   const Layout L = layout(p, nseq, grid);
-  return L.ctl + 2 * L.tag + 2 * L.dtag + L.dpay + L.cnt;
+  return L.ctl + 2 * L.tag + 2 * L.dtag + L.cnt;
 }
 
 void carve_workspace(Params& p, char* w, int nseq, int grid) {
@@ -3307,8 +3393,6 @@ void carve_workspace(Params& p, char* w, int nseq, int grid) {
   w += L.dtag;
   p.dec_rtag = reinterpret_cast<unsigned long long*>(w);
   w += L.dtag;
-  p.dec_pay = reinterpret_cast<unsigned*>(w);
-  w += L.dpay;
   p.cnt = reinterpret_cast<unsigned*>(w);
   w += L.cnt;
   p.seq = w;
@@ -3318,16 +3402,17 @@ void carve_workspace(Params& p, char* w, int nseq, int grid) {
   p.dec_cap = (int)L.dcap;
 }
 
-// SMs whose CTAs run the decisions: about a tenth of the grid's SMs, at
-// least one and never all of them.  The environment variable MDS_DEC_SMS
-// overrides the count (read once per process), for tuning.
-int decision_sms(int grid) {
+// SMs whose CTAs run the decisions, at least one and never all of them: a
+// tenth of the grid's SMs for the weighted schemes, half that for single,
+// whose decisions are short.  The environment variable MDS_DEC_SMS overrides
+// the count (read once per process), for tuning.
+int decision_sms(int grid, int scheme) {
   static const int env = [] {
     const char* e = getenv("MDS_DEC_SMS");
     return e ? atoi(e) : 0;
   }();
   const int sms = grid / kCtasPerSm;
-  int d = env > 0 ? env : (sms + 5) / 10;
+  int d = env > 0 ? env : (scheme == MDS_SINGLE ? (sms + 10) / 20 : (scheme == MDS_WIS0 ? (sms + 3) / 7 : (sms + 5) / 10));
   if (d < 1) d = 1;
   if (d > sms - 1) d = sms - 1;
   return d;
@@ -3416,8 +3501,10 @@ bool plan_geometry(Params& p, int grid) {
   // spread over the GPU.
   const long per_cta = (long)p.B * p.ns / grid;
   p.group = per_cta >= 32 ? 4 : (per_cta >= 16 ? 2 : 1);
+  p.group0 = per_cta >= 8 ? 4 : (per_cta >= 4 ? 2 : 1);   // depth 0: every sequence's slices at once
   p.ng = (p.ns + p.group - 1) / p.group;
-  p.dec_sms = decision_sms(grid);
+  p.ng0 = (p.ns + p.group0 - 1) / p.group0;
+  p.dec_sms = decision_sms(grid, p.scheme);
   return p.dec_sms > 0;
 }
 

@@ -22,10 +22,12 @@ constexpr int kMaxSlicesList = 32;     // slices per row with candidate lists
 constexpr int kMaxSlices = 256;        // slices per row otherwise
 constexpr int kSliceQuantum = 256;     // T is a multiple of this many tokens
 
-// Control words (ctl[]): task head and tail, finished sequences, abort flag,
-// CTAs that left the kernel.  All zero between launches.
-enum { kCtlHead = 0, kCtlTail = 1, kCtlDone = 2, kCtlAbort = 3, kCtlExit = 4, kCtlDecHead = 5, kCtlDecTail = 6,
-       kCtlWords = 16 };
+// Control words (ctl[], one to a 128-byte line: they are polled and counted by
+// every CTA at once): task head and tail, finished sequences, abort flag, CTAs
+// that left the kernel.  All zero between launches.
+constexpr int kCtlLine = 32;
+enum { kCtlHead = 0, kCtlTail = 1 * kCtlLine, kCtlDone = 2 * kCtlLine, kCtlAbort = 3 * kCtlLine,
+       kCtlExit = 4 * kCtlLine, kCtlDecHead = 5 * kCtlLine, kCtlDecTail = 6 * kCtlLine, kCtlWords = 7 * kCtlLine };
 
 struct Params {
   const char* target;                  // [B][K][L+1][V]
@@ -39,9 +41,8 @@ struct Params {
   unsigned* ctl;                       // control words
   unsigned long long* ring_tag;        // [ring_cap] published tasks (launch, lap, sequence, group)
   unsigned long long* ring_rtag;       // [ring_cap] launch and lap of tasks taken
-  unsigned long long* dec_tag;         // [dec_cap] published decision requests
-  unsigned long long* dec_rtag;        // [dec_cap] tags of requests taken
-  unsigned* dec_pay;                   // [dec_cap] the requests
+  unsigned long long* dec_tag;         // [dec_cap] published decision requests (launch, lap, sequence, depth)
+  unsigned long long* dec_rtag;        // [dec_cap] launch and lap of requests taken
   unsigned* cnt;                       // [B] slices of the current pass completed
   char* seq;                           // [B] per-sequence pass and walk state
   float* rec;                          // [B][ns][rec_floats] slice records
@@ -58,8 +59,8 @@ struct Params {
   unsigned lns_rcp;                    // ceil(2^32 / lns): entry / lns by a high product
   int fast_list;                       // the slices' lists are found warp by warp
   int kth;                             // ... each warp's threshold: its kth largest lane maximum
-  int group;                           // slices per task
-  int ng;                              // tasks per pass
+  int group, group0;                   // slices per task (group0: of the depth-0 passes)
+  int ng, ng0;                         // tasks per pass
   int rec_floats;                      // record stride per slice
   int hdr_floats;                      // start of a record's list entries
   int ring_cap;
