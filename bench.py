@@ -176,7 +176,7 @@ def hbm_peak():
 # the translation unit of each kernel and the internal headers it includes
 KERNEL_SOURCES = {
     "flow_kernel": ["mds_flow.cu", "mds_flow.h", "mds_device.cuh", "mds_internal.h"],
-    "verify_kernel": ["mds_kernel.cu", "mds_internal.h"],
+    "verify_kernel": ["mds_kernel.cu", "mds_device.cuh", "mds_internal.h"],
     "topk_kernel": ["mds_topk.cu", "mds_topk.h", "mds_device.cuh", "mds_internal.h"],
 }
 

@@ -233,7 +233,9 @@ int flow_verify(mds_ctx* ctx, const void* target_logits, const void* const* draf
                 void* stream, bool bulk_ok, bool aligned16) {
   const mds_config& c = ctx->cfg;
   mds::flow::Params p{};
-  if (!mds::flow_params(c, ctx->f_grid, scheme, model_of, n_models, bulk_ok, aligned16, p)) return mds::kNotServed;
+  // an export of row statistics wants the engine that writes them
+  if (!mds::flow_params(c, ctx->f_grid, scheme, model_of, n_models, bulk_ok, aligned16, p, ctx->dbg_rows != nullptr))
+    return mds::kNotServed;
   const size_t total = mds::flow::workspace_bytes(p, c.max_B, ctx->f_grid);
   DeviceGuard g(ctx->device);
   if (total > ctx->f_bytes) {
@@ -532,10 +534,26 @@ const char* status_message(unsigned st) {
   return "ok";
 }
 
+// Single draft from one model: a depth is one pass of two rows and a decision
+// of a few instructions, so the per-sequence engine, whose cluster combines a pass in
+// shared memory, beats the dataflow engine's ring, record and request round
+// trips (about 15 us a pass) until a CTA's slice of a row is long: measured at
+// K = 4, L = 4 in bf16, per-sequence against dataflow: slices of 2 to 8 KB 32
+// to 60 against 76 to 247 us, 31 KB 60 against 104, 62 KB 87 to 156 against
+// 107 to 274, 125 KB 144 against 123, 250 KB 267 against 178.  With several
+// models the per-sequence engine would stream every model's row.
+constexpr size_t kSeqSliceMax = 64 * 1024;
+static size_t seq_slice_bytes(const mds_config& c, int grid) {
+  int cn = 1;   // the cluster size the per-sequence engine takes
+  while (cn < kMaxCluster && 2L * cn * c.max_B <= grid) cn *= 2;
+  return (size_t)((c.V + cn - 1) / cn) * (size_t)esize_of(c.dtype);
+}
+
 bool flow_params(const mds_config& c, int grid, int scheme, const int8_t* model_of, int n_models, bool bulk_ok,
-                 bool aligned16, flow::Params& p) {
+                 bool aligned16, flow::Params& p, bool always) {
   if (scheme != MDS_SINGLE && scheme != MDS_WIS && scheme != MDS_WIS0) return false;
   if (grid <= 0 || c.cluster != 0 || c.max_B > 65535) return false;   // ring entries hold 16-bit ids
+  if (scheme == MDS_SINGLE && n_models == 1 && !always && seq_slice_bytes(c, grid) <= kSeqSliceMax) return false;
   p = flow::Params{};
   p.scheme = scheme;
   p.dtype = c.dtype;

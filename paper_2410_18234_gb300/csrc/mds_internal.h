@@ -84,9 +84,10 @@ constexpr int kNotServed = 1;   // a configuration left to the per-sequence engi
 
 // Slice-dataflow engine parameters of a call with configuration c on a grid
 // of `grid` CTAs (geometry sized for c.max_B sequences): false if the engine
-// does not serve the call.  Buffers are filled in by flow_buffers.
+// does not serve the call, or (unless `always`) the per-sequence engine is the
+// faster one for it.  Buffers are filled in by flow_buffers.
 bool flow_params(const mds_config& c, int grid, int scheme, const int8_t* model_of, int n_models, bool bulk_ok,
-                 bool aligned16, flow::Params& p);
+                 bool aligned16, flow::Params& p, bool always = false);
 void flow_buffers(flow::Params& p, const void* target_logits, const void* const* draft_logits,
                   const int32_t* draft_tokens, const float* temperatures, int32_t* out_tokens,
                   int32_t* out_accept_len, float* out_diag, int B, uint64_t seed);

@@ -30,6 +30,7 @@
 #include <cuda_bf16.h>
 #include <cooperative_groups.h>
 
+#include "mds_device.cuh"
 #include "mds_internal.h"
 
 namespace mds {
@@ -41,8 +42,6 @@ constexpr float kPosInf = __builtin_huge_valf();
 constexpr int kWarps = kThreads / 32;
 constexpr int kTop = 8;                 // per-thread candidate list length (>= MDS_MAX_S)
 constexpr int kMaxPairs = MDS_MAX_S * (MDS_MAX_S - 1) / 2;
-constexpr int kLpMaxAugment = 4096;
-constexpr float kLpEpsRel = 1e-6f;
 constexpr long long kWaitLimit = 1ll << 24;
 constexpr int kFastRows = 4;            // WIS candidate path: target + up to 3 draft models
 constexpr int kWStages = 5;             // stages of each warp's streaming ring
@@ -381,25 +380,6 @@ __device__ void warp_merge(Cand (&top)[kTop], Cand* out, int rounds, float& rest
   rest_a = warp_sum(ra);
   rest_b = warp_sum(rb);
 }
-
-// Pair {u, v}, u != v, of tokens below SM: its index in the lexicographic
-// order of (i, j), i < j < SM.
-__host__ __device__ constexpr int pidx(int u, int v, int SM) {
-  return (u < v) ? u * (2 * SM - u - 1) / 2 + (v - u - 1) : v * (2 * SM - v - 1) / 2 + (u - v - 1);
-}
-// Lower token of pair e in that order.
-__host__ __device__ constexpr int pidx_lo(int e, int SM) {
-  int i = 0, n = SM - 1;
-  while (e >= n) {
-    e -= n;
-    ++i;
-    --n;
-  }
-  return i;
-}
-static_assert(pidx(0, 1, 8) == 0 && pidx(1, 2, 8) == 7 && pidx(5, 3, 8) == pidx(3, 5, 8) && pidx(6, 7, 8) == 27 &&
-                  pidx(3, 4, 5) == 9 && pidx_lo(pidx(3, 6, 8), 8) == 3 && pidx_lo(pidx(2, 4, 5), 5) == 2,
-              "pair indexing");
 
 // Insert into a sorted (best first) candidate list; whatever drops out adds
 // its a and b to the running Omega_2 masses.
@@ -1470,262 +1450,33 @@ struct Kernel {
   }
 
   // ---------------------------------------------------------------- WIS: the stage LP
-  // Maximum flow of one stage on the pair/token network, in the fixed order
-  // (a) direct pass over pairs (i, j), i < j, lexicographically: each gives
-  // what it can to token i, then to token j; (b) breadth-first augmenting
-  // paths in token space (sources: tokens of pairs with supply left, each
-  // with the first such pair; u -> v when pair {u, v} gives flow to u;
-  // levels in increasing token order, a token's parent the first frontier
-  // token reaching it; the path ends at the first token with demand left);
-  // (c) the caller splits leftover pair mass 1/2 - 1/2.  Residuals <= eps
-  // count as zero.  SM is the compile-time token capacity (5 covers s <= 5
-  // in registers; 8 covers every s); all state lives in registers indexed
-  // by compile-time constants.  Single thread.
-  template <int SM>
-  __device__ __forceinline__ void lp_flow(int s, float (&rd)[SM], float (&RS)[SM * (SM - 1) / 2],
-                                          float (&FL)[SM * (SM - 1) / 2], float (&FH)[SM * (SM - 1) / 2], float eps) {
-    constexpr int P = SM * (SM - 1) / 2;
-#pragma unroll
-    for (int i = 0; i < SM; ++i) {
-#pragma unroll
-      for (int j = i + 1; j < SM; ++j) {
-        if (j >= s) continue;
-        const int e = pidx(i, j, SM);
-        if (RS[e] > eps && rd[i] > eps) {
-          const float d = fminf(RS[e], rd[i]);
-          FL[e] = __fadd_rn(FL[e], d);
-          RS[e] = __fsub_rn(RS[e], d);
-          rd[i] = __fsub_rn(rd[i], d);
-        }
-        if (RS[e] > eps && rd[j] > eps) {
-          const float d = fminf(RS[e], rd[j]);
-          FH[e] = __fadd_rn(FH[e], d);
-          RS[e] = __fsub_rn(RS[e], d);
-          rd[j] = __fsub_rn(rd[j], d);
-        }
-      }
-    }
-    for (int it = 0; it < kLpMaxAugment; ++it) {
-      // demands first: with none left (or, below, no supply left) no
-      // augmenting path exists
-      uint32_t dm = 0u;
-#pragma unroll
-      for (int t = 0; t < SM; ++t)
-        if (t < s && rd[t] > eps) dm |= 1u << t;
-      if (!dm) return;
-      // adjacency (u -> v when pair {u,v} gives flow to u), sources
-      uint32_t adj[SM];
-#pragma unroll
-      for (int t = 0; t < SM; ++t) adj[t] = 0u;
-      uint32_t srcm = 0u, par = 0u;
-      unsigned long long srcp = 0ull;
-#pragma unroll
-      for (int i = 0; i < SM; ++i) {
-#pragma unroll
-        for (int j = i + 1; j < SM; ++j) {
-          if (j >= s) continue;
-          const int e = pidx(i, j, SM);
-          if (FL[e] > eps) adj[i] |= 1u << j;
-          if (FH[e] > eps) adj[j] |= 1u << i;
-          if (RS[e] > eps) {
-            if (!(srcm >> i & 1u)) {
-              srcm |= 1u << i;
-              srcp |= (unsigned long long)e << (5 * i);
-            }
-            if (!(srcm >> j & 1u)) {
-              srcm |= 1u << j;
-              srcp |= (unsigned long long)e << (5 * j);
-            }
-          }
-        }
-      }
-      if (!srcm) return;
-      uint32_t visited = srcm, frontier = srcm, hit = srcm & dm;
-      for (int level = 0; level < SM && !hit && frontier; ++level) {
-        uint32_t nxt = 0u;
-#pragma unroll
-        for (int u = 0; u < SM; ++u) {
-          if (!(frontier >> u & 1u)) continue;
-          const uint32_t nb = adj[u] & ~(visited | nxt);
-#pragma unroll
-          for (int v = 0; v < SM; ++v)
-            if (nb >> v & 1u) par |= (uint32_t)(u + 1) << (4 * v);
-          nxt |= nb;
-        }
-        visited |= nxt;
-        frontier = nxt;
-        hit = nxt & dm;
-      }
-      if (!hit) return;
-      const int sink = __ffs(hit) - 1;
-      // bottleneck along the path sink <- ... <- t0
-      float delta = 0.f;
-#pragma unroll
-      for (int k = 0; k < SM; ++k)
-        if (k == sink) delta = rd[k];
-      int t = sink, t0 = sink;
-      for (int g = 0; g < SM; ++g) {
-        const int u = (int)((par >> (4 * t)) & 15u) - 1;
-        if (u < 0) {
-          t0 = t;
-          break;
-        }
-        const int e = pidx(u, t, SM);
-        float fl = 0.f;
-#pragma unroll
-        for (int k = 0; k < P; ++k)
-          if (k == e) fl = (u < t) ? FL[k] : FH[k];
-        delta = fminf(delta, fl);
-        t = u;
-      }
-      const int e0 = (int)((srcp >> (5 * t0)) & 31ull);
-      const bool lo0 = pidx_lo(e0, SM) == t0;
-#pragma unroll
-      for (int k = 0; k < P; ++k)
-        if (k == e0) delta = fminf(delta, RS[k]);
-      // push
-#pragma unroll
-      for (int k = 0; k < P; ++k) {
-        if (k == e0) {
-          RS[k] = __fsub_rn(RS[k], delta);
-          if (lo0)
-            FL[k] = __fadd_rn(FL[k], delta);
-          else
-            FH[k] = __fadd_rn(FH[k], delta);
-        }
-      }
-      t = sink;
-      for (int g = 0; g < SM; ++g) {
-        const int u = (int)((par >> (4 * t)) & 15u) - 1;
-        if (u < 0) break;
-        const int e = pidx(u, t, SM);
-        const bool ulo = u < t;
-#pragma unroll
-        for (int k = 0; k < P; ++k) {
-          if (k == e) {
-            if (ulo) {
-              FL[k] = __fsub_rn(FL[k], delta);
-              FH[k] = __fadd_rn(FH[k], delta);
-            } else {
-              FH[k] = __fsub_rn(FH[k], delta);
-              FL[k] = __fadd_rn(FL[k], delta);
-            }
-          }
-        }
-        t = u;
-      }
-#pragma unroll
-      for (int k = 0; k < SM; ++k)
-        if (k == sink) rd[k] = __fsub_rn(rd[k], delta);
-    }
-    atomicOr(p.status, MDS_ST_LP_CAP);
-  }
-
-  // Solve one stage given Omega_1 in S.om (increasing token ids; entries
-  // past s ignored) with q, a, b at those tokens in S.om_q / S.om_a / S.om_b
-  // and the Omega_2 masses: writes p_I on Omega_1 to S.om_x and returns the
-  // stage output for the ordered inputs (A, B) and uniform u.  Single thread.
-  // Pair state: registers for SM = 5, the shared LP scratch for SM = 8.
-  template <int SM>
-  __device__ __forceinline__ int stage_solve_t(int s, float A2, float B2, int A, int Btok, float u) {
-    constexpr int P = SM * (SM - 1) / 2;
-    if constexpr (SM == 5) {
-      float RS[P], FL[P], FH[P];
-      return stage_solve_body<SM>(s, A2, B2, A, Btok, u, RS, FL, FH);
+  // One pairwise stage on the tables om, om_q, om_a, om_b (by warp 0, all its
+  // lanes; entries past s are zero): p_I on Omega_1 to om_x, the stage's
+  // token returned.
+  __device__ int stage_solve(int s, float A2, float B2, int A, int Btok, float u) {
+    const int lane = threadIdx.x & 31;
+    int y;
+    if (s <= 5) {
+      float x;
+      bool capped;
+      y = dev::stage_solve5(A2, B2, A, Btok, u, S.om, S.om_q, S.om_a, S.om_b, x, &capped);
+      if (capped && lane == 0) atomicOr(p.status, MDS_ST_LP_CAP);
+      if (lane < 5) S.om_x[lane] = x;
+      __syncwarp();
     } else {
-      static_assert(P == kMaxPairs, "pair state");
-      return stage_solve_body<SM>(s, A2, B2, A, Btok, u, S.lp_rs, S.lp_fl, S.lp_fh);
+      if (lane == 0) stage_solve_wide(s, A2, B2, A, Btok, u);
+      __syncwarp();
+      y = S.Y;
     }
+    return y;
   }
-
-  template <int SM>
-  __device__ __forceinline__ int stage_solve_body(int s, float A2, float B2, int A, int Btok, float u,
-                                                  float (&RS)[SM * (SM - 1) / 2], float (&FL)[SM * (SM - 1) / 2],
-                                                  float (&FH)[SM * (SM - 1) / 2]) {
-    float ak[SM], bk[SM], x[SM], rd[SM];
-    float eps = 0.f;
-#pragma unroll
-    for (int t = 0; t < SM; ++t) {
-      ak[t] = S.om_a[t];
-      bk[t] = S.om_b[t];
-      const float qk = S.om_q[t];
-      x[t] = __fadd_rn(__fadd_rn(__fmul_rn(ak[t], bk[t]), __fmul_rn(ak[t], B2)), __fmul_rn(bk[t], A2));
-      rd[t] = (t < s) ? fmaxf(0.f, __fsub_rn(qk, x[t])) : 0.f;
-      if (t < s) eps = __fadd_rn(eps, __fadd_rn(qk, x[t]));
-    }
-    eps = __fmul_rn(eps, kLpEpsRel);
-#pragma unroll
-    for (int i = 0; i < SM; ++i) {
-#pragma unroll
-      for (int j = i + 1; j < SM; ++j) {
-        const int e = pidx(i, j, SM);
-        RS[e] = (j < s) ? __fadd_rn(__fmul_rn(ak[i], bk[j]), __fmul_rn(ak[j], bk[i])) : 0.f;
-        FL[e] = 0.f;
-        FH[e] = 0.f;
-      }
-    }
-    lp_flow<SM>(s, rd, RS, FL, FH, eps);
-    // p_I on Omega_1: base + flow + half of the pair mass left over
-#pragma unroll
-    for (int i = 0; i < SM; ++i) {
-#pragma unroll
-      for (int j = i + 1; j < SM; ++j) {
-        if (j >= s) continue;
-        const int e = pidx(i, j, SM);
-        const float half = __fmul_rn(0.5f, RS[e]);
-        x[i] = __fadd_rn(x[i], __fadd_rn(FL[e], half));
-        x[j] = __fadd_rn(x[j], __fadd_rn(FH[e], half));
-      }
-    }
-#pragma unroll
-    for (int t = 0; t < SM; ++t) S.om_x[t] = x[t];
-    // the stage output for the ordered inputs (A, B): only the weight of
-    // the pair {A, B} is needed
-    if (A == Btok) return A;
-    int pa = -1, pb = -1;
-#pragma unroll
-    for (int t = 0; t < SM; ++t) {
-      if (t < s && S.om[t] == A) pa = t;
-      if (t < s && S.om[t] == Btok) pb = t;
-    }
-    if (pa >= 0 && pb >= 0) {
-      const int lo = min(pa, pb), hi = max(pa, pb);
-      const int e = pidx(lo, hi, SM);
-      float fl = 0.f, rs = 0.f, alo = 0.f, ahi = 0.f, blo = 0.f, bhi = 0.f;
-#pragma unroll
-      for (int k = 0; k < SM * (SM - 1) / 2; ++k)
-        if (k == e) {
-          fl = FL[k];
-          rs = RS[k];
-        }
-#pragma unroll
-      for (int t = 0; t < SM; ++t) {
-        if (t == lo) {
-          alo = ak[t];
-          blo = bk[t];
-        }
-        if (t == hi) {
-          ahi = ak[t];
-          bhi = bk[t];
-        }
-      }
-      const float m = __fadd_rn(__fmul_rn(alo, bhi), __fmul_rn(ahi, blo));
-      const float wlo = m > 0.f ? __fdiv_rn(__fadd_rn(fl, __fmul_rn(0.5f, rs)), m) : 0.5f;
-      const float wa = (pa < pb) ? wlo : __fsub_rn(1.f, wlo);
-      return (u < wa) ? A : Btok;
-    }
-    if (pa >= 0) return A;
-    if (pb >= 0) return Btok;
-    return (u < 0.5f) ? A : Btok;
-  }
-
-  // s > 5 is rare (the paper's runs use s = 5 or 7): keep its larger state
-  // out of the inlined hot path.
-  __device__ __noinline__ int stage_solve_wide(int s, float A2, float B2, int A, int Btok, float u) {
-    return stage_solve_t<MDS_MAX_S>(s, A2, B2, A, Btok, u);
-  }
-  __device__ __forceinline__ int stage_solve(int s, float A2, float B2, int A, int Btok, float u) {
-    return (s <= 5) ? stage_solve_t<5>(s, A2, B2, A, Btok, u) : stage_solve_wide(s, A2, B2, A, Btok, u);
+  // s > 5 (the paper's runs use s = 5 or 7): one lane, the pair state in
+  // shared memory.
+  __device__ __noinline__ void stage_solve_wide(int s, float A2, float B2, int A, int Btok, float u) {
+    bool capped;
+    S.Y = dev::stage_solve<MDS_MAX_S>(s, A2, B2, A, Btok, u, S.om, S.om_q, S.om_a, S.om_b, S.om_x, &capped, S.lp_rs,
+                                      S.lp_fl, S.lp_fh);
+    if (capped) atomicOr(p.status, MDS_ST_LP_CAP);
   }
 
   // Law update shared by both paths: generic coefficients gamma.
@@ -1894,13 +1645,14 @@ struct Kernel {
             if (k < s && S.fin[k].id == S.om[t]) qv = qf[k];
           S.om_q[t] = qv;
         }
-        S.Y = stage_solve(s, sa, sb, A, Btok, u);
         S.A2 = sa;
         S.B2 = sb;
       }
       __syncwarp();
-      // law update: special tokens outside Omega_1 (lanes), gamma, Omega_1 values
       const float A2 = S.A2, B2 = S.B2;
+      const int y = stage_solve(s, A2, B2, A, Btok, u);
+      if (lane == 0) S.Y = y;
+      // law update: special tokens outside Omega_1 (lanes), gamma, Omega_1 values
       for (int i = lane; i < S.nspec; i += 32) {
         const int tokn = S.spec_id[i];
         bool in1 = false;
@@ -1993,21 +1745,18 @@ struct Kernel {
           S.om_b[rk] = b;
         }
         __syncwarp();
+        // Omega_2 masses: complement (generic law) + list entries outside Omega_1
+        float A2 = 0.f;
+        for (int r = 1; r < S.nrows; ++r)
+          if (S.gamma[r] != 0.f) A2 = __fmaf_rn(S.gamma[r], __fmul_rn(S.pc[r], S.invZ[r]), A2);
+        const float B2 = __fadd_rn(__fmul_rn(S.pc[rb], izb), rbm);
+        A2 = __fadd_rn(A2, ra);
+        const int y = stage_solve(s, A2, B2, A, Btok, u);
         if (lane == 0) {
-          // Omega_2 masses: complement (generic law) + list entries outside Omega_1
-          float sa = 0.f;
-          for (int r = 1; r < S.nrows; ++r)
-            if (S.gamma[r] != 0.f) sa = __fmaf_rn(S.gamma[r], __fmul_rn(S.pc[r], S.invZ[r]), sa);
-          const float sb = __fadd_rn(__fmul_rn(S.pc[rb], izb), rbm);
-          sa = __fadd_rn(sa, ra);
-          S.Y = stage_solve(s, sa, sb, A, Btok, u);
-          S.A2 = sa;
-          S.B2 = sb;
+          S.Y = y;
           S.fast_ok = 1;
         }
-        __syncwarp();
         // law update on the list: Omega_1 takes its x, other specials mix
-        const float A2 = S.A2, B2 = S.B2;
         if (sel) {
           cm_a[lane] = S.om_x[rk];
           cm_sp[lane] = 1;
@@ -2626,9 +2375,7 @@ struct Kernel {
             S.om_b[rk1] = bb;
           }
           __syncwarp();
-          if (lane == 0) S.Y = stage_solve(sn, A2, B2, cm_id[A], cm_id[Bl], u);
-          __syncwarp();
-          const int Yt = S.Y;
+          const int Yt = stage_solve(sn, A2, B2, cm_id[A], cm_id[Bl], u);
           A = max(0, __ffs(__ballot_sync(FULL, in0 && id == Yt)) - 1);   // Yt is A's or B's token
           a = sel ? S.om_x[rk1] : (in0 ? __fmul_rn(0.5f, __fadd_rn(__fmul_rn(a, B2), __fmul_rn(bb, A2))) : 0.f);
           __syncwarp();

@@ -613,17 +613,21 @@ __device__ int wis_stage(const Params& p, Shared& S, int A, int Btok, int rb, fl
     }
     __syncwarp();
   }
+  int y = 0;
+  if (s <= 5) {
+    float x;
+    bool capped;
+    y = stage_solve5(A2, B2, A, Btok, u, S.om, S.om_q, S.om_a, S.om_b, x, &capped);
+    if (capped && lane == 0) atomicOr(p.status, MDS_ST_LP_CAP);
+    if (lane < 5) S.om_x[lane] = x;
+  }
   if (lane == 0) {
-    bool capped = false;
-    int y;
-    if (s <= 5) {
-      float RS[10], FL[10], FH[10];
-      y = stage_solve<5>(s, A2, B2, A, Btok, u, S.om, S.om_q, S.om_a, S.om_b, S.om_x, &capped, RS, FL, FH);
-    } else {
+    if (s > 5) {
+      bool capped = false;
       y = stage_solve<MDS_MAX_S>(s, A2, B2, A, Btok, u, S.om, S.om_q, S.om_a, S.om_b, S.om_x, &capped, S.RS, S.FL,
                                  S.FH);
+      if (capped) atomicOr(p.status, MDS_ST_LP_CAP);
     }
-    if (capped) atomicOr(p.status, MDS_ST_LP_CAP);
     if (sorted && A != Btok) {
       // both inputs in Omega_2: the one earlier in key order (a token outside U has key 0)
       bool ia = false, ib = false;
@@ -650,7 +654,7 @@ __device__ int wis_stage(const Params& p, Shared& S, int A, int Btok, int rb, fl
                : sorted   ? S.nxt[i]
                           : __fmul_rn(0.5f, __fadd_rn(__fmul_rn(S.cur[i], B2), __fmul_rn(bl[i], A2)));
   }
-  const int y = S.Y;
+  y = S.Y;
   __syncwarp();
   return y;
 }
