@@ -466,6 +466,15 @@ struct Kernel {
   uint32_t wphase;     // parity of each stage of this warp's ring
   int bail;            // this warp's ring gave up on a copy: it streams nothing more
 
+  // A row's constants in registers, for the passes' inner loops (through the
+  // shared state every unit would load them again); prob() is prob_of.
+  struct RowC {
+    float c, mc, iz;
+    __device__ __forceinline__ float arg(float l) const { return __fmaf_rn(l, c, -mc); }
+    __device__ __forceinline__ float prob(float l) const { return __fmul_rn(ex2(arg(l)), iz); }
+  };
+  __device__ __forceinline__ RowC row_c(int r) const { return RowC{S.c[r], __fmul_rn(S.M[r], S.c[r]), S.invZ[r]}; }
+
   __device__ float prob_row(int r, int x) const {
     return prob_of(E::global(S.gptr[r], x), S.M[r], S.c[r], S.invZ[r]);
   }
@@ -1814,7 +1823,7 @@ struct Kernel {
   // sums have a fixed order.  Eight warps x 32 bins x 4 copies take 32 KB
   // (two CTAs per SM); wider ranges of rho take further windows of 32 bins.
   // What bounds it now is issue: about 3 instructions a token in the adds.
-  // Measured (GB300): B = 64, K = 4, V = 32000 594 -> 222 us a call, B = 1024,
+  // Measured (GB300): B = 64, K = 4, V = 32000 590 -> 197 us a call, B = 1024,
   // K = 4, V = 151936 22.1 -> 5.4 ms; p_I(Y) 3e-7 off 64 bits before and after.
 
   // exp(-s e^(d v)) = sum_k z[k] v^k, d = half a bin in ln rho: the series of
@@ -1838,12 +1847,9 @@ struct Kernel {
     const int o = (n >= 0) ? n / kIsSub : -((kIsSub - 1 - n) / kIsSub);
     return ldexpf(ex2((float)(n - o * kIsSub) / kIsSub), o);
   }
-  // log2 rho of a token in bins, from the row's and the target's logit; the
-  // probabilities follow prob_of.
-  __device__ __forceinline__ float is_pos(float lq, float lp, int r) const {
-    const float aq = __fmaf_rn(lq, S.c[0], -__fmul_rn(S.M[0], S.c[0]));
-    const float ap = __fmaf_rn(lp, S.c[r], -__fmul_rn(S.M[r], S.c[r]));
-    return __fmul_rn(__fadd_rn(__fsub_rn(aq, ap), S.is_lz[r]), (float)kIsSub);
+  // log2 rho of a token in bins, from the exponents of its probabilities.
+  __device__ __forceinline__ static float is_pos(float aq, float ap, float lz) {
+    return __fmul_rn(__fadd_rn(__fsub_rn(aq, ap), lz), (float)kIsSub);
   }
 
   // Add this warp's set-aside tokens (v, v^2, p, bin) to its bins.
@@ -1878,6 +1884,8 @@ struct Kernel {
     for (int i = lane; i < kIsWin * 4 * kIsMom; i += 32) bins[i] = 0.f;
     __syncwarp();
     float zero = 0.f;
+    const RowC c0 = row_c(0), cr = row_c(r);
+    const float lz = S.is_lz[r];
     stream(1u | (1u << r), [&](int, bool valid, const auto& L) {
       float lq[VE], lp[VE];
       if (valid) {
@@ -1892,9 +1900,9 @@ struct Kernel {
         int cnt = 0;
 #pragma unroll
         for (int e = e0; e < e0 + 2; ++e) {
-          const float pr = prob_of(lp[e], S.M[r], S.c[r], S.invZ[r]);
-          const float q = prob_of(lq[e], S.M[0], S.c[0], S.invZ[0]);
-          const float x = is_pos(lq[e], lp[e], r);
+          const float aq = c0.arg(lq[e]), ap = cr.arg(lp[e]);
+          const float pr = __fmul_rn(ex2(ap), cr.iz), q = __fmul_rn(ex2(aq), c0.iz);
+          const float x = is_pos(aq, ap, lz);
           const float n = rintf(x);
           const int bin = (int)n - b0;
           const bool pos = pr > 0.f && q > 0.f;
@@ -1962,6 +1970,9 @@ struct Kernel {
     float lo = kPosInf, hi = 0.f;
     for (int r = 1; r < S.nrows; ++r) {
       if (!S.is_cnt[r]) continue;
+      // by the exponents' difference (log2 rho, rounded once per row below)
+      const RowC c0 = row_c(0), cr = row_c(r);
+      float dlo = kPosInf, dhi = kNegInf;
       stream(1u | (1u << r), [&](int, bool valid, const auto& L) {
         if (!valid) return;
         float v[VE], w[VE];
@@ -1969,15 +1980,18 @@ struct Kernel {
         L(r, w);
 #pragma unroll
         for (int e = 0; e < VE; ++e) {
-          const float q = prob_of(v[e], S.M[0], S.c[0], S.invZ[0]);
-          const float pr = prob_of(w[e], S.M[r], S.c[r], S.invZ[r]);
-          if (pr > 0.f && q > 0.f) {
-            const float rho = __fdiv_rn(q, pr);
-            lo = fminf(lo, rho);
-            hi = fmaxf(hi, rho);
+          const float aq = c0.arg(v[e]), ap = cr.arg(w[e]);
+          if (__fmul_rn(ex2(ap), cr.iz) > 0.f && __fmul_rn(ex2(aq), c0.iz) > 0.f) {
+            const float d = __fsub_rn(aq, ap);
+            dlo = fminf(dlo, d);
+            dhi = fmaxf(dhi, d);
           }
         }
       });
+      if (dlo <= dhi) {
+        lo = fminf(lo, exp2f(__fadd_rn(dlo, S.is_lz[r])));
+        hi = fmaxf(hi, exp2f(__fadd_rn(dhi, S.is_lz[r])));
+      }
     }
 #pragma unroll
     for (int o = 16; o; o >>= 1) {
@@ -2005,7 +2019,7 @@ struct Kernel {
         rhi = fmaxf(rhi, S.gat[2 * q + 1]);
       }
       rlo = fmaxf(rlo, 1e-37f);
-      rhi = fmaxf(rhi, rlo);
+      rhi = fminf(fmaxf(rhi, rlo), 3e38f);
       const float h = p.is_h;
       const float ulo = -logf((float)S.nv * rhi) - 40.f;
       const float uhi = logf(40.f / rlo);
@@ -2018,7 +2032,7 @@ struct Kernel {
       // without a token of positive q and p)
       S.is_b0 = 0;
       S.is_nb = 0;
-      if (rlo <= rhi && rhi < kPosInf) {
+      if (rlo <= rhi) {
         S.is_b0 = (int)floorf(kIsSub * log2f(rlo)) - 1;
         S.is_nb = (int)ceilf(kIsSub * log2f(rhi)) + 2 - S.is_b0;
       }
@@ -2572,6 +2586,7 @@ struct Kernel {
           }
           if (!done) {
             const int r1 = S.vrow[0];
+            const RowC c0 = row_c(0), c1 = row_c(r1);
             Z = sample_cdf(
                 1u | (1u << r1),
                 [&](int, const auto& L, float* r) {
@@ -2579,9 +2594,7 @@ struct Kernel {
                   L(0, v);
                   L(r1, w);
 #pragma unroll
-                  for (int e = 0; e < VE; ++e)
-                    r[e] = fmaxf(0.f, __fsub_rn(prob_of(v[e], S.M[0], S.c[0], S.invZ[0]),
-                                                prob_of(w[e], S.M[r1], S.c[r1], S.invZ[r1])));
+                  for (int e = 0; e < VE; ++e) r[e] = fmaxf(0.f, __fsub_rn(c0.prob(v[e]), c1.prob(w[e])));
                 },
                 ures, &tot);
           }
@@ -2697,10 +2710,12 @@ struct Kernel {
         L(rr, lp);
         const float* tab = isBin + (size_t)row * S.is_nb * kIsMom;
         ++row;
+        const RowC c0 = row_c(0), cr = row_c(rr);
+        const float lz = S.is_lz[rr];
 #pragma unroll
         for (int e = 0; e < VE; ++e) {
-          if (!(prob_of(lp[e], S.M[rr], S.c[rr], S.invZ[rr]) > 0.f) || !(q[e] > 0.f)) continue;
-          const float x = is_pos(lq[e], lp[e], rr);
+          if (!(cr.prob(lp[e]) > 0.f) || !(q[e] > 0.f)) continue;
+          const float x = is_pos(c0.arg(lq[e]), cr.arg(lp[e]), lz);
           const float n = rintf(x);
           const int bin = (int)n - S.is_b0;
           if (bin < 0 || bin >= S.is_nb) {
@@ -2747,7 +2762,8 @@ struct Kernel {
   // *Rd: the product of the rounds' residual masses, the probability that
   // every round rejects (1 - the depth's acceptance probability); with
   // acc_prob the rounds after an acceptance are computed for it too, without
-  // changing the token.
+  // changing the token.  The last round's mass pass is the residual draw's own
+  // pass: its weights are the last target up to the factor 1 / R.
   __device__ int spectr(int b, int j, float* qY, float* pIY, int* Yd, float* Rd) {
     const int nv = S.nv;
     int zacc = -1;
@@ -2785,18 +2801,29 @@ struct Kernel {
         }
       }
       // residual mass of this round
-      float part = 0.f;
       const int ri = S.sp_rows[i];
       uint32_t mask = 1u | (1u << ri);
       for (int k = 0; k < i; ++k) mask |= 1u << S.sp_rows[k];
+      const SpectrW sw = spectr_weights(i, ri);
+      if (i == nv - 1 && zacc < 0) {
+        __syncthreads();   // every thread has read the round's state
+        float tot;
+        const int z = sample_cdf(mask, [&](int, const auto& L, float* r) { spectr_resid(L, sw, r); },
+                                 draw_uniform(p.seed, b, j, kDrawResidual), &tot);
+        *Rd = __fmul_rn(prodR, tot);
+        if (tot > 0.f) return z;
+        // no mass (only by rounding, q_i = p_i): the round leaves q_i as it is
+        const SpectrW st = spectr_weights(i, -1);
+        return sample_cdf(mask, [&](int, const auto& L, float* r) { spectr_resid(L, st, r); },
+                          draw_uniform(p.seed, b, j, kDrawResidual), &tot);
+      }
+      float part = 0.f;
       stream(mask, [&](int, bool valid, const auto& L) {
         if (!valid) return;
         float r[VE];
-        spectr_target(L, i, r);
-        float w[VE];
-        L(ri, w);
+        spectr_resid(L, sw, r);
 #pragma unroll
-        for (int e = 0; e < VE; ++e) part += fmaxf(0.f, __fsub_rn(r[e], prob_of(w[e], S.M[ri], S.c[ri], S.invZ[ri])));
+        for (int e = 0; e < VE; ++e) part = __fadd_rn(part, r[e]);
       });
       part = warp_sum(part);
       const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -2819,30 +2846,58 @@ struct Kernel {
       __syncthreads();
     }
     *Rd = prodR;
-    if (zacc >= 0) return zacc;
-    float tot;
-    uint32_t mask = 1u;
-    for (int k = 0; k < nv; ++k) mask |= 1u << S.sp_rows[k];
-    const int z = sample_cdf(mask, [&](int, const auto& L, float* r) { spectr_target(L, nv, r); },
-                             draw_uniform(p.seed, b, j, kDrawResidual), &tot);
-    return z;
+    return zacc;
   }
 
-  // running target after `rounds` rejected rounds, for one unit
+  // Weights of a round: the running target after `rounds` rejected rounds
+  // less the draft row ri (clamped at 0), or (ri < 0) that target itself.
+  // With one draft row in play (i.i.d. drafts) a unit evaluates each of the
+  // two rows once, whatever the round (evaluated anew per earlier round, a
+  // depth that rejects four drafts read 19 rows' worth of exponentials,
+  // against 8): B = 1024, K = 4, V = 151936 1467 -> 1241 us a call.
+  struct SpectrW {
+    RowC q, w;
+    int rounds, ri;
+    bool one;
+  };
+  __device__ __forceinline__ SpectrW spectr_weights(int rounds, int ri) const {
+    return SpectrW{row_c(0), row_c(S.nrows > 1 ? 1 : 0), rounds, ri, S.nrows == 2};
+  }
   template <class LD>
-  __device__ __forceinline__ void spectr_target(const LD& L, int rounds, float* r) const {
+  __device__ __forceinline__ void spectr_resid(const LD& L, const SpectrW& sw, float* r) const {
     float v[VE];
     L(0, v);
 #pragma unroll
-    for (int e = 0; e < VE; ++e) r[e] = prob_of(v[e], S.M[0], S.c[0], S.invZ[0]);
-    for (int k = 0; k < rounds; ++k) {
-      if (!(S.sp_invR[k] > 0.f)) continue;
-      const int rk = S.sp_rows[k];
+    for (int e = 0; e < VE; ++e) r[e] = sw.q.prob(v[e]);
+    if (sw.one) {
+      float w[VE];
+      L(1, w);
+#pragma unroll
+      for (int e = 0; e < VE; ++e) w[e] = sw.w.prob(w[e]);
+      for (int k = 0; k < sw.rounds; ++k) {
+        const float inv = S.sp_invR[k];
+        if (!(inv > 0.f)) continue;
+#pragma unroll
+        for (int e = 0; e < VE; ++e) r[e] = __fmul_rn(fmaxf(0.f, __fsub_rn(r[e], w[e])), inv);
+      }
+      if (sw.ri >= 0) {
+#pragma unroll
+        for (int e = 0; e < VE; ++e) r[e] = fmaxf(0.f, __fsub_rn(r[e], w[e]));
+      }
+      return;
+    }
+    for (int k = 0; k <= sw.rounds; ++k) {
+      const bool last = k == sw.rounds;
+      if (last ? sw.ri < 0 : !(S.sp_invR[k] > 0.f)) continue;
+      const int rk = last ? sw.ri : S.sp_rows[k];
+      const RowC c = row_c(rk);
       float w[VE];
       L(rk, w);
 #pragma unroll
-      for (int e = 0; e < VE; ++e)
-        r[e] = __fmul_rn(fmaxf(0.f, __fsub_rn(r[e], prob_of(w[e], S.M[rk], S.c[rk], S.invZ[rk]))), S.sp_invR[k]);
+      for (int e = 0; e < VE; ++e) {
+        r[e] = fmaxf(0.f, __fsub_rn(r[e], c.prob(w[e])));
+        if (!last) r[e] = __fmul_rn(r[e], S.sp_invR[k]);
+      }
     }
   }
 };
