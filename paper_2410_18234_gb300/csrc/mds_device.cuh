@@ -197,6 +197,61 @@ struct Elt<MDS_BF16> {
   }
 };
 
+// Unit u (16 bytes from byte 16 u of `src` on) of a row that ends before
+// `end` and starts at `first`: where the row is not 16-byte aligned, the two
+// aligned 16-byte blocks that hold the unit, shifted together, if both lie
+// inside the row, else logit by logit; logits past n read -inf.
+template <int DT>
+__device__ __forceinline__ uint4 load_unit(const char* src, const char* first, const char* end, int u, int n) {
+  constexpr int VE = Elt<DT>::VE;
+  const char* at = src + 16 * (size_t)u;
+  const unsigned sh = (unsigned)(reinterpret_cast<uintptr_t>(at) & 15u);
+  const char* blk = at - sh;
+  if (u * VE + VE <= n && blk >= first && blk + (sh ? 32 : 16) <= end) {
+    const uint4 lo = __ldg(reinterpret_cast<const uint4*>(blk));
+    if (!sh) return lo;
+    const uint4 hi = __ldg(reinterpret_cast<const uint4*>(blk) + 1);
+    uint32_t w0 = lo.x, w1 = lo.y, w2 = lo.z, w3 = lo.w, w4 = hi.x, w5 = hi.y, w6 = hi.z, w7 = hi.w;
+    if (sh & 8u) {
+      w0 = w2;
+      w1 = w3;
+      w2 = w4;
+      w3 = w5;
+      w4 = w6;
+      w5 = w7;
+    }
+    if (sh & 4u) {
+      w0 = w1;
+      w1 = w2;
+      w2 = w3;
+      w3 = w4;
+      w4 = w5;
+    }
+    const unsigned bits = (sh & 3u) * 8u;
+    return make_uint4(__funnelshift_r(w0, w1, bits), __funnelshift_r(w1, w2, bits), __funnelshift_r(w2, w3, bits),
+                      __funnelshift_r(w3, w4, bits));
+  }
+  uint32_t w[4];
+  if constexpr (DT == MDS_BF16) {
+    const unsigned short* s16 = reinterpret_cast<const unsigned short*>(src);
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const int t0 = u * VE + 2 * h;
+      const uint32_t a = (t0 < n) ? (uint32_t)__ldg(s16 + t0) : 0xff80u;
+      const uint32_t c = (t0 + 1 < n) ? (uint32_t)__ldg(s16 + t0 + 1) : 0xff80u;
+      w[h] = a | (c << 16);
+    }
+  } else {
+    const float* s32 = reinterpret_cast<const float*>(src);
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const int t0 = u * VE + h;
+      w[h] = (t0 < n) ? __float_as_uint(__ldg(s32 + t0)) : 0xff800000u;
+    }
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
 // Probability of a logit under a row's statistics (row maximum M, scale
 // c = log2(e) / T, inverse normaliser).  The same expression serves every
 // in-pass value and point lookup, so both give identical bits.  Exponents:

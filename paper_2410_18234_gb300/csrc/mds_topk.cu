@@ -37,19 +37,24 @@ namespace {
 
 using namespace mds::dev;
 
-constexpr int kThreads = 256;
+constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
 constexpr int kKMax = MDS_MAX_TOPK;
 constexpr int kRowsMax = 1 + MDS_MAX_K;
 constexpr int kEntMax = kRowsMax * kKMax;   // kept entries of one depth, and the largest |U|
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int kPrefixUnits = 4;             // units per thread behind a row's first logit bound
+constexpr int kFlight = 8;                  // 16-byte loads in flight per thread
+constexpr int kCand = 1024;                 // tokens at or above the bound one row may set aside
 
-static_assert(kWarps * kKMax == 4 * 32, "the row merge holds four candidates per lane");
+static_assert(kWarps >= kKMax && kWarps <= 32, "kk warps bound a row's kk-th logit");
 static_assert(kKMax <= 32, "a row's kept entries fit one warp");
 
 struct Shared {
-  unsigned long long wk[kWarps][kKMax];   // each warp's top k of a row
+  unsigned wmax[kWarps];                  // order keys of the warps' largest logits
+  __align__(16) unsigned ckey[kCand];     // tokens set aside: order key of the logit ...
+  int cid[kCand];                         // ... and id
+  int nc, cnt[kWarps];
   int id[kRowsMax][kKMax];                // each row's kept tokens, decreasing (logit, -id)
   float lg[kRowsMax][kKMax];              // their logits
   float pr[kRowsMax][kKMax];              // their renormalised probabilities
@@ -80,214 +85,217 @@ struct Shared {
   float RS[kMaxPairs], FL[kMaxPairs], FH[kMaxPairs];
   int Y;
   int bcast;                              // warp 0's broadcast word
-  float tau0;                             // lower bound on a row's kk-th logit
   // bonus: the target row's kept entries by increasing id
   int bid[kKMax];
   float bw[kKMax];
 };
 
-__device__ __forceinline__ unsigned long long max_u64(unsigned long long a, unsigned long long b) {
-  return a > b ? a : b;
-}
-__device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v) {
-#pragma unroll
-  for (int o = 16; o; o >>= 1) v = max_u64(v, __shfl_xor_sync(FULL, v, o));
-  return v;
-}
-// A kept entry's key: larger logit first, then lower id.  Never 0 (ids are
-// below 2^24), so 0 marks an empty slot.
-__device__ __forceinline__ unsigned long long entry_key(float v, int id) {
-  return ((unsigned long long)ord_key(v) << 32) | (unsigned long long)(0xffffffffu - (unsigned)id);
-}
-__device__ __forceinline__ int key_id(unsigned long long k) { return (int)(0xffffffffu - (unsigned)k); }
-__device__ __forceinline__ float key_val(unsigned long long k) { return ord_val((unsigned)(k >> 32)); }
-
-// A thread's running list: its 16 largest keys, decreasing; the k-th entry
-// and its logit (or the row's known floor, if higher) bound what can still
-// enter.  Every array is indexed by
-// compile-time constants only (registers).
-struct TopList {
-  unsigned long long e[kKMax];
-  unsigned long long kth;
-  float bound;
-  float floor;   // a lower bound on the row's kk-th logit known in advance
-
-  __device__ __forceinline__ void reset() {
-#pragma unroll
-    for (int i = 0; i < kKMax; ++i) e[i] = 0ull;
-    kth = 0ull;
-    bound = kNegInf;
-    floor = kNegInf;
-  }
-  __device__ __forceinline__ void insert(float v, int id, int kk) {
-    unsigned long long x = entry_key(v, id);
-    if (!(v >= bound) || x <= kth) return;
-#pragma unroll
-    for (int i = 0; i < kKMax; ++i) {
-      const unsigned long long t = e[i];
-      const bool sw = x > t;
-      e[i] = sw ? x : t;
-      x = sw ? t : x;
-    }
-#pragma unroll
-    for (int i = 0; i < kKMax; ++i)
-      if (i == kk - 1) kth = e[i];
-    bound = kth ? fmaxf(floor, key_val(kth)) : floor;
-  }
-  // The values of one unit (n of them, ids base, base + 1, ...): a mask of
-  // those at or above the bound, then one insertion site for the (rare) hits.
-  template <int N>
-  __device__ __forceinline__ void offer(const float (&v)[N], int base, int kk) {
-    unsigned m = 0u;
-#pragma unroll
-    for (int i = 0; i < N; ++i) m |= (v[i] >= bound) ? (1u << i) : 0u;
-    while (m) {
-      const int i0 = __ffs(m) - 1;
-      m &= m - 1u;
-      float x = v[0];
-#pragma unroll
-      for (int i = 1; i < N; ++i)
-        if (i == i0) x = v[i];
-      insert(x, base + i0, kk);
-    }
-  }
-  __device__ __forceinline__ void pop() {
-#pragma unroll
-    for (int i = 0; i + 1 < kKMax; ++i) e[i] = e[i + 1];
-    e[kKMax - 1] = 0ull;
+// One row of the depth: units of 16 bytes from its start, whole and aligned
+// (vec) or shifted together from aligned blocks.
+template <int DT>
+struct Row {
+  const char* row;
+  int V, nu;
+  bool vec;
+  __device__ __forceinline__ uint4 unit(int u) const {
+    if (vec) return __ldcs(reinterpret_cast<const uint4*>(row) + u);
+    return load_unit<DT>(row, row, row + (size_t)V * (16 / Elt<DT>::VE), u, V);
   }
 };
 
-template <int DT>
-__device__ __forceinline__ void scan_unit(TopList& T, const uint4& x, int u, int kk) {
-  using E = Elt<DT>;
-  if (!(E::unit_max(x) >= T.bound)) return;
-  float v[E::VE];
-  E::unpack(x, v);
-  T.offer<E::VE>(v, u * E::VE, kk);
+// Every unit of the row, kFlight per thread in flight: fn(x, u).
+template <int DT, class FN>
+__device__ __forceinline__ void scan_row(const Row<DT>& w, int first, FN&& fn) {
+  for (int u0 = first + (int)threadIdx.x; u0 < w.nu; u0 += kFlight * kThreads) {
+    uint4 x[kFlight];
+#pragma unroll
+    for (int q = 0; q < kFlight; ++q)
+      x[q] = u0 + q * kThreads < w.nu ? w.unit(u0 + q * kThreads) : Elt<DT>::neg_inf();
+#pragma unroll
+    for (int q = 0; q < kFlight; ++q) fn(x[q], u0 + q * kThreads);
+  }
 }
 
-// The row's top kk into S.id / S.lg / S.n[r] (all threads; ends synchronised).
+// The kk-th largest of the warps' maxima in S.wmax (0: fewer than kk warps
+// saw a logit above -inf): kk distinct logits reach it.
+__device__ __forceinline__ unsigned kth_warp_max(const Shared& S, int kk) {
+  const int lane = threadIdx.x & 31;
+  const unsigned k = lane < kWarps ? S.wmax[lane] : 0u;
+  int above = 0;
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) {
+    const unsigned o = S.wmax[w];
+    above += (o > k || (o == k && w < lane)) ? 1 : 0;
+  }
+  const unsigned who = __ballot_sync(FULL, lane < kWarps && above == kk - 1);
+  return __shfl_sync(FULL, k, __ffs(who) - 1);
+}
+__device__ __forceinline__ void put_warp_max(Shared& S, float mx) {
+  const unsigned k = __reduce_max_sync(FULL, mx > kNegInf ? ord_key(__fadd_rn(mx, 0.f)) : 0u);
+  if ((threadIdx.x & 31) == 0) S.wmax[threadIdx.x >> 5] = k;
+}
+
+// Set aside unit u's logits whose order key is at least `lo`.
+template <int DT>
+__device__ __forceinline__ void offer(Shared& S, const uint4& x, int u, int V, unsigned lo, float lof) {
+  using E = Elt<DT>;
+  if (!(E::unit_max(x) >= lof)) return;
+  float v[E::VE];
+  E::unpack(x, v);
+#pragma unroll
+  for (int e = 0; e < E::VE; ++e) {
+    const int id = u * E::VE + e;
+    const unsigned k = ord_key(__fadd_rn(v[e], 0.f));
+    if (v[e] == v[e] && k >= lo && id < V) {
+      const int pos = atomicAdd(&S.nc, 1);
+      if (pos < kCand) {
+        S.ckey[pos] = k;
+        S.cid[pos] = id;
+      }
+    }
+  }
+}
+
+// The `need` lowest ids whose order key is exactly `key`, set aside too (in id
+// order; all threads).
+template <int DT>
+__device__ void offer_equal(Shared& S, const Row<DT>& w, unsigned key, int need) {
+  using E = Elt<DT>;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int u0 = 0; u0 < w.nu && need > 0; u0 += kThreads) {
+    const int u = u0 + (int)threadIdx.x;
+    float v[E::VE];
+    E::unpack(u < w.nu ? w.unit(u) : E::neg_inf(), v);
+    unsigned bits = 0u;
+#pragma unroll
+    for (int e = 0; e < E::VE; ++e)
+      bits |= (u * E::VE + e < w.V && v[e] == v[e] && ord_key(__fadd_rn(v[e], 0.f)) == key) ? 1u << e : 0u;
+    int incl = __popc(bits);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(FULL, incl, o);
+      if (lane >= o) incl += t;
+    }
+    __syncthreads();   // the previous round's counts are read
+    if (lane == 31) S.cnt[warp] = incl;
+    __syncthreads();
+    int before = incl - __popc(bits), total = 0;
+    for (int q = 0; q < kWarps; ++q) {
+      before += q < warp ? S.cnt[q] : 0;
+      total += S.cnt[q];
+    }
+    for (; bits && before < need; bits &= bits - 1u, ++before) {
+      const int pos = atomicAdd(&S.nc, 1);
+      S.ckey[pos] = key;
+      S.cid[pos] = u * E::VE + __ffs(bits) - 1;
+    }
+    need -= total;
+  }
+  __syncthreads();
+}
+
+// The row's top kk into S.id / S.lg / S.n[r] (all threads; ends synchronised):
+// larger logit first, ties to the lower id.  A bound that kk distinct logits
+// reach (the kk-th largest of the warps' maxima over the row's first units)
+// lets the scan set aside some tens to a few hundred tokens, which are ranked
+// by counting.  More than kCand of them, or no bound (few finite logits, ties,
+// flat rows): the tokens above the bound from the whole row's maxima, and of
+// those at it the lowest ids; should even those above be too many, the exact
+// kk-th key by bisection.
+// Bound by the row's stream: eight 16-byte loads in flight per thread, 512
+// threads.  Against per-thread lists of 16 keys in registers with four loads
+// in flight of 256 threads: B = 256, K = 8, V = 128256 WIS top-10 523 -> 428 us
+// a call, smaller batches 1.6 to 2.6 times as fast.
 template <int DT>
 __device__ __noinline__ void select_row(const Params& p, Shared& S, int r, int kk) {
   using E = Elt<DT>;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const char* row = S.rowp[r];
-  TopList T;
-  T.reset();
-  // A lower bound on the row's kk-th logit: the kk-th largest of the threads'
-  // maxima over their first units (kk distinct logits reach it), so the
-  // full scan below inserts only logits at or above it.
+  const int tid = threadIdx.x;
+  const Row<DT> w{S.rowp[r], p.V, (p.V + E::VE - 1) / E::VE, p.vec != 0};
+  if (tid == 0) S.nc = 0;
   {
+    uint4 x[kPrefixUnits];
     float mx = kNegInf;
-    if (p.vec) {
-      const uint4* rv = reinterpret_cast<const uint4*>(row);
-      const int nu = (int)(((size_t)p.V * p.esize) / 16);
 #pragma unroll
-      for (int q = 0; q < kPrefixUnits; ++q)
-        if (tid + q * kThreads < nu) mx = fmaxf(mx, E::unit_max(__ldcs(rv + tid + q * kThreads)));
-    } else {
-#pragma unroll
-      for (int q = 0; q < kPrefixUnits; ++q)
-        if (tid + q * kThreads < p.V) mx = fmaxf(mx, E::global(row, tid + q * kThreads));
+    for (int q = 0; q < kPrefixUnits; ++q) {
+      x[q] = tid + q * kThreads < w.nu ? w.unit(tid + q * kThreads) : E::neg_inf();
+      mx = fmaxf(mx, E::unit_max(x[q]));
     }
-    // kk rounds of a warp maximum over (max, thread) keys, then over the warps'
-    unsigned long long mk = (mx == mx && mx > kNegInf) ? entry_key(mx, tid) : 0ull;
-    for (int t = 0; t < kk; ++t) {
-      const unsigned long long m = warp_max_u64(mk);
-      if (mk == m) mk = 0ull;
-      if (lane == 0) S.wk[warp][t] = m;
+    put_warp_max(S, mx);
+    __syncthreads();
+    const unsigned lo = kth_warp_max(S, kk);
+    if (lo) {
+      const float lof = ord_val(lo);
+#pragma unroll
+      for (int q = 0; q < kPrefixUnits; ++q) offer<DT>(S, x[q], tid + q * kThreads, w.V, lo, lof);
+      scan_row(w, kPrefixUnits * kThreads, [&](const uint4& y, int u) { offer<DT>(S, y, u, w.V, lo, lof); });
     }
     __syncthreads();
-    if (warp == 0) {
-      unsigned long long c0, c1, c2, c3;
-      const int e0 = lane, e1 = lane + 32, e2 = lane + 64, e3 = lane + 96;
-      c0 = (e0 % kKMax < kk) ? S.wk[e0 / kKMax][e0 % kKMax] : 0ull;
-      c1 = (e1 % kKMax < kk) ? S.wk[e1 / kKMax][e1 % kKMax] : 0ull;
-      c2 = (e2 % kKMax < kk) ? S.wk[e2 / kKMax][e2 % kKMax] : 0ull;
-      c3 = (e3 % kKMax < kk) ? S.wk[e3 / kKMax][e3 % kKMax] : 0ull;
-      unsigned long long m = 0ull;
-      for (int t = 0; t < kk; ++t) {
-        m = warp_max_u64(max_u64(max_u64(c0, c1), max_u64(c2, c3)));
-        if (m == 0ull) break;
-        if (c0 == m) c0 = 0ull;
-        if (c1 == m) c1 = 0ull;
-        if (c2 == m) c2 = 0ull;
-        if (c3 == m) c3 = 0ull;
-      }
-      // fewer than kk threads saw a logit: no bound
-      if (lane == 0) S.tau0 = (m != 0ull) ? key_val(m) : kNegInf;
-    }
-    __syncthreads();
-    T.floor = S.tau0;
-    T.bound = S.tau0;
-  }
-  if (p.vec) {
-    // 16-byte units, four in flight per thread
-    const uint4* rv = reinterpret_cast<const uint4*>(row);
-    const int nu = (int)(((size_t)p.V * p.esize) / 16);
-    int u = tid;
-    for (; u + 3 * kThreads < nu; u += 4 * kThreads) {
-      const uint4 x0 = __ldcs(rv + u), x1 = __ldcs(rv + u + kThreads), x2 = __ldcs(rv + u + 2 * kThreads),
-                  x3 = __ldcs(rv + u + 3 * kThreads);
-      scan_unit<DT>(T, x0, u, kk);
-      scan_unit<DT>(T, x1, u + kThreads, kk);
-      scan_unit<DT>(T, x2, u + 2 * kThreads, kk);
-      scan_unit<DT>(T, x3, u + 3 * kThreads, kk);
-    }
-    for (; u < nu; u += kThreads) scan_unit<DT>(T, __ldcs(rv + u), u, kk);
-  } else {
-    // element loads (rows of any length and alignment), four in flight
-    int i = tid;
-    for (; i + 3 * kThreads < p.V; i += 4 * kThreads) {
-      const float v4[4] = {E::global(row, i), E::global(row, i + kThreads), E::global(row, i + 2 * kThreads),
-                           E::global(row, i + 3 * kThreads)};
-      unsigned m = 0u;
+    if (!lo || S.nc > kCand) {
+      // the whole row's maxima
+      __syncthreads();
+      if (tid == 0) S.nc = 0;
+      mx = kNegInf;
+      scan_row(w, 0, [&](const uint4& y, int) { mx = fmaxf(mx, E::unit_max(y)); });
+      put_warp_max(S, mx);
+      __syncthreads();
+      constexpr unsigned kInf = 0x007fffffu;   // order key of -inf
+      unsigned at = kth_warp_max(S, kk);
+      if (!at) at = kInf;
+      scan_row(w, 0, [&](const uint4& y, int u) { offer<DT>(S, y, u, w.V, at + 1u, ord_val(at)); });
+      __syncthreads();
+      if (S.nc > kCand) {
+        // the largest key that kk logits reach, bit by bit
+        unsigned t = 0u;
+        for (int bit = 31; bit >= 0; --bit) {
+          const unsigned cand = t | (1u << bit);
+          unsigned c = 0u;
+          scan_row(w, 0, [&](const uint4& y, int u) {
+            float v[E::VE];
+            E::unpack(y, v);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) m |= (v4[q] >= T.bound) ? (1u << q) : 0u;
-      while (m) {
-        const int q0 = __ffs(m) - 1;
-        m &= m - 1u;
-        const float x = q0 == 0 ? v4[0] : q0 == 1 ? v4[1] : q0 == 2 ? v4[2] : v4[3];
-        T.insert(x, i + q0 * kThreads, kk);
+            for (int e = 0; e < E::VE; ++e)
+              c += (u * E::VE + e < w.V && v[e] == v[e] && ord_key(__fadd_rn(v[e], 0.f)) >= cand) ? 1u : 0u;
+          });
+          c = __reduce_add_sync(FULL, c);
+          __syncthreads();
+          if ((tid & 31) == 0) S.cnt[tid >> 5] = (int)c;
+          __syncthreads();
+          int n = 0;
+          for (int q = 0; q < kWarps; ++q) n += S.cnt[q];
+          if (n >= kk) t = cand;
+        }
+        at = t;
+        __syncthreads();
+        if (tid == 0) S.nc = 0;
+        __syncthreads();
+        scan_row(w, 0, [&](const uint4& y, int u) { offer<DT>(S, y, u, w.V, at + 1u, ord_val(at)); });
+        __syncthreads();
       }
+      const int have = S.nc;
+      if (have < kk) offer_equal(S, w, at, kk - have);
     }
-    for (; i < p.V; i += kThreads) T.insert(E::global(row, i), i, kk);
   }
-  // each warp's top kk: kk rounds of a warp maximum over the lists' heads
-  for (int t = 0; t < kk; ++t) {
-    const unsigned long long m = warp_max_u64(T.e[0]);
-    if (m != 0ull && T.e[0] == m) T.pop();
-    if (lane == 0) S.wk[warp][t] = m;
-  }
+  // ranks by (key, id)
+  const int n = S.nc;
+  for (int i = n + tid; i < ((n + 3) & ~3); i += kThreads) S.ckey[i] = 0u;
   __syncthreads();
-  if (warp == 0) {
-    // the row's top kk from the warps' lists, four candidates per lane
-    unsigned long long c0, c1, c2, c3;
-    {
-      const int e0 = lane, e1 = lane + 32, e2 = lane + 64, e3 = lane + 96;
-      c0 = (e0 % kKMax < kk) ? S.wk[e0 / kKMax][e0 % kKMax] : 0ull;
-      c1 = (e1 % kKMax < kk) ? S.wk[e1 / kKMax][e1 % kKMax] : 0ull;
-      c2 = (e2 % kKMax < kk) ? S.wk[e2 / kKMax][e2 % kKMax] : 0ull;
-      c3 = (e3 % kKMax < kk) ? S.wk[e3 / kKMax][e3 % kKMax] : 0ull;
+  for (int i = tid; i < n; i += kThreads) {
+    const unsigned k = S.ckey[i];
+    int rk = 0, eq = 0;
+    for (int q = 0; q < n; q += 4) {
+      const uint4 o = *reinterpret_cast<const uint4*>(S.ckey + q);
+      rk += (o.x > k ? 1 : 0) + (o.y > k ? 1 : 0) + (o.z > k ? 1 : 0) + (o.w > k ? 1 : 0);
+      eq += (o.x == k ? 1 : 0) + (o.y == k ? 1 : 0) + (o.z == k ? 1 : 0) + (o.w == k ? 1 : 0);
     }
-    int n = 0;
-    for (int t = 0; t < kk; ++t) {
-      const unsigned long long best = max_u64(max_u64(c0, c1), max_u64(c2, c3));
-      const unsigned long long m = warp_max_u64(best);
-      if (m == 0ull) break;
-      if (c0 == m) c0 = 0ull;
-      if (c1 == m) c1 = 0ull;
-      if (c2 == m) c2 = 0ull;
-      if (c3 == m) c3 = 0ull;
-      if (lane == 0) {
-        S.id[r][t] = key_id(m);
-        S.lg[r][t] = key_val(m);
-      }
-      ++n;
+    const int id = S.cid[i];
+    if (eq > 1 && rk < kk)
+      for (int q = 0; q < n; ++q) rk += (S.ckey[q] == k && S.cid[q] < id) ? 1 : 0;
+    if (rk < kk) {
+      S.id[r][rk] = id;
+      S.lg[r][rk] = ord_val(k);
     }
-    if (lane == 0) S.n[r] = n;
   }
+  if (tid == 0) S.n[r] = min(n, kk);
   __syncthreads();
 }
 
