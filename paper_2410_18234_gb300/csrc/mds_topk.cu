@@ -72,6 +72,7 @@ struct Shared {
   short rank[kEntMax];                    // position in U of each kept entry
   unsigned char dup[kEntMax];             // entry repeats a token of an earlier entry
   int nU;
+  __align__(16) unsigned kx[32];          // one word per lane, compared by all
   // the walk
   int X[MDS_MAX_K], vbr[MDS_MAX_K], vrow[MDS_MAX_K];
   int nv;
@@ -372,6 +373,32 @@ __device__ void row_probs(const Params& p, Shared& S, int r) {
 __device__ void build_union(Shared& S) {
   const int lane = threadIdx.x & 31;
   const int nr = S.nrows, ne = nr * kKMax;
+  if (ne <= 32) {
+    // two rows: one kept entry per lane, duplicates by a match, ranks by counting
+    const int r = lane / kKMax, t = lane - r * kKMax;
+    const bool have = r < nr && t < S.n[r < nr ? r : 0];
+    const int id = have ? S.id[r][t] : 0x7fffffff;
+    const unsigned same = __match_any_sync(FULL, id);
+    const bool first = have && (same & ((1u << lane) - 1u)) == 0u;
+    S.kx[lane] = first ? (unsigned)id : 0x7fffffffu;
+    __syncwarp();
+    int k = 0;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const uint4 o = reinterpret_cast<const uint4*>(S.kx)[c];
+      k += (o.x < (unsigned)id ? 1 : 0) + (o.y < (unsigned)id ? 1 : 0) + (o.z < (unsigned)id ? 1 : 0) +
+           (o.w < (unsigned)id ? 1 : 0);
+    }
+    const int nU = __popc(__ballot_sync(FULL, first));
+    if (first) S.uid[k] = id;
+    for (int q = 0; q < nr; ++q)
+      if (lane < nU) S.law[q][lane] = 0.f;
+    if (lane == 0) S.nU = nU;
+    __syncwarp();
+    if (have) S.law[r][k] = S.pr[r][t];
+    __syncwarp();
+    return;
+  }
   for (int e = lane; e < ne; e += 32) {
     const int r = e / kKMax, t = e - r * kKMax;
     unsigned char d = 1;
@@ -667,6 +694,81 @@ __device__ int wis_stage(const Params& p, Shared& S, int A, int Btok, int rb, fl
   return y;
 }
 
+// Warp 0: the pairwise stages of the weighted scheme with the 1/2 rule, one
+// entry of U per lane (nU <= 32, s <= 5), the state in registers; *Yo the
+// stages' token so far.  Returns the first stage with fewer than s positive
+// keys (Omega_1 then takes zero keys, tokens outside U among them), nv if
+// none; the law so far is in S.cur.  Same arithmetic as wis_stage (B = 256,
+// K = 8, V = 128256 top-10 428 us a call with it alone, 321 with this).
+__device__ int wis_stages_small(const Params& p, Shared& S, float ul, int* Yo) {
+  const int lane = threadIdx.x & 31;
+  const int nU = S.nU, nv = S.nv, s = min(p.wis_s, p.V);
+  const bool have = lane < nU;
+  const int id = have ? S.uid[lane] : -1;
+  const float q = have ? S.law[0][lane] : 0.f;
+  float a = have ? S.law[S.vrow[0]][lane] : 0.f;
+  int A = S.X[0], m = 1;
+#pragma unroll 1
+  for (; m < nv; ++m) {
+    const int Btok = S.X[m];
+    const float u = __shfl_sync(FULL, ul, m - 1);
+    const float bq = have ? S.law[S.vrow[m]][lane] : 0.f;
+    const float key = __fadd_rn(__fmaf_rn(-a, bq, q), 0.f);
+    const bool pos = have && key > 0.f;
+    const unsigned kk = pos ? ord_key(key) : 0u;
+    if (__popc(__ballot_sync(FULL, pos)) < s) break;
+    S.kx[lane] = kk;
+    __syncwarp();
+    // Omega_1: the entries with fewer than s larger keys; where the last of
+    // them tie, the smaller token ids (the lower lanes)
+    int above = 0;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const uint4 o = reinterpret_cast<const uint4*>(S.kx)[c];
+      above += (o.x > kk ? 1 : 0) + (o.y > kk ? 1 : 0) + (o.z > kk ? 1 : 0) + (o.w > kk ? 1 : 0);
+    }
+    unsigned selm = __ballot_sync(FULL, pos && above < s);
+    if (__popc(selm) > s) {
+      const int last = (int)__reduce_max_sync(FULL, (selm >> lane & 1u) ? (unsigned)above : 0u);
+      const unsigned tie = __ballot_sync(FULL, pos && above == last);
+      selm = __ballot_sync(FULL, (selm >> lane & 1u) &&
+                                     (above < last || __popc(tie & ((1u << lane) - 1u)) < s - last));
+    }
+    const bool sel = (selm >> lane) & 1u;
+    float ra = (have && !sel) ? a : 0.f, rb = (have && !sel) ? bq : 0.f;
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+      ra = __fadd_rn(ra, __shfl_xor_sync(FULL, ra, o));
+      rb = __fadd_rn(rb, __shfl_xor_sync(FULL, rb, o));
+    }
+    const int rk = __popc(selm & ((1u << lane) - 1u));
+    if (lane >= s && lane < MDS_MAX_S) {
+      S.om[lane] = 0x7fffffff;
+      S.om_q[lane] = 0.f;
+      S.om_a[lane] = 0.f;
+      S.om_b[lane] = 0.f;
+    }
+    if (sel) {
+      S.om[rk] = id;
+      S.om_q[rk] = q;
+      S.om_a[rk] = a;
+      S.om_b[rk] = bq;
+    }
+    __syncwarp();
+    float x;
+    bool capped;
+    A = stage_solve5(ra, rb, A, Btok, u, S.om, S.om_q, S.om_a, S.om_b, x, &capped);
+    if (capped && lane == 0) atomicOr(p.status, MDS_ST_LP_CAP);
+    const float xr = __shfl_sync(FULL, x, rk & 31);
+    a = sel ? xr : __fmul_rn(0.5f, __fadd_rn(__fmul_rn(a, rb), __fmul_rn(bq, ra)));
+    __syncwarp();   // the tables are read before the next stage writes them
+  }
+  if (have) S.cur[lane] = a;
+  __syncwarp();
+  *Yo = A;
+  return m;
+}
+
 // Warp 0: Algorithm 1 on the intermediate token Y with law p_I = a (on U):
 // accept with probability min(1, q(Y) / p_I(Y)), otherwise draw from the
 // residual max(0, q - p_I) in token-id order.  *R: the residual mass after a
@@ -762,12 +864,17 @@ __device__ __noinline__ void decide(const Params& p, Shared& S, int b, int j) {
     int Y = S.X[0];
     const float* a = S.law[S.vrow[0]];
     if ((p.scheme == MDS_WIS || p.scheme == MDS_WISSORT) && nv > 1) {
-      for (int i = lane; i < S.nU; i += 32) S.cur[i] = a[i];
-      __syncwarp();
       // every stage's selection uniform at once (lane m - 1 draws stage m's)
       const float ul = (lane + 1 < nv) ? draw_uniform(p.seed, b, j, kDrawSelect + lane) : 0.f;
       const bool sorted = p.scheme == MDS_WISSORT;
-      for (int m = 1; m < nv; ++m)
+      int m = 1;
+      if (!sorted && S.nU <= 32 && p.wis_s <= 5) {
+        m = wis_stages_small(p, S, ul, &Y);
+      } else {
+        for (int i = lane; i < S.nU; i += 32) S.cur[i] = a[i];
+        __syncwarp();
+      }
+      for (; m < nv; ++m)
         Y = wis_stage(p, S, Y, S.X[m], S.vrow[m], __shfl_sync(FULL, ul, m - 1), sorted);
       a = S.cur;
     }
