@@ -39,8 +39,6 @@ struct mds_ctx {
 
 namespace {
 
-constexpr int kRingBytes = 80 * 1024;   // streaming rings: 8 warps x 5 stages of 2 KB
-constexpr int kRingBytesIs = 40 * 1024; // classical IS: 1 KB stages (two rows), beside its bins two CTAs per SM
 
 struct DeviceGuard {
   int prev = -1;
@@ -97,8 +95,8 @@ int optin_smem(int device) {
   return v;
 }
 
-// Fill the launch geometry (cluster size, slice, ring and list sizes) for
-// n_models distinct draft models.  Rows stream through per-warp rings, so
+// Fill the launch geometry (cluster size, slice and list sizes) for
+// n_models distinct draft models.  Rows stream through registers, so
 // shared memory grows with V only through the special-token bitmap and the
 // segment sums; the cluster size sets the slice each CTA streams per depth.
 // Returns MDS_OK or MDS_EVOCAB.
@@ -107,7 +105,6 @@ int geometry(const mds_ctx* ctx, int scheme, int n_models, mds::Params& p) {
   p.esize = esize_of(c.dtype);
   p.rows_max = 1 + n_models;
   p.scheme = scheme;
-  p.ring_bytes = (scheme == MDS_IS) ? kRingBytesIs : kRingBytes;
   // candidate lists: WIS with at most three draft models in the stats pass;
   // the truncated alphabet always (its Omega_0 comes from the list)
   const bool lists = (scheme == MDS_WIS && p.rows_max <= 4) || scheme == MDS_WIS0;
@@ -122,7 +119,9 @@ int geometry(const mds_ctx* ctx, int scheme, int n_models, mds::Params& p) {
     }
     return mds::smem_bytes(p);
   };
-  const size_t limit = (size_t)optin_smem(ctx->device) - 12 * 1024;  // static shared state
+  // static shared state, and the room a slice's tables leave free (the
+  // vocabularies this bounds: 4 million tokens a CTA)
+  const size_t limit = (size_t)optin_smem(ctx->device) - (12 + (scheme == MDS_IS ? 40 : 80)) * 1024;
   int cn = c.cluster;
   if (cn <= 0) {
     // Every sequence is a serial chain of depths, so as many sequences as
@@ -340,7 +339,6 @@ static int verify_impl(mds_ctx* ctx, const void* target_logits, const void* cons
   p.is_h = c.is_h;
   p.n_models = n_models;
   p.tma_ok = tma_ok ? 1 : 0;
-  p.bulk_ok = bulk_ok ? 1 : 0;
   DeviceGuard g(ctx->device);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   int clusters = clusters_for(ctx, p);

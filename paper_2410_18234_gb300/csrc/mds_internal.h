@@ -38,11 +38,9 @@ struct Params {
   float is_h;
   int cn;                              // CTAs per cluster
   int slice;                           // tokens per CTA (multiple of 8)
-  int ring_bytes;                      // streaming rings of all warps (each warp: 5 stages)
   int rows_max;                        // rows per depth at most (1 + distinct models)
   int n_models;                        // distinct draft models (ids are 0..n_models-1 after remap)
   int tma_ok;                          // rows are 16-byte aligned with a 16-byte-multiple length
-  int bulk_ok;                         // rows may be read with bulk copies (device memory, not mapped host memory)
   int cand_cap;                        // WIS candidate list capacity (kListN; 0: no candidate path)
   int cand_stage;                      // WIS staging capacity (every CTA's list: cn * kListN)
   unsigned long long* dbg_exps;        // IS: quadrature exponentials evaluated (test export), or null

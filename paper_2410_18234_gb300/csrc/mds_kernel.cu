@@ -5,8 +5,7 @@
 // co-resident clusters).  CTA r of the cluster owns tokens
 // [r*slice, (r+1)*slice) of every row.  Per depth j of the walk it
 //   1. streams its slice of the target row and of one row per distinct draft
-//      model through a small shared-memory ring (cp.async.bulk with mbarrier
-//      completion), computing the temperature-softmax statistics online and,
+//      model into registers, computing the temperature-softmax statistics online and,
 //      for the weighted schemes, collecting the candidate tokens; one exchange
 //      over distributed shared memory combines the cluster (the truncated
 //      alphabet streams the target row only: its draft laws on Omega_0 need
@@ -25,8 +24,7 @@
 // sequences are in flight.  Every decision is taken redundantly and
 // identically by every CTA of the cluster from cluster-combined values, so
 // control flow stays uniform and the cluster barriers always match.  No CTA
-// waits on another CTA's flag; the only waits are on this CTA's own bulk
-// copies and they are bounded.
+// waits on another CTA's flag.
 #include <cuda_bf16.h>
 #include <cooperative_groups.h>
 
@@ -42,9 +40,7 @@ constexpr float kPosInf = __builtin_huge_valf();
 constexpr int kWarps = kThreads / 32;
 constexpr int kTop = 8;                 // per-thread candidate list length (>= MDS_MAX_S)
 constexpr int kMaxPairs = MDS_MAX_S * (MDS_MAX_S - 1) / 2;
-constexpr long long kWaitLimit = 1ll << 24;
 constexpr int kFastRows = 4;            // WIS candidate path: target + up to 3 draft models
-constexpr int kWStages = 5;             // stages of each warp's streaming ring
 constexpr int kWarpApp = 64;            // candidate tokens one warp can hold during the stats pass
 constexpr int kIsSub = 4;               // IS: bins of log2 rho per octave
 constexpr int kIsMom = 8;               // IS: moments (Taylor terms) per bin
@@ -92,30 +88,6 @@ __device__ __forceinline__ float ld_dsmem(const float* local, uint32_t rank) {
 __device__ __forceinline__ void st_dsmem(int* local, uint32_t rank, int v) {
   asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(dsmem_addr(local, rank)), "r"(v) : "memory");
 }
-__device__ __forceinline__ void mbar_init(uint64_t* bar) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar)));
-}
-__device__ __forceinline__ void mbar_init_fence() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t done;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(done)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return done != 0;
-}
-__device__ __forceinline__ void bulk_copy(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   smem_u32(dst)),
-               "l"(src), "r"(bytes), "r"(smem_u32(bar))
-               : "memory");
-}
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
 // ---------------------------------------------------------------- Philox4x32-10
 // Salmon, Moraes, Dror, Shaw, SC'11: ten rounds of two 32x32->64 products,
 // round keys bumped by the Weyl constants.  Returns output word 0.
@@ -295,8 +267,6 @@ struct State {
   // CDF search
   int owner, seg;
   float run;
-  // streaming: one ring per warp, one mbarrier per stage
-  uint64_t wbar[kWarps][kWStages];
   int wapp[kWarps];          // tokens each warp set aside (may exceed kWarpApp: overflow)
   float thr_cta;
 };
@@ -404,33 +374,37 @@ __device__ __forceinline__ void cand_insert(Cand (&top)[kTop], const Cand& c, fl
 
 // ------------------------------------------------------------------ the kernel
 
-// Unit lu of row r in the current ring stage (rows of the pass in mask order).
-template <int DT>
-struct StageLoad {
-  const char* base;
-  uint32_t mask;
-  int cb;
-  int lu;
-  __device__ __forceinline__ void operator()(int r, float* v) const {
-    Elt<DT>::unit(base + __popc(mask & ((1u << r) - 1u)) * cb, lu, v);
+// A unit of a pass's rows, held in registers (rows: which row each is).
+template <int DT, int NR>
+struct RegLoad {
+  const uint4 (&x)[NR];
+  const int (&rows)[NR];
+  __device__ __forceinline__ uint4 raw(int r) const {
+    uint4 y = x[0];
+#pragma unroll
+    for (int i = 1; i < NR; ++i)
+      if (rows[i] == r) y = x[i];
+    return y;
   }
+  __device__ __forceinline__ void operator()(int r, float* v) const { Elt<DT>::unpack(raw(r), v); }
 };
-// Unit gu of row r straight from global memory (logits past V read -inf);
-// one 16-byte load when the rows are 16-byte aligned and the unit is whole.
+// Unit gu of row r of a slice straight from global memory (logits past V read
+// -inf): one 16-byte load when the rows are 16-byte aligned, else the aligned
+// blocks that hold the unit, shifted together.
+template <int DT>
+__device__ __forceinline__ uint4 slice_unit(const char* row, int tok0, int V, int gu, bool aligned) {
+  constexpr int VE = Elt<DT>::VE, es = 16 / VE;
+  const char* at = row + (size_t)tok0 * es;
+  if (aligned) return __ldg(reinterpret_cast<const uint4*>(at) + gu);
+  return dev::load_unit<DT>(at, row, row + (size_t)V * es, gu, V - tok0);
+}
 template <int DT>
 struct GlobalLoad {
   const char* const* gptr;
   int tok0, V, gu;
   bool aligned;
-  __device__ __forceinline__ void operator()(int r, float* v) const {
-    const int t0 = tok0 + gu * Elt<DT>::VE;
-    if (aligned && t0 + Elt<DT>::VE <= V) {
-      Elt<DT>::unit_global(gptr[r] + (size_t)t0 * (16 / Elt<DT>::VE), v);
-      return;
-    }
-#pragma unroll
-    for (int e = 0; e < Elt<DT>::VE; ++e) v[e] = (t0 + e < V) ? Elt<DT>::global(gptr[r], t0 + e) : kNegInf;
-  }
+  __device__ __forceinline__ uint4 raw(int r) const { return slice_unit<DT>(gptr[r], tok0, V, gu, aligned); }
+  __device__ __forceinline__ void operator()(int r, float* v) const { Elt<DT>::unpack(raw(r), v); }
 };
 
 template <int DT, int SCHEME>
@@ -440,7 +414,6 @@ struct Kernel {
 
   const Params& p;
   State& S;
-  char* ring;          // streaming rings: kWarps x kWStages stages
   uint32_t* bitmap;    // one bit per 16-byte unit of this CTA's slice that holds a special token
   float* segsum;       // per-segment residual sums
   float* chksum;       // per-chunk (32 segments) residual sums
@@ -463,8 +436,6 @@ struct Kernel {
   int rank, cn, tok0, nvalid, Uv, nseg, nsegv, bm_words;   // nseg: layout (slice); nsegv: written (valid units)
   int xbuf;
   int clbuf;           // which copy of the CTA list the next candidate pass publishes
-  uint32_t wphase;     // parity of each stage of this warp's ring
-  int bail;            // this warp's ring gave up on a copy: it streams nothing more
 
   // A row's constants in registers, for the passes' inner loops (through the
   // shared state every unit would load them again); prob() is prob_of.
@@ -479,105 +450,127 @@ struct Kernel {
     return prob_of(E::global(S.gptr[r], x), S.M[r], S.c[r], S.invZ[r]);
   }
 
-  // ---------------------------------------------------------------- streaming engine
-  // The CTA's slice is cut into chunks of su units (a multiple of 32, one
-  // ring stage) taken round-robin by the warps (warp w: chunks w, w + kWarps,
-  // ...), each walked in groups of 32, one unit per lane:
-  // fn(gu, valid, L) is called by all 32 lanes together, gu the unit's index
-  // in the slice (a group starts at a multiple of 32) and L(r, v) loading
-  // unit gu of row r.  With 16-byte aligned rows the rows of `mask` flow
-  // through the warp's own ring of kWStages stages (cp.async.bulk issued by
-  // lane 0 up to kWStages stages ahead, completion counted on the stage's
-  // mbarrier); otherwise (rows not 16-byte aligned, rows in mapped host
-  // memory, or a stage too small for a group of every row), units are loaded
-  // straight from global memory.  No block barrier is
-  // taken inside a pass, nor at its end: a caller synchronises the block
-  // before reading what other warps wrote.  Every wait is bounded.
-  __device__ __forceinline__ int stage_units(int nrm) const {
-    return ((p.ring_bytes / kWarps / kWStages) / (16 * nrm)) & ~31;
-  }
-
-  // Issue this warp's k-th stage: chunk c = warp + k * kWarps of su units.
-  __device__ __forceinline__ void issue_stage(int k, uint32_t mask, int su) {
-    const int warp = threadIdx.x >> 5;
-    const int stage = k % kWStages;
-    char* dst = ring + (size_t)(warp * kWStages + stage) * (p.ring_bytes / kWarps / kWStages);
-    const int cu0 = (warp + k * kWarps) * su;
-    const int bytes = (min(cu0 + su, Uv) - cu0) * 16;
-    mbar_expect_tx(&S.wbar[warp][stage], (uint32_t)(bytes * __popc(mask)));
-    int pos = 0;
-    for (int r = 0; r < S.nrows; ++r) {
-      if (!(mask >> r & 1u)) continue;
-      bulk_copy(dst + pos * su * 16, S.gptr[r] + ((size_t)tok0 + (size_t)cu0 * VE) * p.esize, (uint32_t)bytes,
-                &S.wbar[warp][stage]);
-      ++pos;
-    }
-  }
-
-  template <class FN>
-  __device__ void stream(uint32_t mask, FN&& fn) {
+  // ---------------------------------------------------------------- streaming
+  // The CTA's slice in groups of 32 units, one unit per lane, dealt to the
+  // warps in turn: fn(gu, valid, L) is called by all 32 lanes together, gu the
+  // unit's index in the slice (a group starts at a multiple of 32) and L(r, v)
+  // giving unit gu of row r (L.raw(r) its 16 bytes; -inf where not valid).
+  // No block barrier is taken: a caller synchronises the block before reading
+  // what other warps wrote.
+  //
+  // stream_rows: NR rows known by the caller, straight into registers, D units
+  // of a thread in flight and the loop unrolled U times.  Two CTAs' warps keep up to
+  // 64 KB an SM in flight, which covers the memory's latency, and a unit costs
+  // no copy, wait or shared-memory read (per-warp rings of bulk copies: 15
+  // instructions a logit at one draft).  Before and after, us a call: sequential
+  // rejection at B = 1024, K = 4, V = 151936 1241 and 931, with two models at
+  // V = 50257 87 and 71, classical IS at V = 32000 197 and 176.  Heavy bodies
+  // (IS moments, several rows) take U = 1: one copy of their code.
+  template <int D, int U, int NR, class FN>
+  __device__ __forceinline__ void stream_rows(const int (&rows)[NR], FN&& fn) {
+    constexpr int kStep = kThreads;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int nrm = __popc(mask);
-    const int su = stage_units(nrm);
-    if (!p.tma_ok || !p.bulk_ok || su < 32) {
-      for (int g = warp * 32; g < Uv; g += kWarps * 32) {
-        const int gu = g + lane;
-        fn(gu, gu < Uv, GlobalLoad<DT>{S.gptr, tok0, p.V, gu, p.tma_ok != 0});
+    uint4 x[D][NR];
+    load_rows(rows, warp * 32 + lane, x);
+#pragma unroll U
+    for (int g = warp * 32; g < Uv; g += kStep) {
+      uint4 y[NR];
+#pragma unroll
+      for (int i = 0; i < NR; ++i) {
+        y[i] = x[0][i];
+#pragma unroll
+        for (int d = 0; d + 1 < D; ++d) x[d][i] = x[d + 1][i];
       }
-      return;
+      uint4 z[1][NR];
+      load_rows(rows, g + D * kStep + lane, z);
+#pragma unroll
+      for (int i = 0; i < NR; ++i) x[D - 1][i] = z[0][i];
+      fn(g + lane, g + lane < Uv, RegLoad<DT, NR>{y, rows});
     }
-    const int nchunk = (Uv + su - 1) / su;
-    const int nk = (nchunk - warp + kWarps - 1) / kWarps;   // this warp's chunks: warp, warp + kWarps, ...
-    if (nk <= 0 || bail) return;
-    if (lane == 0) {
-      fence_proxy_async();
-      for (int k = 0; k < nk && k < kWStages; ++k) issue_stage(k, mask, su);
+  }
+  // Units gu, gu + 256, ... of the rows (-inf past the slice): the loads of a
+  // batch are issued together in either form.
+  template <int N, int NR>
+  __device__ __forceinline__ void load_rows(const int (&rows)[NR], int gu, uint4 (&x)[N][NR]) const {
+    if (p.tma_ok) {
+#pragma unroll
+      for (int d = 0; d < N; ++d)
+#pragma unroll
+        for (int i = 0; i < NR; ++i) x[d][i] = row_unit(rows[i], gu + d * kThreads, true);
+    } else {
+#pragma unroll
+      for (int d = 0; d < N; ++d)
+#pragma unroll
+        for (int i = 0; i < NR; ++i) x[d][i] = row_unit(rows[i], gu + d * kThreads, false);
     }
-    __syncwarp();
-    for (int k = 0; k < nk; ++k) {
-      const int stage = k % kWStages;
-      const char* base = ring + (size_t)(warp * kWStages + stage) * (p.ring_bytes / kWarps / kWStages);
-      long long spins = 0;
-      bool ok = true;
-      while (!mbar_try_wait(&S.wbar[warp][stage], (wphase >> stage) & 1u)) {
-        if (++spins > kWaitLimit) {
-          ok = false;
-          break;
-        }
-      }
-      if (!__all_sync(0xffffffffu, ok)) {
-        // A copy never landed: flag the launch (every sequence still to be
-        // written is then marked -1), issue nothing more from this warp and
-        // give the copies already issued one more bounded wait before the
-        // warp's ring is left for good.
-        if (lane == 0) {
-          atomicOr(p.status, MDS_ST_TIMEOUT);
-          for (int kk = k; kk < nk && kk < k + kWStages; ++kk) {
-            const int st = kk % kWStages;
-            for (long long w = 0; w <= kWaitLimit && !mbar_try_wait(&S.wbar[warp][st], (wphase >> st) & 1u); ++w) {
-            }
-          }
-        }
-        __syncwarp();
-        bail = 1;
-        return;
-      }
-      wphase ^= 1u << stage;
-      const int cu0 = (warp + k * kWarps) * su, cu1 = min(cu0 + su, Uv);
-      for (int g = cu0; g < cu1; g += 32) {
-        const int gu = g + lane;
-        fn(gu, gu < cu1, StageLoad<DT>{base, mask, su * 16, g - cu0 + lane});
-      }
-      __syncwarp();
-      if (lane == 0 && k + kWStages < nk) {
-        fence_proxy_async();
-        issue_stage(k + kWStages, mask, su);
-      }
-      __syncwarp();
+  }
+  __device__ __forceinline__ uint4 row_unit(int r, int gu, bool aligned) const {
+    return gu < Uv ? slice_unit<DT>(S.gptr[r], tok0, p.V, gu, aligned) : dev::Elt<DT>::neg_inf();
+  }
+  // The target row and every draft row, one or two of them in registers.
+  template <class FN>
+  __device__ __forceinline__ void stream_all(FN&& fn) {
+    if (S.nrows == 2)
+      stream_rows<3, 1>({0, 1}, fn);
+    else if (S.nrows == 3)
+      stream_rows<2, 1>({0, 1, 2}, fn);
+    else
+      stream_any(fn);
+  }
+  // Any rows: unit by unit.
+  template <class FN>
+  __device__ __forceinline__ void stream_any(FN&& fn) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int g = warp * 32; g < Uv; g += kWarps * 32) {
+      const int gu = min(g + lane, Uv - 1);
+      fn(g + lane, g + lane < Uv, GlobalLoad<DT>{S.gptr, tok0, p.V, gu, p.tma_ok != 0});
     }
   }
 
   // ---------------------------------------------------------------- softmax statistics
+  // A thread's running max and sum of R rows: a batch of units' maxima first
+  // (packed compares), one rescale, then the exponentials.
+  template <int R>
+  __device__ __forceinline__ void stats_stream(const int (&rows)[R], float (&m)[R], float (&sc)[R],
+                                               const float (&cr)[R]) {
+    using De = dev::Elt<DT>;
+    constexpr int NB = R == 1 ? 8 : (R == 2 ? 4 : 2), kStep = kThreads;
+    for (int g = threadIdx.x; g < Uv; g += kStep * NB) {
+      uint4 x[NB][R];
+      load_rows(rows, g, x);
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        uint4 mx = x[0][r];
+#pragma unroll
+        for (int q = 1; q < NB; ++q) mx = De::max4(mx, x[q][r]);
+        float v[VE];
+        Elt<DT>::unpack(mx, v);
+#pragma unroll
+        for (int e = VE / 2; e; e >>= 1)
+#pragma unroll
+          for (int i = 0; i < e; ++i) v[i] = fmaxf(v[i], v[i + e]);
+        if (v[0] > m[r]) {
+          sc[r] = (m[r] == kNegInf) ? 0.f : __fmul_rn(sc[r], ex2(__fsub_rn(__fmul_rn(m[r], cr[r]), __fmul_rn(v[0], cr[r]))));
+          m[r] = v[0];
+        }
+        if (m[r] > kNegInf) {   // exp of -inf is 0; only -inf - -inf must be avoided
+          const float mc = __fmul_rn(m[r], cr[r]);
+#pragma unroll
+          for (int q = 0; q < NB; ++q) {
+            float t[VE];
+            Elt<DT>::unpack(x[q][r], t);
+#pragma unroll
+            for (int e = 0; e < VE; ++e) t[e] = ex2(__fmaf_rn(t[e], cr[r], -mc));
+#pragma unroll
+            for (int e = VE / 2; e; e >>= 1)
+#pragma unroll
+              for (int i = 0; i < e; ++i) t[i] = __fadd_rn(t[i], t[i + e]);
+            sc[r] = __fadd_rn(sc[r], t[0]);
+          }
+        }
+      }
+    }
+  }
   // Candidate order: larger target logit first, then smaller token id.
   __device__ __forceinline__ static bool cand_before(float la, int ia, float lb, int ib) {
     return la > lb || (la == lb && ia < ib);
@@ -767,8 +760,11 @@ struct Kernel {
     }
     int* wa_id = ap_id + warp * kWarpApp;
     float* wa_l = ap_l + warp * kWarpApp;   // row r at wa_l[r * kWarps * kWarpApp + i]
-    const uint32_t mask = ((1u << R) - 1u) << r0;
-    stream(mask, [&](int gu, bool valid, const auto& L) {
+    int rows[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) rows[r] = r0 + r;
+    if constexpr (!CAND) stats_stream<R>(rows, m, sc, cr);
+    if constexpr (CAND) stream_rows<(R == 2 ? 3 : 2), 1>(rows, [&](int gu, bool valid, const auto& L) {
       // row 0 first: its values decide which tokens are set aside
       float v0[VE];
       if (valid) {
@@ -778,7 +774,6 @@ struct Kernel {
         for (int e = 0; e < VE; ++e) v0[e] = kNegInf;
       }
       const int t0 = tok0 + gu * VE;
-      (void)t0;
       float mu0 = v0[0];
 #pragma unroll
       for (int e = 1; e < VE; ++e) mu0 = fmaxf(mu0, v0[e]);
@@ -815,16 +810,19 @@ struct Kernel {
         }
         if (m[r] > kNegInf) {   // exp of -inf is 0; only -inf - -inf must be avoided
           const float mc = __fmul_rn(m[r], cr[r]);
-          if (!aside) {
+          float t[VE];
 #pragma unroll
-            for (int e = 0; e < VE; ++e) sc[r] = __fadd_rn(sc[r], ex2(__fmaf_rn(v[e], cr[r], -mc)));
-          } else {
+          for (int e = 0; e < VE; ++e) t[e] = ex2(__fmaf_rn(v[e], cr[r], -mc));
+          if (aside) {
 #pragma unroll
-            for (int e = 0; e < VE; ++e) {
-              const float t = ex2(__fmaf_rn(v[e], cr[r], -mc));
-              sc[r] = __fadd_rn(sc[r], ((aside >> e) & 1u) ? 0.f : t);
-            }
+            for (int e = 0; e < VE; ++e)
+              if ((aside >> e) & 1u) t[e] = 0.f;
           }
+#pragma unroll
+          for (int e = VE / 2; e; e >>= 1)
+#pragma unroll
+            for (int i = 0; i < e; ++i) t[i] = __fadd_rn(t[i], t[i + e]);
+          sc[r] = __fadd_rn(sc[r], t[0]);
         }
       }
       if constexpr (CAND) {
@@ -1154,13 +1152,13 @@ struct Kernel {
         default: break;
       }
     }
-    constexpr int step = SCHEME == MDS_IS ? 2 : 4;   // classical IS: its ring holds two rows a stage
+    constexpr int step = 4;
     for (int r0 = 0; r0 < nr; r0 += step) {
       switch (min(step, nr - r0)) {
         case 1: stats_pass<1, false>(r0); break;
         case 2: stats_pass<2, false>(r0); break;
-        case 3: stats_pass<step == 4 ? 3 : 1, false>(r0); break;
-        default: stats_pass<step == 4 ? 4 : 1, false>(r0); break;
+        case 3: stats_pass<3, false>(r0); break;
+        default: stats_pass<4, false>(r0); break;
       }
     }
   }
@@ -1168,15 +1166,15 @@ struct Kernel {
   // ---------------------------------------------------------------- residual / CDF sampling
   // Inverse-CDF draw over this sequence's vocabulary from the nonnegative
   // weights rf(gu, L, r[VE]) in token order: the smallest token whose running
-  // sum exceeds u * (total).  A streaming pass over the rows in `mask` forms
+  // sum exceeds u * (total).  A streaming pass over the rows `pass` names forms
   // the sum of every 32-unit segment (lane partial sums, warp inclusive
   // scan); segments are added in order per CTA and CTAs in rank order; the
   // owner CTA re-reads its one segment from global memory and re-walks the
   // same sums.  Returns the token (cluster-uniform) and the total mass.
-  template <class RF>
-  __device__ int sample_cdf(uint32_t mask, const RF& rf, float u01, float* total) {
+  template <class PASS, class RF>
+  __device__ int sample_cdf(const PASS& pass, const RF& rf, float u01, float* total) {
     const int lane = threadIdx.x & 31;
-    stream(mask, [&](int gu, bool valid, const auto& L) {
+    pass([&](int gu, bool valid, const auto& L) {
       float part = 0.f;
       if (valid) {
         float r[VE];
@@ -1363,7 +1361,7 @@ struct Kernel {
     const float c = S.c[0];
     float wmax = kNegInf, wref = kNegInf;   // warp-uniform; wref = round(wmax c)
     float sc = 0.f;                         // this lane's sum, relative to wref
-    stream(1u, [&](int gu, bool valid, const auto& L) {
+    stream_rows<4, 1>({0}, [&](int gu, bool valid, const auto& L) {
       float v[VE];
       if (valid) {
         L(0, v);
@@ -1542,10 +1540,7 @@ struct Kernel {
     for (int t = 0; t < kTop; ++t) top[t] = CAND_NONE;
     float suma = 0.f, sumb = 0.f;   // masses of tokens dropped from this thread's list
     const int nr = S.nrows;
-    uint32_t mask = 1u | (1u << rb);
-    for (int r = 1; r < nr; ++r)
-      if (S.gamma[r] != 0.f) mask |= 1u << r;
-    stream(mask, [&](int gu, bool valid, const auto& L) {
+    stream_any([&](int gu, bool valid, const auto& L) {
       if (!valid) return;
       const int uu = gu;
       const int tbase = tok0 + uu * VE;
@@ -1886,7 +1881,7 @@ struct Kernel {
     float zero = 0.f;
     const RowC c0 = row_c(0), cr = row_c(r);
     const float lz = S.is_lz[r];
-    stream(1u | (1u << r), [&](int, bool valid, const auto& L) {
+    stream_rows<2, 1>({0, r}, [&](int, bool valid, const auto& L) {
       float lq[VE], lp[VE];
       if (valid) {
         L(0, lq);
@@ -1973,7 +1968,7 @@ struct Kernel {
       // by the exponents' difference (log2 rho, rounded once per row below)
       const RowC c0 = row_c(0), cr = row_c(r);
       float dlo = kPosInf, dhi = kNegInf;
-      stream(1u | (1u << r), [&](int, bool valid, const auto& L) {
+      stream_rows<4, 2>({0, r}, [&](int, bool valid, const auto& L) {
         if (!valid) return;
         float v[VE], w[VE];
         L(0, v);
@@ -2435,7 +2430,7 @@ struct Kernel {
     const bool all0 = S.o0_all != 0;
     float tot;
     int Z = sample_cdf(
-        1u,
+        [&](auto&& fn) { stream_rows<8, 4>({0}, fn); },
         [&](int, const auto& L, float* r) {
           float v[VE];
           L(0, v);
@@ -2447,7 +2442,7 @@ struct Kernel {
       if (Yp >= 0) return Yp;
       if (threadIdx.x == 0 && rank == 0) atomicOr(p.status, MDS_ST_ZERO_RESID);
       Z = sample_cdf(
-          1u,
+          [&](auto&& fn) { stream_rows<2, 1>({0}, fn); },
           [&](int, const auto& L, float* r) {
             float v[VE];
             L(0, v);
@@ -2561,26 +2556,18 @@ struct Kernel {
           bool done = false;
           if constexpr (SCHEME == MDS_WIS) {
             if (S.nv > 1) {
-              uint32_t mask = 1u;
-              for (int r = 1; r < S.nrows; ++r)
-                if (S.gamma[r] != 0.f) mask |= 1u << r;
-              Z = sample_cdf(mask, [&](int gu, const auto& L, float* r) { residual_wis(gu, L, r); }, ures, &tot);
+              Z = sample_cdf([&](auto&& fn) { stream_all(fn); }, [&](int gu, const auto& L, float* r) { residual_wis(gu, L, r); }, ures, &tot);
               done = true;
             }
           }
           if constexpr (SCHEME == MDS_IS) {
             if (S.nv > 1) {
-              uint32_t mask = 1u;
               int rows = 0;
-              for (int r = 1; r < S.nrows; ++r)
-                if (S.is_cnt[r]) {
-                  mask |= 1u << r;
-                  ++rows;
-                }
+              for (int r = 1; r < S.nrows; ++r) rows += S.is_cnt[r] ? 1 : 0;
               if (p.dbg_exps && rank == 0 && tid == 0)   // p_I at every token: one exponential per node and row
                 atomicAdd(p.dbg_exps, (unsigned long long)S.is_n * (unsigned long long)p.V * (unsigned long long)rows);
               is_table();
-              Z = sample_cdf(mask, [&](int, const auto& L, float* r) { residual_is(L, r); }, ures, &tot);
+              Z = sample_cdf([&](auto&& fn) { stream_all(fn); }, [&](int, const auto& L, float* r) { residual_is(L, r); }, ures, &tot);
               done = true;
             }
           }
@@ -2588,7 +2575,7 @@ struct Kernel {
             const int r1 = S.vrow[0];
             const RowC c0 = row_c(0), c1 = row_c(r1);
             Z = sample_cdf(
-                1u | (1u << r1),
+                [&](auto&& fn) { stream_rows<4, 4>({0, r1}, fn); },
                 [&](int, const auto& L, float* r) {
                   float v[VE], w[VE];
                   L(0, v);
@@ -2604,7 +2591,7 @@ struct Kernel {
           } else if (Z < 0) {
             if (tid == 0) atomicOr(p.status, MDS_ST_ZERO_RESID);
             Z = sample_cdf(
-                1u,
+                [&](auto&& fn) { stream_rows<2, 1>({0}, fn); },
                 [&](int, const auto& L, float* r) {
                   float v[VE];
                   L(0, v);
@@ -2642,7 +2629,7 @@ struct Kernel {
     }
     if (rank == 0 && tid == 0) {
       if (*reinterpret_cast<volatile unsigned*>(p.status) & MDS_ST_TIMEOUT) {
-        abandon(b);   // a ring wait gave up during the launch: this walk is not trusted
+        abandon(b);   // a bounded wait gave up on this context: the walk is not trusted
       } else {
         p.out_accept[b] = acc_len;
         for (int j = acc_len + 1; j <= L; ++j) p.out_tokens[(size_t)b * (L + 1) + j] = -1;
@@ -2802,23 +2789,22 @@ struct Kernel {
       }
       // residual mass of this round
       const int ri = S.sp_rows[i];
-      uint32_t mask = 1u | (1u << ri);
-      for (int k = 0; k < i; ++k) mask |= 1u << S.sp_rows[k];
       const SpectrW sw = spectr_weights(i, ri);
+      const auto pass = [&](auto&& fn) { stream_all(fn); };
       if (i == nv - 1 && zacc < 0) {
         __syncthreads();   // every thread has read the round's state
         float tot;
-        const int z = sample_cdf(mask, [&](int, const auto& L, float* r) { spectr_resid(L, sw, r); },
+        const int z = sample_cdf(pass, [&](int, const auto& L, float* r) { spectr_resid(L, sw, r); },
                                  draw_uniform(p.seed, b, j, kDrawResidual), &tot);
         *Rd = __fmul_rn(prodR, tot);
         if (tot > 0.f) return z;
         // no mass (only by rounding, q_i = p_i): the round leaves q_i as it is
         const SpectrW st = spectr_weights(i, -1);
-        return sample_cdf(mask, [&](int, const auto& L, float* r) { spectr_resid(L, st, r); },
+        return sample_cdf(pass, [&](int, const auto& L, float* r) { spectr_resid(L, st, r); },
                           draw_uniform(p.seed, b, j, kDrawResidual), &tot);
       }
       float part = 0.f;
-      stream(mask, [&](int, bool valid, const auto& L) {
+      stream_all([&](int, bool valid, const auto& L) {
         if (!valid) return;
         float r[VE];
         spectr_resid(L, sw, r);
@@ -2915,13 +2901,12 @@ __global__ void __launch_bounds__(kThreads, 2) verify_kernel(const __grid_consta
   k.nseg = (p.slice / Kernel<DT, SCHEME>::VE + 31) / 32;   // same in every CTA: peers map the same offsets
   k.nsegv = (k.Uv + 31) / 32;                                // segments the residual pass writes
   k.bm_words = (p.slice / Kernel<DT, SCHEME>::VE + 31) / 32;   // one bit per 16-byte unit
-  // dynamic shared memory: ring | segment sums | chunk sums | segment references | scheme region
+  // dynamic shared memory: segment sums | chunk sums | segment references | scheme region
   //   IS : bins (the residual's coefficients) | set-aside tokens | nodes t_n | weights W_r(n)
   //   WIS: CTA list (two copies) | warp lists = staging list | merged list, the
   //        last aliased later by the special-token bitmap (only the CTA list
   //        is ever read by other CTAs)
-  k.ring = dsm;
-  k.segsum = reinterpret_cast<float*>(dsm + p.ring_bytes);
+  k.segsum = reinterpret_cast<float*>(dsm);
   k.chksum = k.segsum + ((k.nseg + 3) & ~3);
   k.segref = k.chksum + ((((k.nseg + 31) / 32) + 3) & ~3);
   {
@@ -2955,13 +2940,6 @@ __global__ void __launch_bounds__(kThreads, 2) verify_kernel(const __grid_consta
   }
   k.xbuf = 0;
   k.clbuf = 0;
-  k.wphase = 0u;
-  k.bail = 0;
-  if (threadIdx.x == 0) {
-    for (int w = 0; w < kWarps; ++w)
-      for (int i = 0; i < kWStages; ++i) mbar_init(&S.wbar[w][i]);
-    mbar_init_fence();
-  }
   __syncthreads();
   // A peer's shared memory may be accessed only once every CTA of the
   // cluster is running: one cluster barrier before the first remote store.
@@ -2970,7 +2948,7 @@ __global__ void __launch_bounds__(kThreads, 2) verify_kernel(const __grid_consta
     if (k.rank == 0 && threadIdx.x == 0) {
       int b = (int)(atomicAdd(p.queue, 1u) - p.ticket0);
       if (b < p.B && (*reinterpret_cast<volatile unsigned*>(p.status) & MDS_ST_TIMEOUT)) {
-        k.abandon(b);   // after a ring wait gave up, the remaining sequences are only marked
+        k.abandon(b);   // a bounded wait gave up on this context: the sequences are only marked
         b = -1;
       }
       if (p.cn > 1) {
@@ -3000,7 +2978,7 @@ __global__ void __launch_bounds__(kThreads, 2) verify_kernel(const __grid_consta
 size_t smem_bytes(const Params& p) {
   const int VE = 16 / p.esize;
   const int nseg = (p.slice / VE + 31) / 32;
-  size_t bytes = (size_t)p.ring_bytes + (size_t)((nseg + 3) & ~3) * 4 * 2 + (size_t)((((nseg + 31) / 32) + 3) & ~3) * 4;
+  size_t bytes = (size_t)((nseg + 3) & ~3) * 4 * 2 + (size_t)((((nseg + 31) / 32) + 3) & ~3) * 4;
   if (p.scheme == MDS_IS)
     bytes += (size_t)kIsBinBytes + (size_t)kWarps * kIsStage * 16 + (size_t)kIsNodesMax * 4 * (1 + p.rows_max);
   if (p.scheme == MDS_WIS || p.scheme == MDS_WIS0) {
