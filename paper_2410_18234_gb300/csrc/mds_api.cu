@@ -536,11 +536,13 @@ const char* status_message(unsigned st) {
 // of a few instructions, so the per-sequence engine, whose cluster combines a pass in
 // shared memory, beats the dataflow engine's ring, record and request round
 // trips (about 15 us a pass) until a CTA's slice of a row is long: measured at
-// K = 4, L = 4 in bf16, per-sequence against dataflow: slices of 2 to 8 KB 32
-// to 60 against 76 to 247 us, 31 KB 60 against 104, 62 KB 87 to 156 against
-// 107 to 274, 125 KB 144 against 123, 250 KB 267 against 178.  With several
-// models the per-sequence engine would stream every model's row.
-constexpr size_t kSeqSliceMax = 64 * 1024;
+// K = 4, L = 4, per-sequence against dataflow in us: slices of 2 to 8 KB 32 to
+// 60 against 76 to 247, 31 KB 60 against 104, 62 KB 72 to 121 against 107 to
+// 274, 98 KB 202 against 242, 125 KB 118 against 145 (fp32 102 against 125),
+// 156 KB 133 against 184, 195 KB 179 against 192, 256 KB 194 against 175,
+// 297 KB 225 against 217.  With several models the per-sequence engine would
+// stream every model's row.
+constexpr size_t kSeqSliceMax = 192 * 1024;
 static size_t seq_slice_bytes(const mds_config& c, int grid) {
   int cn = 1;   // the cluster size the per-sequence engine takes
   while (cn < kMaxCluster && 2L * cn * c.max_B <= grid) cn *= 2;

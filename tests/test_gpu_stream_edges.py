@@ -40,3 +40,20 @@ def test_stream_edges(V, cluster, models, dtype):
         res = compare(out.cpu().numpy(), acc.cpu().numpy(), o_out, o_acc, recs, g_diag=diag.cpu().numpy(), scheme=scheme)
         check(res, scheme)
         assert bits == 0
+
+
+@pytest.mark.parametrize("V,dtype", [(98304, "bf16"), (98305, "bf16"), (49152, "f32"), (49153, "f32")])
+def test_single_draft_either_side_of_the_engine_rule(V, dtype):
+    """One CTA a sequence (a batch of 304 at most): slices of 192 KB and just above."""
+    spec = WorkloadSpec(f"v{V}", B=4, K=2, L=2, V=V, dtype=dtype, model_ids=[0, 0], target_scale=3.0,
+                        draft_sigma=[0.8], t_target=0.8, t_draft=[0.8], data_seed=V)
+    w = make_workload(spec, device=DEV)
+    v = mds.Verifier(304, spec.K, spec.L, V, dtype=dtype)
+    out, acc, diag = v.verify(w.target, w.draft_list(), w.model_ids, w.tokens, w.temps, "single", 31, diag=True)
+    torch.cuda.synchronize()
+    bits, _ = v.status()
+    v.close()
+    o_out, o_acc, recs = oracle_verify(*host_copy(w), "single", 31)
+    res = compare(out.cpu().numpy(), acc.cpu().numpy(), o_out, o_acc, recs, g_diag=diag.cpu().numpy(), scheme="single")
+    check(res, "single")
+    assert bits == 0
