@@ -200,9 +200,9 @@ int mds_verify_host(mds_ctx* ctx, const void* target_logits, const void* const* 
  * word, and for single, WIS and WIS0 the slice engine's control words, task
  * ring, per-sequence state and slice records, which grow with B and with the
  * number of slices per row, about V / 8192) lives in a file-scope device
- * array of MDS_NOALLOC_SCRATCH_BYTES (8 MiB) that every GPU loading the
+ * array of MDS_NOALLOC_SCRATCH_BYTES (10 MiB) that every GPU loading the
  * library holds until the process exits; a call whose scratch exceeds it
- * (for llama3-like rows of 128k bf16 logits, beyond roughly 1,500 sequences
+ * (for llama3-like rows of 128k bf16 logits, beyond roughly 2,000 sequences
  * per call) is rejected
  * with MDS_ESHAPE before any launch.  The first call on a device looks up
  * that array's device address and sets kernel attributes, so make it before
@@ -211,7 +211,7 @@ int mds_verify_host(mds_ctx* ctx, const void* target_logits, const void* const* 
  * so calls that overlap on the GPU race.  The status word is not reported
  * (use mds_noalloc_status).  The paper has no counterpart to this entry
  * point: it exists only for callers that cannot allocate. */
-#define MDS_NOALLOC_SCRATCH_BYTES (8u << 20)
+#define MDS_NOALLOC_SCRATCH_BYTES (10u << 20)
 int mds_verify_noalloc(const mds_config* cfg, int device, const void* target_logits,
                        const void* const* draft_logits, const int32_t* draft_model_id,
                        const int32_t* draft_tokens, const float* temperatures, int scheme,

@@ -55,7 +55,7 @@ constexpr int kNBuf = 2;               // slice buffers per CTA
 // descriptor lives on until task k + 3 is issued, which waits for every warp
 // to release task k + 1's buffer, so to have done task k.
 constexpr int kNDesc = kNBuf + 1;
-constexpr int kSlots = 3;              // records between the compute warps and the publishing warpss
+constexpr int kSlots = 3;              // records between the compute warps and the publishing warp
 constexpr int kFastUnits = kBufBytes / 16;   // units of all rows one slice holds
 constexpr int kWarpCand = 32;          // tokens one warp may set aside in a slice
 constexpr int kSlotCand = kCW * kWarpCand;

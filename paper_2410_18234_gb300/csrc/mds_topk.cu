@@ -18,15 +18,14 @@
 // Tokens outside U carry zero mass in every law, so the inverse CDFs in
 // token-id order (residual, bonus) run over U sorted by id.
 //
-// One CTA of 256 threads verifies one sequence.  Per depth: warp 0 plans the
+// One CTA of 512 threads verifies one sequence.  Per depth: warp 0 plans the
 // rows (the target row of the lowest valid branch, one draft row per model
 // among the valid branches, read from its lowest valid branch; the single
-// draft step reads only the first valid branch's).  For each row, every
-// thread first takes the maximum of its first units; the k-th largest of
-// those maxima bounds the row's k-th logit from below.  Then every thread
-// scans its strided share of the row, keeping a sorted list of its 16
-// largest (logit, -id) keys at or above that bound, and the warps merge the
-// lists into the row's top k.  Warp 0 then computes the kept entries'
+// draft step reads only the first valid branch's).  For each row, the warps
+// first take maxima of a share of the row; the k-th largest of them bounds
+// the row's k-th logit from below.  Then every thread scans its share of the
+// row and sets the tokens at or above that bound aside in shared memory,
+// where counting ranks them.  Warp 0 then computes the kept entries'
 // probabilities, the union, the scheme's decision and the walk.
 #include "mds_device.cuh"
 #include "mds_topk.h"

@@ -76,3 +76,22 @@ def test_ties_and_flat_rows(kind):
     for scheme in ("single", "WIS"):
         run(w, scheme)
     run(w, "WIS0", uncertified=True)
+
+
+def test_large_noalloc_batch_fits_the_scratch():
+    """Slice records with 64 run masses (T = 16384) at a batch near the scratch's end."""
+    B, V = 2300, 131072
+    g = torch.Generator(device=DEV).manual_seed(5)
+    target = torch.randn(B, 1, 2, V, generator=g, device=DEV, dtype=torch.bfloat16)
+    draft = torch.randn(B, 1, V, generator=g, device=DEV, dtype=torch.bfloat16)
+    tok = torch.randint(V, (B, 1, 1), generator=g, device=DEV, dtype=torch.int32)
+    temps = torch.ones(B, 2, device=DEV)
+    res = []
+    v = mds.Verifier(B, 1, 1, V, omega0=20)
+    o, a, _ = v.verify(target, [draft], [0], tok, temps, "WIS0", 9)
+    res.append((o.clone(), a.clone()))
+    v.close()
+    o, a = torch.empty_like(o), torch.empty_like(a)
+    mds.mds_verify_noalloc(B, 1, 1, V, target, [draft], [0], tok, temps, "WIS0", 9, o, a, omega0=20)
+    torch.cuda.synchronize()
+    assert torch.equal(o, res[0][0]) and torch.equal(a, res[0][1])
