@@ -27,10 +27,11 @@ struct mds_ctx {
   void* h_buf;
   size_t h_bytes;
   // slice-dataflow engine: workspace (control words, task ring, per-sequence
-  // state and slice records; grown on demand, zero between launches) and the
-  // launch counter that tags the ring's entries
+  // state and slice records; grown on demand), the ring length it was last
+  // laid out for and the launch counter that tags the ring's entries
   void* f_buf;
   size_t f_bytes;
+  int f_cap;
   unsigned epoch;
   int f_grid;
   float* dbg_rows;         // test export of row statistics (caller-owned), or null
@@ -211,6 +212,7 @@ int mds_create(mds_ctx** out, const mds_config* cfg, int device) {
   ctx->h_bytes = 0;
   ctx->f_buf = nullptr;
   ctx->f_bytes = 0;
+  ctx->f_cap = 0;
   ctx->epoch = 0u;
   ctx->f_grid = mds::flow::grid_size(device);
   cudaError_t me = cudaMalloc(&ctx->work, 256);
@@ -225,7 +227,7 @@ int mds_create(mds_ctx** out, const mds_config* cfg, int device) {
 
 // The slice-dataflow engine serves single, WIS and WIS0 where its slice
 // geometry fits (every configuration of the benchmarks); the per-sequence
-// engine serves the rest.  Grows the context's workspace (zeroed) as needed.
+// engine serves the rest.  Grows the context's workspace as needed.
 int flow_verify(mds_ctx* ctx, const void* target_logits, const void* const* draft_logits, const int8_t* model_of,
                 int n_models, const int32_t* draft_tokens, const float* temperatures, int scheme,
                 uint64_t philox_seed, int32_t* out_tokens, int32_t* out_accept_len, float* out_diag, int B,
@@ -245,8 +247,8 @@ int flow_verify(mds_ctx* ctx, const void* target_logits, const void* const* draf
     }
     ctx->f_buf = nullptr;
     ctx->f_bytes = 0;
+    ctx->f_cap = 0;
     cudaError_t e = cudaMalloc(&ctx->f_buf, total);
-    if (e == cudaSuccess) e = cudaMemset(ctx->f_buf, 0, total);
     if (e != cudaSuccess) {
       if (ctx->f_buf) cudaFree(ctx->f_buf);
       ctx->f_buf = nullptr;
@@ -255,6 +257,14 @@ int flow_verify(mds_ctx* ctx, const void* target_logits, const void* const* draf
     ctx->f_bytes = total;
   }
   mds::flow::carve_workspace(p, static_cast<char*>(ctx->f_buf), c.max_B, ctx->f_grid);
+  if (p.ring_cap != ctx->f_cap) {
+    // a new buffer, or a call whose slices (scheme, draft models) move the
+    // rings and the pass counters over words of another kind
+    const cudaError_t e = cudaMemsetAsync(ctx->f_buf, 0, mds::flow::clear_bytes(p, c.max_B, ctx->f_grid),
+                                          static_cast<cudaStream_t>(stream));
+    if (e != cudaSuccess) return cuda_fail(e, "dataflow workspace layout");
+    ctx->f_cap = p.ring_cap;
+  }
   mds::flow_buffers(p, target_logits, draft_logits, draft_tokens, temperatures, out_tokens, out_accept_len, out_diag,
                     B, philox_seed);
   p.status = ctx->work;

@@ -83,9 +83,11 @@ size_t seq_bytes();
 // Workspace of one launch geometry (p after plan_geometry) for up to nseq
 // sequences and a grid of `grid` CTAs: its size in bytes, and the carving of
 // a buffer of that size into p's control words, ring, counters, per-sequence
-// state and records.  The control words and counters must be zero before the
-// first launch on a buffer; the kernel leaves them zero.  clear_bytes() is the
-// length of that prefix (control words, then the ring, then the counters).
+// state and records.  The control words and counters must be zero at a launch
+// and the rings must hold words of earlier launches only; the kernel leaves
+// them so for the same layout (ring_cap).  clear_bytes() is the length of that
+// prefix (control words, then the rings, then the counters): clear it before
+// the first launch on a buffer and whenever ring_cap changes.
 size_t workspace_bytes(const Params& p, int nseq, int grid);
 void carve_workspace(Params& p, char* base, int nseq, int grid);
 size_t clear_bytes(const Params& p, int nseq, int grid);
