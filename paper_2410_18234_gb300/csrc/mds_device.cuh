@@ -268,11 +268,24 @@ __device__ __forceinline__ float ref_shift(float m, float M, float c) {
   return ex2(__fsub_rn(__fmul_rn(m, c), __fmul_rn(M, c)));
 }
 
+// The reference of a partial sum whose largest logit is m: -inf (no
+// reference) also where m c overflows, as for a part masked with the storage
+// type's lowest value.  Its terms are 0 against any reference that does not;
+// against its own they would be inf - inf.
+__device__ __forceinline__ float sum_ref(float m, float c) { return __fmul_rn(m, c) > kNegInf ? m : kNegInf; }
+// round(m c) of a reference m, 0 without one: the terms of such a part are 0,
+// or NaN from a NaN logit.
+__device__ __forceinline__ float ref_exp(float m, float c) { return m > kNegInf ? __fmul_rn(m, c) : 0.f; }
+// A partial sum s against reference m, moved to M >= m (without a reference s
+// is 0 or NaN and stays).
+__device__ __forceinline__ float moved_sum(float s, float m, float M, float c) {
+  return m > kNegInf ? __fmul_rn(s, ref_shift(m, M, c)) : s;
+}
+
 // Combine two (max, sum) pairs of one row.
 __device__ __forceinline__ void combine_ms(float& m, float& s, float m2, float s2, float c) {
   const float M = fmaxf(m, m2);
-  const float a = (m == kNegInf) ? 0.f : __fmul_rn(s, ref_shift(m, M, c));
-  const float b = (m2 == kNegInf) ? 0.f : __fmul_rn(s2, ref_shift(m2, M, c));
+  const float a = moved_sum(s, m, M, c), b = moved_sum(s2, m2, M, c);
   m = M;
   s = __fadd_rn(a, b);
 }

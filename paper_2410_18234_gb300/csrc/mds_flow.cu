@@ -763,7 +763,8 @@ struct Eng {
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const float c = P.row[r].c;
-      const float mc = (m[r] > kNegInf) ? __fmul_rn(m[r], c) : 0.f;
+      m[r] = sum_ref(m[r], c);
+      const float mc = ref_exp(m[r], c);
       float acc = 0.f;
 #pragma unroll
       for (int i = 0; i < NU; ++i) {
@@ -858,7 +859,7 @@ struct Eng {
       float t = kNegInf;
 #pragma unroll
       for (int w = 0; w < kCW; ++w) t = fmaxf(t, S.red[w * kMaxRows + r]);
-      m[r] = t;
+      m[r] = sum_ref(t, c[r]);
     }
     // theta: the smallest of the warps' k-th largest thread maxima (warps
     // with fewer than k tokens left out), so at least LN tokens are >= theta
@@ -924,17 +925,15 @@ struct Eng {
           } else {
             E::unpack(raw(b, r, u), v);
           }
-          if (m[r] > kNegInf) {
-            const float mc = __fmul_rn(m[r], c[r]);
-            if (!cm) {
+          const float mc = ref_exp(m[r], c[r]);
+          if (!cm) {
 #pragma unroll
-              for (int e = 0; e < VE; ++e) sm[r] = __fadd_rn(sm[r], ex2(__fmaf_rn(v[e], c[r], -mc)));
-            } else {
+            for (int e = 0; e < VE; ++e) sm[r] = __fadd_rn(sm[r], ex2(__fmaf_rn(v[e], c[r], -mc)));
+          } else {
 #pragma unroll
-              for (int e = 0; e < VE; ++e) {
-                const float t = ex2(__fmaf_rn(v[e], c[r], -mc));
-                sm[r] = __fadd_rn(sm[r], (cm >> e & 1u) ? 0.f : t);
-              }
+            for (int e = 0; e < VE; ++e) {
+              const float t = ex2(__fmaf_rn(v[e], c[r], -mc));
+              sm[r] = __fadd_rn(sm[r], (cm >> e & 1u) ? 0.f : t);
             }
           }
         }
@@ -1082,17 +1081,15 @@ struct Eng {
     for (int r = 0; r < P.nstream; ++r) {
       float mx = kNegInf;
       for (int u = tid; u < U; u += kCT) mx = fmaxf(mx, E::unit_max(raw(b, r, u)));
-      mx = block_max(mx, S.red);
       const float c = P.row[r].c;
+      mx = sum_ref(block_max(mx, S.red), c);
       float sm = 0.f;
-      if (mx > kNegInf) {
-        const float mc = __fmul_rn(mx, c);
-        for (int u = tid; u < U; u += kCT) {
-          float v[VE];
-          E::unpack(raw(b, r, u), v);
+      const float mc = ref_exp(mx, c);
+      for (int u = tid; u < U; u += kCT) {
+        float v[VE];
+        E::unpack(raw(b, r, u), v);
 #pragma unroll
-          for (int e = 0; e < VE; ++e) sm = __fadd_rn(sm, ex2(__fmaf_rn(v[e], c, -mc)));
-        }
+        for (int e = 0; e < VE; ++e) sm = __fadd_rn(sm, ex2(__fmaf_rn(v[e], c, -mc)));
       }
       sm = block_sum(sm, S.red + kCW);
       if (tid == 0) {
@@ -1380,7 +1377,7 @@ struct Eng {
       float mm = mw;
 #pragma unroll
       for (int o = 4; o; o >>= 1) mm = fmaxf(mm, __shfl_xor_sync(FULLM, mm, o));
-      float v = (mw > kNegInf) ? __fmul_rn(sw, ref_shift(mw, mm, T.c[r])) : 0.f;
+      float v = moved_sum(sw, mw, mm, T.c[r]);
 #pragma unroll
       for (int o = 4; o; o >>= 1) v = __fadd_rn(v, __shfl_xor_sync(FULLM, v, o));
       m[r] = mm;
@@ -1473,7 +1470,7 @@ struct Eng {
           // the chunks' sums, each against its warp's reference, moved to the slice's
           for (int q = lane; q < T.nrun; q += 32) {
             const float mw = T.m[q & (kCW - 1)][0];
-            __stcg(rec + 4 + q, (mw > kNegInf) ? __fmul_rn(T.run[q], ref_shift(mw, m[0], T.c[0])) : 0.f);
+            __stcg(rec + 4 + q, moved_sum(T.run[q], mw, m[0], T.c[0]));
           }
         }
         if (lane == 0) {
@@ -1994,8 +1991,7 @@ struct Dec {
       const float c = D.P.row[r].c;
       float z = 0.f;
       for (int sl = lane; sl < ns; sl += 32) {
-        const float ms = sr[sl * rf + 2 * r];
-        if (ms > kNegInf) z = __fadd_rn(z, __fmul_rn(sr[sl * rf + 2 * r + 1], ref_shift(ms, M, c)));
+        z = __fadd_rn(z, moved_sum(sr[sl * rf + 2 * r + 1], sr[sl * rf + 2 * r], M, c));
       }
       z = warp_sum(z);
       if (lane == 0) {
@@ -2783,8 +2779,7 @@ struct Dec {
     }
     const float c = D.P.row[0].c;
     float Zs = 0.f;
-    for (int q = lane; q < p.ns; q += 32)
-      if (Hm[q] > kNegInf) Zs = __fadd_rn(Zs, __fmul_rn(Rs[q], ref_shift(Hm[q], M, c)));
+    for (int q = lane; q < p.ns; q += 32) Zs = __fadd_rn(Zs, moved_sum(Rs[q], Hm[q], M, c));
     Zs = warp_sum(Zs);
     if (lane == 0) {
       D.P.row[0].M = M;
@@ -2921,8 +2916,8 @@ struct Dec {
         float lr[2], e[2];
 #pragma unroll
         for (int h = 0; h < 2; ++h) lr[h] = in0[h] ? E::global(D.P.row[r].ptr, id[h]) : kNegInf;
-        const float ref = warp_max(fmaxf(lr[0], lr[1]));
         const float cr = D.P.row[r].c;
+        const float ref = sum_ref(warp_max(fmaxf(lr[0], lr[1])), cr);
 #pragma unroll
         for (int h = 0; h < 2; ++h) e[h] = (in0[h] && ref > kNegInf) ? exp_term(lr[h], ref, cr) : 0.f;
         const float Pm = warp_sum(__fadd_rn(e[0], e[1]));

@@ -275,8 +275,7 @@ struct State {
 
 __device__ __forceinline__ void combine_ms(float& m, float& s, float m2, float s2, float c) {
   const float M = fmaxf(m, m2);
-  const float a = (m == kNegInf) ? 0.f : __fmul_rn(s, ex2(__fsub_rn(__fmul_rn(m, c), __fmul_rn(M, c))));
-  const float b = (m2 == kNegInf) ? 0.f : __fmul_rn(s2, ex2(__fsub_rn(__fmul_rn(m2, c), __fmul_rn(M, c))));
+  const float a = dev::moved_sum(s, m, M, c), b = dev::moved_sum(s2, m2, M, c);
   m = M;
   s = __fadd_rn(a, b);
 }
@@ -549,24 +548,23 @@ struct Kernel {
         for (int e = VE / 2; e; e >>= 1)
 #pragma unroll
           for (int i = 0; i < e; ++i) v[i] = fmaxf(v[i], v[i + e]);
-        if (v[0] > m[r]) {
-          sc[r] = (m[r] == kNegInf) ? 0.f : __fmul_rn(sc[r], ex2(__fsub_rn(__fmul_rn(m[r], cr[r]), __fmul_rn(v[0], cr[r]))));
-          m[r] = v[0];
+        const float mu = dev::sum_ref(v[0], cr[r]);
+        if (mu > m[r]) {
+          sc[r] = dev::moved_sum(sc[r], m[r], mu, cr[r]);
+          m[r] = mu;
         }
-        if (m[r] > kNegInf) {   // exp of -inf is 0; only -inf - -inf must be avoided
-          const float mc = __fmul_rn(m[r], cr[r]);
+        const float mc = dev::ref_exp(m[r], cr[r]);
 #pragma unroll
-          for (int q = 0; q < NB; ++q) {
-            float t[VE];
-            Elt<DT>::unpack(x[q][r], t);
+        for (int q = 0; q < NB; ++q) {
+          float t[VE];
+          Elt<DT>::unpack(x[q][r], t);
 #pragma unroll
-            for (int e = 0; e < VE; ++e) t[e] = ex2(__fmaf_rn(t[e], cr[r], -mc));
+          for (int e = 0; e < VE; ++e) t[e] = ex2(__fmaf_rn(t[e], cr[r], -mc));
 #pragma unroll
-            for (int e = VE / 2; e; e >>= 1)
+          for (int e = VE / 2; e; e >>= 1)
 #pragma unroll
-              for (int i = 0; i < e; ++i) t[i] = __fadd_rn(t[i], t[i + e]);
-            sc[r] = __fadd_rn(sc[r], t[0]);
-          }
+            for (int i = 0; i < e; ++i) t[i] = __fadd_rn(t[i], t[i + e]);
+          sc[r] = __fadd_rn(sc[r], t[0]);
         }
       }
     }
@@ -661,7 +659,7 @@ struct Kernel {
       } else if (present) {
 #pragma unroll
         for (int r = 0; r < R; ++r)
-          if (l[r] > kNegInf) add[r] = __fadd_rn(add[r], ex2(__fmaf_rn(l[r], cr[r], -__fmul_rn(pm[r], cr[r]))));
+          if (pm[r] > kNegInf) add[r] = __fadd_rn(add[r], ex2(__fmaf_rn(l[r], cr[r], -__fmul_rn(pm[r], cr[r]))));
       }
       outp += __popc(bal);
       __syncwarp();
@@ -804,11 +802,12 @@ struct Kernel {
 #pragma unroll
           for (int e = 1; e < VE; ++e) mu = fmaxf(mu, v[e]);
         }
+        mu = dev::sum_ref(mu, cr[r]);
         if (mu > m[r]) {
-          sc[r] = (m[r] == kNegInf) ? 0.f : __fmul_rn(sc[r], ex2(__fsub_rn(__fmul_rn(m[r], cr[r]), __fmul_rn(mu, cr[r]))));
+          sc[r] = dev::moved_sum(sc[r], m[r], mu, cr[r]);
           m[r] = mu;
         }
-        if (m[r] > kNegInf) {   // exp of -inf is 0; only -inf - -inf must be avoided
+        if (m[r] > kNegInf) {   // without a reference the terms are 0
           const float mc = __fmul_rn(m[r], cr[r]);
           float t[VE];
 #pragma unroll
@@ -844,7 +843,7 @@ struct Kernel {
                 }
 #pragma unroll
                 for (int e = 0; e < VE; ++e)
-                  if (((back >> e) & 1u) && v[e] > kNegInf)
+                  if (((back >> e) & 1u) && m[r] > kNegInf)
                     sc[r] = __fadd_rn(sc[r], ex2(__fmaf_rn(v[e], cr[r], -__fmul_rn(m[r], cr[r]))));
               }
             }
@@ -951,8 +950,8 @@ struct Kernel {
           }
 #pragma unroll
           for (int r = 0; r < R; ++r) {
-            const float l = ap_l[r * kWarps * kWarpApp + i];
-            const float ev = (l > kNegInf) ? ex2(__fmaf_rn(l, cr[r], -__fmul_rn(S.xch[xbuf][sx * r], cr[r]))) : 0.f;
+            const float l = ap_l[r * kWarps * kWarpApp + i], ref = S.xch[xbuf][sx * r];
+            const float ev = (ref > kNegInf) ? ex2(__fmaf_rn(l, cr[r], -__fmul_rn(ref, cr[r]))) : 0.f;
             if (rk < kListN)
               kp_s[r] = ev;
             else
@@ -1013,8 +1012,7 @@ struct Kernel {
       if (mm > kNegInf)
         for (int q = 0; q < cn; ++q) {
           const float mq = S.gat[q * nx + sx * r];
-          if (!(mq > kNegInf)) continue;
-          const float f = ex2(__fsub_rn(__fmul_rn(mq, cr[r]), __fmul_rn(mm, cr[r])));
+          const float f = mq > kNegInf ? dev::ref_shift(mq, mm, cr[r]) : 1.f;   // without a reference: sums of 0, or NaN
           const float sq = S.gat[q * nx + sx * r + 1];
           ss = __fadd_rn(ss, __fmul_rn(sq, f));
           zz = __fadd_rn(zz, __fmul_rn(CAND ? __fadd_rn(sq, S.gat[q * nx + sx * r + 2]) : sq, f));
@@ -1374,17 +1372,16 @@ struct Kernel {
       for (int e = 1; e < VE; ++e) wm = fmaxf(wm, v[e]);
 #pragma unroll
       for (int o = 16; o; o >>= 1) wm = fmaxf(wm, __shfl_xor_sync(0xffffffffu, wm, o));
+      wm = dev::sum_ref(wm, c);
       if (wm > wmax) {
-        const float nref = __fmul_rn(wm, c);
-        sc = (wmax == kNegInf) ? 0.f : __fmul_rn(sc, ex2(__fsub_rn(wref, nref)));
+        sc = dev::moved_sum(sc, wmax, wm, c);
         wmax = wm;
-        wref = nref;
+        wref = __fmul_rn(wm, c);
       }
       float part = 0.f;
-      if (wmax > kNegInf) {
+      const float ref = dev::ref_exp(wmax, c);
 #pragma unroll
-        for (int e = 0; e < VE; ++e) part = __fadd_rn(part, ex2(__fmaf_rn(v[e], c, -wref)));
-      }
+      for (int e = 0; e < VE; ++e) part = __fadd_rn(part, ex2(__fmaf_rn(v[e], c, -ref)));
       sc = __fadd_rn(sc, part);
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -2322,6 +2319,7 @@ struct Kernel {
 #pragma unroll
         for (int o = 16; o; o >>= 1) ref = fmaxf(ref, __shfl_xor_sync(FULL, ref, o));
         const float cr = S.c[r];
+        ref = dev::sum_ref(ref, cr);
         const float e = (in0 && ref > kNegInf) ? ex2(__fmaf_rn(lr, cr, -__fmul_rn(ref, cr))) : 0.f;
         const float P = warp_sum(e);
         if (lane == 0 && rank == 0 && P != P) atomicOr(p.status, MDS_ST_NONFINITE);
