@@ -125,7 +125,11 @@ struct Elt<MDS_F32> {
     v[2] = __uint_as_float(x.z);
     v[3] = __uint_as_float(x.w);
   }
-  // Largest logit of a unit (NaN entries are ignored unless all are NaN).
+  // Largest logits of a unit's even and odd places (NaN entries are ignored unless all are NaN).
+  __device__ static __forceinline__ float2 unit_max2(const uint4& x) {
+    return make_float2(fmaxf(__uint_as_float(x.x), __uint_as_float(x.z)), fmaxf(__uint_as_float(x.y), __uint_as_float(x.w)));
+  }
+  // Largest logit of a unit.
   __device__ static __forceinline__ float unit_max(const uint4& x) {
     return fmaxf(fmaxf(__uint_as_float(x.x), __uint_as_float(x.y)), fmaxf(__uint_as_float(x.z), __uint_as_float(x.w)));
   }
@@ -168,6 +172,10 @@ struct Elt<MDS_BF16> {
   }
   // Packed bf16x2 maxima (exact: the maximum of bf16 values is one of them).
   __device__ static __forceinline__ float unit_max(const uint4& x) {
+    const float2 m = unit_max2(x);
+    return fmaxf(m.x, m.y);
+  }
+  __device__ static __forceinline__ float2 unit_max2(const uint4& x) {
     uint32_t m;
     asm("{\n\t.reg .b32 t0, t1;\n\t"
         "max.bf16x2 t0, %1, %2;\n\t"
@@ -175,7 +183,7 @@ struct Elt<MDS_BF16> {
         "max.bf16x2 %0, t0, t1;\n\t}"
         : "=r"(m)
         : "r"(x.x), "r"(x.y), "r"(x.z), "r"(x.w));
-    return fmaxf(__uint_as_float(m << 16), __uint_as_float(m & 0xffff0000u));
+    return make_float2(__uint_as_float(m << 16), __uint_as_float(m & 0xffff0000u));
   }
   static constexpr uint32_t kNegInfBits = 0xff80ff80u;   // two logits of -inf
   __device__ static __forceinline__ uint4 neg_inf() {

@@ -21,8 +21,9 @@
 //   full     a full-vocabulary stage of the weighted scheme: the slice's top-s
 //            keys q - a b with a and b, and the Omega_2 masses of the rest;
 //   bonus    the target row's maximum, sum and run sums at depth L.
-// The compute warps work on their own shares of a slice without block
-// barriers and leave partial results in a record slot in shared memory; a
+// The compute warps work on their own shares of a slice (one block barrier
+// where a list is wanted: its bound comes from all of them) and leave partial
+// results in a record slot in shared memory; a
 // publishing warp merges them, stores the record and counts the pass's
 // slices.  The one that counts a pass's last slice posts a decision request.
 // A decision warp combines the records in slice order, runs the importance
@@ -63,6 +64,9 @@ constexpr int kMaxRuns = kFastUnits / 32;    // runs of 32 units of a slice
 constexpr int kCtasPerSm = 2;          // resident CTAs per SM (the launch bound)
 constexpr int kCandCap = 512;          // candidate tokens one slice may set aside
 constexpr int kListMax = 64;           // candidate list length at most
+constexpr int kSliceListMax = 32;      // a slice's list found warp by warp, at most
+constexpr int kRankMax = 64;           // tokens the publishing warp ranks by counting
+constexpr int kGroups = 8;             // groups of a warp's lanes with a maximum each
 constexpr int kHdr = 2 * kMaxRows + 2; // record: (max, sum) per row, tau, list length
 constexpr int kTopF = 8;               // per-thread candidates of a full stage (>= MDS_MAX_S)
 constexpr int kMaxEntries = 512;       // slices x slice list length, at most
@@ -227,13 +231,15 @@ struct __align__(16) Slot {
   int mode, b, slice, kind, j, R, nrun;
   int count;                   // slices to count with this one: its group's, at the group's end (else 0)
   float c[kListRowsMax];
-  int ncand;                   // tokens set aside (zero between slices)
+  int nc[kCW];                 // per warp: tokens set aside
   float tau[kCW];              // per warp: largest target logit not set aside
   float m[kCW][kListRowsMax], s[kCW][kListRowsMax];
   float run[kMaxRuns];
-  __align__(16) unsigned key[kSlotCand];   // order key of the target logit (16-bit logits: and the place, see set_aside)
-  unsigned short loc[kSlotCand], ord[kSlotCand];   // place in the slice; the tokens ranked past the list
-  float l[kListRowsMax][kSlotCand];
+  __align__(16) unsigned sel[kRankMax];    // the tokens ranked for the list: keys ...
+  unsigned short at[kRankMax];             // ... and entries
+  __align__(16) unsigned key[kSlotCand];   // tokens set aside, warp by warp: rank key (see cand_key),
+  unsigned short loc[kSlotCand];           // place in the slice,
+  float l[kListRowsMax][kSlotCand];        // every row's logit
 };
 static_assert(kListRowsMax * kSlotCand >= 2 * kCandCap, "the block-wise list's arrays lie over two slots' logits");
 
@@ -243,6 +249,7 @@ struct FShared {
   FDesc pend;                  // the scheduler's next task, resolved ahead
   float red[kCW * 2 * kMaxRows];
   float wth[kCW];
+  unsigned gmax[kCW * kGroups];   // order keys of the lane groups' largest target logits
   int ncand, issued, consumed;
   float addtau;
   float add[kMaxRows];
@@ -363,6 +370,59 @@ __device__ __noinline__ void load_rows(const FPass& P, int R, char* b, int tok0,
     for (int u = threadIdx.x; u < U; u += kCT)
       *reinterpret_cast<uint4*>(dst + 16 * (size_t)u) = load_unit<DT>(src, first, end, u, n);
   }
+}
+
+// ------------------------------------------------------------------ tokens set aside
+// Their numbers in a slot, warp by warp.
+struct Numbers {
+  int first[kCW + 1];   // each warp's first token
+  __device__ __forceinline__ explicit Numbers(const Slot& T) {
+    first[0] = 0;
+#pragma unroll
+    for (int w = 0; w < kCW; ++w) first[w + 1] = first[w] + T.nc[w];
+  }
+  __device__ __forceinline__ int entry(int j) const {   // slot entry of token j < first[kCW]
+    int at = j;
+#pragma unroll
+    for (int w = 1; w < kCW; ++w) at = j >= first[w] ? w * kWarpCand + j - first[w] : at;
+    return at;
+  }
+};
+// The first LN of n > LN tokens: those with a larger key than x, or x itself
+// and a place of at most y (equal 32-bit logits; 16-bit keys are distinct).
+// Warp-wide; out of line, few slices need it.
+template <int DT>
+__device__ __noinline__ uint2 list_cut(const Slot& T, int n, int LN) {
+  const int lane = threadIdx.x & 31;
+  const Numbers num(T);
+  auto count = [&](auto&& in) {
+    unsigned k = 0u;
+#pragma unroll 1
+    for (int j = lane; j < n; j += 32) k += in(num.entry(j)) ? 1u : 0u;
+    return (int)__reduce_add_sync(FULLM, k);
+  };
+  unsigned thr = 0u, last = 0xffffu;
+  int have = n;
+#pragma unroll 1
+  for (int bit = 31; bit >= 0; --bit) {
+    if (have == LN) break;
+    const unsigned c = thr | (1u << bit);
+    const int k = count([&](int i) { return T.key[i] >= c; });
+    if (k >= LN) {
+      thr = c;
+      have = k;
+    }
+  }
+  if (DT != MDS_BF16 && have > LN) {
+    const int need = LN - count([&](int i) { return T.key[i] > thr; });
+    last = 0u;
+#pragma unroll 1
+    for (int bit = 15; bit >= 0; --bit) {
+      const unsigned c = last | ((1u << bit) - 1u);
+      if (count([&](int i) { return T.key[i] == thr && T.loc[i] <= c; }) < need) last |= 1u << bit;
+    }
+  }
+  return make_uint2(thr, last);
 }
 
 // ------------------------------------------------------------------ the engine
@@ -635,14 +695,20 @@ struct Eng {
   // R rows (compile time) of a slice of at most 2048 / R units a row.  Every
   // thread keeps its units (u = thread, thread + 256, ...: the warps
   // interleave in chunks of 32 units) in registers and every warp works on
-  // its own share, with its own exponent references and no block barrier:
+  // its own share, with its own exponent references:
   // the row maxima (packed), then the sums of 2^(l c - m c).  With LIST the
-  // warp first sets aside the tokens whose target logit reaches theta, the
-  // p.kth-th largest of its lanes' maxima (so at least p.kth tokens where the
-  // warp has as many), and leaves them out of its sums; more than kWarpCand
-  // of them (ties, flat rows) and theta rises to the largest bound that
-  // leaves at most that many.  With RUNS (the bonus row) the chunks' sums are
-  // kept too.  The publishing warp merges the eight warps' results.
+  // warp first sets aside the tokens whose target logit reaches a bound, the
+  // p.kth-th largest of the maxima of the slice's 64 groups of four lanes (one
+  // block barrier), and leaves them out of its sums.  p.kth is the slice's
+  // list length and the maxima are distinct tokens, so none of the slice's
+  // p.kth largest is missed; on independent logits 8.5 tokens a slice are set
+  // aside for p.kth = 8, 18 for 16 and 44 for 32.  More than kWarpCand of them
+  // in one warp (large logits next to each other): the same bound of the
+  // warp's 64 half lanes (every lane's largest at the even and at the odd
+  // places of its units); then the ties at the bound stay out, or, should that
+  // not do, the bound rises to the lowest that leaves at most that many.
+  // With RUNS (the bonus row) the chunks' sums are kept too.  The publishing
+  // warp merges the eight warps' results.
   //
   // Bound by issue (4.5 instructions a logit) and by the loads' latency: two
   // CTAs of eight independent warps an SM.  Against one pass by the whole
@@ -664,30 +730,46 @@ struct Eng {
         x[r][i] = (u < U) ? raw(b, r, u) : E::neg_inf();
       }
     float m[R];
-    unsigned key0 = 0u;   // order key of this lane's largest target logit
+    unsigned h0 = 0u, h1 = 0u;   // order keys of this lane's largest target logits at the units' even and odd places
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       uint4 mx = x[r][0];
 #pragma unroll
       for (int i = 1; i < NU; ++i) mx = E::max4(mx, x[r][i]);
-      const float lm = E::unit_max(mx);
-      const unsigned key = (lm > kNegInf) ? ord_key(__fadd_rn(lm, 0.f)) : 0u;
-      if (r == 0) key0 = key;
-      const unsigned km = __reduce_max_sync(FULLM, key);
+      const float2 lm = E::unit_max2(mx);
+      if (LIST && r == 0) {
+        h0 = lane_key(lm.x);
+        h1 = lane_key(lm.y);
+      }
+      const unsigned km = __reduce_max_sync(FULLM, lane_key(fmaxf(lm.x, lm.y)));
       m[r] = km ? ord_val(km) : kNegInf;
     }
     if constexpr (LIST) {
-      // theta: the kth-th largest lane maximum
-      unsigned km = __reduce_max_sync(FULLM, key0), rest = key0, last = km;
-      for (int t = 1; t < p.kth && km; ++t) {
-        const unsigned who = __ballot_sync(FULLM, rest == km);
-        if (lane == __ffs(who) - 1) rest = 0u;
-        km = __reduce_max_sync(FULLM, rest);
-        if (km) last = km;
+      // 16-bit logits differ in the upper half of their keys only
+      constexpr int kLow = DT == MDS_BF16 ? 16 : 0;
+      // the largest key that p.kth of the lanes' pairs reach (0: fewer have a logit)
+      auto kth_key = [&](unsigned k0, unsigned k1) {
+        const unsigned hi = __reduce_max_sync(FULLM, max(k0, k1)), lo = __reduce_min_sync(FULLM, min(k0, k1));
+        int bit = 31 - __clz(hi ^ lo);   // the keys share the bits above this one (-1: equal)
+        unsigned t = bit < 31 ? hi & (FULLM << max(bit + 1, kLow)) : 0u;
+#pragma unroll 1
+        for (; bit >= kLow; --bit) {
+          const unsigned c = t | (1u << bit);
+          if (__popc(__ballot_sync(FULLM, k0 >= c)) + __popc(__ballot_sync(FULLM, k1 >= c)) >= p.kth) t = c;
+        }
+        return t;
+      };
+      {
+        static_assert(kGroups == 8 && kCW * kGroups == 64, "four lanes a group, two groups a lane");
+        unsigned g = max(h0, h1);
+        g = max(g, __shfl_xor_sync(FULLM, g, 1));
+        g = max(g, __shfl_xor_sync(FULLM, g, 2));
+        if ((lane & 3) == 0) S.gmax[warp * kGroups + (lane >> 2)] = g;
       }
-      float theta = last ? ord_val(last) : kPosInf;
-      unsigned long long bits = 0ull;   // this lane's tokens at or above theta, VE to a unit
-      auto mark = [&]() {
+      cbar();   // the next slice's first barrier comes after this slice's reads
+      unsigned th = kth_key(S.gmax[lane], S.gmax[lane + 32]);
+      unsigned long long bits = 0ull;   // this lane's tokens that reach th, VE to a unit
+      auto mark = [&](float theta) {
         unsigned um = 0u;   // units that hold one
 #pragma unroll
         for (int i = 0; i < NU; ++i) um |= E::unit_max(x[0][i]) >= theta ? 1u << i : 0u;
@@ -701,15 +783,25 @@ struct Eng {
           for (int e = 0; e < VE; ++e) bb |= (v[e] >= theta && v[e] > kNegInf) ? 1u << e : 0u;
           bits |= (unsigned long long)bb << (i * VE);
         }
-        return __popcll(bits);
+        return (int)__reduce_add_sync(FULLM, (unsigned)__popcll(bits));
       };
-      int cnt = mark();
-      if (__reduce_add_sync(FULLM, (unsigned)cnt) > (unsigned)kWarpCand) {
+      int tot = mark(th ? ord_val(th) : kNegInf);
+      if (tot > kWarpCand) {
+        // large logits next to each other: the bound of this warp's half lanes
+        const unsigned own = kth_key(h0, h1);
+        if (own > th) {
+          th = own;
+          tot = mark(ord_val(th));
+        }
+        // ties at the bound (flat rows, rows masked with a finite value) stay out
+        if (tot > kWarpCand && th) tot = mark(ord_val(th + (1u << kLow)));
+      }
+      if (tot > kWarpCand) {
         // the largest key that more than kWarpCand tokens reach, and one up
-        unsigned t = 0u;
+        th = 0u;
 #pragma unroll 1
-        for (int bit = 31; bit >= 0; --bit) {
-          const unsigned cand = t | (1u << bit);
+        for (int bit = 31; bit >= kLow; --bit) {
+          const unsigned cand = th | (1u << bit);
           unsigned c = 0u;
 #pragma unroll 1
           for (int u = tid; u < U; u += kCT) {
@@ -718,15 +810,22 @@ struct Eng {
 #pragma unroll
             for (int e = 0; e < VE; ++e) c += (v[e] == v[e] && ord_key(__fadd_rn(v[e], 0.f)) >= cand) ? 1u : 0u;
           }
-          if (__reduce_add_sync(FULLM, c) > (unsigned)kWarpCand) t = cand;
+          if (__reduce_add_sync(FULLM, c) > (unsigned)kWarpCand) th = cand;
         }
-        theta = ord_val(t + 1u);
-        cnt = mark();
+        tot = mark(ord_val(th + (1u << kLow)));
       }
-      // set aside: into the slot, and out of the slice (-inf in every row;
-      // this thread's own units, read back into its registers)
-      if (cnt) {
-        int pos = atomicAdd(&T.ncand, cnt);
+      if (lane == 0) T.nc[warp] = tot;
+      // set aside: into the slot (lanes in order), and out of the slice (-inf
+      // in every row; this thread's own units, read back into its registers)
+      if (tot) {
+        const int cnt = __popcll(bits);
+        int pos = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int t = __shfl_up_sync(FULLM, pos, o);
+          if (lane >= o) pos += t;
+        }
+        pos += warp * kWarpCand - cnt;
         for (unsigned long long q = bits; q; q &= q - 1ull) {
           const int at = __ffsll((long long)q) - 1;
           const int loc = ((at / VE) * kCT + tid) * VE + at % VE;
@@ -1384,6 +1483,10 @@ struct Eng {
       s[r] = v;
     }
   }
+  // Order key of a lane's largest logit, 0 for none.
+  __device__ __forceinline__ static unsigned lane_key(float m) {
+    return m > kNegInf ? ord_key(__fadd_rn(m, 0.f)) : 0u;
+  }
   // Rank key of a token set aside: larger first.  A 16-bit logit's key needs
   // 16 bits, so the place in the slice (below 65536, smaller first) fits
   // beside it and the keys are distinct; 32-bit logits tie by place apart.
@@ -1393,52 +1496,79 @@ struct Eng {
   }
 
   // The slice's list: the first LN of the tokens set aside, by target logit
-  // (ties: smaller id), with every row's logit; the others rejoin the sums in
-  // rank order, tau covers them and every token not set aside.
+  // (ties: smaller id), with every row's logit; the others rejoin the sums,
+  // tau covers them and every token not set aside.  The tokens are numbered
+  // warp by warp; more than kRankMax of them are first cut to LN by their keys.
   __device__ void merge_list(Slot& T, float* rec, const float (&m)[kListRowsMax], float (&s)[kListRowsMax]) const {
     const int lane = threadIdx.x & 31;
-    const int LN = p.lns, n = T.ncand;
-    int* rid = reinterpret_cast<int*>(rec + kHdr);
+    const int LN = p.lns;
     float tau = (lane < kCW) ? T.tau[lane] : kNegInf;
-    // keys past n count for none
-    for (int i = n + lane; i < ((n + 3) & ~3); i += 32) T.key[i] = 0u;
-    __syncwarp();
-    const int tok0 = T.slice * p.T;
-    for (int i = lane; i < n; i += 32) {
-      const unsigned ki = T.key[i];
-      const int ii = tok0 + T.loc[i];
-      int rk = 0;
-      for (int q = 0; q < n; q += 4) {
-        const uint4 o = *reinterpret_cast<const uint4*>(T.key + q);
-        rk += (o.x > ki ? 1 : 0) + (o.y > ki ? 1 : 0) + (o.z > ki ? 1 : 0) + (o.w > ki ? 1 : 0);
-        if constexpr (DT != MDS_BF16) {
-          const int li = T.loc[i];
-          rk += (o.x == ki && q < n && T.loc[q] < li) ? 1 : 0;
-          rk += (o.y == ki && q + 1 < n && T.loc[q + 1] < li) ? 1 : 0;
-          rk += (o.z == ki && q + 2 < n && T.loc[q + 2] < li) ? 1 : 0;
-          rk += (o.w == ki && q + 3 < n && T.loc[q + 3] < li) ? 1 : 0;
-        }
-      }
-      if (rk < LN) {
-        __stcg(rid + rk, ii);
-#pragma unroll
-        for (int r = 0; r < kListRowsMax; ++r)
-          if (r < T.R) __stcg(rec + kHdr + LN * (1 + r) + rk, T.l[r][i]);
-      } else {
-        T.ord[rk - LN] = (unsigned short)i;
-      }
-    }
-    __syncwarp();
+    const Numbers num(T);
+    auto entry = [&](int j) { return num.entry(j); };
     float add[kListRowsMax];
 #pragma unroll
     for (int r = 0; r < kListRowsMax; ++r) add[r] = 0.f;
-    for (int t = lane; t < n - LN; t += 32) {
-      const int i = T.ord[t];
+    auto rejoin = [&](int i) {
       tau = fmaxf(tau, T.l[0][i]);
 #pragma unroll
       for (int r = 0; r < kListRowsMax; ++r)
         if (r < T.R && m[r] > kNegInf) add[r] = __fadd_rn(add[r], exp_term(T.l[r][i], m[r], T.c[r]));
+    };
+    int n = num.first[kCW];
+    if (n <= kRankMax) {
+#pragma unroll
+      for (int h = 0; h < kRankMax / 32; ++h) {
+        const int j = lane + 32 * h;
+        const int i = j < n ? entry(j) : 0;
+        T.sel[j] = j < n ? T.key[i] : 0u;
+        T.at[j] = (unsigned short)i;
+      }
+    } else {
+      const uint2 cut = list_cut<DT>(T, n, LN);
+      const unsigned thr = cut.x, last = cut.y;
+      int base = 0;
+#pragma unroll 1
+      for (int j0 = 0; j0 < n; j0 += 32) {
+        const int j = j0 + lane, i = j < n ? entry(j) : 0;
+        const unsigned key = j < n ? T.key[i] : 0u;
+        const bool take = j < n && (key > thr || (key == thr && T.loc[i] <= last));
+        const unsigned mk = __ballot_sync(FULLM, take);
+        if (take) {
+          const int at = base + __popc(mk & ((1u << lane) - 1u));
+          T.sel[at] = key;
+          T.at[at] = (unsigned short)i;
+        } else if (j < n) {
+          rejoin(i);
+        }
+        base += __popc(mk);
+      }
+      n = base;   // LN
+      T.sel[n + lane] = 0u;
     }
+    __syncwarp();
+    int* rid = reinterpret_cast<int*>(rec + kHdr);
+#pragma unroll 1
+    for (int j = lane; j < n; j += 32) {
+      const unsigned kj = T.sel[j];
+      const int i = T.at[j], place = T.loc[i];
+      int rk = 0;
+#pragma unroll 4
+      for (int q = 0; q < n; q += 4) {
+        const uint4 o = *reinterpret_cast<const uint4*>(T.sel + q);
+        rk += (o.x > kj ? 1 : 0) + (o.y > kj ? 1 : 0) + (o.z > kj ? 1 : 0) + (o.w > kj ? 1 : 0);
+      }
+      if constexpr (DT != MDS_BF16)
+        for (int q = 0; q < n; ++q) rk += (T.sel[q] == kj && T.loc[T.at[q]] < place) ? 1 : 0;
+      if (rk < LN) {
+        __stcg(rid + rk, T.slice * p.T + place);
+#pragma unroll
+        for (int r = 0; r < kListRowsMax; ++r)
+          if (r < T.R) __stcg(rec + kHdr + LN * (1 + r) + rk, T.l[r][i]);
+      } else {
+        rejoin(i);
+      }
+    }
+    __syncwarp();
     tau = warp_max(tau);
 #pragma unroll
     for (int r = 0; r < kListRowsMax; ++r)
@@ -1502,7 +1632,6 @@ struct Eng {
       const int count = T.count;
       __syncwarp();
       if (lane == 0) {
-        T.ncand = 0;
         mbar_arrive(&S.free[k % kSlots]);
         // the group's records before the count (release; the last one also acquires the others')
         if (count && atom_add_acq_rel(&p.cnt[b], (unsigned)count) == (unsigned)(p.ns - count))
@@ -3215,7 +3344,6 @@ __global__ void __launch_bounds__(kBlock, kCtasPerSm) flow_kernel(const __grid_c
     for (int i = 0; i < kSlots; ++i) {
       mbar_init(&S.done[i], kCW);
       mbar_init(&S.free[i], 1);
-      e.slots[i].ncand = 0;
     }
     S.issued = 0;
     S.consumed = 0;
@@ -3430,11 +3558,11 @@ bool plan_geometry(Params& p, int grid) {
     if ((size_t)ns * p.rec_floats * 4 <= (size_t)kDecStage && ns * p.lns <= kMaxEntries) break;
   }
   // Warp-wise candidate lists where every thread has a unit and the slice's
-  // list is short: each warp sets aside at least half as many tokens as the
-  // list holds, four times its even share, so a needed token is left
-  // out (which only shortens the certified list) about once in 10^6 warps.
-  p.fast_list = (list && p.T * es / 16 >= kCT && p.lns <= kWarpCand) ? 1 : 0;
-  p.kth = p.lns / 2;
+  // list is short.  Each warp's bound is one that as many of its tokens reach
+  // as the slice's list holds, so the list is the slice's largest tokens
+  // wherever they lie (up to ties at the bound).
+  p.fast_list = (list && p.T * es / 16 >= kCT && p.lns <= kSliceListMax) ? 1 : 0;
+  p.kth = p.lns;
   // Slices per task: the scheduler's round trips for one task (claim, ring
   // word, descriptor: about 2 us) are shared by a group of slices where there
   // are many tasks per CTA; one slice a task where a pass's slices should
