@@ -266,7 +266,7 @@ int flow_verify(mds_ctx* ctx, const void* target_logits, const void* const* draf
     ctx->f_cap = p.ring_cap;
   }
   mds::flow_buffers(p, target_logits, draft_logits, draft_tokens, temperatures, out_tokens, out_accept_len, out_diag,
-                    B, philox_seed);
+                    ctx->f_grid, B, philox_seed);
   p.status = ctx->work;
   p.dbg_rows = ctx->dbg_rows;
   ctx->epoch = (ctx->epoch + 1u == 0u) ? 1u : ctx->epoch + 1u;
@@ -585,7 +585,8 @@ bool flow_params(const mds_config& c, int grid, int scheme, const int8_t* model_
 
 void flow_buffers(flow::Params& p, const void* target_logits, const void* const* draft_logits,
                   const int32_t* draft_tokens, const float* temperatures, int32_t* out_tokens,
-                  int32_t* out_accept_len, float* out_diag, int B, uint64_t seed) {
+                  int32_t* out_accept_len, float* out_diag, int grid, int B, uint64_t seed) {
+  flow::plan_tasks(p, grid, B);
   p.target = static_cast<const char*>(target_logits);
   for (int k = 0; k < p.K; ++k) p.drafts[k] = static_cast<const char*>(draft_logits[k]);
   p.tokens = draft_tokens;
@@ -593,7 +594,6 @@ void flow_buffers(flow::Params& p, const void* target_logits, const void* const*
   p.out_tokens = out_tokens;
   p.out_accept = out_accept_len;
   p.out_diag = out_diag;
-  p.B = B;
   p.seed = seed;
 }
 }  // namespace mds

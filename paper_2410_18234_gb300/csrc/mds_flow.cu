@@ -3427,7 +3427,7 @@ struct Layout {
 };
 Layout layout(const Params& p, int nseq, int grid) {
   Layout L;
-  L.cap = (size_t)nseq * p.ng + (size_t)grid + 64;
+  L.cap = (size_t)nseq * p.ng + (size_t)grid + 64;   // every sequence's tasks of one pass, plus the claims
   L.dcap = (size_t)nseq + (size_t)grid * kDecWarps + 64;   // one request per sequence, plus the claims
   L.ctl = kCtlWords * 4;
   L.tag = up256(L.cap * 8);
@@ -3563,17 +3563,24 @@ bool plan_geometry(Params& p, int grid) {
   // wherever they lie (up to ties at the bound).
   p.fast_list = (list && p.T * es / 16 >= kCT && p.lns <= kSliceListMax) ? 1 : 0;
   p.kth = p.lns;
-  // Slices per task: the scheduler's round trips for one task (claim, ring
-  // word, descriptor: about 2 us) are shared by a group of slices where there
-  // are many tasks per CTA; one slice a task where a pass's slices should
-  // spread over the GPU.
-  const long per_cta = (long)p.B * p.ns / grid;
+  p.group = p.group0 = 1;
+  p.ng = p.ng0 = p.ns;
+  p.dec_sms = decision_sms(grid, p.scheme);
+  return p.dec_sms > 0;
+}
+
+// Slices per task: the scheduler's round trips for one task (claim, ring
+// word, descriptor: about 2 us) are shared by a group of slices where there
+// are many tasks per CTA; one slice a task where a pass's slices should
+// spread over the GPU.  By the call's own batch: by the context's largest, a
+// small call's slices went to a few CTAs one after the other.
+void plan_tasks(Params& p, int grid, int B) {
+  const long per_cta = (long)B * p.ns / grid;
   p.group = per_cta >= 32 ? 4 : (per_cta >= 16 ? 2 : 1);
   p.group0 = per_cta >= 8 ? 4 : (per_cta >= 4 ? 2 : 1);   // depth 0: every sequence's slices at once
   p.ng = (p.ns + p.group - 1) / p.group;
   p.ng0 = (p.ns + p.group0 - 1) / p.group0;
-  p.dec_sms = decision_sms(grid, p.scheme);
-  return p.dec_sms > 0;
+  p.B = B;
 }
 
 // Every token's probability under given row statistics, by prob_of.

@@ -58,7 +58,7 @@ struct Params {
   int lns;                             // candidate list length of one slice (<= ln)
   unsigned lns_rcp;                    // ceil(2^32 / lns): entry / lns by a high product
   int fast_list;                       // the slices' lists are found warp by warp
-  int kth;                             // ... each warp's threshold: its kth largest lane maximum
+  int kth;                             // ... and reach the kth largest of the slice's group maxima
   int group, group0;                   // slices per task (group0: of the depth-0 passes)
   int ng, ng0;                         // tasks per pass
   int rec_floats;                      // record stride per slice
@@ -76,6 +76,10 @@ struct Params {
 // false if the configuration is outside what this engine serves (the caller
 // then uses the per-sequence engine).
 bool plan_geometry(Params& p, int grid);
+
+// The tasks of a call of B sequences (p after plan_geometry, which counts one
+// task a slice, the most a workspace's rings need).
+void plan_tasks(Params& p, int grid, int B);
 
 // Bytes of per-sequence state, for the workspace.
 size_t seq_bytes();

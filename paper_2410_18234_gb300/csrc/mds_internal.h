@@ -88,6 +88,6 @@ bool flow_params(const mds_config& c, int grid, int scheme, const int8_t* model_
                  bool aligned16, flow::Params& p, bool always = false);
 void flow_buffers(flow::Params& p, const void* target_logits, const void* const* draft_logits,
                   const int32_t* draft_tokens, const float* temperatures, int32_t* out_tokens,
-                  int32_t* out_accept_len, float* out_diag, int B, uint64_t seed);
+                  int32_t* out_accept_len, float* out_diag, int grid, int B, uint64_t seed);
 
 }  // namespace mds

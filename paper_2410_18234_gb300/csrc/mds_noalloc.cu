@@ -133,13 +133,13 @@ extern "C" int mds_verify_noalloc(const mds_config* cfg_in, int device, const vo
     // the dataflow engine where mds_verify takes it (same geometry: same results)
     mds::flow::Params fp{};
     if (mds::flow_params(c, grid, scheme, p.model_of, n_models, true, tma_ok, fp)) {
+      mds::flow_buffers(fp, target_logits, draft_logits, draft_tokens, temperatures, out_tokens, out_accept_len,
+                        out_diag, grid, B, philox_seed);
       const size_t need = mds::flow::workspace_bytes(fp, B, grid);
       if (kHead + need > MDS_NOALLOC_SCRATCH_BYTES) {
         rc = MDS_ESHAPE;
       } else {
         mds::flow::carve_workspace(fp, reinterpret_cast<char*>(scratch + kHead), B, grid);
-        mds::flow_buffers(fp, target_logits, draft_logits, draft_tokens, temperatures, out_tokens, out_accept_len,
-                          out_diag, B, philox_seed);
         fp.status = reinterpret_cast<unsigned*>(scratch);
         fp.epoch = next_epoch(device);
         cudaError_t e = cudaMemsetAsync(scratch, 0, kHead, st);

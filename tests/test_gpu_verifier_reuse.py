@@ -47,3 +47,27 @@ def test_calls_of_other_layouts(B, V):
         seen = torch.arange(3, device=DEV)[None] <= want[1][:, None]
         assert torch.equal(got[2][seen], want[2][seen]), (scheme, models)
     one.close()
+
+
+@pytest.mark.parametrize("scheme", ["single", "WIS", "WIS0"])
+def test_small_calls_on_a_large_context(scheme):
+    """Tasks are grouped by the call's batch, slices by the context's: a call
+    of a batch's first sequences gives their results, bit for bit."""
+    B, V = 400, 100000
+    w = workload(B, V, 1)
+    v = mds.Verifier(B, 2, 2, V)
+
+    def call(n):
+        out = v.verify(w.target[:n], [d[:n] for d in w.draft_list()], w.model_ids, w.tokens[:n], w.temps[:n], scheme, 9,
+                       diag=True)
+        torch.cuda.synchronize()
+        assert v.status()[0] & ~mds.MDS_ST_OMEGA0 == 0
+        return out
+
+    want = call(B)
+    for n in (1, 5, 64, 150, B):
+        got = call(n)
+        seen = torch.arange(3, device=DEV)[None] <= want[1][:n, None]
+        assert torch.equal(got[0], want[0][:n]) and torch.equal(got[1], want[1][:n]), n
+        assert torch.equal(got[2][seen], want[2][:n][seen]), n
+    v.close()
