@@ -234,7 +234,7 @@ int flow_verify(mds_ctx* ctx, const void* target_logits, const void* const* draf
                 void* stream, bool bulk_ok, bool aligned16) {
   const mds_config& c = ctx->cfg;
   mds::flow::Params p{};
-  // an export of row statistics wants the engine that writes them
+  // an export of row statistics keeps to this engine wherever it serves the call
   if (!mds::flow_params(c, ctx->f_grid, scheme, model_of, n_models, bulk_ok, aligned16, p, ctx->dbg_rows != nullptr))
     return mds::kNotServed;
   const size_t total = mds::flow::workspace_bytes(p, c.max_B, ctx->f_grid);
@@ -337,6 +337,7 @@ static int verify_impl(mds_ctx* ctx, const void* target_logits, const void* cons
   p.out_diag = out_diag;
   p.status = ctx->work;
   p.queue = ctx->work + 1;
+  p.dbg_rows = ctx->dbg_rows;
   p.dbg_exps = ctx->dbg_exps;
   p.seed = philox_seed;
   p.B = B;

@@ -43,6 +43,7 @@ struct Params {
   int tma_ok;                          // rows are 16-byte aligned with a 16-byte-multiple length
   int cand_cap;                        // WIS candidate list capacity (kListN; 0: no candidate path)
   int cand_stage;                      // WIS staging capacity (every CTA's list: cn * kListN)
+  float* dbg_rows;                     // [B][L+1][MDS_DEBUG_ROWS][4] row statistics (test export), or null
   unsigned long long* dbg_exps;        // IS: quadrature exponentials evaluated (test export), or null
   int8_t model_of[MDS_MAX_K];          // remapped model id per branch
 };

@@ -277,8 +277,8 @@ DEBUG_ROWS = 4   # MDS_DEBUG_ROWS
 
 
 def mds_debug_row_stats(ctx, row_stats):
-    """Have the context's later dataflow-engine calls write every visited
-    row's statistics into row_stats (float32 CUDA tensor [max_B][L+1][4][4]:
+    """Have the context's later calls (top_k = 0) write every visited row's
+    statistics into row_stats (float32 CUDA tensor [max_B][L+1][4][4]:
     M, 1/Z, c, source), or stop with None.  Test export."""
     ptr = None if row_stats is None else ctypes.c_void_p(row_stats.data_ptr())
     rc = _lib.mds_debug_row_stats(ctx, ptr)
