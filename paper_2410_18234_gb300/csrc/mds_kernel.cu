@@ -406,6 +406,20 @@ struct GlobalLoad {
   __device__ __forceinline__ void operator()(int r, float* v) const { Elt<DT>::unpack(raw(r), v); }
 };
 
+// Test export: the statistics of a depth's rows (M, 1/Z, c, source: the target
+// row's branch, or 100 + the branch whose draft row it is) to o[r][4].
+__device__ __noinline__ void debug_rows(const State& S, float* o, int rows, unsigned valid) {
+  const int r = (int)threadIdx.x;
+  if (r >= rows || r >= MDS_DEBUG_ROWS) return;
+  int src = __ffs(valid) - 1;
+  for (int i = S.nv - 1; r > 0 && i >= 0; --i)
+    if (S.vrow[i] == r) src = 100 + S.vbr[i];
+  o[4 * r] = S.M[r];
+  o[4 * r + 1] = S.invZ[r];
+  o[4 * r + 2] = S.c[r];
+  o[4 * r + 3] = (float)src;
+}
+
 template <int DT, int SCHEME>
 struct Kernel {
   using E = Elt<DT>;
@@ -2508,7 +2522,9 @@ struct Kernel {
       __syncthreads();
       if (!bonus) {
         depth_stats((SCHEME == MDS_WIS && S.nv > 1) || SCHEME == MDS_WIS0);
-        if (p.dbg_rows) debug_rows(b, j, SCHEME == MDS_WIS0 && p.cand_cap > 0 ? 1 : S.nrows, valid);
+        if (p.dbg_rows && rank == 0)
+          debug_rows(S, p.dbg_rows + ((size_t)b * (L + 1) + j) * MDS_DEBUG_ROWS * 4,
+                     SCHEME == MDS_WIS0 && p.cand_cap > 0 ? 1 : S.nrows, valid);
       }
       int Z;
       float qY = 0.f, pIY = 0.f, Rdiag = 0.f;
@@ -2517,7 +2533,8 @@ struct Kernel {
         float tot;
         Z = bonus_pass(draw_uniform(p.seed, b, j, kDrawBonus), &tot);
         Rdiag = tot;
-        if (p.dbg_rows) debug_rows(b, j, 1, valid);
+        if (p.dbg_rows && rank == 0)
+          debug_rows(S, p.dbg_rows + ((size_t)b * (L + 1) + j) * MDS_DEBUG_ROWS * 4, 1, valid);
       } else if constexpr (SCHEME == MDS_SPECTR) {
         Z = spectr(b, j, &qY, &pIY, &Ydiag, &Rdiag);
       } else if constexpr (SCHEME == MDS_WIS0) {
@@ -2637,21 +2654,6 @@ struct Kernel {
         for (int j = acc_len + 1; j <= L; ++j) p.out_tokens[(size_t)b * (L + 1) + j] = -1;
       }
     }
-  }
-
-  // Test export: the statistics of the depth's rows (M, 1/Z, c, source: the
-  // target row's branch, or 100 + the branch whose draft row it is).
-  __device__ __noinline__ void debug_rows(int b, int j, int rows, unsigned valid) const {
-    const int r = (int)threadIdx.x;
-    if (rank != 0 || r >= rows || r >= MDS_DEBUG_ROWS) return;
-    int src = __ffs(valid) - 1;
-    for (int i = S.nv - 1; r > 0 && i >= 0; --i)
-      if (S.vrow[i] == r) src = 100 + S.vbr[i];
-    float* o = p.dbg_rows + (((size_t)b * (p.L + 1) + j) * MDS_DEBUG_ROWS + r) * 4;
-    o[0] = S.M[r];
-    o[1] = S.invZ[r];
-    o[2] = S.c[r];
-    o[3] = (float)src;
   }
 
   // Outputs of a sequence the launch gives up on: accept length -1, every
