@@ -271,9 +271,29 @@ __device__ __forceinline__ float prob_of(float l, float M, float c, float invZ) 
 }
 // Unnormalised term of a logit against reference m (the row or slice maximum).
 __device__ __forceinline__ float exp_term(float l, float m, float c) { return ex2(__fmaf_rn(l, c, -__fmul_rn(m, c))); }
+// 2^x, x <= 0, to about one unit in the last place (0 below 2^-126): the
+// Taylor series of 2^f, |f| <= 1/2, whose eighth power is below 6e-9.
+__device__ __forceinline__ float exp2_near(float x) {
+  constexpr float l = 0.6931471805599453f;
+  const float n = rintf(x), f = __fmul_rn(__fsub_rn(x, n), l);
+  float y = 1.f / 5040.f;
+  y = __fmaf_rn(y, f, 1.f / 720.f);
+  y = __fmaf_rn(y, f, 1.f / 120.f);
+  y = __fmaf_rn(y, f, 1.f / 24.f);
+  y = __fmaf_rn(y, f, 1.f / 6.f);
+  y = __fmaf_rn(y, f, 0.5f);
+  y = __fmaf_rn(y, f, 1.f);
+  y = __fmaf_rn(y, f, 1.f);
+  return x < -126.f ? 0.f : __fmul_rn(y, __uint_as_float((unsigned)((int)n + 127) << 23));
+}
 // Factor that moves a sum from reference m to reference M >= m.
 __device__ __forceinline__ float ref_shift(float m, float M, float c) {
   return ex2(__fsub_rn(__fmul_rn(m, c), __fmul_rn(M, c)));
+}
+// The same for the sums of whole warps, CTAs or slices: few of them make a
+// row's sum, so the error of a factor does not average out as a term's does.
+__device__ __forceinline__ float ref_shift_near(float m, float M, float c) {
+  return exp2_near(__fsub_rn(__fmul_rn(m, c), __fmul_rn(M, c)));
 }
 
 // The reference of a partial sum whose largest logit is m: -inf (no
@@ -288,6 +308,10 @@ __device__ __forceinline__ float ref_exp(float m, float c) { return m > kNegInf 
 // is 0 or NaN and stays).
 __device__ __forceinline__ float moved_sum(float s, float m, float M, float c) {
   return m > kNegInf ? __fmul_rn(s, ref_shift(m, M, c)) : s;
+}
+
+__device__ __forceinline__ float moved_sum_near(float s, float m, float M, float c) {
+  return m > kNegInf ? __fmul_rn(s, ref_shift_near(m, M, c)) : s;
 }
 
 // Combine two (max, sum) pairs of one row.

@@ -2120,7 +2120,7 @@ struct Dec {
       const float c = D.P.row[r].c;
       float z = 0.f;
       for (int sl = lane; sl < ns; sl += 32) {
-        z = __fadd_rn(z, moved_sum(sr[sl * rf + 2 * r + 1], sr[sl * rf + 2 * r], M, c));
+        z = __fadd_rn(z, moved_sum_near(sr[sl * rf + 2 * r + 1], sr[sl * rf + 2 * r], M, c));
       }
       z = warp_sum(z);
       if (lane == 0) {

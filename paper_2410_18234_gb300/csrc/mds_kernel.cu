@@ -909,14 +909,10 @@ struct Kernel {
     for (int r = 0; r < R; ++r) {
       float mm = m[r], ss = sc[r];
       if (CAND && lane == 0) combine_ms(mm, ss, pm[r], ps[r], cr[r]);
-#pragma unroll
-      for (int o = 16; o; o >>= 1) {
-        const float m2 = __shfl_xor_sync(0xffffffffu, mm, o);
-        const float s2 = __shfl_xor_sync(0xffffffffu, ss, o);
-        combine_ms(mm, ss, m2, s2, cr[r]);
-      }
+      const float wm = dev::warp_max(mm);
+      ss = warp_sum(dev::moved_sum(ss, mm, wm, cr[r]));
       if (lane == 0) {
-        S.red[(warp * kMaxRows + r) * 2] = mm;
+        S.red[(warp * kMaxRows + r) * 2] = wm;
         S.red[(warp * kMaxRows + r) * 2 + 1] = ss;
       }
     }
@@ -927,13 +923,25 @@ struct Kernel {
     __syncthreads();
     constexpr int nx = CAND ? 3 * R + 2 : 2 * R;
     constexpr int sx = CAND ? 3 : 2;   // exchange stride per row: max, complement sum[, list sum]
-    if (threadIdx.x < R) {
-      const int r = threadIdx.x;
-      float mm = kNegInf, ss = 0.f;
-      for (int w = 0; w < kWarps; ++w)
-        combine_ms(mm, ss, S.red[(w * kMaxRows + r) * 2], S.red[(w * kMaxRows + r) * 2 + 1], cr[r]);
-      S.xch[xbuf][sx * r] = mm;
-      S.xch[xbuf][sx * r + 1] = ss;
+    if (warp == 0) {
+      // eight lanes a row, one warp's sums each: every part is moved once and
+      // the sum is a tree, here and over the cluster (moved and added one
+      // after the other, the last few roundings were most of 1/Z's error)
+      static_assert(kWarps == 8 && R <= 4, "eight lanes a row");
+      const int r = lane >> 3, w = lane & 7;
+      const bool on = r < R;
+      const float mw = on ? S.red[(w * kMaxRows + r) * 2] : kNegInf;
+      const float c = S.c[r0 + (on ? r : 0)];
+      float mm = mw;
+#pragma unroll
+      for (int o = 4; o; o >>= 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, o));
+      float ss = on ? dev::moved_sum_near(S.red[(w * kMaxRows + r) * 2 + 1], mw, mm, c) : 0.f;
+#pragma unroll
+      for (int o = 4; o; o >>= 1) ss = __fadd_rn(ss, __shfl_xor_sync(0xffffffffu, ss, o));
+      if (on && w == 0) {
+        S.xch[xbuf][sx * r] = mm;
+        S.xch[xbuf][sx * r + 1] = ss;
+      }
     }
     if constexpr (CAND) {
       __syncthreads();
@@ -1017,27 +1025,27 @@ struct Kernel {
       }
     }
     cluster_gather(S, nx, xbuf, cn);   // also publishes cl_* to the cluster
-    // every CTA: M, Z and the complement sum of each row (rank order)
-    if (threadIdx.x < R) {
-      const int r = threadIdx.x;
-      float mm = kNegInf;
-      for (int q = 0; q < cn; ++q) mm = fmaxf(mm, S.gat[q * nx + sx * r]);
-      float ss = 0.f, zz = 0.f;
-      if (mm > kNegInf)
-        for (int q = 0; q < cn; ++q) {
-          const float mq = S.gat[q * nx + sx * r];
-          const float f = mq > kNegInf ? dev::ref_shift(mq, mm, cr[r]) : 1.f;   // without a reference: sums of 0, or NaN
-          const float sq = S.gat[q * nx + sx * r + 1];
-          ss = __fadd_rn(ss, __fmul_rn(sq, f));
-          zz = __fadd_rn(zz, __fmul_rn(CAND ? __fadd_rn(sq, S.gat[q * nx + sx * r + 2]) : sq, f));
+    // every CTA: M, Z and the complement sum of each row, a warp a row
+    if (warp < R) {
+      static_assert(kMaxCluster <= 32, "one lane a CTA");
+      const int r = warp;
+      const float c = S.c[r0 + r];
+      const bool on = lane < cn;
+      const float mq = on ? S.gat[lane * nx + sx * r] : kNegInf, sq = on ? S.gat[lane * nx + sx * r + 1] : 0.f;
+      float mm = dev::warp_max(mq);
+      const float f = mq > kNegInf ? dev::ref_shift_near(mq, mm, c) : 1.f;   // without a reference: sums of 0, or NaN
+      const float ss = warp_sum(__fmul_rn(sq, f));
+      float zz = ss;
+      if constexpr (CAND) zz = warp_sum(__fmul_rn(on ? __fadd_rn(sq, S.gat[lane * nx + sx * r + 2]) : 0.f, f));
+      if (lane == 0) {
+        if (!(mm > kNegInf) || mm != mm) {
+          atomicOr(p.status, MDS_ST_NONFINITE);
+          mm = 0.f;
         }
-      if (!(mm > kNegInf) || mm != mm) {
-        atomicOr(p.status, MDS_ST_NONFINITE);
-        mm = 0.f;
+        S.M[r0 + r] = mm;
+        S.pc[r0 + r] = ss;
+        finish_row(r0 + r, zz);
       }
-      S.M[r0 + r] = mm;
-      S.pc[r0 + r] = ss;
-      finish_row(r0 + r, zz);
     }
     if constexpr (!CAND) {
       if (threadIdx.x == 0) S.ncand = -1;

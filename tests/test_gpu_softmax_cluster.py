@@ -66,3 +66,33 @@ def test_softmax_rows_match_oracle(name, kw, cluster):
     mds.mds_debug_row_stats(v.ctx, None)
     assert v.status()[0] == 0
     v.close()
+
+
+@pytest.mark.parametrize("V,cluster,scale", [(4096, 16, 3.0), (32003, 8, 4.0)])
+def test_normaliser_error(V, cluster, scale):
+    """1/Z against 64 bits over 640 rows: as near as the dataflow engine's on
+    the same rows (root mean squares within 15%; both are a few tenths of a
+    unit in the last place, set by the last few additions)."""
+    rms = {}
+    for cl in (0, cluster):
+        err = []
+        for seed in range(20):
+            g = torch.Generator(device="cuda:0").manual_seed(seed)
+            target = torch.randn(16, 1, 2, V, generator=g, device="cuda:0") * scale
+            draft = target[:, 0, :1] + torch.randn(16, 1, V, generator=g, device="cuda:0")
+            tokens = torch.randint(V, (16, 1, 1), generator=g, device="cuda:0", dtype=torch.int32)
+            v = mds.Verifier(16, 1, 1, V, dtype="f32", cluster=cl)
+            stats = torch.empty(16, 2, mds.DEBUG_ROWS, 4, device="cuda:0")
+            mds.mds_debug_row_stats(v.ctx, stats)
+            v.verify(target, [draft], [0], tokens, torch.ones(16, 2, device="cuda:0"), "single", 1)
+            torch.cuda.synchronize()
+            assert v.cluster_size == cl
+            v.close()
+            st = stats.double().cpu().numpy()
+            for r, rows in ((0, target[:, 0, 0]), (1, draft[:, 0])):
+                want = torch.softmax(rows.double(), 1).amax(1).cpu().numpy()
+                mc = st[:, 0, r, 0] * st[:, 0, r, 2]   # the largest token's exponent is mc - round(mc)
+                got = st[:, 0, r, 1] * np.exp2(mc - mc.astype(np.float32).astype(np.float64))
+                err.append(got / want - 1.0)
+        rms[cl] = float(np.sqrt(np.mean(np.square(err))))
+    assert rms[cluster] <= 1.15 * rms[0], rms
