@@ -258,9 +258,9 @@ struct State {
   int sp_rows[MDS_MAX_K];
   // IS: quadrature grid, bins of log2 rho (kIsSub to the octave) and the
   // moments of one window of them (one copy for the peers, one combined)
-  int is_mlo, is_n, is_b0, is_nb;
-  int is_cnt[kMaxRows];
-  float is_lz[kMaxRows];        // log2(Z_r / Z_0)
+  int is_mlo, is_n, is_nb;
+  int is_cnt[kMaxRows], is_b0[kMaxRows];
+  float is_rat[kMaxRows];       // Z_r / Z_0
   float is_mom[kIsWin * kIsMom + 1], is_sum[kIsWin * kIsMom + 1];
   float is_ctr[kIsWin];         // the bins' centres
   int is_tab;                   // the residual reads the bins' Taylor coefficients
@@ -1856,14 +1856,17 @@ struct Kernel {
       z[k + 1] = __fmul_rn(__fmul_rn(t, s), -d / (float)(k + 1));
     }
   }
-  // Centre of bin n (the octave's power of two is exact).
-  __device__ __forceinline__ static float is_centre(int n) {
+  // Ratio rho at the centre of row r's bin n (the octave's power of two is
+  // exact): 2^(n / kIsSub) before the rows' normalisers, whose ratio is one
+  // rounding (as a term of every token's logarithm it was two of a larger
+  // number's).
+  __device__ __forceinline__ float is_centre(int r, int n) const {
     const int o = (n >= 0) ? n / kIsSub : -((kIsSub - 1 - n) / kIsSub);
-    return ldexpf(ex2((float)(n - o * kIsSub) / kIsSub), o);
+    return __fmul_rn(ldexpf(ex2((float)(n - o * kIsSub) / kIsSub), o), S.is_rat[r]);
   }
-  // log2 rho of a token in bins, from the exponents of its probabilities.
-  __device__ __forceinline__ static float is_pos(float aq, float ap, float lz) {
-    return __fmul_rn(__fadd_rn(__fsub_rn(aq, ap), lz), (float)kIsSub);
+  // A token's place in bins, from the exponents of its probabilities.
+  __device__ __forceinline__ static float is_pos(float aq, float ap) {
+    return __fmul_rn(__fsub_rn(aq, ap), (float)kIsSub);
   }
 
   // Add this warp's set-aside tokens (v, v^2, p, bin) to its bins.
@@ -1899,7 +1902,6 @@ struct Kernel {
     __syncwarp();
     float zero = 0.f;
     const RowC c0 = row_c(0), cr = row_c(r);
-    const float lz = S.is_lz[r];
     stream_rows<2, 1>({0, r}, [&](int, bool valid, const auto& L) {
       float lq[VE], lp[VE];
       if (valid) {
@@ -1916,7 +1918,7 @@ struct Kernel {
         for (int e = e0; e < e0 + 2; ++e) {
           const float aq = c0.arg(lq[e]), ap = cr.arg(lp[e]);
           const float pr = __fmul_rn(ex2(ap), cr.iz), q = __fmul_rn(ex2(aq), c0.iz);
-          const float x = is_pos(aq, ap, lz);
+          const float x = is_pos(aq, ap);
           const float n = rintf(x);
           const int bin = (int)n - b0;
           const bool pos = pr > 0.f && q > 0.f;
@@ -1940,22 +1942,27 @@ struct Kernel {
     if (lane == 0) S.red[warp] = zero;
     __syncthreads();
     {
-      // one (bin, moment) per thread: warps and copies in order
+      // one (bin, moment) per thread: a tree over the warps and copies
       static_assert(kIsWin * kIsMom == kThreads, "one bin moment per thread");
       const int n = tid / kIsMom, k = tid % kIsMom;
-      float t = 0.f;
-      for (int w = 0; w < kWarps; ++w)
+      float t[kWarps];
 #pragma unroll
-        for (int c = 0; c < 4; ++c)
-          t = __fadd_rn(t, isBin[((w * kIsWin + n) * 4 + c) * kIsMom + k]);
-      S.is_mom[tid] = t;
+      for (int w = 0; w < kWarps; ++w) {
+        const float* c = isBin + (size_t)(w * kIsWin + n) * 4 * kIsMom + k;
+        t[w] = __fadd_rn(__fadd_rn(c[0], c[kIsMom]), __fadd_rn(c[2 * kIsMom], c[3 * kIsMom]));
+      }
+#pragma unroll
+      for (int o = kWarps / 2; o; o >>= 1)
+#pragma unroll
+        for (int w = 0; w < o; ++w) t[w] = __fadd_rn(t[w], t[w + o]);
+      S.is_mom[tid] = t[0];
       if (tid == 0) {
         float z = 0.f;
         for (int w = 0; w < kWarps; ++w) z = __fadd_rn(z, S.red[w]);
         S.is_mom[kThreads] = z;
       }
     }
-    if (tid < kIsWin) S.is_ctr[tid] = is_centre(b0 + tid);
+    if (tid < kIsWin) S.is_ctr[tid] = is_centre(r, b0 + tid);
     __syncthreads();
     if (cn > 1) {
       cluster_sync_all();
@@ -1977,7 +1984,7 @@ struct Kernel {
     if (tid == 0) {
       for (int r = 0; r < kMaxRows; ++r) S.is_cnt[r] = 0;
       for (int i = 0; i < S.nv; ++i) S.is_cnt[S.vrow[i]]++;
-      for (int r = 1; r < S.nrows; ++r) S.is_lz[r] = __fsub_rn(log2f(S.invZ[0]), log2f(S.invZ[r]));
+      for (int r = 1; r < S.nrows; ++r) S.is_rat[r] = __fdiv_rn(S.invZ[0], S.invZ[r]);
     }
     __syncthreads();
     // range of rho = q / p_r over tokens with q > 0 and p_r > 0, a row at a time
@@ -2003,8 +2010,9 @@ struct Kernel {
         }
       });
       if (dlo <= dhi) {
-        lo = fminf(lo, exp2f(__fadd_rn(dlo, S.is_lz[r])));
-        hi = fmaxf(hi, exp2f(__fadd_rn(dhi, S.is_lz[r])));
+        const float lz = log2f(S.is_rat[r]);
+        lo = fminf(lo, exp2f(__fadd_rn(dlo, lz)));
+        hi = fmaxf(hi, exp2f(__fadd_rn(dhi, lz)));
       }
     }
 #pragma unroll
@@ -2043,13 +2051,11 @@ struct Kernel {
       S.is_mlo = mlo;
       S.is_n = mhi - mlo + 1;
       // the bins of that range, a bin to spare on either side (no bins
-      // without a token of positive q and p)
-      S.is_b0 = 0;
+      // without a token of positive q and p); every row's from its own on
       S.is_nb = 0;
-      if (rlo <= rhi) {
-        S.is_b0 = (int)floorf(kIsSub * log2f(rlo)) - 1;
-        S.is_nb = (int)ceilf(kIsSub * log2f(rhi)) + 2 - S.is_b0;
-      }
+      if (rlo <= rhi) S.is_nb = (int)ceilf(kIsSub * (log2f(rhi) - log2f(rlo))) + 4;
+      for (int r = 1; r < S.nrows; ++r)
+        S.is_b0[r] = (int)floorf(kIsSub * (log2f(rlo) - log2f(S.is_rat[r]))) - 1;
       int rows = 0;
       for (int r = 1; r < S.nrows; ++r) rows += S.is_cnt[r] ? 1 : 0;
       S.is_tab = (rows * S.is_nb <= kIsTabBins) ? 1 : 0;
@@ -2070,9 +2076,14 @@ struct Kernel {
     for (int r = 1; r < S.nrows; ++r) {
       if (!S.is_cnt[r]) continue;
       for (int b = 0; b < S.is_nb || b == 0; b += kIsWin) {
-        is_moments(r, S.is_b0 + b, b == 0);
+        is_moments(r, S.is_b0[r] + b, b == 0);
         for (int n = tid; n < nn; n += kThreads) {
-          float acc = (b == 0) ? S.is_sum[kThreads] : isW[r * kIsNodesMax + n];
+          float acc = (b == 0) ? S.is_sum[kThreads] : isW[r * kIsNodesMax + n], comp = 0.f;   // compensated
+          auto add = [&](float m) {
+            const float y = __fsub_rn(m, comp), s = __fadd_rn(acc, y);
+            comp = __fsub_rn(__fsub_rn(s, acc), y);
+            acc = s;
+          };
           const float t = isT[n];
           for (int i = 0; i < kIsWin; ++i) {
             const float* A = S.is_sum + i * kIsMom;
@@ -2080,7 +2091,7 @@ struct Kernel {
             const float s = __fmul_rn(t, S.is_ctr[i]);
             if (!(s < 110.f)) continue;  // exp(-s) is 0 in 32 bits
             if (s < 1e-9f) {
-              acc = __fadd_rn(acc, A[0]);
+              add(A[0]);
               continue;
             }
             float z[kIsMom];
@@ -2088,7 +2099,7 @@ struct Kernel {
             float m = 0.f;
 #pragma unroll
             for (int k = kIsMom - 1; k >= 0; --k) m = __fmaf_rn(A[k], z[k], m);
-            acc = __fadd_rn(acc, m);
+            add(m);
           }
           isW[r * kIsNodesMax + n] = acc;   // M_r(t_n) for now
         }
@@ -2124,7 +2135,7 @@ struct Kernel {
       if (!S.is_cnt[r]) continue;
       const float* W = isW + r * kIsNodesMax;
       for (int n = warp; n < S.is_nb; n += kWarps) {
-        const float ctr = is_centre(S.is_b0 + n);
+        const float ctr = is_centre(r, S.is_b0[r] + n);
         float g[kIsMom];
 #pragma unroll
         for (int k = 0; k < kIsMom; ++k) g[k] = 0.f;
@@ -2166,17 +2177,20 @@ struct Kernel {
     }
     return sum;
   }
-  // The same by a whole warp, the nodes dealt to its lanes.
+  // The same by a whole warp, the nodes dealt to its lanes (a few terms a
+  // lane, added in 64 bits).
   __device__ float is_ratio_warp(const float* rho_r) const {
-    float sum = 0.f;
+    double sum = 0.0;
     for (int r = 1; r < S.nrows; ++r) {
       if (!S.is_cnt[r]) continue;
       const float rl = __fmul_rn(rho_r[r], -kLog2e);
       const float* W = isW + r * kIsNodesMax;
       for (int n = (int)(threadIdx.x & 31); n < S.is_n; n += 32)
-        sum = __fmaf_rn(W[n], ex2(__fmul_rn(isT[n], rl)), sum);
+        sum += (double)W[n] * (double)ex2(__fmul_rn(isT[n], rl));
     }
-    return warp_sum(sum);
+#pragma unroll
+    for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    return (float)sum;
   }
 
   // ---------------------------------------------------------------- importance steps
@@ -2725,13 +2739,12 @@ struct Kernel {
         const float* tab = isBin + (size_t)row * S.is_nb * kIsMom;
         ++row;
         const RowC c0 = row_c(0), cr = row_c(rr);
-        const float lz = S.is_lz[rr];
 #pragma unroll
         for (int e = 0; e < VE; ++e) {
           if (!(cr.prob(lp[e]) > 0.f) || !(q[e] > 0.f)) continue;
-          const float x = is_pos(c0.arg(lq[e]), cr.arg(lp[e]), lz);
+          const float x = is_pos(c0.arg(lq[e]), cr.arg(lp[e]));
           const float n = rintf(x);
-          const int bin = (int)n - S.is_b0;
+          const int bin = (int)n - S.is_b0[rr];
           if (bin < 0 || bin >= S.is_nb) {
             slow |= 1u << e;
             continue;
