@@ -205,6 +205,46 @@ struct Elt<MDS_BF16> {
   }
 };
 
+// Unit u (16 bytes from byte 16 u of `src` on) logit by logit; logits past n
+// read -inf.
+template <int DT>
+__device__ __forceinline__ uint4 load_logits(const char* src, int u, int n) {
+  constexpr int VE = Elt<DT>::VE;
+  uint32_t w[4];
+  if constexpr (DT == MDS_BF16) {
+    const unsigned short* s16 = reinterpret_cast<const unsigned short*>(src);
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const int t0 = u * VE + 2 * h;
+      const uint32_t a = (t0 < n) ? (uint32_t)__ldg(s16 + t0) : 0xff80u;
+      const uint32_t c = (t0 + 1 < n) ? (uint32_t)__ldg(s16 + t0 + 1) : 0xff80u;
+      w[h] = a | (c << 16);
+    }
+  } else {
+    const float* s32 = reinterpret_cast<const float*>(src);
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const int t0 = u * VE + h;
+      w[h] = (t0 < n) ? __float_as_uint(__ldg(s32 + t0)) : 0xff800000u;
+    }
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// The first and last units of a row that is not 16-byte aligned: out of line
+// for 16-bit logits, whose eight loads would stand beside every batched load.
+template <int DT>
+__device__ __noinline__ uint4 load_edge_call(const char* src, int u, int n) {
+  return load_logits<DT>(src, u, n);
+}
+template <int DT>
+__device__ __forceinline__ uint4 load_edge(const char* src, int u, int n) {
+  if constexpr (DT == MDS_BF16)
+    return load_edge_call<DT>(src, u, n);
+  else
+    return load_logits<DT>(src, u, n);
+}
+
 // Unit u (16 bytes from byte 16 u of `src` on) of a row that ends before
 // `end` and starts at `first`: where the row is not 16-byte aligned, the two
 // aligned 16-byte blocks that hold the unit, shifted together, if both lie
@@ -239,25 +279,7 @@ __device__ __forceinline__ uint4 load_unit(const char* src, const char* first, c
     return make_uint4(__funnelshift_r(w0, w1, bits), __funnelshift_r(w1, w2, bits), __funnelshift_r(w2, w3, bits),
                       __funnelshift_r(w3, w4, bits));
   }
-  uint32_t w[4];
-  if constexpr (DT == MDS_BF16) {
-    const unsigned short* s16 = reinterpret_cast<const unsigned short*>(src);
-#pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      const int t0 = u * VE + 2 * h;
-      const uint32_t a = (t0 < n) ? (uint32_t)__ldg(s16 + t0) : 0xff80u;
-      const uint32_t c = (t0 + 1 < n) ? (uint32_t)__ldg(s16 + t0 + 1) : 0xff80u;
-      w[h] = a | (c << 16);
-    }
-  } else {
-    const float* s32 = reinterpret_cast<const float*>(src);
-#pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      const int t0 = u * VE + h;
-      w[h] = (t0 < n) ? __float_as_uint(__ldg(s32 + t0)) : 0xff800000u;
-    }
-  }
-  return make_uint4(w[0], w[1], w[2], w[3]);
+  return load_edge<DT>(src, u, n);
 }
 
 // Probability of a logit under a row's statistics (row maximum M, scale

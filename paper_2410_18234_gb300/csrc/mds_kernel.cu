@@ -402,7 +402,12 @@ struct GlobalLoad {
   const char* const* gptr;
   int tok0, V, gu;
   bool aligned;
-  __device__ __forceinline__ uint4 raw(int r) const { return slice_unit<DT>(gptr[r], tok0, V, gu, aligned); }
+  __device__ __forceinline__ uint4 raw(int r) const {
+    if constexpr (DT == MDS_F32) {   // a unit by itself: four loads, without the shifts
+      if (!aligned) return dev::load_logits<DT>(gptr[r] + (size_t)tok0 * 4, gu, V - tok0);
+    }
+    return slice_unit<DT>(gptr[r], tok0, V, gu, aligned);
+  }
   __device__ __forceinline__ void operator()(int r, float* v) const { Elt<DT>::unpack(raw(r), v); }
 };
 
