@@ -477,13 +477,18 @@ struct Kernel {
   // what other warps wrote.
   //
   // stream_rows: NR rows known by the caller, straight into registers, D units
-  // of a thread in flight and the loop unrolled U times.  Two CTAs' warps keep up to
+  // of a thread in flight and the loop unrolled U times.  The buffer's shifts
+  // vanish by renaming only where U is a multiple of D; else a shift waits for
+  // the youngest load and one pass's loads are in flight, whatever D (cluster
+  // 1, B = 64, V = 151936 truncated alphabet: 4 units with U = 4 207 us, 2, 4 or
+  // 8 with U = 1 240).  Two CTAs' warps keep up to
   // 64 KB an SM in flight, which covers the memory's latency, and a unit costs
   // no copy, wait or shared-memory read (per-warp rings of bulk copies: 15
   // instructions a logit at one draft).  Before and after, us a call: sequential
   // rejection at B = 1024, K = 4, V = 151936 1241 and 931, with two models at
-  // V = 50257 87 and 71, classical IS at V = 32000 197 and 176.  Heavy bodies
-  // (IS moments, several rows) take U = 1: one copy of their code.
+  // V = 50272 87 and 71, classical IS at V = 32000 197 and 176.  Heavy bodies
+  // (IS moments, several rows of sequential rejection) take U = 1: one copy of
+  // their code (B = 256, V = 128256 sequential rejection: 242 us, two copies 248).
   template <int D, int U, int NR, class FN>
   __device__ __forceinline__ void stream_rows(const int (&rows)[NR], FN&& fn) {
     constexpr int kStep = kThreads;
@@ -781,7 +786,7 @@ struct Kernel {
 #pragma unroll
     for (int r = 0; r < R; ++r) rows[r] = r0 + r;
     if constexpr (!CAND) stats_stream<R>(rows, m, sc, cr);
-    if constexpr (CAND) stream_rows<(R == 2 ? 3 : 2), 1>(rows, [&](int gu, bool valid, const auto& L) {
+    if constexpr (CAND) stream_rows<(R == 1 ? 4 : 2), (R == 1 ? 4 : 2)>(rows, [&](int gu, bool valid, const auto& L) {
       // row 0 first: its values decide which tokens are set aside
       float v0[VE];
       if (valid) {
@@ -2467,14 +2472,15 @@ struct Kernel {
     // replace: a draw over the tokens outside Omega_0 in proportion to q
     const float cut = S.o0_cut;
     const bool all0 = S.o0_all != 0;
+    const RowC c0 = row_c(0);
     float tot;
     int Z = sample_cdf(
-        [&](auto&& fn) { stream_rows<8, 4>({0}, fn); },
+        [&](auto&& fn) { stream_rows<4, 4>({0}, fn); },
         [&](int, const auto& L, float* r) {
           float v[VE];
           L(0, v);
 #pragma unroll
-          for (int e = 0; e < VE; ++e) r[e] = (all0 || v[e] > cut) ? 0.f : prob_of(v[e], S.M[0], S.c[0], S.invZ[0]);
+          for (int e = 0; e < VE; ++e) r[e] = (all0 || v[e] > cut) ? 0.f : c0.prob(v[e]);
         },
         draw_uniform(p.seed, b, j, kDrawOutside), &tot);
     if (Z < 0) {   // no target mass outside Omega_0
