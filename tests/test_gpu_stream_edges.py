@@ -34,8 +34,6 @@ def test_stream_edges(V, cluster, models, dtype):
         torch.cuda.synchronize()
         bits, _ = v.status()
         v.close()
-        if scheme == "WIS0" and bits == mds.MDS_ST_OMEGA0:
-            continue   # another Omega_0 than the exact cut: not compared here
         o_out, o_acc, recs = oracle_verify(*host_copy(w), scheme, 31, omega0=10)
         res = compare(out.cpu().numpy(), acc.cpu().numpy(), o_out, o_acc, recs, g_diag=diag.cpu().numpy(), scheme=scheme)
         check(res, scheme)
@@ -52,6 +50,7 @@ def test_single_draft_either_side_of_the_engine_rule(V, dtype):
     out, acc, diag = v.verify(w.target, w.draft_list(), w.model_ids, w.tokens, w.temps, "single", 31, diag=True)
     torch.cuda.synchronize()
     bits, _ = v.status()
+    assert (v.cluster_size > 0) == (V * w.target.element_size() <= 192 * 1024), v.cluster_size
     v.close()
     o_out, o_acc, recs = oracle_verify(*host_copy(w), "single", 31)
     res = compare(out.cpu().numpy(), acc.cpu().numpy(), o_out, o_acc, recs, g_diag=diag.cpu().numpy(), scheme="single")
