@@ -1,5 +1,5 @@
-// Device helpers of the slice-dataflow engine (mds_flow.cu) and the top-k
-// kernel (mds_topk.cu): inline PTX wrappers, the counter-based random
+// Device helpers of the three kernels (mds_flow.cu, mds_kernel.cu,
+// mds_topk.cu): inline PTX wrappers, the counter-based random
 // numbers, logit IO, the exponent convention of every probability, and the
 // stage maximum flow of the weighted scheme.  Not part of the public ABI.
 #pragma once
@@ -102,13 +102,6 @@ struct Elt;
 template <>
 struct Elt<MDS_F32> {
   static constexpr int VE = 4;  // logits per 16-byte unit
-  __device__ static __forceinline__ void unit(const char* row, int u, float* v) {
-    const float4 x = *reinterpret_cast<const float4*>(row + 16 * u);
-    v[0] = x.x;
-    v[1] = x.y;
-    v[2] = x.z;
-    v[3] = x.w;
-  }
   __device__ static __forceinline__ float global(const char* row, int x) {
     return __ldg(reinterpret_cast<const float*>(row) + x);
   }
@@ -150,10 +143,6 @@ struct Elt<MDS_F32> {
 template <>
 struct Elt<MDS_BF16> {
   static constexpr int VE = 8;
-  __device__ static __forceinline__ void unit(const char* row, int u, float* v) {
-    const uint4 x = *reinterpret_cast<const uint4*>(row + 16 * u);
-    unpack(x, v);
-  }
   __device__ static __forceinline__ float global(const char* row, int x) {
     return __uint_as_float((uint32_t)__ldg(reinterpret_cast<const unsigned short*>(row) + x) << 16);
   }

@@ -113,7 +113,7 @@ enum : int {
   kPhListC,             // list tasks: ranking and the record
   kPhPublish,           // a task's record publication (fence, pass counter)
   kPhCombine,           // (unused)
-  kPhLp,                // the stage LPs (one thread)
+  kPhLp,                // the stage LPs
   kPhLpCalls,           // count: stage LPs
   kPhTasks,             // count: slice tasks
   kPhDecisions,         // count: decisions
@@ -210,16 +210,14 @@ struct DState {                // the decision's working state (shared memory)
   int tok;
   // truncated alphabet
   int k_lane[MDS_MAX_K], k_row[MDS_MAX_K];
-  int o0_n, o0_all, o0_Yp;
+  int o0_n, o0_all;
   // inputs of the sequence staged by the decision: draft tokens at the
   // depth (tk0) and the next depth (tk1), temperatures (target, drafts)
   int tk0[MDS_MAX_K], tk1[MDS_MAX_K];
   float tmp[MDS_MAX_K + 1];
   float dr[kDrawsN];           // the depth's uniforms, by kDr*
   int xl_wait;                 // the row logits at the draft tokens are still in flight
-  float o0_cut, o0_pa, o0_R;
-  float rtot;
-  unsigned tbase;
+  float o0_cut, o0_pa;
 };
 static_assert(offsetof(DState, W) == offsetof(DState, P) + sizeof(FPass) && offsetof(FSeq, W) == sizeof(FPass),
               "a sequence's state copies into the decision state in one piece");
@@ -2200,7 +2198,7 @@ struct Dec {
         if (take) {
           D.cm_id[pos] = __float_as_int(e[0]);
           D.cm_l0[pos] = e[LN];
-          } else {
+        } else {
           tau = fmaxf(tau, e[LN]);
         }
 #pragma unroll
@@ -2944,10 +2942,6 @@ struct Dec {
     finish(b, p.L);
   }
   // -------------------------------------------------------------- truncated alphabet
-  // Warp-wide inverse CDF over one weight per lane (lane order = token-id
-  // order of the list): the smallest lane whose running sum exceeds
-  // u * total, the last lane with positive weight if rounding leaves none,
-  // -1 if the total is not positive.
   // Inverse CDF over the list entries in token order, two per lane (entry
   // lane and 32 + lane; weights w0, w1): the first entry whose running sum
   // exceeds u01 * total, else the last with positive weight; -1 when the
@@ -3471,9 +3465,15 @@ void carve_workspace(Params& p, char* w, int nseq, int grid) {
 }
 
 // SMs whose CTAs run the decisions, at least one and never all of them: a
-// tenth of the grid's SMs for the weighted schemes, half that for single,
-// whose decisions are short.  The environment variable MDS_DEC_SMS overrides
-// the count (read once per process), for tuning.
+// twentieth of the grid's SMs for single, whose decisions are short, a tenth
+// for WIS, a seventh for WIS0, which streams one row only per decision.  By
+// scheme alone, set at B = 256, K = 8, V = 128256 and B = 1024, V = 151936
+// (us a call on 152 SMs): single 4 SMs 655, 8 439, 12 451, 18 466; WIS 8 272,
+// 12 226, 15 219, 22 222; WIS0 12 197, 15 181, 18 161, 22 162.  Batches of 64 to
+// 300 at V = 50272 to 151936 move by 2% from 8 SMs on.  Many sequences of short
+// rows want more: B = 1024, V = 32000 WIS 15 SMs 341, 28 229, WIS0 22 221, 28
+// 193.  The environment variable MDS_DEC_SMS overrides the count (read once
+// per process), for tuning.
 int decision_sms(int grid, int scheme) {
   static const int env = [] {
     const char* e = getenv("MDS_DEC_SMS");
@@ -3554,8 +3554,7 @@ bool plan_geometry(Params& p, int grid) {
     const int runs = (T * es / 16 + 31) / 32;
     if (rf < 4 + runs) rf = 4 + runs;
     p.rec_floats = (rf + 3) & ~3;
-    p.hdr_floats = kHdr;
-    if ((size_t)ns * p.rec_floats * 4 <= (size_t)kDecStage && ns * p.lns <= kMaxEntries) break;
+      if ((size_t)ns * p.rec_floats * 4 <= (size_t)kDecStage && ns * p.lns <= kMaxEntries) break;
   }
   // Warp-wise candidate lists where every thread has a unit and the slice's
   // list is short.  Each warp's bound is one that as many of its tokens reach
@@ -3573,7 +3572,12 @@ bool plan_geometry(Params& p, int grid) {
 // word, descriptor: about 2 us) are shared by a group of slices where there
 // are many tasks per CTA; one slice a task where a pass's slices should
 // spread over the GPU.  By the call's own batch: by the context's largest, a
-// small call's slices went to a few CTAs one after the other.
+// small call's slices went to a few CTAs one after the other.  Later passes
+// and depth 0, us a call at 64, 19, 13, 13 and 3 slices a CTA: single B = 1024,
+// V = 151936 1/1 491, 1/4 480, 2/4 436, 4/4 439; B = 300 1/1 164, 1/4 155, 2/4
+// 158, 4/8 164; WIS B = 256, V = 128256 1/1 214, 1/4 218, 2/4 225, 4/4 235; two
+// models B = 128, V = 50272 1/1 150, 1/4 156, 2/4 162, 4/4 178; B = 64,
+// V = 128256 1/1 146, 1/2 144, 2/2 154, 4/4 166.
 void plan_tasks(Params& p, int grid, int B) {
   const long per_cta = (long)B * p.ns / grid;
   p.group = per_cta >= 32 ? 4 : (per_cta >= 16 ? 2 : 1);

@@ -62,7 +62,6 @@ struct Params {
   int group, group0;                   // slices per task (group0: of the depth-0 passes)
   int ng, ng0;                         // tasks per pass
   int rec_floats;                      // record stride per slice
-  int hdr_floats;                      // start of a record's list entries
   int ring_cap;
   int dec_cap;
   int dec_sms;                         // SMs (ids 0..dec_sms-1) whose CTAs run the decisions
@@ -72,7 +71,7 @@ struct Params {
   int8_t model_of[MDS_MAX_K];
 };
 
-// Geometry of one call: fills T, ns, ln, rec_floats, hdr_floats.  Returns
+// Geometry of one call: fills T, ns, ln, rec_floats and the tasks.  Returns
 // false if the configuration is outside what this engine serves (the caller
 // then uses the per-sequence engine).
 bool plan_geometry(Params& p, int grid);

@@ -26,7 +26,6 @@
 // control flow stays uniform and the cluster barriers always match.  No CTA
 // waits on another CTA's flag.
 #include <cuda_bf16.h>
-#include <cooperative_groups.h>
 
 #include "mds_device.cuh"
 #include "mds_internal.h"
@@ -34,12 +33,10 @@
 namespace mds {
 namespace {
 
-constexpr float kLog2e = 1.4426950408889634f;
-constexpr float kNegInf = -__builtin_huge_valf();
-constexpr float kPosInf = __builtin_huge_valf();
+using namespace mds::dev;
+
 constexpr int kWarps = kThreads / 32;
 constexpr int kTop = 8;                 // per-thread candidate list length (>= MDS_MAX_S)
-constexpr int kMaxPairs = MDS_MAX_S * (MDS_MAX_S - 1) / 2;
 constexpr int kFastRows = 4;            // WIS candidate path: target + up to 3 draft models
 constexpr int kWarpApp = 64;            // candidate tokens one warp can hold during the stats pass
 constexpr int kIsSub = 4;               // IS: bins of log2 rho per octave
@@ -50,23 +47,8 @@ constexpr int kIsBinBytes = kThreads / 32 * kIsWin * 4 * kIsMom * 4;   // four c
 constexpr int kIsTabBins = kIsBinBytes / (kIsMom * 4);                 // bins of all rows the residual's table holds
 constexpr int kSampleStride = 4;        // the candidate filter's starting threshold samples 1 unit in 4
 
-// Order-preserving map of floats (not NaN) to unsigned; every key is > 0.
-__device__ __forceinline__ unsigned ord_key(float f) {
-  const unsigned u = __float_as_uint(f);
-  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-__device__ __forceinline__ float ord_val(unsigned k) {
-  return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
-}
-
 // ------------------------------------------------------------------ PTX helpers
 
-__device__ __forceinline__ float ex2(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -87,113 +69,6 @@ __device__ __forceinline__ float ld_dsmem(const float* local, uint32_t rank) {
 }
 __device__ __forceinline__ void st_dsmem(int* local, uint32_t rank, int v) {
   asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(dsmem_addr(local, rank)), "r"(v) : "memory");
-}
-// ---------------------------------------------------------------- Philox4x32-10
-// Salmon, Moraes, Dror, Shaw, SC'11: ten rounds of two 32x32->64 products,
-// round keys bumped by the Weyl constants.  Returns output word 0.
-__device__ __forceinline__ uint32_t philox_w0(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, uint32_t k0,
-                                              uint32_t k1) {
-#pragma unroll
-  for (int r = 0; r < 10; ++r) {
-    if (r) {
-      k0 += 0x9E3779B9u;
-      k1 += 0xBB67AE85u;
-    }
-    const uint32_t hi0 = __umulhi(0xD2511F53u, c0), lo0 = 0xD2511F53u * c0;
-    const uint32_t hi1 = __umulhi(0xCD9E8D57u, c2), lo1 = 0xCD9E8D57u * c2;
-    const uint32_t n0 = hi1 ^ c1 ^ k0, n2 = hi0 ^ c3 ^ k1;
-    c0 = n0;
-    c1 = lo1;
-    c2 = n2;
-    c3 = lo0;
-  }
-  return c0;
-}
-__device__ __forceinline__ float draw_uniform(unsigned long long seed, int b, int j, int draw) {
-  const uint32_t w = philox_w0((uint32_t)b, (uint32_t)j, (uint32_t)draw, 0u, (uint32_t)seed, (uint32_t)(seed >> 32));
-  return (float)(w >> 8) * 0x1p-24f;
-}
-constexpr int kDrawSelect = 0, kDrawAccept = 16, kDrawResidual = 32, kDrawBonus = 33;
-constexpr int kDrawKeep = 34, kDrawOutside = 35;   // truncated alphabet: keep Y', replace it
-
-// ------------------------------------------------------------------ element IO
-
-template <int DT>
-struct Elt;
-template <>
-struct Elt<MDS_F32> {
-  static constexpr int VE = 4;  // logits per 16-byte unit
-  __device__ static __forceinline__ void unit(const char* row, int u, float* v) {
-    const float4 x = *reinterpret_cast<const float4*>(row + 16 * u);
-    v[0] = x.x;
-    v[1] = x.y;
-    v[2] = x.z;
-    v[3] = x.w;
-  }
-  __device__ static __forceinline__ float global(const char* row, int x) {
-    return __ldg(reinterpret_cast<const float*>(row) + x);
-  }
-  __device__ static __forceinline__ void unit_global(const char* at, float* v) {
-    const float4 x = __ldg(reinterpret_cast<const float4*>(at));
-    v[0] = x.x;
-    v[1] = x.y;
-    v[2] = x.z;
-    v[3] = x.w;
-  }
-  __device__ static __forceinline__ void unpack(const uint4& x, float* v) {
-    v[0] = __uint_as_float(x.x);
-    v[1] = __uint_as_float(x.y);
-    v[2] = __uint_as_float(x.z);
-    v[3] = __uint_as_float(x.w);
-  }
-};
-template <>
-struct Elt<MDS_BF16> {
-  static constexpr int VE = 8;
-  __device__ static __forceinline__ void unit(const char* row, int u, float* v) {
-    const uint4 x = *reinterpret_cast<const uint4*>(row + 16 * u);
-    v[0] = __uint_as_float(x.x << 16);
-    v[1] = __uint_as_float(x.x & 0xffff0000u);
-    v[2] = __uint_as_float(x.y << 16);
-    v[3] = __uint_as_float(x.y & 0xffff0000u);
-    v[4] = __uint_as_float(x.z << 16);
-    v[5] = __uint_as_float(x.z & 0xffff0000u);
-    v[6] = __uint_as_float(x.w << 16);
-    v[7] = __uint_as_float(x.w & 0xffff0000u);
-  }
-  __device__ static __forceinline__ float global(const char* row, int x) {
-    return __uint_as_float((uint32_t)__ldg(reinterpret_cast<const unsigned short*>(row) + x) << 16);
-  }
-  __device__ static __forceinline__ void unpack(const uint4& x, float* v) {
-    v[0] = __uint_as_float(x.x << 16);
-    v[1] = __uint_as_float(x.x & 0xffff0000u);
-    v[2] = __uint_as_float(x.y << 16);
-    v[3] = __uint_as_float(x.y & 0xffff0000u);
-    v[4] = __uint_as_float(x.z << 16);
-    v[5] = __uint_as_float(x.z & 0xffff0000u);
-    v[6] = __uint_as_float(x.w << 16);
-    v[7] = __uint_as_float(x.w & 0xffff0000u);
-  }
-  __device__ static __forceinline__ void unit_global(const char* at, float* v) {
-    const uint4 x = __ldg(reinterpret_cast<const uint4*>(at));
-    v[0] = __uint_as_float(x.x << 16);
-    v[1] = __uint_as_float(x.x & 0xffff0000u);
-    v[2] = __uint_as_float(x.y << 16);
-    v[3] = __uint_as_float(x.y & 0xffff0000u);
-    v[4] = __uint_as_float(x.z << 16);
-    v[5] = __uint_as_float(x.z & 0xffff0000u);
-    v[6] = __uint_as_float(x.w << 16);
-    v[7] = __uint_as_float(x.w & 0xffff0000u);
-  }
-};
-
-// Probability of a logit under a row's statistics.  The same expression is
-// used for in-pass values and point lookups so both give identical bits.
-// Exponents: a term is 2^fma(l, c, -round(M c)) (one rounding, l c exact
-// inside the FMA); a partial sum moves from reference m to M by the factor
-// 2^(round(m c) - round(M c)), so every term of a row shares one reference.
-__device__ __forceinline__ float prob_of(float l, float M, float c, float invZ) {
-  return __fmul_rn(ex2(__fmaf_rn(l, c, -__fmul_rn(M, c))), invZ);
 }
 
 // ------------------------------------------------------------------ shared state
@@ -268,23 +143,11 @@ struct State {
   int owner, seg;
   float run;
   int wapp[kWarps];          // tokens each warp set aside (may exceed kWarpApp: overflow)
-  float thr_cta;
 };
 
 // ------------------------------------------------------------------ reductions
 
-__device__ __forceinline__ void combine_ms(float& m, float& s, float m2, float s2, float c) {
-  const float M = fmaxf(m, m2);
-  const float a = dev::moved_sum(s, m, M, c), b = dev::moved_sum(s2, m2, M, c);
-  m = M;
-  s = __fadd_rn(a, b);
-}
 
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-  for (int o = 16; o; o >>= 1) v = __fadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
 
 // Every CTA contributes n floats (S.xch[buf][0..n)); afterwards S.gat[r*n+i]
 // holds CTA r's values.  One cluster barrier; the two halves of S.xch
