@@ -708,10 +708,10 @@ struct Eng {
   // With RUNS (the bonus row) the chunks' sums are kept too.  The publishing
   // warp merges the eight warps' results.
   //
-  // Bound by issue (4.5 instructions a logit) and by the loads' latency: two
-  // CTAs of eight independent warps an SM.  Against one pass by the whole
-  // block with five barriers and the publication in it (GB300, a 32 KB slice
-  // of two rows): with a list 17k -> 3.5k SM cycles, without 8k -> 2.7k.
+  // Against one pass by the whole block with five barriers and the publication
+  // in it (GB300, a 32 KB slice of two rows): with a list 17k -> 4k SM cycles,
+  // without 8k -> 2.7k; the publishing warp takes 4.5k beside it, and a CTA
+  // turns a slice over about every 5.5k.
   template <int R, bool LIST, bool RUNS>
   __device__ __forceinline__ void stats_fast(const FPass& P, int bi, int tok0, int n, Slot& T) {
     char* b = buf(bi);
