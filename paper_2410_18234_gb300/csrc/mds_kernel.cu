@@ -1709,7 +1709,7 @@ struct Kernel {
   // an instruction share an address, the bank of every lane is fixed and the
   // sums have a fixed order.  Eight warps x 32 bins x 4 copies take 32 KB
   // (two CTAs per SM); wider ranges of rho take further windows of 32 bins.
-  // What bounds it now is issue: about 3 instructions a token in the adds.
+  // The adds take about 3 instructions a token.
   // Measured (GB300): B = 64, K = 4, V = 32000 590 -> 197 us a call, B = 1024,
   // K = 4, V = 151936 22.1 -> 5.4 ms; p_I(Y) 3e-7 off 64 bits before and after.
 
